@@ -35,7 +35,7 @@ from . import binding as eb
 NEVER = 1 << 20
 LAYOUT_CANDIDATES = {
     "coeff_cw_min_width": (640, NEVER),
-    "sor_tma_min_per_sm": (2, 4, NEVER),
+    "sor_tma_min_per_sm": (1, 4, NEVER),
     "sor_row_waves": (0, 2),
     "var_cluster_max": (8, 16),
     "coeff_cw_rows": (4, 16),

@@ -125,6 +125,7 @@ struct ebof_stream {
         std::vector<char> h_call;
         // scratch sets 1 .. kFlows - 1 (set 0: the stream's own buffers)
         float *up[kFlows] = {}, *Ua[kFlows] = {}, *Ub[kFlows] = {}, *work[kFlows] = {};
+        CoefMaps cmaps[kFlows];  // tensor maps of work[f]
         int head = 0;            // slot of the newest window
         bool has_prev = false;   // the newest window is in these slots
         bool latest = false;     // these slots, not the ordinary ones, hold the newest window
@@ -295,10 +296,25 @@ cudaError_t dmalloc(T **ptr, size_t bytes)
     return cudaMalloc((void **)ptr, std::max<size_t>(bytes, 256));
 }
 
+// A dense flow buffer (Ua, Ub): it starts one element past its allocation, so
+// that the pixel pairs of the SOR regions, which begin on odd columns, are
+// aligned 8-byte pairs (rows and planes hold an even number of elements).
+cudaError_t flow_alloc(float **u, size_t floats)
+{
+    const cudaError_t e = dmalloc(u, sizeof(float) * (floats + 1));
+    if (e == cudaSuccess) ++*u;
+    return e;
+}
+
+void flow_free(float *u)
+{
+    cudaFree(u ? u - 1 : nullptr);
+}
+
 void free_all(ebof_stream *s)
 {
     cudaFree(s->E); cudaFree(s->Ed); cudaFree(s->Edf); cudaFree(s->g); cudaFree(s->pyr);
-    cudaFree(s->up); cudaFree(s->Ua); cudaFree(s->Ub); cudaFree(s->work);
+    cudaFree(s->up); flow_free(s->Ua); flow_free(s->Ub); cudaFree(s->work);
     cudaFree(s->dstats); cudaFree(s->d_dropped_time); cudaFree(s->d_err);
     cudaFree(s->flow_stage); cudaFree(s->ev_stage); cudaFree(s->d_call);
     for (int b = 0; b < 2; ++b)
@@ -333,8 +349,8 @@ void free_all(ebof_stream *s)
     cudaFree(L.call);
     for (int f = 0; f < ebof_stream::Pipeline::kFlows; ++f) {
         cudaFree(L.up[f]);
-        cudaFree(L.Ua[f]);
-        cudaFree(L.Ub[f]);
+        flow_free(L.Ua[f]);
+        flow_free(L.Ub[f]);
         cudaFree(L.work[f]);
     }
     if (L.front) cudaStreamDestroy(L.front);
@@ -680,10 +696,15 @@ void pipeline_release(ebof_stream *s)
         *b = nullptr;
     }
     for (int f = 0; f < kPipeFlows; ++f)
-        for (float **b : {&L.up[f], &L.Ua[f], &L.Ub[f], &L.work[f]}) {
+    {
+        flow_free(L.Ua[f]);
+        flow_free(L.Ub[f]);
+        L.Ua[f] = L.Ub[f] = nullptr;
+        for (float **b : {&L.up[f], &L.work[f]}) {
             cudaFree(*b);
             *b = nullptr;
         }
+    }
 }
 
 // Streams, events, slots, descriptor blocks and the extra scratch sets of
@@ -704,14 +725,15 @@ ebof_status pipeline_ready(ebof_stream *s)
          dmalloc(&L.call, kPipeSlots * kPipeCallBytes) == cudaSuccess;
     for (int f = 1; f < kPipeFlows && ok; ++f)
         ok = dmalloc(&L.up[f], sizeof(float) * s->up_fs) == cudaSuccess &&
-             dmalloc(&L.Ua[f], sizeof(float) * s->u_fs) == cudaSuccess &&
-             dmalloc(&L.Ub[f], sizeof(float) * s->u_fs) == cudaSuccess &&
+             flow_alloc(&L.Ua[f], s->u_fs) == cudaSuccess &&
+             flow_alloc(&L.Ub[f], s->u_fs) == cudaSuccess &&
              dmalloc(&L.work[f], sizeof(float) * s->work_fs) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         pipeline_release(s);
         return EBOF_ERR_OOM;
     }
+    for (int f = 1; f < kPipeFlows; ++f) make_coef_maps(L.work[f], s->geo, 1, &L.cmaps[f]);
     L.h_call.assign(kPipeSlots * kPipeCallBytes, 0);
     L.ready = true;
     return EBOF_OK;
@@ -781,7 +803,7 @@ ebof_status run_pipelined(ebof_stream *s, const uint16_t *x, const uint16_t *y, 
     // slot j's flow stream and scratch set (kSlots is a multiple of kFlows,
     // so consecutive windows take consecutive sets)
     const int f = j % kPipeFlows;
-    const FlowScratch setf = {L.up[f], L.Ua[f], L.Ub[f], L.work[f], nullptr};
+    const FlowScratch setf = {L.up[f], L.Ua[f], L.Ub[f], L.work[f], &L.cmaps[f]};
     const FlowScratch *sc = f ? &setf : nullptr;  // set 0: the stream's own buffers
     cudaStream_t fl = L.flow[f];
     if (graphs) {
@@ -847,7 +869,7 @@ void free_group(ebof_group *g)
     for (int b = 0; b < 2; ++b)
         if (g->graph[b]) cudaGraphExecDestroy(g->graph[b]);
     cudaFree(g->E); cudaFree(g->Ed); cudaFree(g->Edf); cudaFree(g->g); cudaFree(g->pyr);
-    cudaFree(g->up); cudaFree(g->Ua); cudaFree(g->Ub); cudaFree(g->work); cudaFree(g->flow);
+    cudaFree(g->up); flow_free(g->Ua); flow_free(g->Ub); cudaFree(g->work); cudaFree(g->flow);
     cudaFree(g->dstats); cudaFree(g->d_dropped_time); cudaFree(g->d_err); cudaFree(g->d_desc);
     delete[] g->h_events;
     if (g->cap) cudaStreamDestroy(g->cap);
@@ -1332,11 +1354,12 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
                 r.w = lv.w;
                 r.h = lv.h;
                 r.pitch = lv.pitch;
-                r.R = n_half > 0 ? n_half - 1 : 0;
+                r.R = sor_halo(p.var_sor);
                 r.n_half = n_half;
                 r.omega = fp.omega;
-                r.gx = (lv.w + sor_tile_x(r.R) - 1) / sor_tile_x(r.R);
-                r.gy = (lv.h + sor_tile_y(r.R) - 1) / sor_tile_y(r.R);
+                const int tile = sor_tile(r.R);
+                r.gx = (lv.w + tile - 1) / tile;
+                r.gy = (lv.h + tile - 1) / tile;
                 sor.push_back({r, r.gx * r.gy * v.x->g->n});
                 std::swap(v.a, v.b);
                 v.x->U = v.a;
@@ -1413,9 +1436,7 @@ void ebof_default_params(ebof_params *p, int32_t width, int32_t height)
     p->surface = EBOF_SURFACE_EXP;
     p->d_sat = 6.0f;
     p->coeff_cw_min_width = 1024;
-    // the copy-ahead SOR kernel: 1280 x 720 batches of 40 windows ran 3 %
-    // faster without it (same flow); 346 x 260 groups slightly faster with it
-    p->sor_tma_min_per_sm = width >= 1024 ? (1 << 20) : 4;
+    p->sor_tma_min_per_sm = 2;
     p->sor_row_waves = 1;
     // the cluster-resident refinement of small levels gives the same flow but
     // measured no faster inside a graph (1544 vs 1573 frames/s at 1280 x 720):
@@ -1461,8 +1482,8 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     s->es = p->storage == EBOF_STORAGE_FP16 ? 2 : 4;
     ok &= dmalloc(&s->pyr, s->es * s->pyr_fs * s->nslots) == cudaSuccess;
     ok &= dmalloc(&s->up, sizeof(float) * s->up_fs * B) == cudaSuccess;
-    ok &= dmalloc(&s->Ua, sizeof(float) * s->u_fs * B) == cudaSuccess;
-    ok &= dmalloc(&s->Ub, sizeof(float) * s->u_fs * B) == cudaSuccess;
+    ok &= flow_alloc(&s->Ua, s->u_fs * B) == cudaSuccess;
+    ok &= flow_alloc(&s->Ub, s->u_fs * B) == cudaSuccess;
     ok &= dmalloc(&s->work, sizeof(float) * s->work_fs * B) == cudaSuccess;
     ok &= dmalloc(&s->dstats, sizeof(DevStats) * B) == cudaSuccess;
     ok &= dmalloc(&s->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
@@ -1506,7 +1527,7 @@ int64_t ebof_stream_device_bytes(const ebof_params *p)
     auto r = [](size_t b) { return std::max<size_t>(b, 256); };
     size_t total = 3 * r(plane0 * B) + r(4 * plane0 * B) + r(es * geo.pyr_floats * (B + 1));
     total += r(4 * 2 * (size_t)std::max(geo.max_patches, 1) * B);
-    total += 2 * r(4 * 2 * plane0 * B) + r(4 * 9 * plane0 * B);
+    total += 2 * r(4 * (2 * plane0 * B + 1)) + r(4 * 9 * plane0 * B);
     total += r(sizeof(DevStats) * B) + 2 * 256 + r(4 * 2 * (size_t)p->width * p->height) +
              r((sizeof(ebof_window_desc) + sizeof(float *)) * B);
     return (int64_t)total;
@@ -1990,8 +2011,8 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     ok &= dmalloc(&g->g, sizeof(int32_t) * g->g_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->pyr, g->es * g->pyr_fs * n * 2) == cudaSuccess;
     ok &= dmalloc(&g->up, sizeof(float) * g->up_fs * n) == cudaSuccess;
-    ok &= dmalloc(&g->Ua, sizeof(float) * g->u_fs * n) == cudaSuccess;
-    ok &= dmalloc(&g->Ub, sizeof(float) * g->u_fs * n) == cudaSuccess;
+    ok &= flow_alloc(&g->Ua, g->u_fs * n) == cudaSuccess;
+    ok &= flow_alloc(&g->Ub, g->u_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->work, sizeof(float) * g->work_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->flow, sizeof(float) * 2 * (size_t)q.width * q.height * n) == cudaSuccess;
     ok &= dmalloc(&g->dstats, sizeof(DevStats) * n) == cudaSuccess;

@@ -155,7 +155,7 @@ void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_
 
 // Tensor maps (TMA descriptors) of the variational coefficient planes of
 // each pyramid level in a stream's or group's work buffer: level l holds
-// frames x 9 planes of pitch_l x h_l floats, frame stride 9 planes.
+// frames x coeff_planes() planes of pitch_l x h_l floats.
 struct CoefMaps {
     bool ok[kMaxLevels];
     CUtensorMap map[kMaxLevels];

@@ -6,34 +6,44 @@
 // of the warped image and the smoothness weights, and writes every pixel's
 // 2x2 linear system (data and gradient-constancy terms normalised, weights
 // lagged at dU = 0): omega/a11, omega/a22 (the SOR relaxation factor folded
-// into the inverted diagonal), a12, b1, b2 and the left and upper edge
-// weights, as seven planes (the right and lower weights are the neighbours'
-// left and upper ones).  Only the staging halo is shared between tiles.  On
-// levels from 1024 px wide the same systems come from var_coeff_cw_kernel,
-// a column walk with the rows in registers.
+// into the inverted diagonal), a12, b1, b2 and the smoothness weight, as six
+// planes.  Only the staging halo is shared between tiles.  On levels from
+// 1024 px wide the same systems come from var_coeff_cw_kernel, a column walk
+// with the rows in registers.
 //
-// var_sor_kernel: one block owns a 64x64 region and refines the flow of its
+// SOR: one block owns a 64x64 region and refines the flow of its
 // (64 - 2R)^2 interior, R = 2 * sweeps - 1.  It loads the region's linear
 // systems into registers and runs the red-black SOR sweeps there: a thread
 // owns a 2-column x 4-row strip, so one horizontal neighbour is its own and
-// the other is a lane shuffle away, and the rows at strip ends are exchanged
-// through shared memory once per half sweep.  (A 2 x 2 strip with 1024
-// threads, twice the resident warps, measured no faster.)  The region border keeps
+// the other is a lane shuffle away, and the pixels at strip ends are exchanged
+// through shared memory once per half sweep.  The region border keeps
 // du = 0; after h half sweeps only pixels within h - 1 px of that border
 // differ from the whole-image red-black iteration, and those lie in the
 // discarded halo, so the interior is exactly the whole-image iteration (up to
 // floating-point rounding).  It writes U + dU for its interior.
 //
-// var_sor_tma_kernel: the same sweeps in a persistent grid (one block per
-// SM) that walks over the regions, for grids of at least four regions per
-// SM.  One thread loads each region's coefficient planes into shared memory
-// with a single TMA tensor copy (cp.async.bulk.tensor, completion on an
-// mbarrier); once every thread has
-// moved its values into registers, the copy of the block's next region is
-// issued and runs during the sweeps.  The box starts at the region's first
-// column rounded down to a multiple of 4 (the 16-byte rule of tensor
-// copies) and is 4 columns wider; elements outside the level are filled
-// with zero, as the direct loads do, so both kernels give the same result.
+// What bounds it: the issue slots and the latency between the barriers of the
+// half sweeps (four warps a scheduler; the register file holds no more), and
+// the L2 bandwidth of the planes, read 1.93 times for the halo.  So (u, v) are
+// updated as packed pairs, only the pixels just updated are exchanged, the
+// first half sweep (whose neighbours are 0) runs without an exchange, the edge
+// weights are rebuilt from one plane, regions begin on odd columns that every
+// buffer aligns to 8 bytes, and the interior's flow is fetched behind the
+// sweeps.  Measured per 1280x720 launch on a GB300, inside a graph, against
+// the scalar form of 7 planes and a full exchange: 18.3 -> 15.6 us for one
+// frame, 165 -> 126 us for eight.
+//
+// var_sor_tma_kernel: the same regions in a persistent grid (one block per
+// SM).  One thread loads each region's planes into shared memory with a
+// single TMA tensor copy (cp.async.bulk.tensor, completion on an mbarrier);
+// once every thread has moved its values into registers, the copy of the
+// block's next region is issued and runs during the sweeps.  The box starts at
+// the region's first column rounded down to the 16-byte rule of tensor copies
+// and is 4 columns wider; elements outside the level are filled with zero, as
+// the direct loads do, so both kernels give the same result.  It needs at
+// least two regions an SM to hide a copy: measured against the direct form (in
+// a graph, 7 planes) 6.8 vs 6.1 us for 112 regions, 10.4 vs 9.8 for 154, 14.7
+// vs 15.6 for 448, 27.0 vs 30.4 for 896, 101 vs 126 for 3584.
 #include "dev_common.cuh"
 #include "ebof_internal.cuh"
 #include "profiler.cuh"
@@ -50,17 +60,32 @@ constexpr int kVR = 64;                  // region side
 constexpr int kVS = 4;                   // rows per thread strip
 constexpr int kVWarps = kVR / kVS;       // warps per block (stacked strips)
 constexpr int kVThreads = 32 * kVWarps;  // 512
-constexpr size_t kVSmemFloats = 2 * 2 * kVWarps * 2 * 64;  // strip-end exchange
-constexpr size_t kVSmemFloats2 = 2 * 2 * 32 * 2 * 64;       // the same for 32 warps
+constexpr int kVSmallRows = 32;          // region rows of the small form
+constexpr int kVSmallVS = 2;             // and its rows per strip
+static_assert(kVSmallRows / kVSmallVS == kVWarps, "both forms run 16 warps");
 // Coefficient planes of a pixel's system: omega/a11, omega/a22, a12, b1, b2
-// and the left and upper edge weights.  The right and lower weights of a pixel are
-// the left and upper ones of its neighbours (each the mean of the same two
-// smoothness weights, so equal bit for bit) and are not stored.
-enum { kCI11 = 0, kCI22, kCA12, kCB1, kCB2, kCWL, kCWU, kCPlanes };
+// and the smoothness weight.  An edge's weight is the mean of its two pixels'
+// smoothness weights, one sum and one product that the sweeps' kernels do
+// themselves: one plane instead of the left and upper edge weights' two, a
+// seventh of the bytes they load.
+//
+// The planes are stored one element to the right of their base, column x at
+// x + 1: a region starts on an odd column (its halo is odd, its interior
+// even), so a lane's two columns are then one aligned 8-byte pair.  The flow
+// buffers are offset the same way by their owner.
+enum { kCI11 = 0, kCI22, kCA12, kCB1, kCB2, kCAS, kCPlanes };
+constexpr int kCoefShift = 1;
 
 constexpr int kTmaBoxW = kVR + 4;  // region columns + the rounding of the box start
 constexpr size_t kTmaCoefFloats = (size_t)kCPlanes * kVR * kTmaBoxW;
-constexpr size_t kTmaSmemBytes = (kTmaCoefFloats + kVSmemFloats) * sizeof(float);
+// the interior's flow, staged while the sweeps run: (u, v) pairs of a strip's rows
+template <int VS, int WARPS>
+constexpr size_t flow_stage_bytes()
+{
+    return (size_t)VS * 2 * WARPS * 32 * sizeof(float2);
+}
+constexpr size_t kTmaSmemBytes =
+    kTmaCoefFloats * sizeof(float) + flow_stage_bytes<kVS, kVWarps>();
 constexpr int kMaxDevs = 64;
 int g_num_sms[kMaxDevs];
 // coefficient tile: 384 threads at 40 registers, four blocks per SM, so a
@@ -91,117 +116,178 @@ __device__ __forceinline__ float2 ldf2(const float *p)
 }
 
 
-// One red-black half sweep of colour C on a thread's 2-column x VS-row
-// strip; P is the parity of (x + y) at the strip's first pixel.  Pixel
-// (row r, column q) has colour (P + r + q) & 1.  The strip's first and last
-// rows are read by the warps above and below from xch (double-buffered by
-// half sweep, so one barrier per half sweep suffices).  WARPS strips are
-// stacked in a block.
-template <int VS, int WARPS, int P, int C>
-__device__ __forceinline__ void sor_half(float (&du)[VS][2], float (&dv)[VS][2],
-                                         const float (&i11)[VS][2], const float (&i22)[VS][2],
-                                         const float (&a12)[VS][2], const float (&b1)[VS][2],
-                                         const float (&b2)[VS][2], const float (&wl)[VS][2],
-                                         const float (&wr)[VS][2], const float (&wu)[VS][2],
-                                         const float (&wd)[VS][2], const float *xtop,
-                                         const float *xbot, int lane, int wp, float omega)
+// (u, v) pairs in one 64-bit register: the packed FP32 instructions round each
+// half as the scalar ones do.  A packed multiply-add holds the FMA pipe as long
+// as two scalar ones (measured: 2.0 cycles a warp against 1.0), but takes one
+// issue slot: the sweeps are bound by issue, not by that pipe.
+typedef unsigned long long pair_t;
+__device__ __forceinline__ pair_t pk(float a, float b)
 {
-    const float om1 = 1.0f - omega;
+    pair_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 upk(pair_t v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ pair_t ffma2(pair_t a, pair_t b, pair_t c)
+{
+    pair_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ pair_t fmul2(pair_t a, pair_t b)
+{
+    pair_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// A thread's strip of 2 columns x VS rows: the pixels' systems, the weights of
+// their edges (right: of column 1 only, column 0's is column 1's left one;
+// down: of the last row only) and (du, dv).
+template <int VS>
+struct Strip {
+    float i11[VS][2], i22[VS][2], a12[VS][2];
+    pair_t b[VS][2];
+    float wl[VS][2], wr[VS], wu[VS][2], wd[2];
+    pair_t d[VS][2];
+};
+
+// Shared memory of the strip ends, double-buffered by half sweep.  Of a strip's
+// first and last row only the pixels just updated are published: a half sweep
+// reads the other colour.  top[.][k] is warp k's first row, bot[.][k + 1] its
+// last; the entries past either end stay 0.
+template <int WARPS>
+struct StripEnds {
+    pair_t top[2][WARPS + 1][32], bot[2][WARPS + 1][32];
+};
+template <int WARPS>
+__device__ __forceinline__ void clear_ends(StripEnds<WARPS> &x)
+{
+    const int t = threadIdx.x, lane = t & 31, k = (t >> 5) & 1;
+    if (t < 64) x.bot[k][0][lane] = 0;
+    else if (t < 128) x.top[k][WARPS][lane] = 0;
+}
+
+// One red-black half sweep: row r's pixel of column (Q + r) & 1.  up, dn: the
+// neighbours above the strip's first and below its last row.
+template <int VS, int Q>
+__device__ __forceinline__ void sor_half(Strip<VS> &s, pair_t up, pair_t dn, pair_t om1)
+{
 #pragma unroll
     for (int r = 0; r < VS; ++r) {
-        const int q = (C + P + r) & 1;  // compile-time after unrolling
+        const int q = (Q + r) & 1;  // compile-time after unrolling
         // lane 0's left and lane 31's right neighbours lie outside the
         // region: the shuffles return the lane's own (finite) values there,
-        // and the edge weights wl / wr of those pixels are 0
-        float lu, lv, ru, rv;
+        // and the weights of those edges are 0
+        pair_t l, rt;
         if (q == 0) {
-            lu = __shfl_up_sync(kFull, du[r][1], 1);
-            lv = __shfl_up_sync(kFull, dv[r][1], 1);
-            ru = du[r][1];
-            rv = dv[r][1];
+            const float2 n = upk(s.d[r][1]);
+            l = pk(__shfl_up_sync(kFull, n.x, 1), __shfl_up_sync(kFull, n.y, 1));
+            rt = s.d[r][1];
         } else {
-            ru = __shfl_down_sync(kFull, du[r][0], 1);
-            rv = __shfl_down_sync(kFull, dv[r][0], 1);
-            lu = du[r][0];
-            lv = dv[r][0];
+            const float2 n = upk(s.d[r][0]);
+            rt = pk(__shfl_down_sync(kFull, n.x, 1), __shfl_down_sync(kFull, n.y, 1));
+            l = s.d[r][0];
         }
-        const int col = q * 32 + lane;  // the exchange rows hold the q = 0 column first
-        float uu, uv, dnu, dnv;
-        if (r > 0) {
-            uu = du[r - 1][q];
-            uv = dv[r - 1][q];
-        } else {
-            uu = wp > 0 ? xbot[((wp - 1) * 2 + 0) * 64 + col] : 0.0f;
-            uv = wp > 0 ? xbot[((wp - 1) * 2 + 1) * 64 + col] : 0.0f;
-        }
-        if (r < VS - 1) {
-            dnu = du[r + 1][q];
-            dnv = dv[r + 1][q];
-        } else {
-            dnu = wp < WARPS - 1 ? xtop[((wp + 1) * 2 + 0) * 64 + col] : 0.0f;
-            dnv = wp < WARPS - 1 ? xtop[((wp + 1) * 2 + 1) * 64 + col] : 0.0f;
-        }
+        const pair_t u = r > 0 ? s.d[r > 0 ? r - 1 : 0][q] : up;
+        const pair_t d = r < VS - 1 ? s.d[r < VS - 1 ? r + 1 : r][q] : dn;
+        const float wl = s.wl[r][q], wr = q == 0 ? s.wl[r][1] : s.wr[r];
+        const float wu = s.wu[r][q], wd = r < VS - 1 ? s.wu[r < VS - 1 ? r + 1 : r][q] : s.wd[q];
         // i11 = omega / a11, i22 = omega / a22; fixed rounding order (every
         // SOR layout gives the same values)
-        float tu = ffma(wl[r][q], lu, b1[r][q]);
-        tu = ffma(wr[r][q], ru, tu);
-        tu = ffma(wu[r][q], uu, tu);
-        tu = ffma(wd[r][q], dnu, tu);
-        tu = ffma(-a12[r][q], dv[r][q], tu);
-        const float nu = ffma(tu, i11[r][q], fmul(om1, du[r][q]));
-        float tv = ffma(wl[r][q], lv, b2[r][q]);
-        tv = ffma(wr[r][q], rv, tv);
-        tv = ffma(wu[r][q], uv, tv);
-        tv = ffma(wd[r][q], dnv, tv);
-        tv = ffma(-a12[r][q], nu, tv);
-        const float nv = ffma(tv, i22[r][q], fmul(om1, dv[r][q]));
-        du[r][q] = nu;
-        dv[r][q] = nv;
+        pair_t t = ffma2(pk(wl, wl), l, s.b[r][q]);
+        t = ffma2(pk(wr, wr), rt, t);
+        t = ffma2(pk(wu, wu), u, t);
+        t = ffma2(pk(wd, wd), d, t);
+        const float2 tt = upk(t), own = upk(s.d[r][q]), o = upk(fmul2(om1, s.d[r][q]));
+        const float nu = ffma(ffma(-s.a12[r][q], own.y, tt.x), s.i11[r][q], o.x);
+        const float nv = ffma(ffma(-s.a12[r][q], nu, tt.y), s.i22[r][q], o.y);
+        s.d[r][q] = pk(nu, nv);
     }
 }
 
-// n_half half sweeps, red first.  pw = parity of (x + y) at this warp's
-// strip start (block-uniform when VS is even, alternating per warp when VS
-// is odd); the branch on it is warp-uniform and every barrier is outside it.
-template <int VS, int WARPS>
-__device__ __forceinline__ void sor_sweeps(float (&du)[VS][2], float (&dv)[VS][2],
-                                           const float (&i11)[VS][2], const float (&i22)[VS][2],
-                                           const float (&a12)[VS][2], const float (&b1)[VS][2],
-                                           const float (&b2)[VS][2], const float (&wl)[VS][2],
-                                           const float (&wr)[VS][2], const float (&wu)[VS][2],
-                                           const float (&wd)[VS][2], float *xch, int lane, int wp,
-                                           int pw, int n_half, float omega)
+// Publishes the pixels that the last half sweep updated (row r's of column
+// (Q + r) & 1) at the strip's ends, waits for the block, and reads the
+// neighbours' of the next half sweep.
+template <int VS, int WARPS, int Q>
+__device__ __forceinline__ void swap_ends(const Strip<VS> &s, StripEnds<WARPS> &x, int buf,
+                                          int lane, int wp, pair_t &up, pair_t &dn)
 {
-    for (int hs = 0; hs < n_half; ++hs) {
-        // exchange buffer of this half sweep: [top|bottom][warp][du|dv][q][lane]
-        // (a lane's two columns 32 floats apart: conflict-free accesses)
-        float *xb = xch + (hs & 1) * (2 * WARPS * 2 * 64);
-        float *xtop = xb, *xbot = xb + WARPS * 2 * 64;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            xtop[(wp * 2 + 0) * 64 + q * 32 + lane] = du[0][q];
-            xtop[(wp * 2 + 1) * 64 + q * 32 + lane] = dv[0][q];
-            xbot[(wp * 2 + 0) * 64 + q * 32 + lane] = du[VS - 1][q];
-            xbot[(wp * 2 + 1) * 64 + q * 32 + lane] = dv[VS - 1][q];
-        }
-        __syncthreads();
-        if (pw == 0) {
-            if ((hs & 1) == 0)
-                sor_half<VS, WARPS, 0, 0>(du, dv, i11, i22, a12, b1, b2, wl, wr, wu, wd, xtop,
-                                          xbot, lane, wp, omega);
-            else
-                sor_half<VS, WARPS, 0, 1>(du, dv, i11, i22, a12, b1, b2, wl, wr, wu, wd, xtop,
-                                          xbot, lane, wp, omega);
-        } else {
-            if ((hs & 1) == 0)
-                sor_half<VS, WARPS, 1, 0>(du, dv, i11, i22, a12, b1, b2, wl, wr, wu, wd, xtop,
-                                          xbot, lane, wp, omega);
-            else
-                sor_half<VS, WARPS, 1, 1>(du, dv, i11, i22, a12, b1, b2, wl, wr, wu, wd, xtop,
-                                          xbot, lane, wp, omega);
+    x.top[buf][wp][lane] = s.d[0][Q];
+    x.bot[buf][wp + 1][lane] = s.d[VS - 1][(Q + VS - 1) & 1];
+    __syncthreads();
+    up = x.bot[buf][wp][lane];
+    dn = x.top[buf][wp + 1][lane];
+}
+
+// n_half half sweeps from dU = 0; P: the column of the red pixel in the strip's
+// first row.  The first one has no neighbour to read, so n_half - 1 barriers.
+template <int VS, int WARPS, int P>
+__device__ __forceinline__ void sor_sweeps_p(Strip<VS> &s, StripEnds<WARPS> &x, int lane, int wp,
+                                             int n_half, pair_t om1)
+{
+    if (n_half <= 0) return;
+    sor_half<VS, P>(s, 0, 0, om1);
+    pair_t up, dn;
+#pragma unroll 1
+    for (int hs = 1; hs < n_half; hs += 2) {
+        swap_ends<VS, WARPS, P>(s, x, 0, lane, wp, up, dn);
+        sor_half<VS, 1 - P>(s, up, dn, om1);
+        if (hs + 1 < n_half) {
+            swap_ends<VS, WARPS, 1 - P>(s, x, 1, lane, wp, up, dn);
+            sor_half<VS, P>(s, up, dn, om1);
         }
     }
-    __syncthreads();
+}
+
+// par: parity of (x + y) at the strip's first pixel, the same in every warp
+// (VS is even).
+template <int VS, int WARPS>
+__device__ __forceinline__ void sor_sweeps(Strip<VS> &s, StripEnds<WARPS> &x, int lane, int wp,
+                                           int par, int n_half, float omega)
+{
+    static_assert((VS & 1) == 0, "one parity per block");
+    const float o = 1.0f - omega;
+    const pair_t om1 = pk(o, o);
+#pragma unroll
+    for (int r = 0; r < VS; ++r) s.d[r][0] = s.d[r][1] = 0;
+    if (par == 0)
+        sor_sweeps_p<VS, WARPS, 0>(s, x, lane, wp, n_half, om1);
+    else
+        sor_sweeps_p<VS, WARPS, 1>(s, x, lane, wp, n_half, om1);
+}
+
+// The strip's edge weights from the smoothness weights of its rows and of the
+// rows above and below it (as[0], as[VS + 1]); (gx, gy): its first pixel.  An
+// edge that leaves the level (not INSIDE) or the region has weight 0; past the
+// region's ends lie pixels whose dU stays 0.
+template <int VS, bool INSIDE>
+__device__ __forceinline__ void edge_weights(Strip<VS> &s, const float (&as)[VS + 2][2], int lane,
+                                             bool first, bool last, int gx, int gy, int w, int h)
+{
+    auto mean = [](float a, float b) { return fmul(0.5f, fadd(a, b)); };
+    const bool x0 = lane > 0 && (INSIDE || (gx > 0 && gx < w));
+    const bool x1 = INSIDE || (gx >= 0 && gx + 1 < w);
+    const bool x2 = lane < 31 && (INSIDE || (gx + 1 >= 0 && gx + 2 < w));
+#pragma unroll
+    for (int r = 0; r < VS; ++r) {
+        const float l = __shfl_up_sync(kFull, as[r + 1][1], 1);
+        const float n = __shfl_down_sync(kFull, as[r + 1][0], 1);
+        s.wl[r][0] = x0 ? mean(as[r + 1][0], l) : 0.0f;
+        s.wl[r][1] = x1 ? mean(as[r + 1][1], as[r + 1][0]) : 0.0f;
+        s.wr[r] = x2 ? mean(as[r + 1][1], n) : 0.0f;
+        const bool yu = !(r == 0 && first) && (INSIDE || (gy + r > 0 && gy + r < h));
+#pragma unroll
+        for (int q = 0; q < 2; ++q) s.wu[r][q] = yu ? mean(as[r + 1][q], as[r][q]) : 0.0f;
+    }
+    const bool yd = !last && (INSIDE || (gy + VS > 0 && gy + VS < h));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) s.wd[q] = yd ? mean(as[VS + 1][q], as[VS][q]) : 0.0f;
 }
 
 // Smoothness weight alpha_s Psi'(|grad u|^2 + |grad v|^2) with forward
@@ -241,7 +327,7 @@ __device__ __forceinline__ void stage_derivs(const float *sW, const float *sU, c
 }
 
 struct PixelSystem {
-    float i11, i22, a12, b1, b2, cl, cr, cu, cd;
+    float i11, i22, a12, b1, b2;
 };
 
 // The 2x2 system of pixel (gx, gy) from its neighbourhood.  ix, iy: the
@@ -279,17 +365,17 @@ __device__ __forceinline__ PixelSystem pixel_system_vals(
         ag = 0.0f;
     }
     PixelSystem ps;
-    ps.cl = bl ? fmul(0.5f, fadd(asp, asl)) : 0.0f;
-    ps.cr = br ? fmul(0.5f, fadd(asp, asr)) : 0.0f;
-    ps.cu = bu ? fmul(0.5f, fadd(asp, asu)) : 0.0f;
-    ps.cd = bd ? fmul(0.5f, fadd(asp, asd)) : 0.0f;
-    const float sw = fadd(fadd(fadd(ps.cl, ps.cr), ps.cu), ps.cd);
-    const float su0 = ffma(ps.cd, fsub(ud, u),
-                           ffma(ps.cu, fsub(uu, u), ffma(ps.cr, fsub(ur, u),
-                                                         fmul(ps.cl, fsub(ul, u)))));
-    const float sv0 = ffma(ps.cd, fsub(vd, v),
-                           ffma(ps.cu, fsub(vu, v), ffma(ps.cr, fsub(vr, v),
-                                                         fmul(ps.cl, fsub(vl, v)))));
+    const float cl = bl ? fmul(0.5f, fadd(asp, asl)) : 0.0f;
+    const float cr = br ? fmul(0.5f, fadd(asp, asr)) : 0.0f;
+    const float cu = bu ? fmul(0.5f, fadd(asp, asu)) : 0.0f;
+    const float cd = bd ? fmul(0.5f, fadd(asp, asd)) : 0.0f;
+    const float sw = fadd(fadd(fadd(cl, cr), cu), cd);
+    const float su0 = ffma(cd, fsub(ud, u),
+                           ffma(cu, fsub(uu, u), ffma(cr, fsub(ur, u),
+                                                         fmul(cl, fsub(ul, u)))));
+    const float sv0 = ffma(cd, fsub(vd, v),
+                           ffma(cu, fsub(vu, v), ffma(cr, fsub(vr, v),
+                                                         fmul(cl, fsub(vl, v)))));
     const float adx = fmul(ad, Ix), ady = fmul(ad, Iy);
     ps.i11 = __fdividef(omega, fadd(ffma(ag, ffma(Ixy, Ixy, fmul(Ixx, Ixx)), fmul(adx, Ix)), sw));
     ps.i22 = __fdividef(omega, fadd(ffma(ag, ffma(Iyy, Iyy, fmul(Ixy, Ixy)), fmul(ady, Iy)), sw));
@@ -392,8 +478,7 @@ __device__ __forceinline__ void coeff_tile(
     cf[kCA12 * pl] = ps.a12;
     cf[kCB1 * pl] = ps.b1;
     cf[kCB2 * pl] = ps.b2;
-    cf[kCWL * pl] = ps.cl;
-    cf[kCWU * pl] = ps.cu;
+    cf[kCAS * pl] = sAs[ty + 1][tx + 1];
 }
 
 // (bx, by): the tile, f: the frame.
@@ -435,7 +520,7 @@ seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
     const SegCoeff &a = seg_of(tab, b);
     const int r = b / a.gx;
     var_coeff_body((const T *)a.I0, (const T *)a.I0x, (const T *)a.I0y, (const T *)a.I1, a.w, a.h,
-                   a.pitch, a.pfs, a.U, a.ufs, a.plane, a.coef, a.cfs, a.delta, a.gamma,
+                   a.pitch, a.pfs, a.U, a.ufs, a.plane, a.coef + kCoefShift, a.cfs, a.delta, a.gamma,
                    a.alpha_s, a.omega, b % a.gx, r % a.gy, r / a.gy);
 }
 
@@ -558,8 +643,7 @@ __device__ __forceinline__ void coeff_strip(const T *__restrict__ I0, const T *_
             c[kCA12 * pl] = ps.a12;
             c[kCB1 * pl] = ps.b1;
             c[kCB2 * pl] = ps.b2;
-            c[kCWL * pl] = ps.cl;
-            c[kCWU * pl] = ps.cu;
+            c[kCAS * pl] = as0;
         }
         // move the windows down one row
         ixm = ix0; iym = iy0; asm_ = as0;
@@ -598,243 +682,195 @@ var_coeff_cw_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                               out_lane, delta, gamma, alpha_s, omega);
 }
 
-// Left and right halo of a region in columns: R rounded up to even, so that
-// every region starts on an even column and a lane's two columns are one
-// aligned 8-byte pair in every plane (pitches and plane sizes are even).
-__host__ __device__ __forceinline__ int sor_halo_x(int R) { return R + (R & 1); }
-
-// Interior output of a lane's pair (columns gx0, gx0 + 1 of row gy; the
-// pair is interior or not as a whole): U + dU, as pairs where both columns
-// are in the level.
-template <bool COH = false>
-__device__ __forceinline__ void store_pair(const float *Uin, float *Uout, size_t plane, int p,
-                                           int gx0, int w, float du0, float du1, float dv0,
-                                           float dv1)
+__device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
-    if (gx0 + 1 < w) {
-        const float2 u = ldf2<COH>(Uin + p);
-        const float2 v = ldf2<COH>(Uin + plane + p);
-        *reinterpret_cast<float2 *>(Uout + p) = make_float2(u.x + du0, u.y + du1);
-        *reinterpret_cast<float2 *>(Uout + plane + p) = make_float2(v.x + dv0, v.y + dv1);
-    } else if (gx0 < w) {
-        Uout[p] = ldf<COH>(Uin + p) + du0;
-        (Uout + plane)[p] = ldf<COH>(Uin + plane + p) + dv0;
-    }
+    return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// The right and lower edge weights of a thread's strip from the stored left
-// and upper ones: w_r(x) = w_l(x + 1) (the next lane's first column for the
-// strip's second column; 0 past the region's last column, whose right
-// neighbour holds dU = 0) and w_d(y) = w_u(y + 1) (wub: w_u of the row below
-// the strip).
-template <int VS>
-__device__ __forceinline__ void lower_right_weights(const float (&wl)[VS][2],
-                                                    const float (&wu)[VS][2],
-                                                    const float (&wub)[2], int lane,
-                                                    float (&wr)[VS][2], float (&wd)[VS][2])
+__device__ __forceinline__ void copy_async8(uint32_t dst, const float *src, int bytes)
 {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes)
+                 : "memory");
+}
+
+// Where a thread's strip lies: the region's first pixel, the strip's, and
+// which of its pixels the region outputs.
+template <int VS, int WARPS>
+struct StripPlace {
+    int gx, gy;    // the strip's first pixel
+    int pitch, w, h;
+    bool c0, c1;   // column 0 / 1 is an output column
+    int r0, r1;    // rows r0 <= r < r1 of the strip are output rows
+    __device__ __forceinline__ StripPlace(int bx, int by, int R, int w_, int h_, int pitch_,
+                                          int lane, int wp)
+        : pitch(pitch_), w(w_), h(h_)
+    {
+        const int tx = kVR - 2 * R, ty = VS * WARPS - 2 * R;
+        gx = bx * tx - R + 2 * lane;
+        gy = by * ty - R + wp * VS;
+        c0 = 2 * lane >= R && 2 * lane < R + tx && gx < w;
+        c1 = 2 * lane + 1 >= R && 2 * lane + 1 < R + tx && gx + 1 < w;
+        r0 = max(R - wp * VS, 0);
+        r1 = min(min(R + ty - wp * VS, VS), h - gy);
+    }
+    // the region lies in the level (block-uniform)
+    __device__ __forceinline__ bool inside(int lane, int wp) const
+    {
+        const int rx = gx - 2 * lane, ry = gy - wp * VS;
+        return rx >= 0 && ry >= 0 && rx + kVR <= w && ry + VS * WARPS <= h;
+    }
+};
+
+// Starts the copy of the output pixels' flow into the thread's own slots of
+// su ([VS][2][threads] pairs), read back by store_flow: the loads' latency
+// passes behind the sweeps.
+template <int VS, int WARPS>
+__device__ __forceinline__ void stage_flow(const StripPlace<VS, WARPS> &p, const float *Uin,
+                                           size_t plane, uint32_t su)
+{
+    const int bytes = (p.c0 || p.c1) ? (p.gx + 1 < p.w ? 8 : 4) : 0;
+#pragma unroll
+    for (int r = 0; r < VS; ++r)
+        if (bytes && r >= p.r0 && r < p.r1) {
+            const float *c = Uin + (p.gy + r) * p.pitch + p.gx;
+            copy_async8(su + (2 * r) * 32 * WARPS * 8, c, bytes);
+            copy_async8(su + (2 * r + 1) * 32 * WARPS * 8, c + plane, bytes);
+        }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// U + dU of the output pixels.  staged: this thread's slots after stage_flow,
+// or null: the flow is read here, through L2 (another SM may have written it
+// earlier in the launch).
+template <int VS, int WARPS>
+__device__ __forceinline__ void store_flow(const StripPlace<VS, WARPS> &p, const Strip<VS> &s,
+                                           const float *Uin, float *Uout, size_t plane,
+                                           const float2 *staged)
+{
+    if (staged) asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
     for (int r = 0; r < VS; ++r) {
-        const float n = __shfl_down_sync(kFull, wl[r][0], 1);
-        wr[r][0] = wl[r][1];
-        wr[r][1] = lane < 31 ? n : 0.0f;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) wd[r][q] = r + 1 < VS ? wu[r + 1][q] : wub[q];
+        if (r < p.r0 || r >= p.r1) continue;
+        const int o = (p.gy + r) * p.pitch + p.gx;
+        const float2 d0 = upk(s.d[r][0]), d1 = upk(s.d[r][1]);
+        float2 u = make_float2(0.0f, 0.0f), v = u;
+        if (staged) {
+            u = staged[(2 * r) * 32 * WARPS];
+            v = staged[(2 * r + 1) * 32 * WARPS];
+        } else {
+            if (p.c0) u.x = __ldcg(Uin + o), v.x = __ldcg(Uin + plane + o);
+            if (p.c1) u.y = __ldcg(Uin + o + 1), v.y = __ldcg(Uin + plane + o + 1);
+        }
+        if (p.c0 && p.c1) {
+            *reinterpret_cast<float2 *>(Uout + o) = make_float2(u.x + d0.x, u.y + d1.x);
+            *reinterpret_cast<float2 *>(Uout + plane + o) = make_float2(v.x + d0.y, v.y + d1.y);
+        } else if (p.c0) {
+            Uout[o] = u.x + d0.x;
+            (Uout + plane)[o] = v.x + d0.y;
+        } else if (p.c1) {
+            Uout[o + 1] = u.y + d1.x;
+            (Uout + plane)[o + 1] = v.y + d1.y;
+        }
     }
 }
 
-// The region's first column (lane 0's first) has its left neighbour outside
-// the region, where dU stays 0; a zero edge weight there lets the SOR update
-// take the shuffled value without a select (0 times a finite value adds
-// exactly 0).  Its right neighbour's weight is unaffected: a pixel's right
-// weight is read from the next lane.
-template <int VS>
-__device__ __forceinline__ void zero_region_left_weights(float (&wl)[VS][2], int lane)
-{
-    if (lane == 0) {
-#pragma unroll
-        for (int r = 0; r < VS; ++r) wl[r][0] = 0.0f;
-    }
-}
-
-// A lane's two adjacent values of one plane (c: the first); EVEN: one
-// aligned 8-byte load.
-template <bool EVEN, bool COH = false>
-__device__ __forceinline__ void set_pair(float (&a)[2], const float *c)
-{
-    if (EVEN) {
-        const float2 v = ldf2<COH>(c);
-        a[0] = v.x;
-        a[1] = v.y;
-    } else {
-        a[0] = ldf<COH>(c);
-        a[1] = ldf<COH>(c + 1);
-    }
-}
-
-// Region of 64 columns x RH rows, strips of VS rows: RH / VS warps.  EVEN:
-// column halo rounded up to even (pairs loaded and stored as 8 bytes); else
-// a halo of R columns (narrower halo, scalar accesses).
-template <int VS, int RH, bool EVEN, bool COH>
+// A region of 64 columns x VS * WARPS rows, its coefficients loaded straight
+// into registers.  COH: the planes and U were written earlier in the launch.
+// su: the block's flow stage (COH: none).
+template <int VS, int WARPS, bool COH>
 __device__ __forceinline__ void sor_region(int bx, int by, int f, int w, int h, int pitch,
                                            const float *__restrict__ Uinb,
                                            float *__restrict__ Uoutb, size_t ufs, size_t plane,
                                            const float *__restrict__ coefb, size_t cfs, int R,
-                                           int n_half, float omega, float *xch)
+                                           int n_half, float omega, StripEnds<WARPS> &ends,
+                                           float2 *su)
 {
-    constexpr int WARPS = RH / VS;
-    const int hx = EVEN ? sor_halo_x(R) : R;
-    const int tile_x = kVR - 2 * hx, tile_y = RH - 2 * R;
-    const int rx0 = bx * tile_x - hx, ry0 = by * tile_y - R;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const StripPlace<VS, WARPS> p(bx, by, R, w, h, pitch, lane, wp);
     const float *Uin = Uinb + (size_t)f * ufs;
-    float *Uout = Uoutb + (size_t)f * ufs;
     const float *cf = coefb + (size_t)f * cfs;
     const int pl = (int)plane;  // offsets within a frame fit in 32 bits
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    float i11[VS][2], i22[VS][2], a12[VS][2], b1[VS][2], b2[VS][2];
-    float wl[VS][2], wr[VS][2], wu[VS][2], wd[VS][2];
-    float du[VS][2], dv[VS][2];
-    const int gx0 = rx0 + 2 * lane;  // the lane's pair of columns (even when EVEN)
-    const bool inside = rx0 >= 0 && ry0 >= 0 && rx0 + kVR <= w && ry0 + RH <= h;  // block-uniform
-#pragma unroll
-    for (int r = 0; r < VS; ++r) {
-        const int gy = ry0 + wp * VS + r;
-        if (inside) {
-            // the whole region lies in the level: loads without bounds tests
-            du[r][0] = du[r][1] = 0.0f;
-            dv[r][0] = dv[r][1] = 0.0f;
-            const float *c = cf + gy * pitch + gx0;
-            set_pair<EVEN, COH>(i11[r], c + kCI11 * pl);
-            set_pair<EVEN, COH>(i22[r], c + kCI22 * pl);
-            set_pair<EVEN, COH>(a12[r], c + kCA12 * pl);
-            set_pair<EVEN, COH>(b1[r], c + kCB1 * pl);
-            set_pair<EVEN, COH>(b2[r], c + kCB2 * pl);
-            set_pair<EVEN, COH>(wl[r], c + kCWL * pl);
-            set_pair<EVEN, COH>(wu[r], c + kCWU * pl);
-            continue;
-        }
-        if (!EVEN) {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                du[r][q] = 0.0f;
-                dv[r][q] = 0.0f;
-                const int gx = gx0 + q;
-                const bool in = gx >= 0 && gx < w && gy >= 0 && gy < h;
-                const float *c = cf + (in ? gy * pitch + gx : 0);
-                i11[r][q] = in ? ldf<COH>(c + kCI11 * pl) : 0.0f;
-                i22[r][q] = in ? ldf<COH>(c + kCI22 * pl) : 0.0f;
-                a12[r][q] = in ? ldf<COH>(c + kCA12 * pl) : 0.0f;
-                b1[r][q] = in ? ldf<COH>(c + kCB1 * pl) : 0.0f;
-                b2[r][q] = in ? ldf<COH>(c + kCB2 * pl) : 0.0f;
-                wl[r][q] = in ? ldf<COH>(c + kCWL * pl) : 0.0f;
-                wu[r][q] = in ? ldf<COH>(c + kCWU * pl) : 0.0f;
-            }
-            continue;
-        }
-        // gx0 >= 0 implies both columns >= 0; the second may be w (odd w),
-        // still inside the row's pitch: loaded and masked
-        const bool in0 = gx0 >= 0 && gx0 < w && gy >= 0 && gy < h;
-        const bool in1 = in0 && gx0 + 1 < w;
-        const float *c = cf + (in0 ? gy * pitch + gx0 : 0);
-        float2 v[kCPlanes];
-#pragma unroll
-        for (int k = 0; k < kCPlanes; ++k)
-            v[k] = in0 ? ldf2<COH>(c + k * pl) : make_float2(0.0f, 0.0f);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const bool in = q ? in1 : in0;
-            du[r][q] = 0.0f;
-            dv[r][q] = 0.0f;
-            i11[r][q] = in ? (q ? v[kCI11].y : v[kCI11].x) : 0.0f;
-            i22[r][q] = in ? (q ? v[kCI22].y : v[kCI22].x) : 0.0f;
-            a12[r][q] = in ? (q ? v[kCA12].y : v[kCA12].x) : 0.0f;
-            b1[r][q] = in ? (q ? v[kCB1].y : v[kCB1].x) : 0.0f;
-            b2[r][q] = in ? (q ? v[kCB2].y : v[kCB2].x) : 0.0f;
-            wl[r][q] = in ? (q ? v[kCWL].y : v[kCWL].x) : 0.0f;
-            wu[r][q] = in ? (q ? v[kCWU].y : v[kCWU].x) : 0.0f;
-        }
-    }
-
-    // upper weights of the row below the strip (the next strip's first row;
-    // none below the region's last strip, whose lower neighbours hold dU = 0)
-    float wub[2] = {0.0f, 0.0f};
-    if (wp < WARPS - 1) {
-        const int gy = ry0 + (wp + 1) * VS;
-        if (inside) {
-            set_pair<EVEN, COH>(wub, cf + gy * pitch + gx0 + kCWU * pl);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int gx = gx0 + q;
-                if (gx >= 0 && gx < w && gy >= 0 && gy < h)
-                    wub[q] = ldf<COH>(cf + gy * pitch + gx + kCWU * pl);
-            }
-        }
-    }
-    lower_right_weights<VS>(wl, wu, wub, lane, wr, wd);
-    zero_region_left_weights<VS>(wl, lane);
-
-    // red-black SOR; red = (x + y) even, first.  Given the parity of (x + y)
-    // at a strip's first pixel, the column of a given colour in a given row
-    // is a compile-time constant.
-    sor_sweeps<VS, WARPS>(du, dv, i11, i22, a12, b1, b2, wl, wr, wu, wd, xch, lane, wp,
-                          (rx0 + ry0 + wp * VS) & 1, n_half, omega);
-
-    if (!EVEN) {
-#pragma unroll
-        for (int r = 0; r < VS; ++r)
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int lx = 2 * lane + q, ly = wp * VS + r;
-                const int gx = rx0 + lx, gy = ry0 + ly;
-                if (lx < hx || lx >= hx + tile_x || ly < R || ly >= R + tile_y || gx >= w ||
-                    gy >= h)
-                    continue;
-                const int p = gy * pitch + gx;
-                Uout[p] = ldf<COH>(Uin + p) + du[r][q];
-                (Uout + plane)[p] = ldf<COH>(Uin + plane + p) + dv[r][q];
-            }
-        return;
-    }
-    const int lx0 = 2 * lane;
-    if (lx0 >= hx && lx0 < hx + tile_x) {
+    const bool inside = p.inside(lane, wp);
+    const bool first = wp == 0, last = wp == WARPS - 1;
+    Strip<VS> s;
+    float as[VS + 2][2];
+    if (inside) {
+        // the whole region lies in the level: loads without bounds tests
+        const float *c0 = cf + p.gy * pitch + p.gx;
 #pragma unroll
         for (int r = 0; r < VS; ++r) {
-            const int ly = wp * VS + r, gy = ry0 + ly;
-            if (ly < R || ly >= R + tile_y || gy >= h) continue;
-            store_pair<COH>(Uin, Uout, plane, gy * pitch + gx0, gx0, w, du[r][0], du[r][1],
-                            dv[r][0], dv[r][1]);
+            const float *c = c0 + r * pitch;
+            const float2 i1 = ldf2<COH>(c + kCI11 * pl), i2 = ldf2<COH>(c + kCI22 * pl);
+            const float2 a = ldf2<COH>(c + kCA12 * pl), g = ldf2<COH>(c + kCAS * pl);
+            const float2 b1 = ldf2<COH>(c + kCB1 * pl), b2 = ldf2<COH>(c + kCB2 * pl);
+            s.i11[r][0] = i1.x, s.i11[r][1] = i1.y;
+            s.i22[r][0] = i2.x, s.i22[r][1] = i2.y;
+            s.a12[r][0] = a.x, s.a12[r][1] = a.y;
+            as[r + 1][0] = g.x, as[r + 1][1] = g.y;
+            s.b[r][0] = pk(b1.x, b2.x);
+            s.b[r][1] = pk(b1.y, b2.y);
+        }
+        const float *ca = c0 + kCAS * pl;
+        const float2 z = make_float2(0.0f, 0.0f);
+        const float2 gu = first ? z : ldf2<COH>(ca - pitch);
+        const float2 gd = last ? z : ldf2<COH>(ca + VS * pitch);
+        as[0][0] = gu.x, as[0][1] = gu.y;
+        as[VS + 1][0] = gd.x, as[VS + 1][1] = gd.y;
+    } else {
+#pragma unroll
+        for (int r = -1; r <= VS; ++r) {
+            const int gy = p.gy + r;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int gx = p.gx + q;
+                const bool in = gx >= 0 && gx < w && gy >= 0 && gy < h;
+                const float *c = cf + (in ? gy * pitch + gx : 0);
+                auto ld = [&](int k) { return in ? ldf<COH>(c + k * pl) : 0.0f; };
+                as[r + 1][q] = ld(kCAS);
+                if (r >= 0 && r < VS) {
+                    s.i11[r][q] = ld(kCI11);
+                    s.i22[r][q] = ld(kCI22);
+                    s.a12[r][q] = ld(kCA12);
+                    s.b[r][q] = pk(ld(kCB1), ld(kCB2));
+                }
+            }
         }
     }
+    float2 *slot = su + threadIdx.x;
+    if (!COH) stage_flow(p, Uin, plane, smem_u32(slot));
+    clear_ends(ends);
+    if (inside)
+        edge_weights<VS, true>(s, as, lane, first, last, p.gx, p.gy, w, h);
+    else
+        edge_weights<VS, false>(s, as, lane, first, last, p.gx, p.gy, w, h);
+    sor_sweeps<VS, WARPS>(s, ends, lane, wp, (p.gx + p.gy) & 1, n_half, omega);
+    store_flow(p, s, Uin, Uoutb + (size_t)f * ufs, plane, COH ? nullptr : slot);
 }
 
-template <int VS, int RH, bool EVEN>
-__global__ void __launch_bounds__(32 * (RH / VS), 1)
+template <int VS>
+__global__ void __launch_bounds__(kVThreads, 1)
 var_sor_kernel(int w, int h, int pitch, const float *__restrict__ Uinb,
                float *__restrict__ Uoutb, size_t ufs, size_t plane,
                const float *__restrict__ coefb, size_t cfs, int R, int n_half, float omega)
 {
-    extern __shared__ float xch[];  // strip-end exchange, two buffers
-    sor_region<VS, RH, EVEN, false>(blockIdx.x, blockIdx.y, blockIdx.z, w, h, pitch, Uinb, Uoutb,
-                                    ufs, plane, coefb, cfs, R, n_half, omega, xch);
+    extern __shared__ float2 su[];
+    __shared__ StripEnds<kVWarps> ends;
+    sor_region<VS, kVWarps, false>(blockIdx.x, blockIdx.y, blockIdx.z, w, h, pitch, Uinb, Uoutb,
+                                   ufs, plane, coefb, cfs, R, n_half, omega, ends, su);
 }
 
-// The even-halo 64 x 64 regions of several groups' levels in one launch.
+// The 64 x 64 regions of several groups' levels in one launch.
 __global__ void __launch_bounds__(kVThreads, 1)
 seg_var_sor_kernel(const __grid_constant__ SegTable<SegSor> tab)
 {
-    extern __shared__ float xch[];
+    extern __shared__ float2 su[];
+    __shared__ StripEnds<kVWarps> ends;
     int b;
     const SegSor &a = seg_of(tab, b);
     const int r = b / a.gx;
-    sor_region<kVS, kVR, true, false>(b % a.gx, r % a.gy, r / a.gy, a.w, a.h, a.pitch, a.Uin,
-                                      a.Uout, a.ufs, a.plane, a.coef, a.cfs, a.R, a.n_half,
-                                      a.omega, xch);
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
+    sor_region<kVS, kVWarps, false>(b % a.gx, r % a.gy, r / a.gy, a.w, a.h, a.pitch, a.Uin,
+                                    a.Uout, a.ufs, a.plane, a.coef + kCoefShift, a.cfs, a.R,
+                                    a.n_half, a.omega, ends, su);
 }
 
 // Bounded wait for the mbarrier phase with the given parity: at most
@@ -858,16 +894,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
 __global__ void __launch_bounds__(kVThreads, 1)
 var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int pitch,
                    const float *__restrict__ Uinb, float *__restrict__ Uoutb, size_t ufs,
-                   size_t plane, int R, int tile, int nrx, int nry, int total, int n_half,
-                   float omega, long long wait_limit, int *err)
+                   size_t plane, int R, int nrx, int nry, int total, int n_half, float omega,
+                   long long wait_limit, int *err)
 {
     extern __shared__ __align__(1024) float tsm[];
-    float *cbuf = tsm;                  // [kCPlanes][kVR][kTmaBoxW]
-    float *xch = tsm + kTmaCoefFloats;  // strip-end exchange, two buffers
+    float *cbuf = tsm;  // [kCPlanes][kVR][kTmaBoxW]
+    float2 *slot = reinterpret_cast<float2 *>(tsm + kTmaCoefFloats) + threadIdx.x;
+    __shared__ StripEnds<kVWarps> ends;
     __shared__ __align__(8) unsigned long long mbar_s;
     const uint32_t mbar = smem_u32(&mbar_s);
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
-    const int per_frame = nrx * nry;
+    const int per_frame = nrx * nry, tile = kVR - 2 * R;
     const unsigned long long map_addr = (unsigned long long)&cmap;
     const uint32_t dst = smem_u32(cbuf);
 
@@ -875,13 +912,13 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int p
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    clear_ends(ends);
     __syncthreads();
-    const int hx = sor_halo_x(R), tile_x = kVR - 2 * hx;
+    // the tensor map's column x + 1 is the level's column x
     auto issue = [&](int r) {  // thread 0: the tensor copy of region r
         const int f = r / per_frame, rem = r - f * per_frame;
         const int ry = rem / nrx, rx = rem - ry * nrx;
-        const int bx0 = (rx * tile_x - hx) & ~3;
-        const int by0 = ry * tile - R;
+        const int bx0 = (rx * tile - R + kCoefShift) & ~3, by0 = ry * tile - R;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar),
                      "r"((unsigned)(kTmaCoefFloats * sizeof(float)))
                      : "memory");
@@ -894,8 +931,42 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int p
     int r = blockIdx.x;
     if (t == 0 && r < total) issue(r);
     uint32_t parity = 0;
+#pragma unroll 1
     for (; r < total; r += gridDim.x) {
         const bool ok = mbar_wait(mbar, parity, wait_limit);
+        const int f = r / per_frame, rem = r - f * per_frame;
+        const int ry = rem / nrx, rx = rem - ry * nrx;
+        const StripPlace<kVS, kVWarps> p(rx, ry, R, w, h, pitch, lane, wp);
+        const bool first = wp == 0, last = wp == kVWarps - 1;
+        // a left border's column -1 holds the end of the row before: masked
+        const bool out = p.gx < 0;
+        Strip<kVS> s;
+        float as[kVS + 2][2];
+        constexpr int P = kVR * kTmaBoxW;
+        const float *c0 = cbuf + wp * kVS * kTmaBoxW + ((rx * tile - R + kCoefShift) & 3) + 2 * lane;
+        auto ld = [&](const float *c) {
+            float2 v = *reinterpret_cast<const float2 *>(c);
+            if (out) v.x = 0.0f;
+            return v;
+        };
+#pragma unroll
+        for (int k = 0; k < kVS; ++k) {
+            const float *c = c0 + k * kTmaBoxW;
+            const float2 i1 = ld(c + kCI11 * P), i2 = ld(c + kCI22 * P), a = ld(c + kCA12 * P);
+            const float2 b1 = ld(c + kCB1 * P), b2 = ld(c + kCB2 * P), g = ld(c + kCAS * P);
+            s.i11[k][0] = i1.x, s.i11[k][1] = i1.y;
+            s.i22[k][0] = i2.x, s.i22[k][1] = i2.y;
+            s.a12[k][0] = a.x, s.a12[k][1] = a.y;
+            as[k + 1][0] = g.x, as[k + 1][1] = g.y;
+            s.b[k][0] = pk(b1.x, b2.x);
+            s.b[k][1] = pk(b1.y, b2.y);
+        }
+        const float *ca = c0 + kCAS * P;
+        const float2 z = make_float2(0.0f, 0.0f);
+        const float2 gu = first ? z : ld(ca - kTmaBoxW), gd = last ? z : ld(ca + kVS * kTmaBoxW);
+        as[0][0] = gu.x, as[0][1] = gu.y;
+        as[kVS + 1][0] = gd.x, as[kVS + 1][1] = gd.y;
+        // every thread holds its coefficients: the buffer is free
         if (__syncthreads_or(!ok)) {
             if (t == 0) {
                 atomicOr(err, kErrTimeout);
@@ -906,63 +977,18 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int p
             return;
         }
         parity ^= 1u;
-        const int f = r / per_frame, rem = r - f * per_frame;
-        const int ry = rem / nrx, rx = rem - ry * nrx;
-        const int rx0 = rx * tile_x - hx, ry0 = ry * tile - R;
-        const int ox = rx0 - (rx0 & ~3);  // region column 0 within the box: 0 or 2
-        float i11[kVS][2], i22[kVS][2], a12[kVS][2], b1[kVS][2], b2[kVS][2];
-        float wl[kVS][2], wr[kVS][2], wu[kVS][2], wd[kVS][2];
-        float du[kVS][2], dv[kVS][2];
-#pragma unroll
-        for (int rr = 0; rr < kVS; ++rr) {
-            const float *c = cbuf + (wp * kVS + rr) * kTmaBoxW + ox + 2 * lane;
-            constexpr int P = kVR * kTmaBoxW;
-            float2 v[kCPlanes];
-#pragma unroll
-            for (int k = 0; k < kCPlanes; ++k) v[k] = *reinterpret_cast<const float2 *>(c + k * P);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                du[rr][q] = 0.0f;
-                dv[rr][q] = 0.0f;
-                i11[rr][q] = q ? v[kCI11].y : v[kCI11].x;
-                i22[rr][q] = q ? v[kCI22].y : v[kCI22].x;
-                a12[rr][q] = q ? v[kCA12].y : v[kCA12].x;
-                b1[rr][q] = q ? v[kCB1].y : v[kCB1].x;
-                b2[rr][q] = q ? v[kCB2].y : v[kCB2].x;
-                wl[rr][q] = q ? v[kCWL].y : v[kCWL].x;
-                wu[rr][q] = q ? v[kCWU].y : v[kCWU].x;
-            }
-        }
-        {
-            float wub[2] = {0.0f, 0.0f};
-            if (wp < kVWarps - 1) {
-                const float2 v = *reinterpret_cast<const float2 *>(
-                    cbuf + kCWU * kVR * kTmaBoxW + (wp + 1) * kVS * kTmaBoxW + ox + 2 * lane);
-                wub[0] = v.x;
-                wub[1] = v.y;
-            }
-            lower_right_weights<kVS>(wl, wu, wub, lane, wr, wd);
-            zero_region_left_weights<kVS>(wl, lane);
-        }
-        __syncthreads();  // every thread holds its coefficients: the buffer is free
         if (t == 0 && r + (int)gridDim.x < total) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             issue(r + gridDim.x);
         }
         const float *Uin = Uinb + (size_t)f * ufs;
-        float *Uout = Uoutb + (size_t)f * ufs;
-        sor_sweeps<kVS, kVWarps>(du, dv, i11, i22, a12, b1, b2, wl, wr, wu, wd, xch, lane, wp,
-                                 (rx0 + ry0) & 1, n_half, omega);
-        const int lx0 = 2 * lane, gx0 = rx0 + lx0;
-        if (lx0 >= hx && lx0 < hx + tile_x) {
-#pragma unroll
-            for (int rr = 0; rr < kVS; ++rr) {
-                const int ly = wp * kVS + rr, gy = ry0 + ly;
-                if (ly < R || ly >= R + tile || gy >= h) continue;
-                store_pair(Uin, Uout, plane, gy * pitch + gx0, gx0, w, du[rr][0], du[rr][1],
-                           dv[rr][0], dv[rr][1]);
-            }
-        }
+        stage_flow(p, Uin, plane, smem_u32(slot));
+        if (p.inside(lane, wp))
+            edge_weights<kVS, true>(s, as, lane, first, last, p.gx, p.gy, w, h);
+        else
+            edge_weights<kVS, false>(s, as, lane, first, last, p.gx, p.gy, w, h);
+        sor_sweeps<kVS, kVWarps>(s, ends, lane, wp, (p.gx + p.gy) & 1, n_half, omega);
+        store_flow(p, s, Uin, Uoutb + (size_t)f * ufs, plane, slot);
     }
 }
 
@@ -992,7 +1018,7 @@ var_level_cluster_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                          int nry, int ncx, int ncy, float delta, float gamma, float alpha_s,
                          float omega)
 {
-    extern __shared__ float xch[];  // strip-end exchange of the SOR regions
+    __shared__ StripEnds<kVWarps> ends;
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
@@ -1017,9 +1043,12 @@ var_level_cluster_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                                                 y0, out_lane, delta, gamma, alpha_s, omega);
         }
         cluster.sync();
-        for (int r = rank; r < nreg; r += C)
-            sor_region<2, 32, true, true>(r % nrx, r / nrx, f, w, h, pitch, a, b, ufs, plane,
-                                          coefb, cfs, R, n_half, omega, xch);
+        for (int r = rank; r < nreg; r += C) {
+            sor_region<kVSmallVS, kVWarps, true>(r % nrx, r / nrx, f, w, h, pitch, a, b, ufs,
+                                                 plane, coefb, cfs, R, n_half, omega, ends,
+                                                 nullptr);
+            __syncthreads();  // the next region publishes its strip ends
+        }
         cluster.sync();
         float *t = a;
         a = b;
@@ -1061,7 +1090,7 @@ void make_coef_maps(float *work, const Geometry &geo, int frames, CoefMaps *m)
     if (!enc || !work) return;
     for (int l = 0; l < geo.levels; ++l) {
         const Level &lv = geo.lv[l];
-        const cuuint64_t dims[4] = {(cuuint64_t)lv.w, (cuuint64_t)lv.h, (cuuint64_t)kCPlanes,
+        const cuuint64_t dims[4] = {(cuuint64_t)lv.w + kCoefShift, (cuuint64_t)lv.h, (cuuint64_t)kCPlanes,
                                     (cuuint64_t)frames};
         const cuuint64_t strides[3] = {(cuuint64_t)lv.pitch * sizeof(float),
                                        (cuuint64_t)lv.plane * sizeof(float),
@@ -1078,8 +1107,7 @@ void make_coef_maps(float *work, const Geometry &geo, int frames, CoefMaps *m)
 
 bool var_fused_supported(int var_sor)
 {
-    const int R = var_sor > 0 ? 2 * var_sor - 1 : 0;
-    return kVR - 2 * sor_halo_x(R) >= 16;
+    return kVR - 2 * sor_halo(var_sor) >= 16;
 }
 
 void init_var_attributes()
@@ -1092,8 +1120,10 @@ void init_var_attributes()
     }
     cudaFuncSetAttribute(var_sor_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kTmaSmemBytes);
-    cudaFuncSetAttribute(var_sor_kernel<1, 32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(kVSmemFloats2 * sizeof(float)));
+    cudaFuncSetAttribute(var_sor_kernel<kVS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)flow_stage_bytes<kVS, kVWarps>());
+    cudaFuncSetAttribute(seg_var_sor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)flow_stage_bytes<kVS, kVWarps>());
     // clusters of up to 16 blocks for the level-resident refinement: the
     // largest size whose cluster can be resident with one block per SM
     cudaFuncSetAttribute(var_level_cluster_kernel<2, float>,
@@ -1109,7 +1139,7 @@ void init_var_attributes()
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(c, 1, 1);
         cfg.blockDim = dim3(kVThreads, 1, 1);
-        cfg.dynamicSmemBytes = kVSmemFloats * sizeof(float);
+        cfg.dynamicSmemBytes = 0;
         cudaLaunchAttribute at;
         at.id = cudaLaunchAttributeClusterDimension;
         at.val.clusterDim.x = c;
@@ -1135,8 +1165,8 @@ void init_var_attributes()
 
 }
 
-int sor_tile_x(int R) { return kVR - 2 * sor_halo_x(R); }
-int sor_tile_y(int R) { return kVR - 2 * R; }
+int sor_halo(int var_sor) { return var_sor > 0 ? 2 * var_sor - 1 : 1; }
+int sor_tile(int R) { return kVR - 2 * R; }
 void coeff_tile_shape(int &x, int &y)
 {
     x = kAX;
@@ -1154,7 +1184,7 @@ void launch_seg_coeff(const SegTable<SegCoeff> &t, int blocks, bool half, cudaSt
 void launch_seg_sor(const SegTable<SegSor> &t, int blocks, cudaStream_t st)
 {
     StageScope sc(kStVarSor, 1, st);
-    seg_var_sor_kernel<<<blocks, kVThreads, kVSmemFloats * sizeof(float), st>>>(t);
+    seg_var_sor_kernel<<<blocks, kVThreads, flow_stage_bytes<kVS, kVWarps>(), st>>>(t);
 }
 
 float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y,
@@ -1169,9 +1199,10 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
     cudaGetDevice(&dev);
     const int nsm = (dev >= 0 && dev < kMaxDevs && g_num_sms[dev] > 0) ? g_num_sms[dev] : 0;
     const int n_half = 2 * fp.var_sor;
-    const int R = n_half > 0 ? n_half - 1 : 0;
-    const int tile = kVR - 2 * R;                    // interior rows of a 64-row region
-    const int tile_x = kVR - 2 * sor_halo_x(R);      // interior columns
+    const int R = sor_halo(fp.var_sor);
+    const int tile = sor_tile(R);           // interior side of a 64 x 64 region
+    const int small = kVSmallRows - 2 * R;  // interior rows of a 64 x 32 region
+    coef += kCoefShift;
     const dim3 cgrd((lv.w + kAX - 1) / kAX, (lv.h + kAY - 1) / kAY, frames);
     // the coefficient kernel's form depends on the level's width and the
     // stream's parameters only, so single, batched and grouped windows of a
@@ -1183,7 +1214,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
                                                                        : kCWRows;
     const dim3 wgrd((lv.w + kCWOut - 1) / kCWOut,
                     ((lv.h + cw_rows - 1) / cw_rows + kCWWarps - 1) / kCWWarps, frames);
-    const dim3 sgrd((lv.w + tile_x - 1) / tile_x, (lv.h + tile - 1) / tile, frames);
+    const dim3 sgrd((lv.w + tile - 1) / tile, (lv.h + tile - 1) / tile, frames);
     // small levels: every outer iteration in one cluster launch per frame
     // (same flow bit for bit), where one cluster holds the level's work and
     // all the frames' clusters fit one wave
@@ -1191,11 +1222,9 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
         // strips of 2 rows if the cluster can hold them, else of 4
         const int cmax = std::min((dev >= 0 && dev < kMaxDevs) ? g_cluster_max[dev] : 0,
                                   fp.var_cluster_max);
-        // SOR regions of 64 x 32 (2-row strips, 16 warps): the interior is
-        // 32 - 2R rows high
-        const int ty32 = 32 - 2 * R;
-        const int nrx = (lv.w + tile_x - 1) / tile_x;
-        const int nry = ty32 > 0 ? (lv.h + ty32 - 1) / ty32 : 1 << 20;
+        // SOR regions of 64 x 32 (2-row strips, 16 warps)
+        const int nrx = (lv.w + tile - 1) / tile;
+        const int nry = small > 0 ? (lv.h + small - 1) / small : 1 << 20;
         const int ncx = (lv.w + kCWOut - 1) / kCWOut, nreg = nrx * nry;
         auto need = [&](int sr) {
             const int ncy_ = (lv.h + sr - 1) / sr;
@@ -1207,7 +1236,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(C, 1, frames);
             cfg.blockDim = dim3(kVThreads, 1, 1);
-            cfg.dynamicSmemBytes = kVSmemFloats * sizeof(float);
+            cfg.dynamicSmemBytes = 0;
             cfg.stream = st;
             cudaLaunchAttribute at;
             at.id = cudaLaunchAttributeClusterDimension;
@@ -1279,45 +1308,22 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
         {
             StageScope sc(kStVarSor, 1, st);
             const int total = (int)(sgrd.x * sgrd.y * sgrd.z);
-            // the persistent copy-ahead kernel pays off once every SM has
-            // several regions to walk (batched and grouped windows); both
-            // kernels see the same coefficients, so the choice never changes
-            // the result
-            // grids of under one wave are latency bound: where 64 x 32
-            // regions of 1-row strips (1024 threads, one pixel update each
-            // per half sweep) still fit in one wave, they replace the 4-row
-            // strips.  Every layout computes the interior's whole-image
-            // iteration, so the choice never changes the result.
-            const dim3 g1((lv.w + tile_x - 1) / tile_x,
-                          (lv.h + (32 - 2 * R) - 1) / (32 - 2 * R), frames);
             const int row_waves = fp.sor_row_waves;
-            const bool small = nsm > 0 && row_waves > 0 && total < row_waves * nsm;
-            // even-halo regions (8-byte pairs) unless they take more waves
-            // than regions with an R-column halo
-            const int todd = kVR - 2 * R;
-            const dim3 godd((lv.w + todd - 1) / todd, sgrd.y, frames);
-            const int wave = nsm > 0 ? nsm : 1;
-            const bool even = (total + wave - 1) / wave <=
-                              ((int)(godd.x * godd.y * godd.z) + wave - 1) / wave;
+            const dim3 g1(sgrd.x, small > 0 ? (lv.h + small - 1) / small : 1, frames);
             if (coef_map && nsm > 0 && (long long)total >= (long long)fp.sor_tma_min_per_sm * nsm)
-                var_sor_tma_kernel<<<nsm, kVThreads, kTmaSmemBytes, st>>>(
-                    *coef_map, lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, R, tile,
+                var_sor_tma_kernel<<<std::min(nsm, total), kVThreads, kTmaSmemBytes, st>>>(
+                    *coef_map, lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, R,
                     (int)sgrd.x, (int)sgrd.y, total, n_half, fp.omega,
                     fp.wait_limit >= 0 ? fp.wait_limit : kWaitLimitDefault, err);
-            else if (small && 32 - 2 * R >= 8 && (int)(g1.x * g1.y * g1.z) <= row_waves * nsm)
-                var_sor_kernel<1, 32, true><<<g1, 32 * 32, kVSmemFloats2 * sizeof(float), st>>>(
-                    lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, coef,
-                    coef_frame_stride, R, n_half, fp.omega);
-            else if (even)
-                var_sor_kernel<kVS, kVR, true>
-                    <<<sgrd, kVThreads, kVSmemFloats * sizeof(float), st>>>(
+            else if (small >= 8 && (long long)(g1.x * g1.y * g1.z) <= (long long)row_waves * nsm)
+                var_sor_kernel<kVSmallVS>
+                    <<<g1, kVThreads, flow_stage_bytes<kVSmallVS, kVWarps>(), st>>>(
                         lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, coef,
                         coef_frame_stride, R, n_half, fp.omega);
             else
-                var_sor_kernel<kVS, kVR, false>
-                    <<<godd, kVThreads, kVSmemFloats * sizeof(float), st>>>(
-                        lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, coef,
-                        coef_frame_stride, R, n_half, fp.omega);
+                var_sor_kernel<kVS><<<sgrd, kVThreads, flow_stage_bytes<kVS, kVWarps>(), st>>>(
+                    lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, coef,
+                    coef_frame_stride, R, n_half, fp.omega);
         }
         float *t = a;
         a = b;

@@ -166,8 +166,8 @@ size_t edt_rows_smem(int W, int rows);  // dynamic shared memory of such a block
 void edt_cols_chunks(int H, int &CH, int &nch);
 int search_patches_per_block(int ps, bool wide);
 bool search_wide(int n_patches);
-int sor_tile_x(int R);                 // interior columns of a SOR region
-int sor_tile_y(int R);                 // interior rows of a SOR region
+int sor_halo(int var_sor);             // halo of a SOR region (odd)
+int sor_tile(int R);                   // interior side of a 64 x 64 SOR region
 void coeff_tile_shape(int &x, int &y);  // pixels of a coefficient tile
 int coeff_planes();                    // coefficient planes per level and frame
 int seg_max_levels();                  // pyramid levels the fused pyramid kernels build
