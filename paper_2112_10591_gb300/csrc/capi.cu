@@ -1078,7 +1078,7 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
     // A3
     {
         std::vector<std::pair<SegEdtCols, int>> segs;
-        int nch_max = 1;
+        int max_h = 1;
         for (GS &x : gs) {
             ebof_group *g = x.g;
             SegEdtCols a = {};
@@ -1089,13 +1089,12 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
             a.epitch = a.gpitch = g->pitch0;
             a.W = g->p.width;
             a.H = g->p.height;
-            edt_cols_chunks(a.H, a.CH, a.nch);
             a.gx = (a.W + 31) / 32;
-            nch_max = std::max(nch_max, a.nch);
+            max_h = std::max(max_h, a.H);
             segs.push_back({a, a.gx * g->n});
         }
-        emit_seg(P, segs, [nch_max](const SegTable<SegEdtCols> &t, int b, cudaStream_t st) {
-            launch_seg_edt_cols(t, b, nch_max, st);
+        emit_seg(P, segs, [max_h](const SegTable<SegEdtCols> &t, int b, cudaStream_t st) {
+            launch_seg_edt_cols(t, b, max_h, st);
         });
     }
     // A4 (keyed by storage): rows of one warp
@@ -1962,9 +1961,20 @@ ebof_status ebof_edt(const uint8_t *d_edge, int32_t width, int32_t height, int32
     cudaStream_t st = (cudaStream_t)cuda_stream;
     cudaGetLastError();
     const size_t plane = (size_t)width * height;
-    launch_edt_columns(d_edge, width, plane, width, height, d_scratch, width, plane, 1, st);
-    launch_edt_rows_surface(d_scratch, width, plane, width, height, alpha, d_edt, d_surface,
-                            nullptr, width, plane, 1, false, st);
+    // a row's words serve 32 rows, so the scratch must outlive the first
+    // results: where the caller lets it overlap them, the column distances are
+    // read off the edge image instead
+    auto overlaps = [&](const void *out) {
+        return out && (const char *)out < (const char *)(d_scratch + plane) &&
+               (const char *)d_scratch < (const char *)out + 4 * plane;
+    };
+    if (overlaps(d_edt) || overlaps(d_surface)) {
+        launch_edt_direct(d_edge, width, height, alpha, d_edt, d_surface, st);
+    } else {
+        launch_edt_columns(d_edge, width, plane, width, height, d_scratch, width, plane, 1, st);
+        launch_edt_rows_surface(d_scratch, width, plane, width, height, alpha, d_edt, d_surface,
+                                nullptr, width, plane, 1, false, st);
+    }
     return cudaGetLastError() == cudaSuccess ? EBOF_OK : EBOF_ERR_CUDA;
 }
 

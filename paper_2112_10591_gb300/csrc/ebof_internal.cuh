@@ -108,7 +108,8 @@ void launch_denoise_fill(const uint8_t *E, uint8_t *Ed, uint8_t *Edf, int W, int
                          size_t frame_stride, int frames, int conn, int n_d, int n_f,
                          uint8_t *export_dense, DevStats *stats, cudaStream_t st);
 
-// A3: per-column distance to the nearest edge pixel (G_INF = W + H if none).
+// A3: per column and 32 rows, the edge pixels' bits and the nearest edge rows
+// above and below; g: at least g_pitch * H int32 a frame.
 void launch_edt_columns(const uint8_t *E, int edge_pitch, size_t edge_frame_stride, int W,
                         int H, int32_t *g, int g_pitch, size_t g_frame_stride, int frames,
                         cudaStream_t st);
@@ -124,6 +125,11 @@ void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_strid
                              float alpha, int32_t *D_dense, float *S_dense, void *I0,
                              int i_pitch, size_t i_frame_stride, int frames, bool half,
                              cudaStream_t st);
+
+// A3 and A4 with the Eq. 1 surface straight from a dense edge image, without
+// scratch (slower: every pixel walks its column).
+void launch_edt_direct(const uint8_t *edge, int W, int H, float alpha, int32_t *D_dense,
+                       float *S_dense, cudaStream_t st);
 
 // Per-device kernel attributes (opt-in shared memory); call with the device current.
 void init_front_attributes();

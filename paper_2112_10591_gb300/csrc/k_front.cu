@@ -320,161 +320,200 @@ seg_denoise_fill_kernel(const __grid_constant__ SegTable<SegDenoise> tab)
 }
 
 // ---------------------------------------------------------------- A3
-// Column pass: g(x, y) = distance to the nearest edge pixel in column x, or
-// G_INF = W + H for a column without any (larger than any in-image
-// distance).  A block covers 32 columns; thread (c, k) owns column c's
-// chunk k of CH rows (CH a multiple of 32, at most 512).  It packs its
-// chunk into bit masks, publishes the first and last edge row of the chunk,
-// and after one barrier finds, for each row, the nearest edge pixel above
-// (highest set bit at or above the row, else the previous chunks) and below
-// (lowest set bit at or below, else the next chunks) with bit scans.  Row
-// writes of a warp are 32 consecutive int32.
-constexpr int kColMaxWords = 16;   // CH <= 512 rows
-constexpr int kColMaxChunks = 32;  // chunks per column
+// Column pass.  A column's edge pixels as 32-row bit words, and for every word
+// the nearest edge rows outside it: the last one above (-32768: none) and the
+// first one below (32767: none), 16 bits each.  The row pass turns a pixel's
+// two words into its column distance with two bit scans.  That is 8 bytes per
+// 32 pixels of a column where the distances themselves took 128, and the pass
+// is one read of the edge image.  An image of one word a column (H <= 32) has
+// no second plane, so the words always fit W * H int32.
+// Measured against distances written by this pass (column and row pass in one
+// stream): see the row pass.
+//
+// A block covers 32 columns; a warp packs the words ty, ty + blockDim.y, ...
+// of its columns (a word's 32 byte loads in flight together) and publishes
+// their first and last edge rows; one warp then runs down and one up the
+// column's words.
+constexpr int kColWarps = 32;
+constexpr int kNoneAbove = -32768, kNoneBelow = 32767;
 
-// bx: the block of 32 columns, f: the frame; nch chunks (at most blockDim.y:
-// threads of chunks past the last one only take part in the barrier).
+__host__ __device__ __forceinline__ int col_words(int H) { return (H + 31) / 32; }
+// shared memory of a block: the first and last edge rows of its words
+__host__ __device__ __forceinline__ size_t cols_smem_bytes(int nw)
+{
+    return (size_t)nw * 32 * 2 * sizeof(int16_t);
+}
+// the nearest edge rows above and below, 16 bits each
+__device__ __forceinline__ int pack_rows(int above, int below)
+{
+    return (int)((uint32_t)(above & 0xffff) | ((uint32_t)below << 16));
+}
+__device__ __forceinline__ int row_above(int v) { return (int)(int16_t)(v & 0xffff); }
+__device__ __forceinline__ int row_below(int v) { return v >> 16; }
+
+// bx: the block of 32 columns, f: the frame.
 __device__ __forceinline__ void edt_cols_body(const uint8_t *__restrict__ E, int epitch,
-                                              size_t efs, int W, int H,
-                                              int32_t *__restrict__ g, int gpitch, size_t gfs,
-                                              int CH, int nch, unsigned bx, unsigned f)
+                                              size_t efs, int W, int H, int32_t *__restrict__ g,
+                                              int gpitch, size_t gfs, unsigned bx, unsigned f)
 {
-    __shared__ int s_first[kColMaxChunks][32], s_last[kColMaxChunks][32];
-    const int c = threadIdx.x, k = threadIdx.y;
-    const int x = bx * 32 + c;
-    const bool colok = x < W;  // chunks k >= nch start at or below row H: nothing to do
-    const uint8_t *e = E + (size_t)f * efs;
-    const int y0 = k * CH, y1 = min(H, y0 + CH);
-    const int nw = (CH + 31) / 32;
-    unsigned mask[kColMaxWords];
-    int first = -1, last = -1;
+    extern __shared__ int16_t s_rows[];
+    const int nw = col_words(H), c = threadIdx.x, x = bx * 32 + c;
+    int16_t *s_last = s_rows + c, *s_first = s_last + nw * 32;
+    const bool colok = x < W;
+    const uint8_t *e = E + (size_t)f * efs + min(x, W - 1);
+    uint32_t *words = reinterpret_cast<uint32_t *>(g + (size_t)f * gfs) + x;
+    for (int wi = threadIdx.y; wi < nw; wi += blockDim.y) {
+        // all 32 loads in flight before the first test (rows past the image
+        // read its last row and are masked out)
+        uint8_t ev[32];
 #pragma unroll
-    for (int wi = 0; wi < kColMaxWords; ++wi) {
-        unsigned m = 0;
-        if (wi < nw && colok) {
-            // all 32 loads in flight before the first test (rows past the
-            // chunk read its last row and are masked out)
-            uint8_t ev[32];
+        for (int b = 0; b < 32; ++b) ev[b] = e[(size_t)min(wi * 32 + b, H - 1) * epitch];
+        uint32_t m = 0;
 #pragma unroll
-            for (int b = 0; b < 32; ++b)
-                ev[b] = e[(size_t)min(y0 + wi * 32 + b, y1 - 1) * epitch + x];
-#pragma unroll
-            for (int b = 0; b < 32; ++b)
-                if (y0 + wi * 32 + b < y1 && ev[b]) m |= 1u << b;
-        }
-        mask[wi] = m;
-        if (m) {
-            if (first < 0) first = y0 + wi * 32 + __ffs(m) - 1;
-            last = y0 + wi * 32 + 31 - __clz(m);
-        }
+        for (int b = 0; b < 32; ++b)
+            if (ev[b]) m |= 1u << b;
+        if (wi == nw - 1 && (H & 31)) m &= (1u << (H & 31)) - 1;
+        if (colok) words[(size_t)wi * gpitch] = m;
+        s_last[wi * 32] = (int16_t)(m ? wi * 32 + 31 - __clz(m) : kNoneAbove);
+        s_first[wi * 32] = (int16_t)(m ? wi * 32 + __ffs(m) - 1 : kNoneBelow);
     }
-    s_first[k][c] = first;
-    s_last[k][c] = last;
+    if (nw == 1) return;
     __syncthreads();
-    if (!colok || y0 >= H) return;
-    int above = -1, below = -1;
-    for (int j = k - 1; j >= 0; --j)
-        if (s_last[j][c] >= 0) { above = s_last[j][c]; break; }
-    for (int j = k + 1; j < nch; ++j)
-        if (s_first[j][c] >= 0) { below = s_first[j][c]; break; }
-    const int ginf = W + H;
-    int32_t *gc = g + (size_t)f * gfs + x;
-    int run_above = above;  // nearest edge row before word wi
+    // one warp runs down the column's words and one up, eight at a time (the
+    // loads before the chain of maxima)
+    constexpr int kRun = 8;
+    if (threadIdx.y == 0) {  // last edge row above each word
+        int run = kNoneAbove;
+        for (int w0 = 0; w0 < nw; w0 += kRun) {
+            int l[kRun];
 #pragma unroll
-    for (int wi = 0; wi < kColMaxWords; ++wi) {
-        if (wi >= nw) break;
-        int next_first = below;  // nearest edge row after word wi
+            for (int k = 0; k < kRun; ++k) l[k] = s_last[min(w0 + k, nw - 1) * 32];
 #pragma unroll
-        for (int wj = kColMaxWords - 1; wj > wi; --wj)
-            if (wj < nw && mask[wj]) next_first = y0 + wj * 32 + __ffs(mask[wj]) - 1;
-        const unsigned m = mask[wi];
-        for (int b = 0; b < 32; ++b) {
-            const int y = y0 + wi * 32 + b;
-            if (y >= y1) break;
-            const unsigned up = m & (0xffffffffu >> (31 - b));  // bits 0..b
-            const unsigned dn = m & (0xffffffffu << b);         // bits b..31
-            const int a = up ? y0 + wi * 32 + 31 - __clz(up) : run_above;
-            const int bl = dn ? y0 + wi * 32 + __ffs(dn) - 1 : next_first;
-            int d = ginf;
-            if (a >= 0) d = y - a;
-            if (bl >= 0 && bl - y < d) d = bl - y;
-            gc[(size_t)y * gpitch] = d;
+            for (int k = 0; k < kRun; ++k) {
+                if (w0 + k < nw) s_last[(w0 + k) * 32] = (int16_t)run;
+                run = max(run, l[k]);
+            }
         }
-        if (m) run_above = y0 + wi * 32 + 31 - __clz(m);
     }
+    if (threadIdx.y == (blockDim.y > 1 ? 1 : 0)) {  // first edge row below
+        int run = kNoneBelow;
+        for (int w0 = nw - 1; w0 >= 0; w0 -= kRun) {
+            int l[kRun];
+#pragma unroll
+            for (int k = 0; k < kRun; ++k) l[k] = s_first[max(w0 - k, 0) * 32];
+#pragma unroll
+            for (int k = 0; k < kRun; ++k) {
+                if (w0 - k >= 0) s_first[(w0 - k) * 32] = (int16_t)run;
+                run = min(run, l[k]);
+            }
+        }
+    }
+    __syncthreads();
+    if (!colok) return;
+    for (int wi = threadIdx.y; wi < nw; wi += blockDim.y)
+        words[(size_t)(nw + wi) * gpitch] = pack_rows(s_last[wi * 32], s_first[wi * 32]);
 }
 
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(32 * kColWarps)
 edt_cols_kernel(const uint8_t *__restrict__ E, int epitch, size_t efs, int W, int H,
-                int32_t *__restrict__ g, int gpitch, size_t gfs, int CH)
+                int32_t *__restrict__ g, int gpitch, size_t gfs)
 {
-    edt_cols_body(E, epitch, efs, W, H, g, gpitch, gfs, CH, blockDim.y, blockIdx.x, blockIdx.y);
+    edt_cols_body(E, epitch, efs, W, H, g, gpitch, gfs, blockIdx.x, blockIdx.y);
 }
 
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(32 * kColWarps)
 seg_edt_cols_kernel(const __grid_constant__ SegTable<SegEdtCols> tab)
 {
     int b;
     const SegEdtCols &a = seg_of(tab, b);
-    edt_cols_body(a.E, a.epitch, a.efs, a.W, a.H, a.g, a.gpitch, a.gfs, a.CH, a.nch, b % a.gx,
-                  b / a.gx);
+    edt_cols_body(a.E, a.epitch, a.efs, a.W, a.H, a.g, a.gpitch, a.gfs, b % a.gx, b / a.gx);
 }
 
 // ---------------------------------------------------------------- A4
-// Row pass: D(x) = min over columns s of (x - s)^2 + h(s), h(s) = g(s, y)^2,
-// the lower envelope of the row's parabolas evaluated at every pixel.  With
-// F(s) = s^2 + h(s) it reads D(x) = x^2 + min_s (F(s) - 2 x s): a minimum of
-// lines in x, so the sites that own part of the envelope are exactly the
-// vertices of the lower convex hull of the points (s, F(s)).  One warp (two
-// or four for single frames of wide rows) serves a row, and each lane owns a
-// band of B consecutive columns (B odd, so that the lanes' accesses to F fall
-// in distinct shared-memory banks).
-//  1. The row's F is staged in shared memory (-1: column without edge pixels).
-//  2. Each lane builds the lower hull of its band's points with a stack
-//     (orientation tests exact in 64-bit integers; a point on the segment of
-//     its neighbours is dropped, which never changes a minimum).
-//  3. Rounds merge the hulls of neighbouring groups of 1, 2, 4, ... bands
-//     (five for 32 bands, seven for 128).  The group's first lane finds the
-//     lower bridge of the two hulls
-//     by walking from their inner ends (the left hull's last vertex moves left
-//     and the right hull's first vertex moves right while the vertex is not
-//     strictly below the line through the other two); the right hull's
-//     surviving vertices are then moved down behind the left hull's, so a
-//     group's hull always starts at its first column.
-//  4. Each lane walks its band's pixels left to right with a pointer into the
-//     row's hull (binary search for the first pixel): along a strictly convex
-//     hull the owner of x never moves left as x grows.
-//  5. Eq. 1 (or an ablation surface) and the 8-bit scale, coalesced stores.
+// Row pass: D(x) = min over columns s of (x - s)^2 + h(s), h(s) = g(s, y)^2.
+// With F(s) = s^2 + h(s) it reads D(x) = x^2 + min_s (F(s) - 2 x s).  The
+// column that attains the minimum never moves left as x grows: for s < t,
+// (F(t) - 2 x t) - (F(s) - 2 x s) falls with x.  So the columns that attain it
+// at x0 and x1 bound the ones between them, whichever of equal ones is taken.
+//  1. The row's F is staged in shared memory (a column without edge pixels: a
+//     value above every distance).
+//  2. The columns that own the pixels 32, 64, ... are found coarse to fine: a
+//     pixel half way (or an eighth of the way) between two known ones is
+//     searched by a warp's lanes over the columns between their owners only.
+//  3. A band of 32 pixels, one per lane, takes the minimum over the columns
+//     between the owners of its ends: every lane reads the same columns, four
+//     at a time, so the bands of a row together cost W evaluations a lane, each
+//     a multiply-add and a minimum.
+//  4. Eq. 1 (or an ablation surface) and the 8-bit scale, coalesced stores.
 // Every step is an exact integer minimum, so D is bit-identical to any exact
-// EDT.  The work per pixel is a few hull steps whatever the distance to the
-// nearest edge, and the lanes of a warp stay in step.
+// EDT.  No step depends on the distance to the nearest edge, and the lanes of
+// a warp never diverge.  It replaced the lower convex hull of the points
+// (s, F(s)), built and merged band by band, whose stack and bridge walks were
+// serial chains of 64-bit orientation tests.  Bound by the integer pipes (a
+// row issues on 75 % of cycles).  Measured, the hull form's time in brackets:
+// 6.5 us at 346x260 (17.7), 29.6 at 1920x1080 (39.7), 10.9 a frame in 1280x720
+// batches (17.4).
 
-// With hull points a < b < c (columns; F as above): is b on or above the
-// segment from a to c, i.e. not a strict vertex of the lower hull?
-__device__ __forceinline__ bool above_chord(int a, int b, int c, const int32_t *F)
-{
-    const long long fa = F[a], fb = F[b], fc = F[c];
-    return (fc - fb) * (long long)(b - a) <= (fb - fa) * (long long)(c - b);
-}
-
-// (x - s)^2 + h(s) from F(s) = s^2 + h(s); every term is below 2^29 for
-// images up to 16384 px a side.
-__device__ __forceinline__ int para(int x, int s, const int32_t *F)
-{
-    const int d = x - s;
-    return d * d + (F[s] - s * s);
-}
+// (x - s)^2 + h(s) is below 2^29 for images up to 16384 px a side; a column
+// without edge pixels gets h = 2^30.
+constexpr int kNoColumn = 1 << 30;
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRowsPerBlock = 4;                  // rows (warps) per block
-constexpr int kRowLoads = 8;                      // column distances in flight per lane
-constexpr size_t kRowsSmemCap = 200 * 1024;       // bytes; 16384-px rows fit one per block
+constexpr int kRowLoads = 4;                      // pixels in flight per lane
+constexpr size_t kRowsSmemCap = 200 * 1024;       // bytes; 16384-px rows fit
 
-// Shared memory of one row, in bytes: F and D (int32) and the hull's columns
-// (int16: every column is below 2^14), padded to a multiple of 4 bytes.
+// Shared memory of one row, in bytes: F (int32, padded to a multiple of 4) and
+// the owners of the band ends.
 __host__ __device__ __forceinline__ size_t rows_smem_bytes(int W)
 {
-    return 8 * (size_t)W + 2 * (((size_t)W + 1) & ~(size_t)1);
+    const size_t nb = ((size_t)W + 31) / 32;
+    return 4 * (((size_t)W + 3) & ~(size_t)3) + ((4 * (nb + 1) + 15) & ~(size_t)15);
+}
+
+// Column distance from a pixel's words; above kMaxDim - 1: no edge pixel.
+__device__ __forceinline__ int word_distance(uint32_t m, int ab, int y)
+{
+    const int b = y & 31;
+    const uint32_t us = m << (31 - b), ds = m >> b;
+    const int up = us ? __clz(us) : y - row_above(ab);
+    const int dn = ds ? __clz(__brev(ds)) : row_below(ab) - y;
+    return min(up, dn);
+}
+
+// Owners of the NP pixels x, x + dx, ... (NP * dx columns of pixels) among the
+// columns lo .. hi, into own[0], own[stride], ...: a warp's lanes share the
+// columns; the minima first, then, for each pixel, the column among the
+// minimum lane's that attains it.
+template <int NP>
+__device__ __forceinline__ void find_owners(const int32_t *F, int lo, int hi, int x, int dx,
+                                            int32_t *own, int stride, int lane)
+{
+    int best[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) best[k] = INT32_MAX;
+#pragma unroll 2
+    for (int s = lo + lane; s <= hi; s += 32) {
+        const int f = F[s];
+#pragma unroll
+        for (int k = 0; k < NP; ++k) best[k] = min(best[k], f - 2 * (x + k * dx) * s);
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int m = __reduce_min_sync(0xffffffffu, best[k]);
+        const int l = __ffs(__ballot_sync(0xffffffffu, best[k] == m)) - 1;
+        const int n2x = -2 * (x + k * dx);
+        int arg = hi;
+        for (int s0 = lo + l; s0 <= hi; s0 += 32 * 32) {
+            const int s = s0 + 32 * lane;
+            const unsigned hit = __ballot_sync(0xffffffffu, s <= hi && F[s] + n2x * s == m);
+            if (hit) {
+                arg = s0 + 32 * (__ffs(hit) - 1);
+                break;
+            }
+        }
+        if (lane == 0) own[k * stride] = arg;
+    }
 }
 
 // Level-0 intensity of the flow block.  FP32 storage keeps I = 255 d_exp.
@@ -505,201 +544,128 @@ __device__ __forceinline__ float ablation_surface(const SurfaceMap &sm, float d)
     return sm.mode == 1 ? d : (sm.mode == 2 ? fminf(d, sm.d_sat) : log1pf(d));
 }
 
-// Lower bridge of two hulls of one row whose columns are x-separated: the
-// left hull hs[aL, aL + nL), the right one hs[aR, aR + nR), both non-empty.
-// On return the merged hull is hs[aL, aL + i] followed by hs[aR + j, aR + nR).
-// The left end moves left and the right end moves right while the vertex is
-// not strictly below the line through the other two; each move drops a
-// vertex, so the walk ends after at most nL + nR steps.
-__device__ __forceinline__ void bridge(const int16_t *hs, const int32_t *F, int aL, int nL,
-                                       int aR, int nR, int &i, int &j)
-{
-    i = nL - 1;
-    j = 0;
-    int li = hs[aL + i], rj = hs[aR];
-    for (;;) {
-        bool moved = false;
-        while (j + 1 < nR) {
-            const int rn = hs[aR + j + 1];
-            if (!above_chord(li, rj, rn, F)) break;
-            rj = rn;
-            ++j;
-            moved = true;
-        }
-        while (i > 0) {
-            const int lp = hs[aL + i - 1];
-            if (!above_chord(lp, li, rj, F)) break;
-            li = lp;
-            --i;
-            moved = true;
-        }
-        if (!moved) break;
-    }
-}
-
-// WPR warps serve a row (32 WPR bands).  WPR = 1: rows_per_block rows of one
-// warp each, warp-level barriers only.  WPR > 1: one row per block; the merge
-// rounds of groups wider than a warp go through shared memory and block
-// barriers.  D is exact whatever WPR, so the layout never changes a result.
-// bx: the block of rows, f: the frame.  A warp past the block's
-// rows_per_block rows (a fused launch sized for another segment's) exits
-// (WPR = 1 has warp-level barriers only).
+// WPR warps serve a row.  WPR = 1: rows_per_block rows of one warp each,
+// warp-level barriers only.  WPR > 1: one row per block.  D is exact whatever
+// WPR, so the layout never changes a result.  bx: the block of rows, f: the
+// frame.  A warp past the block's rows_per_block rows (a fused launch sized for
+// another segment's) exits (WPR = 1 has warp-level barriers only).  Edge: where
+// set, the column distances are read off the edge image itself instead of g.
 template <int WPR, typename T>
 __device__ __forceinline__ void edt_rows_surface_body(
     const int32_t *__restrict__ g, int gpitch, size_t gfs, int W, int H, int rows_per_block,
-    const SurfaceMap &sm, int32_t *__restrict__ D_dense, float *__restrict__ S_dense,
-    T *__restrict__ I0, int ipitch, size_t ifs, int bx, int f)
+    const SurfaceMap &sm, int32_t *D_dense, float *__restrict__ S_dense,
+    T *__restrict__ I0, int ipitch, size_t ifs, int bx, int f,
+    const uint8_t *__restrict__ edge = nullptr)
 {
-    constexpr int NB = 32 * WPR;
-    extern __shared__ int32_t smem[];
-    __shared__ int s_cnt[NB];         // hull sizes of the group leaders (WPR > 1)
-    __shared__ int s_move[NB / 64 + 1][3];  // src, dst, len of a cross-warp group's move
+    constexpr int NT = 32 * WPR;
+    constexpr int FAC = 4;  // how many times finer each level of step 2 is
+    extern __shared__ __align__(16) int32_t smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rib = warp / WPR;                 // row within the block
-    const int tr = (warp % WPR) * 32 + lane;    // this lane's band
+    const int rib = warp / WPR, wr = warp % WPR;  // row within the block, warp within the row
+    const int tr = wr * 32 + lane;
     const int y = bx * rows_per_block + rib;
     // WPR = 1: the whole warp; WPR > 1: never (one row per block)
     if (rib >= rows_per_block || y >= H) return;
+    const int Wp = (W + 3) & ~3, nb = (W + 31) / 32;
     int32_t *F = smem + (size_t)rib * (rows_smem_bytes(W) / 4);
-    int32_t *res = F + W;  // D of the row's pixels
-    // hull columns; a group's hull starts at its first column
-    int16_t *hs = reinterpret_cast<int16_t *>(res + W);
+    int32_t *own = F + Wp;  // own[b]: owner of pixel 32 b (bounds at both ends)
     auto row_sync = [] {
         if (WPR == 1) __syncwarp();
         else __syncthreads();
     };
-    const int ginf = W + H;
-    const int32_t *grow = g + (size_t)f * gfs + (size_t)y * gpitch;
-    // loads issued in batches of kRowLoads before their first use
-    for (int x0 = tr; x0 < W; x0 += NB * kRowLoads) {
-        int gv[kRowLoads];
+    // 1. loads issued in batches of kRowLoads before their first use
+    {
+        const int nw = col_words(H);
+        const uint32_t *words =
+            reinterpret_cast<const uint32_t *>(g + (size_t)f * gfs) + (size_t)(y >> 5) * gpitch;
+        const size_t ab_off = (size_t)nw * gpitch;
+        const int none = pack_rows(kNoneAbove, kNoneBelow);
+        for (int x0 = tr; x0 < Wp; x0 += NT * kRowLoads) {
+            uint32_t m[kRowLoads];
+            int ab[kRowLoads], d[kRowLoads];
 #pragma unroll
-        for (int u = 0; u < kRowLoads; ++u) {
-            const int x = x0 + NB * u;
-            gv[u] = x < W ? grow[x] : ginf;
+            for (int u = 0; u < kRowLoads; ++u) {
+                const int x = x0 + NT * u;
+                m[u] = 0;
+                ab[u] = none;
+                if (x < W && !edge) {
+                    m[u] = words[x];
+                    if (nw > 1) ab[u] = (int)words[ab_off + x];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kRowLoads; ++u) d[u] = word_distance(m[u], ab[u], y);
+            if (edge) {
+#pragma unroll 1
+                for (int u = 0; u < kRowLoads; ++u) {
+                    const int x = x0 + NT * u;
+                    d[u] = kMaxDim;
+                    for (int k = 0; x < W && k < H; ++k) {
+                        if ((y - k >= 0 && edge[(size_t)(y - k) * W + x]) ||
+                            (y + k < H && edge[(size_t)(y + k) * W + x])) {
+                            d[u] = k;
+                            break;
+                        }
+                        if (y - k < 0 && y + k >= H) break;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kRowLoads; ++u) {
+                const int x = x0 + NT * u;
+                if (x < Wp) F[x] = x * x + (d[u] < kMaxDim ? d[u] * d[u] : kNoColumn);
+            }
         }
-#pragma unroll
-        for (int u = 0; u < kRowLoads; ++u) {
-            const int x = x0 + NB * u;
-            if (x < W) F[x] = gv[u] >= ginf ? -1 : gv[u] * gv[u] + x * x;
+    }
+    if (tr == 0) {
+        own[0] = 0;
+        own[nb] = W - 1;
+    }
+    // 2. owners of the band ends; the FAC - 1 pixels between two known ones
+    // share their columns: one warp takes them all, or, while there are fewer
+    // such intervals than warps, one each
+    int step = 1;
+    while (step * FAC < nb) step *= FAC;
+    for (; step >= 1; step /= FAC) {
+        row_sync();  // F and the coarser owners
+        const int wide = step * FAC, ni = (nb + wide - 1) / wide;
+        const bool split = WPR > 1 && ni < WPR;
+        for (int u = wr; u < (split ? ni * (FAC - 1) : ni); u += WPR) {
+            const int i = split ? u / (FAC - 1) : u;
+            const int b0 = i * wide + step * (split ? 1 + u % (FAC - 1) : 1);
+            if (b0 >= nb) continue;
+            const int lo = own[i * wide], hi = own[min(i * wide + wide, nb)];
+            if (!split && b0 + (FAC - 2) * step < nb) {
+                find_owners<FAC - 1>(F, lo, hi, 32 * b0, 32 * step, own + b0, step, lane);
+            } else {
+                for (int b = b0; b < min(split ? b0 + 1 : nb, (i + 1) * wide); b += step)
+                    find_owners<1>(F, lo, hi, 32 * b, 0, own + b, 0, lane);
+            }
         }
     }
     row_sync();
 
-    // 2. the lower hull of the lane's band
-    const int B = ((W + NB - 1) / NB) | 1;
-    const int a = min(W, tr * B), b = min(W, a + B);
-    int cnt = 0;
-    for (int q = a; q < b; ++q) {
-        if (F[q] < 0) continue;
-        while (cnt >= 2 && above_chord(hs[a + cnt - 2], hs[a + cnt - 1], q, F)) --cnt;
-        hs[a + cnt++] = (int16_t)q;
-    }
-    __syncwarp();
-
-    // 3. merge rounds within the warp; the first lane of a group holds the
-    // group's hull size
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const int gs = 2 << k, half = 1 << k;
-        const int nR = __shfl_down_sync(kFull, cnt, half);  // read by group leaders only
-        const int leader = lane & ~(gs - 1);
-        int src = 0, dst = 0, len = 0;
-        if (lane == leader) {
-            const int AR = min(W, (tr + half) * B);  // the right half's first column
-            int i = cnt - 1, j = 0;
-            if (cnt > 0 && nR > 0) bridge(hs, F, a, cnt, AR, nR, i, j);
-            src = AR + j;
-            dst = a + i + 1;
-            len = nR - j;
-            cnt = i + 1 + len;
-        }
-        src = __shfl_sync(kFull, src, leader);
-        dst = __shfl_sync(kFull, dst, leader);
-        len = __shfl_sync(kFull, len, leader);
-        // move the right hull's survivors down (dst <= src: every read of a
-        // later step lies above every write of an earlier one)
-        const int steps = __reduce_max_sync(kFull, (unsigned)((len + gs - 1) / gs));
-        const int e0 = lane - leader;
-        for (int t = 0; t < steps; ++t) {
-            const int e = t * gs + e0;
-            int v = 0;
-            if (e < len) v = hs[src + e];
-            __syncwarp();
-            if (e < len) hs[dst + e] = (int16_t)v;
-            __syncwarp();
-        }
-    }
-    int n;  // the row's hull: hs[0, n)
-    if (WPR == 1) {
-        n = __shfl_sync(kFull, cnt, 0);
-    } else {
-        // merge rounds across the row's warps
-        if (lane == 0) s_cnt[tr] = cnt;
-        __syncthreads();
-#pragma unroll
-        for (int k = 5; (2 << k) <= NB; ++k) {
-            const int gs = 2 << k, half = 1 << k;
-            const int grp = tr / gs, leader = grp * gs;
-            if (tr == leader) {
-                const int nL = s_cnt[tr], nR = s_cnt[tr + half];
-                const int AR = min(W, (tr + half) * B);
-                int i = nL - 1, j = 0;
-                if (nL > 0 && nR > 0) bridge(hs, F, a, nL, AR, nR, i, j);
-                s_move[grp][0] = AR + j;
-                s_move[grp][1] = a + i + 1;
-                s_move[grp][2] = nR - j;
-                s_cnt[tr] = i + 1 + nR - j;
-            }
-            __syncthreads();
-            const int src = s_move[grp][0], dst = s_move[grp][1], len = s_move[grp][2];
-            int steps = 0;
-#pragma unroll
-            for (int q = 0; q < NB / gs; ++q) steps = max(steps, (s_move[q][2] + gs - 1) / gs);
-            const int e0 = tr - leader;
-            for (int t = 0; t < steps; ++t) {
-                const int e = t * gs + e0;
-                int v = 0;
-                if (e < len) v = hs[src + e];
-                __syncthreads();
-                if (e < len) hs[dst + e] = (int16_t)v;
-                __syncthreads();
-            }
-            __syncthreads();  // s_move is rewritten by the next round
-        }
-        n = s_cnt[0];
-    }
-
-    // 4. D of the lane's pixels
-    if (n > 0 && a < b) {
-        int lo = 0, hi = n - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (para(a, hs[mid + 1], F) <= para(a, hs[mid], F)) lo = mid + 1;
-            else hi = mid;
-        }
-        int kk = lo, sk = hs[lo];
-        for (int x = a; x < b; ++x) {
-            int cur = para(x, sk, F);
-            while (kk + 1 < n) {
-                const int sn = hs[kk + 1];
-                const int nx = para(x, sn, F);
-                if (nx > cur) break;
-                cur = nx;
-                sk = sn;
-                ++kk;
-            }
-            res[x] = cur;
-        }
-    }
-    row_sync();
-
-    // 5. surface and intensity (n == 0: the image has no edge pixel)
+    // 3. the bands; 4. surface and intensity
     T *irow = I0 ? I0 + (size_t)f * ifs + (size_t)y * ipitch : nullptr;
     const size_t dbase = (size_t)f * W * H + (size_t)y * W;
     const float inv_alpha = 1.0f / sm.alpha;
-    for (int x = tr; x < W; x += NB) {
-        const int32_t D = n > 0 ? res[x] : kInfD;
+    for (int b = wr; b < nb; b += WPR) {
+        const int x = 32 * b + lane, lo = own[b] & ~3, hi = own[b + 1];
+        const int n2x = -2 * x;
+        int m = INT32_MAX, o = n2x * lo;
+#pragma unroll 2
+        for (int s = lo; s <= hi; s += 4) {
+            // min(a + b, c) is one instruction
+            const int4 q = *reinterpret_cast<const int4 *>(F + s);
+            int v = __viaddmin_s32(q.y, n2x, q.x);
+            v = __viaddmin_s32(q.z, 2 * n2x, v);
+            v = __viaddmin_s32(q.w, 3 * n2x, v);
+            m = __viaddmin_s32(v, o, m);
+            o += 4 * n2x;
+        }
+        if (x >= W) continue;
+        m += x * x;
+        const int32_t D = m < kNoColumn ? m : kInfD;  // kInfD: the image has no edge pixel
         float S = 1.0f, C = 0.0f;  // d_exp of Eq. 1 and its complement 1 - d_exp
         if (sm.mode == 0) {
             if (D != kInfD) {
@@ -725,6 +691,15 @@ edt_rows_surface_kernel(const int32_t *__restrict__ g, int gpitch, size_t gfs, i
 {
     edt_rows_surface_body<WPR, T>(g, gpitch, gfs, W, H, rows_per_block, sm, D_dense, S_dense, I0,
                                   ipitch, ifs, blockIdx.x, blockIdx.y);
+}
+
+// The row pass straight from a dense edge image, without scratch.
+__global__ void __launch_bounds__(32 * kRowsPerBlock)
+edt_direct_kernel(const uint8_t *__restrict__ edge, int W, int H, SurfaceMap sm,
+                  int32_t *__restrict__ D_dense, float *__restrict__ S_dense)
+{
+    edt_rows_surface_body<kRowsPerBlock, float>(nullptr, 0, 0, W, H, 1, sm, D_dense, S_dense,
+                                                nullptr, 0, 0, blockIdx.x, 0, edge);
 }
 
 template <typename T>
@@ -797,25 +772,17 @@ void launch_denoise_fill(const uint8_t *E, uint8_t *Ed, uint8_t *Edf, int W, int
                                              export_dense, stats);
 }
 
-void edt_cols_chunks(int H, int &CH, int &nch)
-{
-    // chunks of CH rows, CH a multiple of 32: at most 32 chunks of at most 512 rows
-    nch = (H + 31) / 32;
-    if (nch > kColMaxChunks) nch = kColMaxChunks;
-    CH = ((H + nch - 1) / nch + 31) / 32 * 32;
-    nch = (H + CH - 1) / CH;
-}
+int edt_cols_warps(int H) { return std::min(col_words(H), kColWarps); }
+size_t edt_cols_smem(int H) { return cols_smem_bytes(col_words(H)); }
 
 void launch_edt_columns(const uint8_t *E, int edge_pitch, size_t edge_frame_stride, int W,
                         int H, int32_t *g, int g_pitch, size_t g_frame_stride, int frames,
                         cudaStream_t st)
 {
     StageScope sc(kStEdtCols, 1, st);
-    int CH, nch;
-    edt_cols_chunks(H, CH, nch);
-    dim3 blk(32, nch), grd((W + 31) / 32, frames);
-    edt_cols_kernel<<<grd, blk, 0, st>>>(E, edge_pitch, edge_frame_stride, W, H, g, g_pitch,
-                                         g_frame_stride, CH);
+    dim3 blk(32, edt_cols_warps(H)), grd((W + 31) / 32, frames);
+    edt_cols_kernel<<<grd, blk, edt_cols_smem(H), st>>>(E, edge_pitch, edge_frame_stride, W, H, g,
+                                                        g_pitch, g_frame_stride);
 }
 
 int edt_rows_block_rows(int W)
@@ -827,39 +794,35 @@ int edt_rows_block_rows(int W)
 
 size_t edt_rows_smem(int W, int rows) { return (size_t)rows * rows_smem_bytes(W); }
 
-// Warps per row: one for batches (fewest instructions per frame) and rows
-// under 512 px; single windows (one or two frames per launch) of wider rows
-// use two, or four from 1024 px, one row per block, to shorten the serial
-// work of a lane.
-int edt_rows_wpr(int W, int frames)
-{
-    if (frames > 2 || W < 512) return 1;
-    return W >= 1024 ? 4 : 2;
-}
+// Warps per row: one for batches (fewest instructions per frame), four for
+// single windows (one or two frames per launch), one row per block, to shorten
+// a row's chain.
+int edt_rows_wpr(int frames) { return frames > 2 ? 1 : kRowsPerBlock; }
 
 template <typename T>
 void edt_rows_t(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
                 const SurfaceMap &sm, int32_t *D_dense, float *S_dense, T *I0, int i_pitch,
                 size_t i_frame_stride, int frames, cudaStream_t st)
 {
-    const int wpr = edt_rows_wpr(W, frames);
+    const int wpr = edt_rows_wpr(frames);
     // one warp a row: four rows per block, fewer where a row's shared memory
-    // is large; wider layouts: one row per block
+    // is large; the wider layout: one row per block
     const int rows = wpr == 1 ? edt_rows_block_rows(W) : 1;
     const size_t smem = edt_rows_smem(W, rows);
     dim3 grd((H + rows - 1) / rows, frames);
-    if (wpr == 4)
-        edt_rows_surface_kernel<4, T><<<grd, 128, smem, st>>>(
-            g, g_pitch, g_frame_stride, W, H, 1, sm, D_dense, S_dense, I0, i_pitch,
-            i_frame_stride);
-    else if (wpr == 2)
-        edt_rows_surface_kernel<2, T><<<grd, 64, smem, st>>>(
-            g, g_pitch, g_frame_stride, W, H, 1, sm, D_dense, S_dense, I0, i_pitch,
-            i_frame_stride);
-    else
-        edt_rows_surface_kernel<1, T><<<grd, 32 * rows, smem, st>>>(
-            g, g_pitch, g_frame_stride, W, H, rows, sm, D_dense, S_dense, I0, i_pitch,
-            i_frame_stride);
+    auto kern = wpr == 1 ? edt_rows_surface_kernel<1, T>
+                         : edt_rows_surface_kernel<kRowsPerBlock, T>;
+    kern<<<grd, 32 * (wpr == 1 ? rows : wpr), smem, st>>>(g, g_pitch, g_frame_stride, W, H, rows,
+                                                          sm, D_dense, S_dense, I0, i_pitch,
+                                                          i_frame_stride);
+}
+
+void launch_edt_direct(const uint8_t *edge, int W, int H, float alpha, int32_t *D_dense,
+                       float *S_dense, cudaStream_t st)
+{
+    StageScope sc(kStEdtRows, 1, st);
+    edt_direct_kernel<<<H, 32 * kRowsPerBlock, edt_rows_smem(W, 1), st>>>(
+        edge, W, H, exp_surface(alpha), D_dense, S_dense);
 }
 
 void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
@@ -891,11 +854,12 @@ void init_front_attributes()
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemCap);
     };
     opt_in((const void *)edt_rows_surface_kernel<1, float>);
-    opt_in((const void *)edt_rows_surface_kernel<2, float>);
-    opt_in((const void *)edt_rows_surface_kernel<4, float>);
+    opt_in((const void *)edt_rows_surface_kernel<kRowsPerBlock, float>);
     opt_in((const void *)edt_rows_surface_kernel<1, __half>);
-    opt_in((const void *)edt_rows_surface_kernel<2, __half>);
-    opt_in((const void *)edt_rows_surface_kernel<4, __half>);
+    opt_in((const void *)edt_rows_surface_kernel<kRowsPerBlock, __half>);
+    opt_in((const void *)edt_direct_kernel);
+    opt_in((const void *)edt_cols_kernel);
+    opt_in((const void *)seg_edt_cols_kernel);
     opt_in((const void *)seg_edt_rows_kernel<float>);
     opt_in((const void *)seg_edt_rows_kernel<__half>);
 }
@@ -912,11 +876,10 @@ void launch_seg_denoise_fill(const SegTable<SegDenoise> &t, int blocks, cudaStre
     seg_denoise_fill_kernel<<<blocks, dim3(kDfX, kDfY), 0, st>>>(t);
 }
 
-void launch_seg_edt_cols(const SegTable<SegEdtCols> &t, int blocks, int nch_max,
-                         cudaStream_t st)
+void launch_seg_edt_cols(const SegTable<SegEdtCols> &t, int blocks, int max_h, cudaStream_t st)
 {
     StageScope sc(kStEdtCols, 1, st);
-    seg_edt_cols_kernel<<<blocks, dim3(32, nch_max), 0, st>>>(t);
+    seg_edt_cols_kernel<<<blocks, dim3(32, edt_cols_warps(max_h)), edt_cols_smem(max_h), st>>>(t);
 }
 
 void launch_seg_edt_rows(const SegTable<SegEdtRows> &t, int blocks, int rows_max, size_t smem,

@@ -66,12 +66,12 @@ struct SegDenoise {
     int W, H, pitch, conn, n_d, n_f, gx, gy;
 };
 
-// A3: gx blocks of 32 columns per frame, chunks of CH rows.
+// A3: gx blocks of 32 columns per frame.
 struct SegEdtCols {
     const uint8_t *E;
     int32_t *g;
     size_t efs, gfs;
-    int epitch, gpitch, W, H, CH, nch, gx;
+    int epitch, gpitch, W, H, gx;
 };
 
 // A4: gx blocks of `rows` rows (one warp each) per frame.
@@ -144,8 +144,8 @@ struct SegFlowOut {
 // is sized on the host, every block walks the work list).
 void launch_seg_scatter(const ScatterWin *wins, int n_wins, int blocks, cudaStream_t st);
 void launch_seg_denoise_fill(const SegTable<SegDenoise> &t, int blocks, cudaStream_t st);
-void launch_seg_edt_cols(const SegTable<SegEdtCols> &t, int blocks, int nch_max,
-                         cudaStream_t st);
+// max_h: the largest frame height of the table
+void launch_seg_edt_cols(const SegTable<SegEdtCols> &t, int blocks, int max_h, cudaStream_t st);
 void launch_seg_edt_rows(const SegTable<SegEdtRows> &t, int blocks, int rows_max,
                          size_t smem, bool half, cudaStream_t st);
 void launch_seg_pyr_means(const SegTable<SegPyr> &t, int blocks, bool half, cudaStream_t st);
@@ -163,7 +163,6 @@ void launch_seg_flow_out(const SegTable<SegFlowOut> &t, int blocks, cudaStream_t
 // Block shapes the host needs to build the tables.
 int edt_rows_block_rows(int W);        // rows per block of the one-warp row layout
 size_t edt_rows_smem(int W, int rows);  // dynamic shared memory of such a block
-void edt_cols_chunks(int H, int &CH, int &nch);
 int search_patches_per_block(int ps, bool wide);
 bool search_wide(int n_patches);
 int sor_halo(int var_sor);             // halo of a SOR region (odd)
