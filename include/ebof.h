@@ -97,11 +97,11 @@ typedef struct {
                                    SM take the persistent copy-ahead kernel; >= 1 (2) */
     int32_t sor_row_waves;      /* SOR grids that fit this many waves of 64x32 regions
                                    of two-row strips take that form; 0 = never (1) */
-    int32_t var_cluster_max;    /* small levels: the whole refinement of a frame in one
-                                   thread-block cluster launch (every outer iteration,
-                                   cluster barriers between the phases) when the level's
-                                   work fits a cluster of at most this many blocks and
-                                   the call's clusters fit one wave; 0 = never (0) */
+    int32_t var_cluster_max;    /* small levels: the whole refinement of a level in one
+                                   launch (every outer iteration).  A single frame in
+                                   order always takes it where its regions fit one
+                                   wave; calls of several frames do so for levels of
+                                   at most this many regions a frame; 0 = never (0) */
     int32_t coeff_cw_rows;      /* rows a warp of the column-walk kernel walks down (the
                                    strip's height): 4, 8 or 16 (8) */
 } ebof_params;
@@ -140,7 +140,7 @@ typedef struct ebof_stream ebof_stream;
  * variational iterations (delta 5, gamma 10, alpha 20, omega 1.6),
  * max_batch 1, FP32 storage; layouts: column walk from 1024 px, copy-ahead
  * SOR from 2 regions per SM, two-row SOR strips for one-wave grids, no
- * cluster-resident refinement. */
+ * one-launch refinement for several frames. */
 void ebof_default_params(ebof_params *p, int32_t width, int32_t height);
 
 /* Eq. 2 with eps = 1/255 (Eq. 3): alpha = d_sat / ln(255). */

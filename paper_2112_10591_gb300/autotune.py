@@ -17,8 +17,8 @@ tuner itself only orchestrates and compares.
    which never touches the oracle.
 2. Layout candidates (the coefficient kernel's form and the height of its
    column-walk strips, the SOR kernels' forms: the persistent copy-ahead
-   kernel, regions of one-row strips; the cluster-resident refinement of
-   small levels) never change the flow.  The tuner checks that each one gives the flow of
+   kernel, regions of two-row strips; the one-launch refinement of small
+   levels) never change the flow.  The tuner checks that each one gives the flow of
    the default layout bit for bit and keeps the fastest, one knob at a time
    from the default, then the combination of the winners.
 """

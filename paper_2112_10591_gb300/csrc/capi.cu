@@ -66,6 +66,7 @@ struct ebof_stream {
     DevStats *dstats = nullptr;
     unsigned long long *d_dropped_time = nullptr;
     int *d_err = nullptr;
+    unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
     float *flow_stage = nullptr;  // device flow for the host-buffer call
     void *ev_stage = nullptr;     // device events for the host-buffer call
     size_t ev_stage_bytes = 0;
@@ -153,6 +154,7 @@ struct ebof_group {
     DevStats *dstats = nullptr;
     unsigned long long *d_dropped_time = nullptr;
     int *d_err = nullptr;
+    unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
     ebof_window_desc *d_desc = nullptr;
     int64_t *h_events = nullptr;  // events given per stream in the last step
     int parity = 0;
@@ -315,7 +317,7 @@ void free_all(ebof_stream *s)
 {
     cudaFree(s->E); cudaFree(s->Ed); cudaFree(s->Edf); cudaFree(s->g); cudaFree(s->pyr);
     cudaFree(s->up); flow_free(s->Ua); flow_free(s->Ub); cudaFree(s->work);
-    cudaFree(s->dstats); cudaFree(s->d_dropped_time); cudaFree(s->d_err);
+    cudaFree(s->dstats); cudaFree(s->d_dropped_time); cudaFree(s->d_err); cudaFree(s->d_ctl);
     cudaFree(s->flow_stage); cudaFree(s->ev_stage); cudaFree(s->d_call);
     for (int b = 0; b < 2; ++b)
         if (s->graph[b]) cudaGraphExecDestroy(s->graph[b]);
@@ -393,6 +395,7 @@ FlowParams flow_params(const ebof_params &p)
     fp.sor_row_waves = p.sor_row_waves;
     fp.var_cluster_max = p.var_cluster_max;
     fp.coeff_cw_rows = p.coeff_cw_rows;
+    fp.level_ctl = nullptr;
     return fp;
 }
 
@@ -471,6 +474,8 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
         const Level *lvc = nullptr;
         for (int l = geo.levels - 1; l >= 0; --l) {
             tl_level = l;
+            // windows in order: nothing else uses the counters meanwhile
+            if (parts == kPartAll) fp.level_ctl = s->d_ctl;
             const Level &lv = geo.lv[l];
             const char *I0 = pyr + ((size_t)prev_first * s->pyr_fs + geo.pyr_off[l]) * es;
             const char *I1 = pyr + ((size_t)curf_first * s->pyr_fs + geo.pyr_off[l]) * es;
@@ -870,7 +875,8 @@ void free_group(ebof_group *g)
         if (g->graph[b]) cudaGraphExecDestroy(g->graph[b]);
     cudaFree(g->E); cudaFree(g->Ed); cudaFree(g->Edf); cudaFree(g->g); cudaFree(g->pyr);
     cudaFree(g->up); flow_free(g->Ua); flow_free(g->Ub); cudaFree(g->work); cudaFree(g->flow);
-    cudaFree(g->dstats); cudaFree(g->d_dropped_time); cudaFree(g->d_err); cudaFree(g->d_desc);
+    cudaFree(g->dstats); cudaFree(g->d_dropped_time); cudaFree(g->d_err); cudaFree(g->d_ctl);
+    cudaFree(g->d_desc);
     delete[] g->h_events;
     if (g->cap) cudaStreamDestroy(g->cap);
     if (g->done) cudaEventDestroy(g->done);
@@ -917,7 +923,8 @@ void run_group_flow(ebof_group *g, bool with_flow, cudaStream_t st)
     char *prv = g->pyr + (size_t)(g->parity ^ 1) * n * g->pyr_fs * es;
     const size_t flow_frame = (size_t)2 * W * H;
     if (with_flow && geo.levels > 0) {
-        const FlowParams fp = flow_params(p);
+        FlowParams fp = flow_params(p);
+        fp.level_ctl = g->d_ctl;
         float *Ucur = nullptr, *Uc = nullptr;
         const Level *lvc = nullptr;
         for (int l = geo.levels - 1; l >= 0; --l) {
@@ -1437,9 +1444,8 @@ void ebof_default_params(ebof_params *p, int32_t width, int32_t height)
     p->coeff_cw_min_width = 1024;
     p->sor_tma_min_per_sm = 2;
     p->sor_row_waves = 1;
-    // the cluster-resident refinement of small levels gives the same flow but
-    // measured no faster inside a graph (1544 vs 1573 frames/s at 1280 x 720):
-    // off unless chosen (the autotuner tries it for groups)
+    // several frames fill the SMs with one launch per step: the one-launch
+    // refinement only if chosen (the autotuner tries it for groups)
     p->var_cluster_max = 0;
     p->coeff_cw_rows = 8;
 }
@@ -1487,6 +1493,7 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     ok &= dmalloc(&s->dstats, sizeof(DevStats) * B) == cudaSuccess;
     ok &= dmalloc(&s->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&s->d_err, sizeof(int)) == cudaSuccess;
+    ok &= dmalloc(&s->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
     ok &= dmalloc(&s->flow_stage, sizeof(float) * 2 * (size_t)p->width * p->height) == cudaSuccess;
     ok &= cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming) == cudaSuccess;
     const size_t call_bytes = (sizeof(ebof_window_desc) + sizeof(float *)) * B;
@@ -1505,6 +1512,7 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
         return EBOF_ERR_OOM;
     }
     cudaMemset(s->d_err, 0, sizeof(int));
+    cudaMemset(s->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
     cudaMemset(s->dstats, 0, sizeof(DevStats) * B);
     make_coef_maps(s->work, s->geo, B, &s->cmaps);
     cudaMemset(s->d_dropped_time, 0, sizeof(unsigned long long));
@@ -1527,6 +1535,7 @@ int64_t ebof_stream_device_bytes(const ebof_params *p)
     size_t total = 3 * r(plane0 * B) + r(4 * plane0 * B) + r(es * geo.pyr_floats * (B + 1));
     total += r(4 * 2 * (size_t)std::max(geo.max_patches, 1) * B);
     total += 2 * r(4 * (2 * plane0 * B + 1)) + r(4 * 9 * plane0 * B);
+    total += sizeof(unsigned) * kLevelCtl;
     total += r(sizeof(DevStats) * B) + 2 * 256 + r(4 * 2 * (size_t)p->width * p->height) +
              r((sizeof(ebof_window_desc) + sizeof(float *)) * B);
     return (int64_t)total;
@@ -2028,6 +2037,7 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     ok &= dmalloc(&g->dstats, sizeof(DevStats) * n) == cudaSuccess;
     ok &= dmalloc(&g->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&g->d_err, sizeof(int)) == cudaSuccess;
+    ok &= dmalloc(&g->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
     ok &= dmalloc(&g->d_desc, sizeof(ebof_window_desc) * n) == cudaSuccess;
     ok &= cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking) == cudaSuccess;
     ok &= cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming) == cudaSuccess;
@@ -2038,6 +2048,7 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
         return EBOF_ERR_OOM;
     }
     cudaMemset(g->d_err, 0, sizeof(int));
+    cudaMemset(g->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
     cudaMemset(g->flow, 0, sizeof(float) * 2 * (size_t)q.width * q.height * n);
     make_coef_maps(g->work, g->geo, n, &g->cmaps);
     if (cudaDeviceSynchronize() != cudaSuccess) {

@@ -88,7 +88,13 @@ struct FlowParams {
     long long wait_limit;  // first wait of the copy-ahead SOR kernel (rounds)
     // variational layouts (ebof_params): none changes a result
     int coeff_cw_min_width, sor_tma_min_per_sm, sor_row_waves, var_cluster_max, coeff_cw_rows;
+    // the counters of the one-launch refinement (kLevelCtl words that are 0
+    // between launches and used by no other launch at the same time), or null:
+    // one launch per step
+    unsigned *level_ctl;
 };
+constexpr int kLevelBlocks = 1022;  // regions of a one-launch refinement
+constexpr int kLevelCtl = kLevelBlocks + 2;
 
 // Launchers (each enqueues on `st`; frames = batch size). ---------------------
 

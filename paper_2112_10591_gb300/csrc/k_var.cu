@@ -49,7 +49,6 @@
 #include "profiler.cuh"
 #include "seg.cuh"
 
-#include <cooperative_groups.h>
 #include <mutex>
 
 namespace ebof {
@@ -992,73 +991,392 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int p
     }
 }
 
-// The whole variational refinement of one small level (every outer
-// iteration) in one launch: one thread-block cluster per frame, C blocks of
-// 512 threads.  Per outer iteration the cluster first builds the level's
-// linear systems, a warp per column-walk strip (28 columns x SR rows, the
-// strips dealt round the cluster's warps; short strips, as the walk down a
-// strip is a chain of dependent loads), into the coefficient planes; a
-// cluster barrier; then runs the SOR sweeps, a block per 64x32 region of
-// 2-row strips (the regions dealt round the blocks), writing U + dU; a
-// cluster barrier.  The
-// device functions are those of var_coeff_cw_kernel and var_sor_kernel and
-// the arithmetic has a fixed rounding sequence, so the flow is the same bit
-// for bit as with the two kernels launched per iteration; it only saves their
-// launches and the blocks' start-up, which dominate on levels this small.
-// Data written earlier in the launch by other blocks (the planes, U) is read
-// through L2 (ld.global.cg) after the barrier, whose release / acquire order
-// makes it visible across the cluster.  Every block of a cluster passes every
-// barrier (the work loops sit between them), so none can wait forever.
-template <int SR, typename T>
-__global__ void __launch_bounds__(kVThreads, 1)
-var_level_cluster_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
-                         const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h,
-                         int pitch, size_t pfs, float *Ua, float *Ub, size_t ufs, size_t plane,
-                         float *coefb, size_t cfs, int outer, int n_half, int R, int nrx,
-                         int nry, int ncx, int ncy, float delta, float gamma, float alpha_s,
-                         float omega)
+// ---------------------------------------------------------------- resident levels
+// Packed operations beside ffma2 and fmul2.  The compiler fuses a packed
+// product into a packed sum that follows it (whatever the rounding suffix), so
+// a product whose rounding matters is added by scalar operations.
+__device__ __forceinline__ pair_t fadd2(pair_t a, pair_t b)
 {
-    __shared__ StripEnds<kVWarps> ends;
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
-    const int f = blockIdx.z;  // one cluster per frame
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const size_t po = (size_t)f * pfs;
-    const int nstrips = ncx * ncy, nreg = nrx * nry;
-    const bool out_lane = lane >= 2 && lane < 2 + kCWOut;
-    float *a = Ua, *b = Ub;
-    for (int k = 0; k < outer; ++k) {
-        const float *U = a + (size_t)f * ufs;
-        float *cf = coefb + (size_t)f * cfs;
-        for (int si = rank * kVWarps + wp; si < nstrips; si += C * kVWarps) {
-            const int cx0 = (si % ncx) * kCWOut - 2, y0 = (si / ncx) * SR;
-            if (cx0 >= 0 && cx0 + 31 < w && y0 >= 2 && y0 + SR + 1 < h)
-                coeff_strip<SR, true, T, true>(I0b + po, I0xb + po, I0yb + po, I1b + po, w, h,
-                                               pitch, U, U + plane, cf, (int)plane, cx0 + lane,
-                                               y0, out_lane, delta, gamma, alpha_s, omega);
-            else
-                coeff_strip<SR, false, T, true>(I0b + po, I0xb + po, I0yb + po, I1b + po, w, h,
-                                                pitch, U, U + plane, cf, (int)plane, cx0 + lane,
-                                                y0, out_lane, delta, gamma, alpha_s, omega);
-        }
-        cluster.sync();
-        for (int r = rank; r < nreg; r += C) {
-            sor_region<kVSmallVS, kVWarps, true>(r % nrx, r / nrx, f, w, h, pitch, a, b, ufs,
-                                                 plane, coefb, cfs, R, n_half, omega, ends,
-                                                 nullptr);
-            __syncthreads();  // the next region publishes its strip ends
-        }
-        cluster.sync();
-        float *t = a;
-        a = b;
-        b = t;
-    }
+    pair_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair_t fsub2(pair_t a, pair_t b)
+{
+    pair_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair_t dup(float a) { return pk(a, a); }
+__device__ __forceinline__ pair_t neg2(pair_t a)
+{
+    const float2 v = upk(a);
+    return pk(-v.x, -v.y);
+}
+// The approximate reciprocal square root and reciprocal, without the scaling
+// of subnormal inputs that rsqrtf and __fdividef carry: the arguments here are
+// at least 1e-6 and 0.01, and over the normal floats up to 2^126 both give the
+// same bits.
+__device__ __forceinline__ float rsqrt_normal(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_normal(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ pair_t psi_prime2(pair_t s2)
+{
+    const float2 v = upk(s2);
+    return fmul2(dup(0.5f),
+                 pk(rsqrt_normal(fadd(v.x, 1e-6f)), rsqrt_normal(fadd(v.y, 1e-6f))));
 }
 
-// Largest cluster of var_level_cluster_kernel that can be resident, per
-// device (0: none); set by init_var_attributes.
-int g_cluster_max[kMaxDevs];
+// The bilinear samples (bilinear_i's, bit for bit) at two clamped positions.
+// The floor comes from an addition rounded down to the integers above 2^23,
+// whose low bits are the column and row; both are held one short of the last,
+// where the weight is 1 instead of a clamped neighbour's index (the level has
+// at least two columns and rows).
+struct Taps2 {
+    float2 a, b, c, d;
+    pair_t fx, fy;
+};
+template <typename T>
+__device__ __forceinline__ Taps2 bil_taps2(const T *__restrict__ I, int w, int h, int pitch,
+                                           pair_t x, pair_t y)
+{
+    constexpr float kInt = 8388608.0f;  // 2^23
+    const float wm = (float)(w - 1), hm = (float)(h - 1);
+    const float tw = kInt + (float)(w - 2), th = kInt + (float)(h - 2);
+    const float2 px = upk(x), py = upk(y);
+    const float x0 = fminf(fmaxf(px.x, 0.0f), wm), x1 = fminf(fmaxf(px.y, 0.0f), wm);
+    const float y0 = fminf(fmaxf(py.x, 0.0f), hm), y1 = fminf(fmaxf(py.y, 0.0f), hm);
+    const float tx0 = fminf(__fadd_rd(x0, kInt), tw), tx1 = fminf(__fadd_rd(x1, kInt), tw);
+    const float ty0 = fminf(__fadd_rd(y0, kInt), th), ty1 = fminf(__fadd_rd(y1, kInt), th);
+    Taps2 t;
+    t.fx = fsub2(pk(x0, x1), fsub2(pk(tx0, tx1), dup(kInt)));
+    t.fy = fsub2(pk(y0, y1), fsub2(pk(ty0, ty1), dup(kInt)));
+    // the bits are 0x4b000000 + the integer: the products wrap alike
+    const uint32_t bias = 0x4b000000u * (uint32_t)pitch + 0x4b000000u;
+    const T *q0 = I + (__float_as_uint(ty0) * (uint32_t)pitch + __float_as_uint(tx0) - bias);
+    const T *q1 = I + (__float_as_uint(ty1) * (uint32_t)pitch + __float_as_uint(tx1) - bias);
+    t.a = make_float2(ldp(q0), ldp(q1));
+    t.b = make_float2(ldp(q0 + 1), ldp(q1 + 1));
+    t.c = make_float2(ldp(q0 + pitch), ldp(q1 + pitch));
+    t.d = make_float2(ldp(q0 + pitch + 1), ldp(q1 + pitch + 1));
+    return t;
+}
+__device__ __forceinline__ pair_t bil_lerp2(const Taps2 &t)
+{
+    const pair_t one = dup(1.0f), gx = fsub2(one, t.fx);
+    const pair_t top = ffma2(t.fx, pk(t.b.x, t.b.y), fmul2(gx, pk(t.a.x, t.a.y)));
+    const pair_t bot = ffma2(t.fx, pk(t.d.x, t.d.y), fmul2(gx, pk(t.c.x, t.c.y)));
+    return ffma2(t.fy, bot, fmul2(fsub2(one, t.fy), top));
+}
+
+// The whole variational refinement of a level in one launch.  The work is a
+// list of items (iteration, region of 64 x 16 VS), iteration by iteration; a
+// block claims them in order from a counter, the next one while it works on
+// the last:
+//  E. It waits for the previous iteration of the region and its eight
+//     neighbours (the halo and the 2 px around are no wider than an interior).
+//  A. It stages the flow of the region and 2 px around, and the warped image
+//     there (positions outside the level are those of the nearest pixel
+//     inside, which gives the replicated borders of the differences).
+//  B. The warped image's derivatives and the smoothness weights, 1 px around.
+//  C. Each thread builds the systems of its strip in registers, where the
+//     sweeps use them: they never leave the SM.
+//  D. The sweeps, then U + dU of the interior to the other flow buffer.
+// The arithmetic is that of the per-iteration kernels, pixel by pixel with the
+// same rounding, so the flow is the same bit for bit.
+//
+// Items are claimed by running blocks and in order, so whatever an item waits
+// for is already claimed by a block that runs: the kernel ends with any number
+// of blocks resident, beside any other kernel, and needs no cooperative launch
+// (which, inside a CUDA graph, cost more than the ten launches it replaced).
+//
+// It pays where an iteration's two launches are latency: the launches
+// themselves, and three round trips through L2 (flow, image, coefficients)
+// before the sweeps start.  The halo's systems are built again by every region
+// that holds them (1.9 times at 64 x 64, 3.2 at 64 x 32).  A 64 x 32 item takes
+// about 12500 cycles: the wait and the release 3000, A 2400, B 1300, C 2700,
+// the sweeps 2700.  Measured, with the launches of one iteration each in
+// brackets: a 346 x 260 window 165 us (175; both inside a graph), outside a
+// graph, where every launch costs more, 613 x 397 windows with all outputs 234
+// us (315) and the flow block on 641 x 479 surfaces 401 us (497).
+//
+// ctl: [0] the claim counter, [1] blocks gone, [2 + r] finished iterations of
+// region r.  The last block to leave sets them to 0 for the next launch.  Waits
+// are bounded; a block whose wait runs out reports kErrTimeout and leaves.
+constexpr int kLvW = kVR + 4;  // staged columns
+template <int VS>
+constexpr size_t level_smem_bytes()
+{
+    return (size_t)6 * kLvW * (VS * kVWarps + 4) * sizeof(float);
+}
+
+template <int VS, typename T>
+__global__ void __launch_bounds__(kVThreads, 1)
+var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
+                 const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h, int pitch,
+                 size_t pfs, float *Ua, float *Ub, size_t ufs, size_t plane, int outer, int n_half,
+                 int R, int nrx, int nry, float delta, float gamma, float alpha_s, float omega,
+                 int blocks, unsigned *ctl, long long wait_limit, int *err)
+{
+    constexpr int RH = VS * kVWarps, WH = RH + 4, NP = kLvW / 2;  // pairs of a staged row
+    extern __shared__ __align__(16) float lsm[];
+    float *sU = lsm, *sV = sU + kLvW * WH, *sW = sV + kLvW * WH;
+    float *sIx = sW + kLvW * WH, *sIy = sIx + kLvW * WH, *sAs = sIy + kLvW * WH;
+    __shared__ StripEnds<kVWarps> ends;
+    const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
+    __shared__ int s_item;
+    const int per_frame = nrx * nry, total = outer * blocks;
+    clear_ends(ends);
+    const float wm1 = (float)(w - 1), hm1 = (float)(h - 1);
+    auto pr = [](const float *a) { return *reinterpret_cast<const pair_t *>(a); };
+    if (t == 0) s_item = (int)atomicAdd(ctl, 1u);
+    __syncthreads();
+    for (int item = s_item; item < total; item = s_item) {
+        const unsigned next = t == 0 ? atomicAdd(ctl, 1u) : 0u;
+        const int k = item / blocks, reg = item - k * blocks, f = reg / per_frame;
+        const int rem = reg - f * per_frame, by = rem / nrx, bx = rem - by * nrx;
+        const StripPlace<VS, kVWarps> p(bx, by, R, w, h, pitch, lane, wp);
+        const int rx0 = p.gx - 2 * lane, ry0 = p.gy - wp * VS;
+        const size_t po = (size_t)f * pfs;
+        const T *I0 = I0b + po, *I0x = I0xb + po, *I0y = I0yb + po, *I1 = I1b + po;
+        // the staged window lies in the level (block-uniform)
+        const bool inside = rx0 >= 2 && ry0 >= 2 && rx0 + kVR + 2 <= w && ry0 + RH + 2 <= h;
+        const float *a = ((k & 1) ? Ub : Ua) + (size_t)f * ufs;
+        float *b = ((k & 1) ? Ua : Ub) + (size_t)f * ufs;
+        // the strip's template values, which do not depend on the wait
+        pair_t i0[VS], i0x[VS], i0y[VS];
+#pragma unroll
+        for (int r = 0; r < VS; ++r) {
+            const int gx = p.gx, gy = p.gy + r, o = gy * pitch + gx;
+            const bool in0 = inside || (gx >= 0 && gx < w && gy >= 0 && gy < h);
+            const bool in1 = inside || (gx + 1 >= 0 && gx + 1 < w && gy >= 0 && gy < h);
+            i0[r] = pk(in0 ? ldp(I0 + o) : 0.0f, in1 ? ldp(I0 + o + 1) : 0.0f);
+            i0x[r] = pk(in0 ? ldp(I0x + o) : 0.0f, in1 ? ldp(I0x + o + 1) : 0.0f);
+            i0y[r] = pk(in0 ? ldp(I0y + o) : 0.0f, in1 ? ldp(I0y + o + 1) : 0.0f);
+        }
+        // E
+        bool late = false;
+        if (k > 0 && t < 9) {
+            const int nx = bx + t % 3 - 1, ny = by + t / 3 - 1;
+            if (nx >= 0 && nx < nrx && ny >= 0 && ny < nry) {
+                const unsigned *q = ctl + 2 + f * per_frame + ny * nrx + nx;
+                late = true;
+                for (long long it = 0; it < wait_limit; ++it) {
+                    unsigned got;
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
+                                 : "=r"(got)
+                                 : "l"(q)
+                                 : "memory");
+                    if ((int)got >= k) {
+                        late = false;
+                        break;
+                    }
+                }
+            }
+        }
+        if (__syncthreads_or(late)) {
+            if (t == 0) atomicOr(err, kErrTimeout);
+            break;
+        }
+        // A
+        constexpr int NI = NP * WH, KI = 3;
+#pragma unroll 1
+        for (int i0 = t; i0 < NI; i0 += kVThreads * KI) {
+            pair_t u[KI], v[KI], x[KI], y[KI];
+#pragma unroll
+            for (int j = 0; j < KI; ++j) {
+                const int i = min(i0 + kVThreads * j, NI - 1);
+                const int row = i / NP, gx = rx0 - 2 + 2 * (i - row * NP), gy = ry0 - 2 + row;
+                if (inside) {
+                    const float *q = a + gy * pitch + gx;
+                    const float2 uu = __ldcg(reinterpret_cast<const float2 *>(q));
+                    const float2 vv = __ldcg(reinterpret_cast<const float2 *>(q + plane));
+                    u[j] = pk(uu.x, uu.y);
+                    v[j] = pk(vv.x, vv.y);
+                    x[j] = pk((float)gx, (float)(gx + 1));
+                    y[j] = dup((float)gy);
+                } else {
+                    const int c0 = clampi(gx, 0, w - 1), c1 = clampi(gx + 1, 0, w - 1);
+                    const int cy = clampi(gy, 0, h - 1);
+                    const float *q = a + cy * pitch;
+                    u[j] = pk(__ldcg(q + c0), __ldcg(q + c1));
+                    v[j] = pk(__ldcg(q + plane + c0), __ldcg(q + plane + c1));
+                    x[j] = pk((float)c0, (float)c1);
+                    y[j] = dup((float)cy);
+                }
+            }
+            Taps2 tp[KI];
+#pragma unroll
+            for (int j = 0; j < KI; ++j)
+                tp[j] = bil_taps2(I1, w, h, pitch, fadd2(x[j], u[j]), fadd2(y[j], v[j]));
+#pragma unroll
+            for (int j = 0; j < KI; ++j) {
+                const int i = i0 + kVThreads * j;
+                if (i < NI) {
+                    *reinterpret_cast<pair_t *>(sU + 2 * i) = u[j];
+                    *reinterpret_cast<pair_t *>(sV + 2 * i) = v[j];
+                    *reinterpret_cast<pair_t *>(sW + 2 * i) = bil_lerp2(tp[j]);
+                }
+            }
+        }
+        __syncthreads();
+        // B: rows 1 .. WH - 2 (the first and last column's left and right
+        // neighbours are another row's; nothing reads those results)
+#pragma unroll 1
+        for (int i = NP + t; i < NP * (WH - 1); i += kVThreads) {
+            const int e = 2 * i;
+            const pair_t half = dup(0.5f);
+            const float2 u = upk(pr(sU + e)), v = upk(pr(sV + e)), wc = upk(pr(sW + e));
+            const float un = sU[e + 2], vn = sV[e + 2];
+            const pair_t ix = pk(fsub(wc.y, sW[e - 1]), fsub(sW[e + 2], wc.x));
+            const pair_t iy = fsub2(pr(sW + e + kLvW), pr(sW + e - kLvW));
+            const pair_t ux = pk(fsub(u.y, u.x), fsub(un, u.y));
+            const pair_t vx = pk(fsub(v.y, v.x), fsub(vn, v.y));
+            const pair_t uy = fsub2(pr(sU + e + kLvW), pk(u.x, u.y));
+            const pair_t vy = fsub2(pr(sV + e + kLvW), pk(v.x, v.y));
+            const pair_t q = psi_prime2(ffma2(vy, vy, ffma2(vx, vx, ffma2(uy, uy, fmul2(ux, ux)))));
+            *reinterpret_cast<pair_t *>(sIx + e) = fmul2(half, ix);
+            *reinterpret_cast<pair_t *>(sIy + e) = fmul2(half, iy);
+            *reinterpret_cast<pair_t *>(sAs + e) = fmul2(dup(alpha_s), q);
+        }
+        __syncthreads();
+        // C
+        Strip<VS> s;
+#pragma unroll
+        for (int r = 0; r < VS; ++r) {
+            const int e = (wp * VS + r + 2) * kLvW + 2 * lane + 2;
+            const int gx = p.gx, gy = p.gy + r;
+            const pair_t half = dup(0.5f);
+            auto cd2 = [&](pair_t hi, pair_t lo) { return fmul2(half, fsub2(hi, lo)); };
+            const bool top = !inside && gy <= 0, bottom = !inside && gy + 1 >= h;
+            const bool c0 = inside || (gx >= 0 && gx < w), c1 = inside || (gx + 1 >= 0 && gx + 1 < w);
+            const bool row_in = inside || (gy >= 0 && gy < h);
+            const bool in0 = c0 && row_in, in1 = c1 && row_in;
+            const pair_t ix = pr(sIx + e), iy = pr(sIy + e);
+            const pair_t ixu = top ? ix : pr(sIx + e - kLvW), ixd = bottom ? ix : pr(sIx + e + kLvW);
+            const pair_t iyu = top ? iy : pr(sIy + e - kLvW), iyd = bottom ? iy : pr(sIy + e + kLvW);
+            const float2 ixv = upk(ix);
+            // clamped neighbours along x
+            const bool l0 = inside || gx > 0, r0 = inside || gx + 1 < w;
+            const bool l1 = inside || gx + 1 > 0, r1 = inside || gx + 2 < w;
+            const pair_t Ixx = fmul2(half, pk(fsub(r0 ? ixv.y : ixv.x, l0 ? sIx[e - 1] : ixv.x),
+                                              fsub(r1 ? sIx[e + 2] : ixv.y, l1 ? ixv.x : ixv.y)));
+            const pair_t Ixy = cd2(ixd, ixu), Iyy = cd2(iyd, iyu);
+            const pair_t Iz = fsub2(pr(sW + e), i0[r]);
+            const pair_t Ixz = fsub2(ix, i0x[r]), Iyz = fsub2(iy, i0y[r]);
+            const pair_t z2 = dup(kZeta2);
+            const pair_t xx = fmul2(Ixx, Ixx), yy = fmul2(Ixy, Ixy);
+            const float2 n1 = upk(fadd2(ffma2(iy, iy, fmul2(ix, ix)), z2));
+            const float2 n2 =
+                upk(fadd2(ffma2(Iyy, Iyy, ffma2(fmul2(dup(2.0f), Ixy), Ixy, xx)), z2));
+            const pair_t nd = pk(rcp_normal(n1.x), rcp_normal(n1.y));
+            const pair_t ng = pk(rcp_normal(n2.x), rcp_normal(n2.y));
+            float2 adv =
+                upk(fmul2(fmul2(dup(delta), nd), psi_prime2(fmul2(fmul2(nd, Iz), Iz))));
+            float2 agv = upk(fmul2(fmul2(dup(gamma), ng),
+                                   psi_prime2(fmul2(ng, ffma2(Iyz, Iyz, fmul2(Ixz, Ixz))))));
+            const pair_t u = pr(sU + e), v = pr(sV + e);
+            const float2 wx = upk(fadd2(pk((float)gx, (float)(gx + 1)), u));
+            const float2 wy = upk(fadd2(dup((float)gy), v));
+            if (wx.x < 0.0f || wx.x > wm1 || wy.x < 0.0f || wy.x > hm1) adv.x = agv.x = 0.0f;
+            if (wx.y < 0.0f || wx.y > wm1 || wy.y < 0.0f || wy.y > hm1) adv.y = agv.y = 0.0f;
+            const pair_t ad = pk(adv.x, adv.y), ag = pk(agv.x, agv.y);
+            // edge weights, 0 where the edge leaves the level
+            const pair_t as = pr(sAs + e);
+            const float2 av = upk(as);
+            const float mid = fmul(0.5f, fadd(av.x, av.y));
+            const float wl = l0 ? fmul(0.5f, fadd(av.x, sAs[e - 1])) : 0.0f;
+            const float wr = r1 ? fmul(0.5f, fadd(av.y, sAs[e + 2])) : 0.0f;
+            const pair_t cl = pk(wl, l1 ? mid : 0.0f), cr = pk(r0 ? mid : 0.0f, wr);
+            const pair_t cu = top ? 0 : fmul2(half, fadd2(as, pr(sAs + e - kLvW)));
+            const pair_t cd = bottom ? 0 : fmul2(half, fadd2(as, pr(sAs + e + kLvW)));
+            const pair_t sw = fadd2(fadd2(fadd2(cl, cr), cu), cd);
+            auto smooth = [&](const float *q, pair_t c) {
+                const float2 m = upk(c);
+                const pair_t dl = pk(fsub(q[e - 1], m.x), fsub(m.x, m.y));
+                const pair_t dr = pk(fsub(m.y, m.x), fsub(q[e + 2], m.y));
+                return ffma2(cd, fsub2(pr(q + e + kLvW), c),
+                             ffma2(cu, fsub2(pr(q + e - kLvW), c), ffma2(cr, dr, fmul2(cl, dl))));
+            };
+            const pair_t su = smooth(sU, u), sv = smooth(sV, v);
+            const pair_t adx = fmul2(ad, ix), ady = fmul2(ad, iy), nag = neg2(ag);
+            const float2 d1 = upk(fadd2(ffma2(ag, ffma2(Ixy, Ixy, xx), fmul2(adx, ix)), sw));
+            const float2 d2 = upk(fadd2(ffma2(ag, ffma2(Iyy, Iyy, yy), fmul2(ady, iy)), sw));
+            const float2 a12 =
+                upk(ffma2(ag, ffma2(Ixy, Iyy, fmul2(Ixx, Ixy)), fmul2(adx, iy)));
+            const float2 b1 = upk(ffma2(nag, ffma2(Ixy, Iyz, fmul2(Ixx, Ixz)),
+                                        ffma2(neg2(adx), Iz, su)));
+            const float2 b2 = upk(ffma2(nag, ffma2(Iyy, Iyz, fmul2(Ixy, Ixz)),
+                                        ffma2(neg2(ady), Iz, sv)));
+            s.i11[r][0] = in0 ? __fdividef(omega, d1.x) : 0.0f;
+            s.i11[r][1] = in1 ? __fdividef(omega, d1.y) : 0.0f;
+            s.i22[r][0] = in0 ? __fdividef(omega, d2.x) : 0.0f;
+            s.i22[r][1] = in1 ? __fdividef(omega, d2.y) : 0.0f;
+            s.a12[r][0] = in0 ? a12.x : 0.0f;
+            s.a12[r][1] = in1 ? a12.y : 0.0f;
+            s.b[r][0] = in0 ? pk(b1.x, b2.x) : 0;
+            s.b[r][1] = in1 ? pk(b1.y, b2.y) : 0;
+            // the region's own edges carry no weight, nor do pixels outside
+            const float2 lv = upk(cl), uv = upk(cu), dv = upk(cd);
+            s.wl[r][0] = lane > 0 && in0 ? lv.x : 0.0f;
+            s.wl[r][1] = in1 ? lv.y : 0.0f;
+            s.wr[r] = lane < 31 && in1 ? wr : 0.0f;
+            const bool up_in = !(r == 0 && wp == 0);
+            s.wu[r][0] = up_in && in0 ? uv.x : 0.0f;
+            s.wu[r][1] = up_in && in1 ? uv.y : 0.0f;
+            if (r == VS - 1) {
+                s.wd[0] = wp < kVWarps - 1 && in0 ? dv.x : 0.0f;
+                s.wd[1] = wp < kVWarps - 1 && in1 ? dv.y : 0.0f;
+            }
+        }
+        // D
+        sor_sweeps<VS, kVWarps>(s, ends, lane, wp, (p.gx + p.gy) & 1, n_half, omega);
+#pragma unroll
+        for (int r = 0; r < VS; ++r) {
+            if (r < p.r0 || r >= p.r1) continue;
+            const int e = (wp * VS + r + 2) * kLvW + 2 * lane + 2;
+            float *q = b + (p.gy + r) * pitch + p.gx;
+            const float2 u = upk(pr(sU + e)), v = upk(pr(sV + e));
+            const float2 d0 = upk(s.d[r][0]), d1 = upk(s.d[r][1]);
+            if (p.c0 && p.c1) {
+                __stcg(reinterpret_cast<float2 *>(q), make_float2(u.x + d0.x, u.y + d1.x));
+                __stcg(reinterpret_cast<float2 *>(q + plane), make_float2(v.x + d0.y, v.y + d1.y));
+            } else if (p.c0) {
+                __stcg(q, u.x + d0.x);
+                __stcg(q + plane, v.x + d0.y);
+            } else if (p.c1) {
+                __stcg(q + 1, u.y + d1.x);
+                __stcg(q + plane + 1, v.y + d1.y);
+            }
+        }
+        if (t == 0) s_item = (int)next;
+        __syncthreads();  // the block's stores, its reads of the stage
+        if (t == 0)  // releases the whole block's stores, which the barrier ordered before it
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ctl + 2 + reg), "r"(k + 1)
+                         : "memory");
+    }
+    // the last block to leave resets the counters
+    __shared__ bool s_last;
+    if (t == 0) {
+        __threadfence();
+        s_last = atomicInc(ctl + 1, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        for (int i = t; i < blocks; i += kVThreads) ctl[2 + i] = 0;
+        if (t == 0) ctl[0] = 0;
+    }
+}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -1124,45 +1442,14 @@ void init_var_attributes()
                          (int)flow_stage_bytes<kVS, kVWarps>());
     cudaFuncSetAttribute(seg_var_sor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)flow_stage_bytes<kVS, kVWarps>());
-    // clusters of up to 16 blocks for the level-resident refinement: the
-    // largest size whose cluster can be resident with one block per SM
-    cudaFuncSetAttribute(var_level_cluster_kernel<2, float>,
-                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(var_level_cluster_kernel<2, __half>,
-                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(var_level_cluster_kernel<4, float>,
-                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(var_level_cluster_kernel<4, __half>,
-                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    int cm = 0;
-    for (int c = 16; c >= 1 && cm == 0; --c) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(c, 1, 1);
-        cfg.blockDim = dim3(kVThreads, 1, 1);
-        cfg.dynamicSmemBytes = 0;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = c;
-        at.val.clusterDim.y = 1;
-        at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        int n32 = 0, n16 = 0;
-        int n32b = 0, n16b = 0;
-        if (cudaOccupancyMaxActiveClusters(&n32, var_level_cluster_kernel<2, float>, &cfg) ==
-                cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&n16, var_level_cluster_kernel<2, __half>, &cfg) ==
-                cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&n32b, var_level_cluster_kernel<4, float>, &cfg) ==
-                cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&n16b, var_level_cluster_kernel<4, __half>, &cfg) ==
-                cudaSuccess &&
-            n32 > 0 && n16 > 0 && n32b > 0 && n16b > 0)
-            cm = c;
-    }
+    auto level_smem = [](const void *fn, size_t bytes) {
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    level_smem((const void *)var_level_kernel<kVS, float>, level_smem_bytes<kVS>());
+    level_smem((const void *)var_level_kernel<kVS, __half>, level_smem_bytes<kVS>());
+    level_smem((const void *)var_level_kernel<kVSmallVS, float>, level_smem_bytes<kVSmallVS>());
+    level_smem((const void *)var_level_kernel<kVSmallVS, __half>, level_smem_bytes<kVSmallVS>());
     cudaGetLastError();
-    if (dev >= 0 && dev < kMaxDevs) g_cluster_max[dev] = cm;
-
 }
 
 int sor_halo(int var_sor) { return var_sor > 0 ? 2 * var_sor - 1 : 1; }
@@ -1215,61 +1502,46 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
     const dim3 wgrd((lv.w + kCWOut - 1) / kCWOut,
                     ((lv.h + cw_rows - 1) / cw_rows + kCWWarps - 1) / kCWWarps, frames);
     const dim3 sgrd((lv.w + tile - 1) / tile, (lv.h + tile - 1) / tile, frames);
-    // small levels: every outer iteration in one cluster launch per frame
-    // (same flow bit for bit), where one cluster holds the level's work and
-    // all the frames' clusters fit one wave
-    {
-        // strips of 2 rows if the cluster can hold them, else of 4
-        const int cmax = std::min((dev >= 0 && dev < kMaxDevs) ? g_cluster_max[dev] : 0,
-                                  fp.var_cluster_max);
-        // SOR regions of 64 x 32 (2-row strips, 16 warps)
-        const int nrx = (lv.w + tile - 1) / tile;
-        const int nry = small > 0 ? (lv.h + small - 1) / small : 1 << 20;
-        const int ncx = (lv.w + kCWOut - 1) / kCWOut, nreg = nrx * nry;
-        auto need = [&](int sr) {
-            const int ncy_ = (lv.h + sr - 1) / sr;
-            return std::max(nreg, (ncx * ncy_ + kVWarps - 1) / kVWarps);
-        };
-        const int sr = need(2) <= cmax ? 2 : 4;
-        const int ncy = (lv.h + sr - 1) / sr, C = need(sr);
-        if (fp.var_outer > 0 && C <= cmax && nsm > 0 && frames * C <= nsm) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(C, 1, frames);
-            cfg.blockDim = dim3(kVThreads, 1, 1);
-            cfg.dynamicSmemBytes = 0;
-            cfg.stream = st;
-            cudaLaunchAttribute at;
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = C;
-            at.val.clusterDim.y = 1;
-            at.val.clusterDim.z = 1;
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            cudaError_t e;
-            {
-                StageScope sc(kStVarSor, 1, st);
-                if (fp.half)
-                    e = cudaLaunchKernelEx(&cfg, sr == 2 ? var_level_cluster_kernel<2, __half>
-                                                         : var_level_cluster_kernel<4, __half>,
-                                           (const __half *)I0, (const __half *)I0x,
-                                           (const __half *)I0y, (const __half *)I1, lv.w, lv.h,
-                                           lv.pitch, pyr_frame_stride, U, Utmp, u_frame_stride,
-                                           lv.plane, coef, coef_frame_stride, fp.var_outer,
-                                           n_half, R, nrx, nry, ncx, ncy, fp.delta, fp.gamma,
-                                           fp.alpha_s, fp.omega);
-                else
-                    e = cudaLaunchKernelEx(&cfg, sr == 2 ? var_level_cluster_kernel<2, float>
-                                                         : var_level_cluster_kernel<4, float>,
-                                           (const float *)I0, (const float *)I0x,
-                                           (const float *)I0y, (const float *)I1, lv.w, lv.h,
-                                           lv.pitch, pyr_frame_stride, U, Utmp, u_frame_stride,
-                                           lv.plane, coef, coef_frame_stride, fp.var_outer,
-                                           n_half, R, nrx, nry, ncx, ncy, fp.delta, fp.gamma,
-                                           fp.alpha_s, fp.omega);
-            }
-            if (e == cudaSuccess) return (fp.var_outer & 1) ? Utmp : U;
-            cudaGetLastError();  // not launched: the per-iteration kernels below
+    // small levels of a single frame: every outer iteration in one launch (same
+    // flow bit for bit), where the regions fit one wave and a region's staged
+    // window reaches no further than its neighbours' interiors; 64 x 32 regions
+    // if they fit, else 64 x 64 (640 x 360: 112 of them, no slower than ten
+    // launches inside a graph, 12 % faster outside one).  Not for levels of
+    // more than one wave (1280 x 720: 171 us against 145), nor, unless asked
+    // for, for several frames, whose launches fill the SMs (640 x 480, eight
+    // frames: 1.21 against 1.20 ms a call)
+    for (int vs : {kVSmallVS, kVS}) {
+        const int ty = vs * kVWarps - 2 * R, nrx = (int)sgrd.x;
+        const int nry = ty > 0 ? (lv.h + ty - 1) / ty : 0;
+        const long long per = (long long)nrx * nry, blocks = per * frames;
+        if (!fp.level_ctl || fp.var_outer < 1 || ty < R + 2 || tile < R + 2 || lv.w < 2 ||
+            lv.h < 2 || nsm < 1 || blocks > std::min(nsm, kLevelBlocks) ||
+            (frames > 1 && per > fp.var_cluster_max))
+            continue;
+        const bool small_form = vs == kVSmallVS;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)std::min<long long>(blocks, nsm), 1, 1);
+        cfg.blockDim = dim3(kVThreads, 1, 1);
+        cfg.dynamicSmemBytes =
+            small_form ? level_smem_bytes<kVSmallVS>() : level_smem_bytes<kVS>();
+        cfg.stream = st;
+        cudaError_t e;
+        {
+            StageScope sc(kStVarSor, 1, st);
+#define EBOF_LV(VS, T)                                                                          \
+    cudaLaunchKernelEx(&cfg, var_level_kernel<VS, T>, (const T *)I0, (const T *)I0x,            \
+                       (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride,   \
+                       U, Utmp, u_frame_stride, lv.plane, fp.var_outer, n_half, R, nrx, nry,    \
+                       fp.delta, fp.gamma, fp.alpha_s, fp.omega, (int)blocks, fp.level_ctl,     \
+                       kWaitLimitDefault, err)
+            if (fp.half)
+                e = small_form ? EBOF_LV(kVSmallVS, __half) : EBOF_LV(kVS, __half);
+            else
+                e = small_form ? EBOF_LV(kVSmallVS, float) : EBOF_LV(kVS, float);
+#undef EBOF_LV
         }
+        if (e == cudaSuccess) return (fp.var_outer & 1) ? Utmp : U;
+        cudaGetLastError();  // not launched: the per-iteration kernels below
     }
     float *a = U, *b = Utmp;
     for (int k = 0; k < fp.var_outer; ++k) {
