@@ -1268,8 +1268,7 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
                 a.stride = p.stride;
                 a.iters = p.gn_iters;
                 a.kappa = p.gn_damping;
-                const int ppb = search_patches_per_block(p.patch, wide);
-                a.gx = (np + ppb - 1) / ppb;
+                a.gx = search_blocks(p.patch, wide, lv.npx, lv.npy);
                 search.push_back({(half << 40) | ((long long)p.patch << 8) | (wide ? 1 : 0),
                                   {a, a.gx * g->n}});
             }

@@ -16,6 +16,7 @@
 #include "dev_common.cuh"
 #include "seg.cuh"
 
+#include <climits>
 #include <type_traits>
 
 namespace ebof {
@@ -315,6 +316,17 @@ struct SearchShape {
 };
 constexpr int kWideSearchPatches = 8192;
 
+// A warp's patches form a tile (4 x 2, 2 x 2, 2 x 1): neighbours stop together.
+__host__ __device__ constexpr int search_tile_w(int patches)
+{
+    return patches >= 8 ? 4 : (patches >= 2 ? 2 : 1);
+}
+// Threads per block: the wide layout's 168 registers a thread leave twelve
+// warps an SM, and its warps stop at different iterations, so a block is one
+// warp (a block's slots are free only once its last warp is done).
+constexpr int kNarrowThreads = 128;
+int search_threads(bool wide) { return wide ? 32 : kNarrowThreads; }
+
 // bx: the block of patches, f: the frame.
 template <int PS, int CG, int RG, typename T>
 __device__ __forceinline__ void patch_search_body(
@@ -327,12 +339,15 @@ __device__ __forceinline__ void patch_search_body(
     constexpr int G = CG * RG;
     constexpr int CPL = (PS + CG - 1) / CG;
     constexpr int RPL = (PS + RG - 1) / RG;
+    constexpr int TW = search_tile_w(32 / G), TH = 32 / G / TW;
     const int c = threadIdx.x % G;
     const int np = npx * npy;
-    const int pid_raw = bx * (128 / G) + threadIdx.x / G;
-    const bool real = pid_raw < np;
-    const int pid = real ? pid_raw : np - 1;
-    const int i = pid % npx, j = pid / npx;
+    const int tx = (npx + TW - 1) / TW;  // a warp's tiles of TW x TH patches
+    const int tile = bx * (blockDim.x / 32) + threadIdx.x / 32, q = threadIdx.x % 32 / G;
+    const int i_raw = tile % tx * TW + q % TW, j_raw = tile / tx * TH + q / TW;
+    const bool real = i_raw < npx && j_raw < npy;
+    const int i = min(i_raw, npx - 1), j = min(j_raw, npy - 1);
+    const int pid = j * npx + i;
     const int x0 = min(i * stride, w - PS), y0 = min(j * stride, h - PS);
     const int c0 = (c % CG) * CPL;  // first column of this lane
     const int r0 = (c / CG) * RPL;  // first row of this lane
@@ -399,6 +414,24 @@ __device__ __forceinline__ void patch_search_body(
 
     float u = u0, v = v0;
     const float lim = (float)(w + h);
+    // The warped patch's texels, (RPL + 1) x (CPL + 1) a lane, stay in
+    // registers, two rows a pair: an iteration reads them again only where the
+    // whole-pixel part of the displacement changed (at 1280x720 one patch in
+    // eight and four warps in ten an iteration, most of them in the first
+    // ones), and a warp stops when no patch of it moves any more: where the
+    // step leaves a displacement as it is, every later one does.  Guarded
+    // patches never move (42 % of a 1280x720 level 0).  Bound by the L1 loads
+    // before (52 a lane and iteration, L1 at 70 %), now by issue at the nine to
+    // twelve warps an SM that 168 registers leave: 1280x720 level 0, eight
+    // frames, 397 -> 316 us (FP16 storage 640x480 141 -> 125), its narrow
+    // layouts 106 -> 93 and 66 -> 50.
+    constexpr int NR2 = (RPL + 2) / 2;  // pairs of rows (the last may be half used)
+    pair_t tex[NR2][CPL + 1];
+    int wx = INT_MIN, wy = INT_MIN;  // the texels' origin
+#pragma unroll
+    for (int i = 0; i < NR2; ++i)
+#pragma unroll
+        for (int k = 0; k <= CPL; ++k) tex[i][k] = 0;
     for (int it = 0; it < iters; ++it) {
         // b = sum g ((w - mean w) - (T - mean T)); the mean-normalised
         // gradients sum to zero, so both means drop out: b = sum g w - sum g T
@@ -415,56 +448,84 @@ __device__ __forceinline__ void patch_search_body(
         // window leaves the level; inside it the clamps do nothing, so the
         // form a warp takes never changes a value.
         const float uc = fminf(fmaxf(u, -lim), lim), vc = fminf(fmaxf(v, -lim), lim);
-        const float fu = floorf(uc), fv = floorf(vc);
-        const int sx0 = x0 + (int)fu, sy0 = y0 + (int)fv;
-        const float ax = uc - fu, ay = vc - fv;
+        // floor by an addition rounded down to the integers (|uc| < 2^22): the
+        // FMA pipe's, where floorf and the conversion take the slow one
+        constexpr float kInt = 12582912.0f;  // 3 * 2^22
+        const float tu = __fadd_rd(uc, kInt), tv = __fadd_rd(vc, kInt);
+        const int sx0 = x0 + (__float_as_int(tu) - 0x4b400000);
+        const int sy0 = y0 + (__float_as_int(tv) - 0x4b400000);
+        const float ax = uc - (tu - kInt), ay = vc - (tv - kInt);
         const bool inside = sx0 >= 0 && sy0 >= 0 && sx0 + PS <= w - 1 && sy0 + PS <= h - 1;
         // columns c0 .. c0 + CPL and rows r0 .. r0 + RPL of the window (the
         // last of each only as the right / lower neighbour); no column or row
         // beyond PS is read
-        auto window = [&](auto clamped) {
-            constexpr bool C = decltype(clamped)::value;
-            int cx[CPL + 1];
+        const bool moved = sx0 != wx || sy0 != wy;
+        if (__any_sync(0xffffffffu, moved)) {
+            const bool all_in = __all_sync(0xffffffffu, inside);
+            if (moved) {
+                wx = sx0;
+                wy = sy0;
+                auto window = [&](auto clamped) {
+                    constexpr bool C = decltype(clamped)::value;
+                    int cx[CPL + 1];
 #pragma unroll
-            for (int k = 0; k <= CPL; ++k)
-                cx[k] = C ? clampi(sx0 + c0 + k, 0, w - 1) : sx0 + c0 + k;
-            auto row = [&](int rr) {
-                return I1 + (C ? clampi(sy0 + rr, 0, h - 1) : sy0 + rr) * pitch;
-            };
-            float hp[CPL];
-            {
-                const T *q = row(r0);
-                float s[CPL + 1];
+                    for (int k = 0; k <= CPL; ++k)
+                        cx[k] = C ? clampi(sx0 + c0 + k, 0, w - 1) : sx0 + c0 + k;
 #pragma unroll
-                for (int k = 0; k <= CPL; ++k)
-                    s[k] = c0 + k <= PS && r0 <= PS ? ldp(&q[cx[k]]) : 0.0f;
+                    for (int i = 0; i < NR2; ++i) {
+                        float lo[CPL + 1], hi[CPL + 1];
 #pragma unroll
-                for (int k = 0; k < CPL; ++k) hp[k] = s[k] + ax * (s[k + 1] - s[k]);
+                        for (int j = 0; j < 2; ++j) {
+                            const int r = 2 * i + j;
+                            const int gy = sy0 + r0 + r;
+                            const T *q = I1 + (C ? clampi(gy, 0, h - 1) : gy) * pitch;
+#pragma unroll
+                            for (int k = 0; k <= CPL; ++k)
+                                (j ? hi : lo)[k] = r <= RPL && c0 + k <= PS && r0 + r <= PS
+                                                       ? ldp(&q[cx[k]])
+                                                       : 0.0f;
+                        }
+#pragma unroll
+                        for (int k = 0; k <= CPL; ++k) tex[i][k] = pk(lo[k], hi[k]);
+                    }
+                };
+                if (all_in)
+                    window(std::integral_constant<bool, false>());
+                else
+                    window(std::integral_constant<bool, true>());
             }
+        }
+        {
+            const pair_t ax2 = pk(ax, ax);
+            float hp[CPL];
 #pragma unroll
-            for (int r = 0; r < RPL; ++r) {
-                const T *q = row(r0 + r + 1);
-                const bool rin = r0 + r + 1 <= PS;
-                float s[CPL + 1];
+            for (int i = 0; i < NR2; ++i) {
+                float2 hl[CPL];
 #pragma unroll
-                for (int k = 0; k <= CPL; ++k) s[k] = c0 + k <= PS && rin ? ldp(&q[cx[k]]) : 0.0f;
+                for (int k = 0; k < CPL; ++k)
+                    hl[k] = upk(ffma2(ax2, fsub2(tex[i][k + 1], tex[i][k]), tex[i][k]));
 #pragma unroll
-                for (int k = 0; k < CPL; ++k) {
-                    const float hn = s[k] + ax * (s[k + 1] - s[k]);
-                    const float wv = hp[k] + ay * (hn - hp[k]);
-                    hp[k] = hn;
-                    b1 += GX[r][k] * wv;
-                    b2 += GY[r][k] * wv;
+                for (int j = 0; j < 2; ++j) {
+                    const int r = 2 * i + j;  // the window's row; output row r - 1
+                    if (r > RPL) continue;
+#pragma unroll
+                    for (int k = 0; k < CPL; ++k) {
+                        const float hn = j ? hl[k].y : hl[k].x;
+                        if (r > 0) {
+                            const float wv = hp[k] + ay * (hn - hp[k]);
+                            b1 += GX[r - 1][k] * wv;
+                            b2 += GY[r - 1][k] * wv;
+                        }
+                        hp[k] = hn;
+                    }
                 }
             }
-        };
-        if (__all_sync(0xffffffffu, inside))
-            window(std::integral_constant<bool, false>());
-        else
-            window(std::integral_constant<bool, true>());
+        }
         b1 = group_sum<G>(b1 - tb1); b2 = group_sum<G>(b2 - tb2);
+        const float up = u, vp = v;
         u -= (a22 * b1 - h12 * b2) * inv_det;
         v -= (a11 * b2 - h12 * b1) * inv_det;
+        if (__all_sync(0xffffffffu, guard || (u == up && v == vp))) break;
     }
     if (guard || !(hypotf(u - u0, v - v0) <= (float)PS)) { u = u0; v = v0; }
     if (real && c == 0) {
@@ -475,7 +536,7 @@ __device__ __forceinline__ void patch_search_body(
 }
 
 template <int PS, int CG, int RG, typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kNarrowThreads)
 patch_search_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                     const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h,
                     int pitch, size_t pfs, int npx, int npy, const float *__restrict__ Ucb, int wc,
@@ -488,7 +549,7 @@ patch_search_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
 }
 
 template <int PS, int CG, int RG, typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kNarrowThreads)
 seg_patch_search_kernel(const __grid_constant__ SegTable<SegSearch> tab)
 {
     int b;
@@ -785,14 +846,11 @@ void search_ps(const T *I0, const T *I0x, const T *I0y, const T *I1,
                float *up, size_t upfs, int frames, const FlowParams &fp, int *err, cudaStream_t st)
 {
     using SS = SearchShape<PS>;
-    const int np = lv.npx * lv.npy;
-    const bool wide = search_wide(np);
-    const int G = wide ? SS::kWideCG * SS::kWideRG : SS::kNarrowCG * SS::kNarrowRG;
-    const int per_block = 128 / G;
-    dim3 grd((np + per_block - 1) / per_block, frames);
+    const bool wide = search_wide(lv.npx * lv.npy);
+    dim3 grd(search_blocks(PS, wide, lv.npx, lv.npy), frames);
     auto kern = wide ? patch_search_kernel<PS, SS::kWideCG, SS::kWideRG, T>
                      : patch_search_kernel<PS, SS::kNarrowCG, SS::kNarrowRG, T>;
-    kern<<<grd, 128, 0, st>>>(
+    kern<<<grd, search_threads(wide), 0, st>>>(
         I0, I0x, I0y, I1, lv.w, lv.h, lv.pitch, pfs, lv.npx, lv.npy, Uc, lvc ? lvc->w : 0,
         lvc ? lvc->h : 0, lvc ? lvc->pitch : 0, lvc ? lvc->plane : 0, ucfs, up, upfs, fp.stride,
         fp.gn_iters, fp.gn_damping, err);
@@ -1003,9 +1061,9 @@ float *launch_variational(const void *I0, const void *I0x, const void *I0y, cons
 
 bool search_wide(int n_patches) { return n_patches >= kWideSearchPatches; }
 
-int search_patches_per_block(int ps, bool wide)
+int search_blocks(int ps, bool wide, int npx, int npy)
 {
-    int G = 0;
+    int G = 32;
 #define EBOF_G(N)                                                                                \
     case N:                                                                                      \
         G = wide ? SearchShape<N>::kWideCG * SearchShape<N>::kWideRG                             \
@@ -1017,7 +1075,10 @@ int search_patches_per_block(int ps, bool wide)
         default: break;
     }
 #undef EBOF_G
-    return G > 0 ? 128 / G : 0;
+    const int tw = search_tile_w(32 / G), th = 32 / G / tw;
+    const int warps = ((npx + tw - 1) / tw) * ((npy + th - 1) / th);
+    const int per_block = search_threads(wide) / 32;
+    return (warps + per_block - 1) / per_block;
 }
 
 void launch_seg_pyr_means(const SegTable<SegPyr> &t, int blocks, bool half, cudaStream_t st)
@@ -1046,11 +1107,11 @@ void launch_seg_search(const SegTable<SegSearch> &t, int blocks, int ps, bool wi
         if (half)                                                                                \
             (wide ? seg_patch_search_kernel<N, SS::kWideCG, SS::kWideRG, __half>                 \
                   : seg_patch_search_kernel<N, SS::kNarrowCG, SS::kNarrowRG, __half>)            \
-                <<<blocks, 128, 0, st>>>(t);                                                     \
+                <<<blocks, search_threads(wide), 0, st>>>(t);                                    \
         else                                                                                     \
             (wide ? seg_patch_search_kernel<N, SS::kWideCG, SS::kWideRG, float>                  \
                   : seg_patch_search_kernel<N, SS::kNarrowCG, SS::kNarrowRG, float>)             \
-                <<<blocks, 128, 0, st>>>(t);                                                     \
+                <<<blocks, search_threads(wide), 0, st>>>(t);                                    \
         break;                                                                                   \
     }
     switch (ps) {

@@ -115,36 +115,6 @@ __device__ __forceinline__ float2 ldf2(const float *p)
 }
 
 
-// (u, v) pairs in one 64-bit register: the packed FP32 instructions round each
-// half as the scalar ones do.  A packed multiply-add holds the FMA pipe as long
-// as two scalar ones (measured: 2.0 cycles a warp against 1.0), but takes one
-// issue slot: the sweeps are bound by issue, not by that pipe.
-typedef unsigned long long pair_t;
-__device__ __forceinline__ pair_t pk(float a, float b)
-{
-    pair_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 upk(pair_t v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ pair_t ffma2(pair_t a, pair_t b, pair_t c)
-{
-    pair_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ pair_t fmul2(pair_t a, pair_t b)
-{
-    pair_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // A thread's strip of 2 columns x VS rows: the pixels' systems, the weights of
 // their edges (right: of column 1 only, column 0's is column 1's left one;
 // down: of the last row only) and (du, dv).
@@ -992,21 +962,6 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int p
 }
 
 // ---------------------------------------------------------------- resident levels
-// Packed operations beside ffma2 and fmul2.  The compiler fuses a packed
-// product into a packed sum that follows it (whatever the rounding suffix), so
-// a product whose rounding matters is added by scalar operations.
-__device__ __forceinline__ pair_t fadd2(pair_t a, pair_t b)
-{
-    pair_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ pair_t fsub2(pair_t a, pair_t b)
-{
-    pair_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
 __device__ __forceinline__ pair_t dup(float a) { return pk(a, a); }
 __device__ __forceinline__ pair_t neg2(pair_t a)
 {

@@ -163,7 +163,7 @@ void launch_seg_flow_out(const SegTable<SegFlowOut> &t, int blocks, cudaStream_t
 // Block shapes the host needs to build the tables.
 int edt_rows_block_rows(int W);        // rows per block of the one-warp row layout
 size_t edt_rows_smem(int W, int rows);  // dynamic shared memory of such a block
-int search_patches_per_block(int ps, bool wide);
+int search_blocks(int ps, bool wide, int npx, int npy);
 bool search_wide(int n_patches);
 int sor_halo(int var_sor);             // halo of a SOR region (odd)
 int sor_tile(int R);                   // interior side of a 64 x 64 SOR region
