@@ -1288,7 +1288,8 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
                 a.npx = lv.npx;
                 a.npy = lv.npy;
                 a.ps = p.patch;
-                a.stride = p.stride;
+                a.stride = std::min(p.stride, kMaxDim);
+                a.magic = densify_magic(a.stride);
                 a.gx = (lv.w + 31) / 32;
                 a.gy = (lv.h + 7) / 8;
                 const int nc = (p.patch + p.stride - 1) / p.stride;

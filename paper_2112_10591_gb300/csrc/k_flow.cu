@@ -561,14 +561,23 @@ seg_patch_search_kernel(const __grid_constant__ SegTable<SegSearch> tab)
 }
 
 // ---------------------------------------------------------------- A7
-__device__ __forceinline__ void cover_range(int x, int n, int ps, int stride, int cnt, int &lo,
-                                            int &hi, bool &last)
+// x / s for 0 <= x < 2^15 and 1 <= s < 2^15: x s < 2^31, so rounding the
+// reciprocal up never reaches the next integer.  magic = 2^31 / s + 1.
+inline uint32_t stride_magic(int s) { return (uint32_t)((1u << 31) / (uint32_t)s + 1); }
+__device__ __forceinline__ int div_stride(int x, uint32_t magic)
+{
+    return (int)(((unsigned long long)(uint32_t)x * magic) >> 31);
+}
+
+// The patches that cover x along an axis of n: the regular ones lo .. hi, and
+// whether the last one does.
+__device__ __forceinline__ void cover_range(int x, int n, int ps, int stride, uint32_t magic,
+                                            int cnt, int &lo, int &hi, bool &last)
 {
     // regular patches k < cnt - 1 have origin k * stride; the last one is
     // flush with the border at n - ps
-    const int t = x - ps + 1;
-    lo = t <= 0 ? 0 : (t + stride - 1) / stride;
-    hi = min(cnt - 2, x / stride);
+    lo = div_stride(max(x - ps + stride, 0), magic);
+    hi = min(cnt - 2, div_stride(x, magic));
     last = x >= n - ps;
 }
 
@@ -597,55 +606,125 @@ __device__ __forceinline__ float dense_sample(const T *__restrict__ I1, int w, i
     return bilinear_i(I1, w, h, pitch, (float)x + u, (float)y + v);
 }
 
-// (bx, by): the 32 x 8 tile, f: the frame.
+// The patches that cover a block's tile, staged once: their displacement, its
+// fraction and its whole-pixel part as an offset.  At most 36 x 12 of them
+// where NC <= 4 (a stride of 1 with 4 x 4 patches).
+constexpr int kDenseX = 36, kDenseY = 12;
+
+// (bx, by): the 32 x 8 tile, f: the frame.  NC > 0: a block whose patches'
+// samples all lie inside the level takes them from the staged values, without
+// the floors, conversions and border tests of every pixel (each on the slow
+// pipe, nine times a pixel at 12 x 12 patches and stride 4); other blocks
+// sample patch by patch.  The arithmetic is the same.
 template <typename T, int NC>
 __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T *__restrict__ I1b,
                                              int w, int h, int pitch, size_t pfs,
                                              const float *__restrict__ upb, size_t upfs, int npx,
                                              int npy, float *__restrict__ Ub, size_t ufs,
-                                             size_t plane, int ps, int stride, unsigned bx,
-                                             unsigned by, unsigned f)
+                                             size_t plane, int ps, int stride, uint32_t magic,
+                                             unsigned bx, unsigned by, unsigned f)
 {
     const int x = bx * 32 + threadIdx.x;
     const int y = by * 8 + threadIdx.y;
-    if (x >= w || y >= h) return;
+    const bool px = x < w && y < h;
     const T *I0 = I0b + (size_t)f * pfs, *I1 = I1b + (size_t)f * pfs;
     const float *up = upb + (size_t)f * upfs;
     const float *vp = up + npx * npy;
+    const int p = y * pitch + x;
+    const float i0 = px ? ldp(&I0[p]) : 0.0f;
     int ilo, ihi, jlo, jhi;
     bool ilast, jlast;
-    cover_range(x, w, ps, stride, npx, ilo, ihi, ilast);
-    cover_range(y, h, ps, stride, npy, jlo, jhi, jlast);
-    const float i0 = ldp(&I0[y * pitch + x]);
+    cover_range(x, w, ps, stride, magic, npx, ilo, ihi, ilast);
+    cover_range(y, h, ps, stride, magic, npy, jlo, jhi, jlast);
     float nu = 0.0f, nv = 0.0f, den = 0.0f;
-    auto add = [&](int id) {
-        const float u = up[id], v = vp[id];
-        const float r = dense_sample(I1, w, h, pitch, x, y, u, v) - i0;
+    auto weigh = [&](float sample, float u, float v) {
+        const float r = sample - i0;
         const float lam = 1.0f / fmaxf(1.0f, fabsf(r));
         nu += lam * u; nv += lam * v; den += lam;
     };
-    // the patches of row j: regular columns, then the flush one
-    auto row = [&](int j) {
-        const int base = j * npx;
-        if (NC > 0) {
-#pragma unroll
-            for (int di = 0; di < (NC > 0 ? NC : 1); ++di)
-                if (ilo + di <= ihi) add(base + ilo + di);
-        } else {
-            for (int i = ilo; i <= ihi; ++i) add(base + i);
-        }
-        if (ilast) add(base + npx - 1);
-    };
+    bool staged = false;
     if (NC > 0) {
+        __shared__ float4 s_uv[kDenseY][kDenseX];
+        __shared__ int s_off[kDenseY][kDenseX];
+        // the tile's patches: columns ti .. ti + ni - 1, then the flush one
+        int ti, tj, ie, je, lo;
+        bool fx, fy;
+        cover_range(min((int)bx * 32 + 31, w - 1), w, ps, stride, magic, npx, lo, ie, fx);
+        cover_range(min((int)by * 8 + 7, h - 1), h, ps, stride, magic, npy, lo, je, fy);
+        ti = div_stride(max((int)bx * 32 - ps + stride, 0), magic);
+        tj = div_stride(max((int)by * 8 - ps + stride, 0), magic);
+        const int ni = max(ie - ti + 1, 0), nj = max(je - tj + 1, 0);
+        bool in = true;
+        for (int jj = threadIdx.y; jj < nj + fy; jj += 8)
+            for (int ii = threadIdx.x; ii < ni + fx; ii += 32) {
+                const int i = ii < ni ? ti + ii : npx - 1, j = jj < nj ? tj + jj : npy - 1;
+                const float u = up[j * npx + i], v = vp[j * npx + i];
+                const float fu = floorf(u), fv = floorf(v);
+                const float ox = (float)min(i * stride, w - ps) + fu;
+                const float oy = (float)min(j * stride, h - ps) + fv;
+                const bool ok = ox >= 0.0f && ox + (float)ps <= (float)(w - 1) && oy >= 0.0f &&
+                                oy + (float)ps <= (float)(h - 1);
+                in = in && ok;
+                s_uv[jj][ii] = make_float4(u, v, u - fu, v - fv);
+                s_off[jj][ii] = ok ? (int)fv * pitch + (int)fu : 0;
+            }
+        staged = __syncthreads_and(in);
+        if (staged && px) {
+            const T *q = I1 + p;
+            auto add = [&](const float4 *m4, const int *off) {
+                const float4 m = *m4;
+                const float ax = m.z, ay = m.w;
+                const T *r0 = q + *off, *r1 = r0 + pitch;
+                const float a = ldp(&r0[0]), b = ldp(&r0[1]), c = ldp(&r1[0]), d = ldp(&r1[1]);
+                weigh((1.0f - ay) * ((1.0f - ax) * a + ax * b) +
+                          ay * ((1.0f - ax) * c + ax * d),
+                      m.x, m.y);
+            };
+            // every pixel of the tile has exactly NC x NC regular patches:
+            // no test stands between the loads of one patch and the next
+            if (NC * stride == ps && (int)bx * 32 >= ps - stride && ie <= npx - 2 && !fx &&
+                (int)by * 8 >= ps - stride && je <= npy - 2 && !fy &&
+                div_stride(min((int)bx * 32 + 31, w - 1), magic) <= npx - 2 &&
+                div_stride(min((int)by * 8 + 7, h - 1), magic) <= npy - 2) {
+                const float4 *m = &s_uv[jlo - tj][ilo - ti];
+                const int *o = &s_off[jlo - tj][ilo - ti];
 #pragma unroll
-        for (int dj = 0; dj < (NC > 0 ? NC : 1); ++dj)
-            if (jlo + dj <= jhi) row(jlo + dj);
-    } else {
-        for (int j = jlo; j <= jhi; ++j) row(j);
+                for (int dj = 0; dj < (NC > 0 ? NC : 1); ++dj)
+#pragma unroll
+                    for (int di = 0; di < (NC > 0 ? NC : 1); ++di)
+                        add(m + dj * kDenseX + di, o + dj * kDenseX + di);
+                ilo = INT_MAX / 2;  // done
+                ilast = jlast = false;
+                jhi = -1;
+            }
+            auto row = [&](int jj) {
+                const float4 *m = &s_uv[jj][ilo - ti];
+                const int *o = &s_off[jj][ilo - ti];
+#pragma unroll
+                for (int di = 0; di < (NC > 0 ? NC : 1); ++di)
+                    if (ilo + di <= ihi) add(m + di, o + di);
+                if (ilast) add(&s_uv[jj][ni], &s_off[jj][ni]);
+            };
+#pragma unroll
+            for (int dj = 0; dj < (NC > 0 ? NC : 1); ++dj)
+                if (jlo + dj <= jhi) row(jlo - tj + dj);
+            if (jlast) row(nj);
+        }
     }
-    if (jlast) row(npy - 1);
+    if (!px) return;
+    if (!staged) {
+        auto add = [&](int id) {
+            const float u = up[id], v = vp[id];
+            weigh(dense_sample(I1, w, h, pitch, x, y, u, v), u, v);
+        };
+        auto row = [&](int j) {
+            for (int i = ilo; i <= ihi; ++i) add(j * npx + i);
+            if (ilast) add(j * npx + npx - 1);
+        };
+        for (int j = jlo; j <= jhi; ++j) row(j);
+        if (jlast) row(npy - 1);
+    }
     float *U = Ub + (size_t)f * ufs;
-    const int p = y * pitch + x;
     U[p] = den > 0.0f ? nu / den : 0.0f;
     (U + plane)[p] = den > 0.0f ? nv / den : 0.0f;
 }
@@ -654,10 +733,11 @@ template <typename T, int NC>
 __global__ void __launch_bounds__(256)
 densify_kernel(const T *__restrict__ I0b, const T *__restrict__ I1b, int w, int h, int pitch,
                size_t pfs, const float *__restrict__ upb, size_t upfs, int npx, int npy,
-               float *__restrict__ Ub, size_t ufs, size_t plane, int ps, int stride)
+               float *__restrict__ Ub, size_t ufs, size_t plane, int ps, int stride,
+               uint32_t magic)
 {
     densify_body<T, NC>(I0b, I1b, w, h, pitch, pfs, upb, upfs, npx, npy, Ub, ufs, plane, ps,
-                        stride, blockIdx.x, blockIdx.y, blockIdx.z);
+                        stride, magic, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 template <typename T, int NC>
@@ -668,8 +748,8 @@ seg_densify_kernel(const __grid_constant__ SegTable<SegDensify> tab)
     const SegDensify &a = seg_of(tab, b);
     const int r = b / a.gx;
     densify_body<T, NC>((const T *)a.I0, (const T *)a.I1, a.w, a.h, a.pitch, a.pfs, a.up, a.upfs,
-                        a.npx, a.npy, a.U, a.ufs, a.plane, a.ps, a.stride, b % a.gx, r % a.gy,
-                        r / a.gy);
+                        a.npx, a.npy, a.U, a.ufs, a.plane, a.ps, a.stride, a.magic, b % a.gx,
+                        r % a.gy, r / a.gy);
 }
 
 // ---------------------------------------------------------------- A8
@@ -980,11 +1060,14 @@ void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_
     const dim3 grd = grid2d(lv.w, lv.h, frames, blk);
     // regular patches covering a pixel per axis: at most ceil(ps / stride)
     const int nc = (fp.ps + fp.stride - 1) / fp.stride;
+    // no patch beyond the border: a longer stride is the same grid
+    const int stride = std::min(fp.stride, kMaxDim);
+    const uint32_t magic = stride_magic(stride);
 #define EBOF_DENSE(T, N)                                                                         \
     densify_kernel<T, N><<<grd, blk, 0, st>>>((const T *)I0, (const T *)I1, lv.w, lv.h,         \
                                               lv.pitch, pyr_frame_stride, up, up_frame_stride,   \
                                               lv.npx, lv.npy, U, u_frame_stride, lv.plane, fp.ps,\
-                                              fp.stride)
+                                              stride, magic)
     if (fp.half) {
         if (nc == 2) EBOF_DENSE(__half, 2);
         else if (nc == 3) EBOF_DENSE(__half, 3);
@@ -1058,6 +1141,8 @@ float *launch_variational(const void *I0, const void *I0x, const void *I0y, cons
                           work_frame_stride, frames, fp, st);
     return U;
 }
+
+uint32_t densify_magic(int stride) { return stride_magic(stride); }
 
 bool search_wide(int n_patches) { return n_patches >= kWideSearchPatches; }
 

@@ -110,6 +110,7 @@ struct SegDensify {
     float *U;
     size_t pfs, upfs, ufs, plane;
     int w, h, pitch, npx, npy, ps, stride, gx, gy;
+    uint32_t magic;  // densify_magic(stride)
 };
 
 // A8: the coefficient tiles (gx x gy per frame) of one outer iteration.
@@ -163,6 +164,7 @@ void launch_seg_flow_out(const SegTable<SegFlowOut> &t, int blocks, cudaStream_t
 // Block shapes the host needs to build the tables.
 int edt_rows_block_rows(int W);        // rows per block of the one-warp row layout
 size_t edt_rows_smem(int W, int rows);  // dynamic shared memory of such a block
+uint32_t densify_magic(int stride);      // the stride's reciprocal (at most kMaxDim)
 int search_blocks(int ps, bool wide, int npx, int npy);
 bool search_wide(int n_patches);
 int sor_halo(int var_sor);             // halo of a SOR region (odd)
