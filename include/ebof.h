@@ -90,9 +90,8 @@ typedef struct {
      * never what is computed.  Every setting gives the same flow bit for bit
      * (the per-pixel arithmetic has a fixed rounding sequence in every kernel
      * form), so the autotuner picks them by time alone. */
-    int32_t coeff_cw_min_width; /* levels at least this wide build their linear systems
-                                   with the column-walk kernel (a warp per 28 columns x 8
-                                   rows), narrower ones with 32x12 tiles; >= 1 (1024) */
+    int32_t coeff_cw_min_width; /* >= 1 (1024); checked, without effect: the coefficient
+                                   kernel has one form and picks its tile by the grid */
     int32_t sor_tma_min_per_sm; /* SOR grids with at least this many 64x64 regions per
                                    SM take the persistent copy-ahead kernel; >= 1 (2) */
     int32_t sor_row_waves;      /* SOR grids that fit this many waves of 64x32 regions
@@ -102,8 +101,7 @@ typedef struct {
                                    order always takes it where its regions fit one
                                    wave; calls of several frames do so for levels of
                                    at most this many regions a frame; 0 = never (0) */
-    int32_t coeff_cw_rows;      /* rows a warp of the column-walk kernel walks down (the
-                                   strip's height): 4, 8 or 16 (8) */
+    int32_t coeff_cw_rows;      /* 4, 8 or 16 (8); checked, without effect */
 } ebof_params;
 
 /* Distance surface built from the EDT (§III-C) and handed to the flow block.
@@ -138,9 +136,9 @@ typedef struct ebof_stream ebof_stream;
  * of 12x12 patches from 640 px, stride 4, 12 Gauss-Newton iterations with
  * damping 0.1, 5 x 5
  * variational iterations (delta 5, gamma 10, alpha 20, omega 1.6),
- * max_batch 1, FP32 storage; layouts: column walk from 1024 px, copy-ahead
- * SOR from 2 regions per SM, two-row SOR strips for one-wave grids, no
- * one-launch refinement for several frames. */
+ * max_batch 1, FP32 storage; layouts: copy-ahead SOR from 2 regions per SM,
+ * two-row SOR strips for one-wave grids, no one-launch refinement for several
+ * frames. */
 void ebof_default_params(ebof_params *p, int32_t width, int32_t height);
 
 /* Eq. 2 with eps = 1/255 (Eq. 3): alpha = d_sat / ln(255). */

@@ -15,8 +15,7 @@ tuner itself only orchestrates and compares.
    path of a candidate configuration matches the FP64 oracle is a property
    of the library, covered by its tests; the tuner runs in the product path,
    which never touches the oracle.
-2. Layout candidates (the coefficient kernel's form and the height of its
-   column-walk strips, the SOR kernels' forms: the persistent copy-ahead
+2. Layout candidates (the SOR kernels' forms: the persistent copy-ahead
    kernel, regions of two-row strips; the one-launch refinement of small
    levels) never change the flow.  The tuner checks that each one gives the flow of
    the default layout bit for bit and keeps the fastest, one knob at a time
@@ -34,11 +33,9 @@ from . import binding as eb
 # and the values tried besides the default.
 NEVER = 1 << 20
 LAYOUT_CANDIDATES = {
-    "coeff_cw_min_width": (640, NEVER),
     "sor_tma_min_per_sm": (1, 4, NEVER),
     "sor_row_waves": (0, 2),
     "var_cluster_max": (8, 16),
-    "coeff_cw_rows": (4, 16),
 }
 
 

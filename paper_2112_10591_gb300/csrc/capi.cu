@@ -390,11 +390,9 @@ FlowParams flow_params(const ebof_params &p)
     fp.alpha_s = p.var_alpha;
     fp.omega = p.sor_omega;
     fp.wait_limit = kWaitLimitDefault;
-    fp.coeff_cw_min_width = p.coeff_cw_min_width;
     fp.sor_tma_min_per_sm = p.sor_tma_min_per_sm;
     fp.sor_row_waves = p.sor_row_waves;
     fp.var_cluster_max = p.var_cluster_max;
-    fp.coeff_cw_rows = p.coeff_cw_rows;
     fp.level_ctl = nullptr;
     return fp;
 }
@@ -1184,8 +1182,6 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
     // left runs that group's own launches (with its own layouts).
     int Lmax = 0;
     for (GS &x : gs) Lmax = std::max(Lmax, x.g->geo.levels);
-    int cax = 32, cay = 12;
-    coeff_tile_shape(cax, cay);
     for (int j = 0; j < Lmax; ++j) {
         int active = 0;
         for (GS &x : gs) active += j < x.g->geo.levels;
@@ -1342,8 +1338,8 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
                 c.w = lv.w;
                 c.h = lv.h;
                 c.pitch = lv.pitch;
-                c.gx = (lv.w + cax - 1) / cax;
-                c.gy = (lv.h + cay - 1) / cay;
+                c.gx = coeff_tiles_x(lv.w);
+                c.gy = coeff_tiles_y(lv.h);
                 c.delta = fp.delta;
                 c.gamma = fp.gamma;
                 c.alpha_s = fp.alpha_s;

@@ -87,7 +87,7 @@ struct FlowParams {
     float delta, gamma, alpha_s, omega;
     long long wait_limit;  // first wait of the copy-ahead SOR kernel (rounds)
     // variational layouts (ebof_params): none changes a result
-    int coeff_cw_min_width, sor_tma_min_per_sm, sor_row_waves, var_cluster_max, coeff_cw_rows;
+    int sor_tma_min_per_sm, sor_row_waves, var_cluster_max;
     // the counters of the one-launch refinement (kLevelCtl words that are 0
     // between launches and used by no other launch at the same time), or null:
     // one launch per step

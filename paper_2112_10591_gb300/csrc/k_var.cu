@@ -1,15 +1,21 @@
 // k_var.cu -- variational refinement (reading F6): two kernels per
 // fixed-point iteration.
 //
-// var_coeff_kernel, one thread per pixel: stages U and the warped image
-// I1(x + U) for a 32x12 tile plus 2 px in shared memory, builds derivatives
-// of the warped image and the smoothness weights, and writes every pixel's
-// 2x2 linear system (data and gradient-constancy terms normalised, weights
-// lagged at dU = 0): omega/a11, omega/a22 (the SOR relaxation factor folded
-// into the inverted diagonal), a12, b1, b2 and the smoothness weight, as six
-// planes.  Only the staging halo is shared between tiles.  On levels from
-// 1024 px wide the same systems come from var_coeff_cw_kernel, a column walk
-// with the rows in registers.
+// var_coeff_kernel: a block stages U and the warped image I1(x + U) for a tile
+// of 64 columns plus 2 px in shared memory, builds the derivatives of the
+// warped image and the smoothness weights, and writes every pixel's 2x2 linear
+// system (data and gradient-constancy terms normalised, weights lagged at
+// dU = 0): omega/a11, omega/a22 (the SOR relaxation factor folded into the
+// inverted diagonal), a12, b1, b2 and the smoothness weight, as six planes.
+// Everything is done on pairs of adjacent pixels with packed FP32 operations.
+// What bounds it: issue slots (a scalar form took 340 instructions a pixel row
+// of 32) and, once those are halved, the latency of the flow and the image's
+// taps, which is why the rows are staged by a block of independent threads: a
+// warp that walks its columns down with the rows in registers needs as few
+// instructions but only four warps a scheduler fit.  Measured in a graph,
+// against the scalar column walk (levels from 1024 px) and scalar 32x12 tiles:
+// 1280x720 14.3 -> 12.7 us for one frame, 103 -> 89 for eight (pairs in a
+// column walk: 12.1 and 92); 640x360 5.8 -> 5.0 and 34 -> 25; 160x90 3.1 -> 2.9.
 //
 // SOR: one block owns a 64x64 region and refines the flow of its
 // (64 - 2R)^2 interior, R = 2 * sweeps - 1.  It loads the region's linear
@@ -87,11 +93,6 @@ constexpr size_t kTmaSmemBytes =
     kTmaCoefFloats * sizeof(float) + flow_stage_bytes<kVS, kVWarps>();
 constexpr int kMaxDevs = 64;
 int g_num_sms[kMaxDevs];
-// coefficient tile: 384 threads at 40 registers, four blocks per SM, so a
-// 640 x 360 level (600 tiles) takes one wave where 32 x 16 tiles took two
-constexpr int kAX = 32, kAY = 12;
-constexpr int kAEX = kAX + 4, kAEY = kAY + 4;  // staging window: tile + 2 px
-constexpr int kADX = kAX + 2, kADY = kAY + 2;  // derivative window: tile + 1 px
 constexpr unsigned kFull = 0xffffffffu;
 
 // Loads of data that the same launch may have written on another SM earlier
@@ -257,398 +258,6 @@ __device__ __forceinline__ void edge_weights(Strip<VS> &s, const float (&as)[VS 
     const bool yd = !last && (INSIDE || (gy + VS > 0 && gy + VS < h));
 #pragma unroll
     for (int q = 0; q < 2; ++q) s.wd[q] = yd ? mean(as[VS + 1][q], as[VS][q]) : 0.0f;
-}
-
-// Smoothness weight alpha_s Psi'(|grad u|^2 + |grad v|^2) with forward
-// differences (ur, ud: U to the right and below; hx, hy: those neighbours are
-// in the level, else the difference is 0).
-__device__ __forceinline__ float smooth_weight(float u, float ur, float ud, float v, float vr,
-                                               float vd, bool hx, bool hy, float alpha_s)
-{
-    const float ux = hx ? fsub(ur, u) : 0.0f;
-    const float uy = hy ? fsub(ud, u) : 0.0f;
-    const float vx = hx ? fsub(vr, v) : 0.0f;
-    const float vy = hy ? fsub(vd, v) : 0.0f;
-    return fmul(alpha_s, psi_prime(ffma(vy, vy, ffma(vx, vx, ffma(uy, uy, fmul(ux, ux))))));
-}
-
-__device__ __forceinline__ float cdiff(float hi, float lo) { return fmul(0.5f, fsub(hi, lo)); }
-
-// Derivatives of the warped image and the smoothness weight at a pixel of a
-// staging window (row stride ES; (e) the pixel, at image position gx, gy).
-// IN: the pixel and its neighbours lie inside the level, so the clamps and
-// border tests are known to pass and are left out (same values).
-template <bool IN>
-__device__ __forceinline__ void stage_derivs(const float *sW, const float *sU, const float *sV,
-                                             int ES, int e, int ex0, int ey0, int gx, int gy,
-                                             int w, int h, float alpha_s, float &ix, float &iy,
-                                             float &as)
-{
-    const int xp = (IN ? gx + 1 : min(gx + 1, w - 1)) - ex0;
-    const int xm = (IN ? gx - 1 : max(gx - 1, 0)) - ex0;
-    const int yp = (IN ? gy + 1 : min(gy + 1, h - 1)) - ey0;
-    const int ym = (IN ? gy - 1 : max(gy - 1, 0)) - ey0;
-    const int ex = gx - ex0, ey = gy - ey0;
-    ix = cdiff(sW[ey * ES + xp], sW[ey * ES + xm]);
-    iy = cdiff(sW[yp * ES + ex], sW[ym * ES + ex]);
-    as = smooth_weight(sU[e], sU[e + 1], sU[e + ES], sV[e], sV[e + 1], sV[e + ES],
-                       IN || gx + 1 < w, IN || gy + 1 < h, alpha_s);
-}
-
-struct PixelSystem {
-    float i11, i22, a12, b1, b2;
-};
-
-// The 2x2 system of pixel (gx, gy) from its neighbourhood.  ix, iy: the
-// warped image's derivatives at the pixel; ixl, ixr: Ix at the clamped left
-// and right neighbours, ixu, ixd and iyu, iyd: Ix and Iy at the clamped upper
-// and lower ones; iw: the warped sample; as*: smoothness weights at the pixel
-// and its four neighbours, used only where that neighbour is in the level
-// (bl, br, bu, bd); u*, v*: the flow at the pixel and its four neighbours (0
-// outside the level); i0, i0x, i0y: the template image and its gradient.
-// The diagonal is stored inverted and scaled by the SOR relaxation factor:
-// i11 = omega / a11, i22 = omega / a22.
-__device__ __forceinline__ PixelSystem pixel_system_vals(
-    float ix, float iy, float ixl, float ixr, float ixu, float ixd, float iyu, float iyd,
-    float iw, float asp, float asl, float asr, float asu, float asd, float u, float ul, float ur,
-    float uu, float ud, float v, float vl, float vr, float vu, float vd, bool bl, bool br,
-    bool bu, bool bd, int gx, int gy, int w, int h, float i0, float i0x, float i0y, float delta,
-    float gamma, float omega)
-{
-    // every operation with a fixed rounding (fmul, fadd, fsub, ffma), so that
-    // the two kernel forms that call this function give the same systems
-    const float Ix = ix, Iy = iy;
-    const float Ixx = cdiff(ixr, ixl);
-    const float Ixy = cdiff(ixd, ixu);
-    const float Iyy = cdiff(iyd, iyu);
-    const float Iz = fsub(iw, i0);
-    const float Ixz = fsub(Ix, i0x), Iyz = fsub(Iy, i0y);
-    const float nd = __fdividef(1.0f, fadd(ffma(Iy, Iy, fmul(Ix, Ix)), kZeta2));
-    const float ng = __fdividef(
-        1.0f, fadd(ffma(Iyy, Iyy, ffma(fmul(2.0f, Ixy), Ixy, fmul(Ixx, Ixx))), kZeta2));
-    float ad = fmul(fmul(delta, nd), psi_prime(fmul(fmul(nd, Iz), Iz)));
-    float ag = fmul(fmul(gamma, ng), psi_prime(fmul(ng, ffma(Iyz, Iyz, fmul(Ixz, Ixz)))));
-    const float wx = fadd((float)gx, u), wy = fadd((float)gy, v);
-    if (wx < 0.0f || wx > (float)(w - 1) || wy < 0.0f || wy > (float)(h - 1)) {
-        ad = 0.0f;
-        ag = 0.0f;
-    }
-    PixelSystem ps;
-    const float cl = bl ? fmul(0.5f, fadd(asp, asl)) : 0.0f;
-    const float cr = br ? fmul(0.5f, fadd(asp, asr)) : 0.0f;
-    const float cu = bu ? fmul(0.5f, fadd(asp, asu)) : 0.0f;
-    const float cd = bd ? fmul(0.5f, fadd(asp, asd)) : 0.0f;
-    const float sw = fadd(fadd(fadd(cl, cr), cu), cd);
-    const float su0 = ffma(cd, fsub(ud, u),
-                           ffma(cu, fsub(uu, u), ffma(cr, fsub(ur, u),
-                                                         fmul(cl, fsub(ul, u)))));
-    const float sv0 = ffma(cd, fsub(vd, v),
-                           ffma(cu, fsub(vu, v), ffma(cr, fsub(vr, v),
-                                                         fmul(cl, fsub(vl, v)))));
-    const float adx = fmul(ad, Ix), ady = fmul(ad, Iy);
-    ps.i11 = __fdividef(omega, fadd(ffma(ag, ffma(Ixy, Ixy, fmul(Ixx, Ixx)), fmul(adx, Ix)), sw));
-    ps.i22 = __fdividef(omega, fadd(ffma(ag, ffma(Iyy, Iyy, fmul(Ixy, Ixy)), fmul(ady, Iy)), sw));
-    ps.a12 = ffma(ag, ffma(Ixy, Iyy, fmul(Ixx, Ixy)), fmul(adx, Iy));
-    ps.b1 = ffma(-ag, ffma(Ixy, Iyz, fmul(Ixx, Ixz)), ffma(-adx, Iz, su0));
-    ps.b2 = ffma(-ag, ffma(Iyy, Iyz, fmul(Ixy, Ixz)), ffma(-ady, Iz, sv0));
-    return ps;
-}
-
-// The same system read from the staging and derivative windows: d indexes
-// the derivative window (row stride DS, origin dx0, dy0), e the staging
-// window (row stride ES).  Every index read lies in the windows (their rings
-// hold 0 outside the level).  IN as in stage_derivs.
-template <bool IN>
-__device__ __forceinline__ PixelSystem pixel_system(const float *sIx, const float *sIy,
-                                                    const float *sAs, int DS, int dx0, int dy0,
-                                                    const float *sW, const float *sU,
-                                                    const float *sV, int ES, int e, int gx,
-                                                    int gy, int w, int h, float i0, float i0x,
-                                                    float i0y, float delta, float gamma,
-                                                    float omega)
-{
-    const int xp = (IN ? gx + 1 : min(gx + 1, w - 1)) - dx0;
-    const int xm = (IN ? gx - 1 : max(gx - 1, 0)) - dx0;
-    const int yp = (IN ? gy + 1 : min(gy + 1, h - 1)) - dy0;
-    const int ym = (IN ? gy - 1 : max(gy - 1, 0)) - dy0;
-    const int dx = gx - dx0, dy = gy - dy0;
-    const int d = dy * DS + dx;
-    return pixel_system_vals(
-        sIx[d], sIy[d], sIx[dy * DS + xm], sIx[dy * DS + xp], sIx[ym * DS + dx],
-        sIx[yp * DS + dx], sIy[ym * DS + dx], sIy[yp * DS + dx], sW[e], sAs[d], sAs[d - 1],
-        sAs[d + 1], sAs[d - DS], sAs[d + DS], sU[e], sU[e - 1], sU[e + 1], sU[e - ES],
-        sU[e + ES], sV[e], sV[e - 1], sV[e + 1], sV[e - ES], sV[e + ES], IN || gx > 0,
-        IN || gx + 1 < w, IN || gy > 0, IN || gy + 1 < h, gx, gy, w, h, i0, i0x, i0y, delta,
-        gamma, omega);
-}
-
-// One coefficient tile.  IN: the tile's staging window (tile + 2 px) lies
-// inside the level, so no load or neighbour needs a bounds test.
-template <bool IN, typename T>
-__device__ __forceinline__ void coeff_tile(
-    float (&sU)[kAEY][kAEX], float (&sV)[kAEY][kAEX], float (&sW)[kAEY][kAEX],
-    float (&sIx)[kADY][kADX], float (&sIy)[kADY][kADX], float (&sAs)[kADY][kADX],
-    const T *__restrict__ I0b, const T *__restrict__ I0xb, const T *__restrict__ I0yb,
-    const T *__restrict__ I1b, int w, int h, int pitch, size_t pfs, const float *__restrict__ Ub,
-    size_t ufs, size_t plane, float *__restrict__ coefb, size_t cfs, float delta, float gamma,
-    float alpha_s, float omega, unsigned bx, unsigned by, unsigned f)
-{
-    const int tx0 = bx * kAX, ty0 = by * kAY;
-    const int ex0 = tx0 - 2, ey0 = ty0 - 2, dx0 = tx0 - 1, dy0 = ty0 - 1;
-    // frame base pointers once; offsets within a frame fit in 32 bits
-    const size_t po = (size_t)f * pfs;
-    const T *I1 = I1b + po;
-    const float *U = Ub + (size_t)f * ufs;
-    const float *V = U + plane;
-    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 12 threads, one per tile pixel
-
-    const int t = ty * kAX + tx;
-    constexpr int kN = kAX * kAY;
-    for (int i = t; i < kAEX * kAEY; i += kN) {
-        const int lx = i % kAEX, ly = i / kAEX;
-        const int gx = ex0 + lx, gy = ey0 + ly;
-        float u = 0.0f, v = 0.0f, wv = 0.0f;
-        if (IN || (gx >= 0 && gx < w && gy >= 0 && gy < h)) {
-            const int p = gy * pitch + gx;
-            u = U[p];
-            v = V[p];
-            wv = bilinear_i(I1, w, h, pitch, (float)gx + u, (float)gy + v);
-        }
-        sU[ly][lx] = u;
-        sV[ly][lx] = v;
-        sW[ly][lx] = wv;
-    }
-    __syncthreads();
-    for (int i = t; i < kADX * kADY; i += kN) {
-        const int lx = i % kADX, ly = i / kADX;
-        const int gx = dx0 + lx, gy = dy0 + ly;
-        float ix = 0.0f, iy = 0.0f, as = 0.0f;
-        if (IN || (gx >= 0 && gx < w && gy >= 0 && gy < h))
-            stage_derivs<IN>(&sW[0][0], &sU[0][0], &sV[0][0], kAEX,
-                             (gy - ey0) * kAEX + (gx - ex0), ex0, ey0, gx, gy, w, h, alpha_s,
-                             ix, iy, as);
-        sIx[ly][lx] = ix;
-        sIy[ly][lx] = iy;
-        sAs[ly][lx] = as;
-    }
-    __syncthreads();
-
-    const int gx = tx0 + threadIdx.x, gy = ty0 + threadIdx.y;
-    if (!IN && (gx >= w || gy >= h)) return;
-    const int p = gy * pitch + gx;
-    const PixelSystem ps = pixel_system<IN>(
-        &sIx[0][0], &sIy[0][0], &sAs[0][0], kADX, dx0, dy0, &sW[0][0], &sU[0][0], &sV[0][0], kAEX,
-        (gy - ey0) * kAEX + (gx - ex0), gx, gy, w, h, ldp(&(I0b + po)[p]), ldp(&(I0xb + po)[p]),
-        ldp(&(I0yb + po)[p]), delta, gamma, omega);
-    const int pl = (int)plane;
-    float *cf = coefb + (size_t)f * cfs + p;
-    cf[kCI11 * pl] = ps.i11;
-    cf[kCI22 * pl] = ps.i22;
-    cf[kCA12 * pl] = ps.a12;
-    cf[kCB1 * pl] = ps.b1;
-    cf[kCB2 * pl] = ps.b2;
-    cf[kCAS * pl] = sAs[ty + 1][tx + 1];
-}
-
-// (bx, by): the tile, f: the frame.
-template <typename T>
-__device__ __forceinline__ void var_coeff_body(
-    const T *__restrict__ I0b, const T *__restrict__ I0xb, const T *__restrict__ I0yb,
-    const T *__restrict__ I1b, int w, int h, int pitch, size_t pfs, const float *__restrict__ Ub,
-    size_t ufs, size_t plane, float *__restrict__ coefb, size_t cfs, float delta, float gamma,
-    float alpha_s, float omega, unsigned bx, unsigned by, unsigned f)
-{
-    __shared__ float sU[kAEY][kAEX], sV[kAEY][kAEX], sW[kAEY][kAEX];
-    __shared__ float sIx[kADY][kADX], sIy[kADY][kADX], sAs[kADY][kADX];
-    const int tx0 = bx * kAX, ty0 = by * kAY;
-    if (tx0 >= 2 && ty0 >= 2 && tx0 + kAX + 2 <= w && ty0 + kAY + 2 <= h)
-        coeff_tile<true>(sU, sV, sW, sIx, sIy, sAs, I0b, I0xb, I0yb, I1b, w, h, pitch, pfs, Ub,
-                         ufs, plane, coefb, cfs, delta, gamma, alpha_s, omega, bx, by, f);
-    else
-        coeff_tile<false>(sU, sV, sW, sIx, sIy, sAs, I0b, I0xb, I0yb, I1b, w, h, pitch, pfs, Ub,
-                          ufs, plane, coefb, cfs, delta, gamma, alpha_s, omega, bx, by, f);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kAX * kAY)
-var_coeff_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
-                 const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h,
-                 int pitch, size_t pfs, const float *__restrict__ Ub, size_t ufs, size_t plane,
-                 float *__restrict__ coefb, size_t cfs, float delta, float gamma, float alpha_s,
-                 float omega)
-{
-    var_coeff_body(I0b, I0xb, I0yb, I1b, w, h, pitch, pfs, Ub, ufs, plane, coefb, cfs, delta,
-                   gamma, alpha_s, omega, blockIdx.x, blockIdx.y, blockIdx.z);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kAX * kAY)
-seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
-{
-    int b;
-    const SegCoeff &a = seg_of(tab, b);
-    const int r = b / a.gx;
-    var_coeff_body((const T *)a.I0, (const T *)a.I0x, (const T *)a.I0y, (const T *)a.I1, a.w, a.h,
-                   a.pitch, a.pfs, a.U, a.ufs, a.plane, a.coef + kCoefShift, a.cfs, a.delta, a.gamma,
-                   a.alpha_s, a.omega, b % a.gx, r % a.gy, r / a.gy);
-}
-
-// Column-walk form of the same kernel.  A warp owns 28 output columns: lane
-// l holds column x = x0 - 2 + l, lanes 2..29 are outputs and lanes 0, 1, 30,
-// 31 the halo that the central differences and the forward differences of
-// the smoothness term need.  The warp walks R output rows down and keeps
-// the rows it needs in registers: W (the warped sample I1(x + U)) of rows
-// y .. y + 2, Ix, Iy and the smoothness weight of rows y - 1 .. y + 1, U and
-// V of rows y - 1 .. y + 2; horizontal neighbours come from lane shuffles.
-// Each row's U, V loads are issued two iterations and its bilinear taps one
-// iteration before their use.  Values of positions outside the level are 0,
-// as in the staging windows of coeff_tile, and every clamp and border test
-// is the tile form's; the arithmetic has a fixed rounding sequence (fmul,
-// fadd, ffma), so both forms write the same coefficients bit for bit.  Seven
-// blocks of 72 registers per SM: a 1280 x 720 level's 1058 blocks take one
-// wave (at eight blocks, 64 registers, the kernel spilled).
-constexpr int kCWOut = 28;   // output columns per warp
-constexpr int kCWWarps = 4;  // warps per block, row strips stacked
-constexpr int kCWRows = 8;   // output rows per warp (default; ebof_params.coeff_cw_rows)
-
-template <int R, bool IN, typename T, bool COH = false>
-__device__ __forceinline__ void coeff_strip(const T *__restrict__ I0, const T *__restrict__ I0x,
-                                            const T *__restrict__ I0y, const T *__restrict__ I1,
-                                            int w, int h, int pitch, const float *__restrict__ U,
-                                            const float *__restrict__ V, float *__restrict__ cf,
-                                            int pl, int x, int y0, bool out_lane, float delta,
-                                            float gamma, float alpha_s, float omega)
-{
-    const bool xin = IN || (x >= 0 && x < w);
-    const bool hx = IN || x + 1 < w;
-    const bool bl = IN || x > 0;
-    const int ylast = y0 + R + 1;  // last row whose W, U and V are read
-    auto row_in = [&](int r) { return IN || (r >= 0 && r < h); };
-    auto load_uv = [&](int r, float &u, float &v) {
-        u = 0.0f;
-        v = 0.0f;
-        if (row_in(r) && xin) {
-            const int p = r * pitch + x;
-            u = ldf<COH>(U + p);
-            v = ldf<COH>(V + p);
-        }
-    };
-    auto taps = [&](int r, float u, float v) {
-        BilTaps t = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (row_in(r) && xin) t = bil_taps_i(I1, w, h, pitch, (float)x + u, (float)r + v);
-        return t;
-    };
-    // neighbour in x with the clamp of the central differences
-    auto right = [&](float c) {
-        const float n = __shfl_down_sync(kFull, c, 1);
-        return (IN || x + 1 < w) ? n : c;
-    };
-    auto left = [&](float c) {
-        const float n = __shfl_up_sync(kFull, c, 1);
-        return (IN || x > 0) ? n : c;
-    };
-    // Ix, Iy and the smoothness weight of row r from W of rows r - 1 .. r + 1
-    // and U, V of rows r, r + 1
-    auto derive = [&](int r, float wm, float w0, float wp, float u0, float u1, float v0,
-                      float v1, float &ix, float &iy, float &as) {
-        ix = cdiff(right(w0), left(w0));
-        iy = cdiff((IN || r + 1 < h) ? wp : w0, (IN || r > 0) ? wm : w0);
-        as = smooth_weight(u0, __shfl_down_sync(kFull, u0, 1), u1, v0,
-                           __shfl_down_sync(kFull, v0, 1), v1, hx, IN || r + 1 < h, alpha_s);
-    };
-
-    // prologue: U, V of rows y0 - 2 .. y0 + 3, W of rows y0 - 2 .. y0 + 1,
-    // the derivatives of rows y0 - 1 and y0, the taps of row y0 + 2
-    float ua, va, ub, vb, uc, vc, ud, vd, u2, v2, u3, v3;
-    load_uv(y0 - 2, ua, va);
-    load_uv(y0 - 1, ub, vb);
-    load_uv(y0, uc, vc);
-    load_uv(y0 + 1, ud, vd);
-    load_uv(y0 + 2, u2, v2);
-    load_uv(y0 + 3, u3, v3);
-    const float wa = bil_lerp(taps(y0 - 2, ua, va));
-    const float wb = bil_lerp(taps(y0 - 1, ub, vb));
-    float wc = bil_lerp(taps(y0, uc, vc));
-    float wd = bil_lerp(taps(y0 + 1, ud, vd));
-    BilTaps t2 = taps(y0 + 2, u2, v2);
-    float ixm, iym, asm_, ix0, iy0, as0;
-    derive(y0 - 1, wa, wb, wc, ub, uc, vb, vc, ixm, iym, asm_);
-    derive(y0, wb, wc, wd, uc, ud, vc, vd, ix0, iy0, as0);
-    auto ld_t = [&](const T *a, int p) { return ldp(&a[p]); };
-    int p = y0 * pitch + x;
-    const bool pin = row_in(y0) && xin;
-    float i0 = pin ? ld_t(I0, p) : 0.0f, i0x = pin ? ld_t(I0x, p) : 0.0f;
-    float i0y = pin ? ld_t(I0y, p) : 0.0f;
-
-#pragma unroll 1
-    for (int y = y0; y < y0 + R; ++y) {
-        if (!IN && y >= h) break;
-        // W, derivatives of row y + 1
-        const float we = bil_lerp(t2);
-        float ixp, iyp, asp_;
-        derive(y + 1, wc, wd, we, ud, u2, vd, v2, ixp, iyp, asp_);
-        // loads for the next iterations
-        BilTaps t3 = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (y + 3 <= ylast) t3 = taps(y + 3, u3, v3);
-        float u4 = 0.0f, v4 = 0.0f;
-        if (y + 4 <= ylast) load_uv(y + 4, u4, v4);
-        const int pn = p + pitch;
-        const bool nin = y + 1 < y0 + R && row_in(y + 1) && xin;
-        const float n_i0 = nin ? ld_t(I0, pn) : 0.0f, n_i0x = nin ? ld_t(I0x, pn) : 0.0f;
-        const float n_i0y = nin ? ld_t(I0y, pn) : 0.0f;
-        // the system of row y
-        const PixelSystem ps = pixel_system_vals(
-            ix0, iy0, left(ix0), right(ix0), (IN || y > 0) ? ixm : ix0,
-            (IN || y + 1 < h) ? ixp : ix0, (IN || y > 0) ? iym : iy0,
-            (IN || y + 1 < h) ? iyp : iy0, wc, as0, __shfl_up_sync(kFull, as0, 1),
-            __shfl_down_sync(kFull, as0, 1), asm_, asp_, uc, __shfl_up_sync(kFull, uc, 1),
-            __shfl_down_sync(kFull, uc, 1), ub, ud, vc, __shfl_up_sync(kFull, vc, 1),
-            __shfl_down_sync(kFull, vc, 1), vb, vd, bl, hx, IN || y > 0, IN || y + 1 < h, x, y,
-            w, h, i0, i0x, i0y, delta, gamma, omega);
-        if (out_lane && xin) {
-            float *c = cf + p;
-            c[kCI11 * pl] = ps.i11;
-            c[kCI22 * pl] = ps.i22;
-            c[kCA12 * pl] = ps.a12;
-            c[kCB1 * pl] = ps.b1;
-            c[kCB2 * pl] = ps.b2;
-            c[kCAS * pl] = as0;
-        }
-        // move the windows down one row
-        ixm = ix0; iym = iy0; asm_ = as0;
-        ix0 = ixp; iy0 = iyp; as0 = asp_;
-        wc = wd; wd = we;
-        ub = uc; vb = vc; uc = ud; vc = vd; ud = u2; vd = v2; u2 = u3; v2 = v3; u3 = u4; v3 = v4;
-        t2 = t3;
-        p = pn;
-        i0 = n_i0; i0x = n_i0x; i0y = n_i0y;
-    }
-}
-
-template <int R, typename T>
-__global__ void __launch_bounds__(32 * kCWWarps, 7)
-var_coeff_cw_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
-                    const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h,
-                    int pitch, size_t pfs, const float *__restrict__ Ub, size_t ufs,
-                    size_t plane, float *__restrict__ coefb, size_t cfs, float delta,
-                    float gamma, float alpha_s, float omega)
-{
-    const int lane = threadIdx.x;
-    const int y0 = (blockIdx.y * kCWWarps + threadIdx.y) * R;
-    if (y0 >= h) return;  // the whole warp
-    const int f = blockIdx.z;
-    const int cx0 = blockIdx.x * kCWOut - 2;  // column of lane 0
-    const size_t po = (size_t)f * pfs;
-    const float *U = Ub + (size_t)f * ufs;
-    const bool out_lane = lane >= 2 && lane < 2 + kCWOut;
-    if (cx0 >= 0 && cx0 + 31 < w && y0 >= 2 && y0 + R + 1 < h)
-        coeff_strip<R, true>(I0b + po, I0xb + po, I0yb + po, I1b + po, w, h, pitch, U, U + plane,
-                             coefb + (size_t)f * cfs, (int)plane, cx0 + lane, y0, out_lane,
-                             delta, gamma, alpha_s, omega);
-    else
-        coeff_strip<R, false>(I0b + po, I0xb + po, I0yb + po, I1b + po, w, h, pitch, U,
-                              U + plane, coefb + (size_t)f * cfs, (int)plane, cx0 + lane, y0,
-                              out_lane, delta, gamma, alpha_s, omega);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
@@ -1033,6 +642,260 @@ __device__ __forceinline__ pair_t bil_lerp2(const Taps2 &t)
     return ffma2(t.fy, bot, fmul2(fsub2(one, t.fy), top));
 }
 
+constexpr int kLvW = kVR + 4;  // staged columns: 64 and 2 around
+
+// The windows of a tile of 64 columns, WH - 4 rows and 2 px around, from pixel
+// (ex, ey), ex odd.
+template <int WH>
+struct Windows {
+    float *U, *V, *W, *Ix, *Iy, *As;
+    __device__ __forceinline__ explicit Windows(float *m)
+        : U(m), V(U + kLvW * WH), W(V + kLvW * WH), Ix(W + kLvW * WH), Iy(Ix + kLvW * WH),
+          As(Iy + kLvW * WH)
+    {
+    }
+    static constexpr size_t kBytes = (size_t)6 * kLvW * WH * sizeof(float);
+};
+__device__ __forceinline__ pair_t ld_pair(const float *a)
+{
+    return *reinterpret_cast<const pair_t *>(a);
+}
+__device__ __forceinline__ void st_pair(float *a, pair_t v)
+{
+    *reinterpret_cast<pair_t *>(a) = v;
+}
+
+// The flow of the window and the warped image there.  Positions outside the
+// level are those of the nearest pixel inside: the replicated borders of the
+// differences.  inside: the window lies in the level (block-uniform).  COH as
+// in ldf.
+template <int WH, int NT, int KI, bool COH, typename T>
+__device__ __forceinline__ void stage_window(const Windows<WH> &m, const float *a, size_t plane,
+                                             const T *__restrict__ I1, int w, int h, int pitch,
+                                             int ex, int ey, bool inside)
+{
+    constexpr int NP = kLvW / 2, NI = NP * WH;
+#pragma unroll 1
+    for (int i0 = threadIdx.x; i0 < NI; i0 += NT * KI) {
+        pair_t u[KI], v[KI], x[KI], y[KI];
+#pragma unroll
+        for (int j = 0; j < KI; ++j) {
+            const int i = min(i0 + NT * j, NI - 1);
+            const int row = i / NP, gx = ex + 2 * (i - row * NP), gy = ey + row;
+            if (inside) {
+                const float *q = a + gy * pitch + gx;
+                const float2 uu = ldf2<COH>(q), vv = ldf2<COH>(q + plane);
+                u[j] = pk(uu.x, uu.y);
+                v[j] = pk(vv.x, vv.y);
+                x[j] = pk((float)gx, (float)(gx + 1));
+                y[j] = dup((float)gy);
+            } else {
+                const int c0 = clampi(gx, 0, w - 1), c1 = clampi(gx + 1, 0, w - 1);
+                const int cy = clampi(gy, 0, h - 1);
+                const float *q = a + cy * pitch;
+                u[j] = pk(ldf<COH>(q + c0), ldf<COH>(q + c1));
+                v[j] = pk(ldf<COH>(q + plane + c0), ldf<COH>(q + plane + c1));
+                x[j] = pk((float)c0, (float)c1);
+                y[j] = dup((float)cy);
+            }
+        }
+        Taps2 tp[KI];
+#pragma unroll
+        for (int j = 0; j < KI; ++j)
+            tp[j] = bil_taps2(I1, w, h, pitch, fadd2(x[j], u[j]), fadd2(y[j], v[j]));
+#pragma unroll
+        for (int j = 0; j < KI; ++j) {
+            const int i = i0 + NT * j;
+            if (i < NI) {
+                st_pair(m.U + 2 * i, u[j]);
+                st_pair(m.V + 2 * i, v[j]);
+                st_pair(m.W + 2 * i, bil_lerp2(tp[j]));
+            }
+        }
+    }
+}
+
+// The warped image's derivatives and the smoothness weights 1 px around the
+// tile, rows 1 .. WH - 2 (the first and last column's left and right
+// neighbours are another row's; nothing reads those results).
+template <int WH, int NT>
+__device__ __forceinline__ void derive_window(const Windows<WH> &m, float alpha_s)
+{
+    constexpr int NP = kLvW / 2;
+#pragma unroll 1
+    for (int i = NP + threadIdx.x; i < NP * (WH - 1); i += NT) {
+        const int e = 2 * i;
+        const pair_t half = dup(0.5f);
+        const float2 u = upk(ld_pair(m.U + e)), v = upk(ld_pair(m.V + e));
+        const float2 wc = upk(ld_pair(m.W + e));
+        const float un = m.U[e + 2], vn = m.V[e + 2];
+        const pair_t ix = pk(fsub(wc.y, m.W[e - 1]), fsub(m.W[e + 2], wc.x));
+        const pair_t iy = fsub2(ld_pair(m.W + e + kLvW), ld_pair(m.W + e - kLvW));
+        const pair_t ux = pk(fsub(u.y, u.x), fsub(un, u.y));
+        const pair_t vx = pk(fsub(v.y, v.x), fsub(vn, v.y));
+        const pair_t uy = fsub2(ld_pair(m.U + e + kLvW), pk(u.x, u.y));
+        const pair_t vy = fsub2(ld_pair(m.V + e + kLvW), pk(v.x, v.y));
+        const pair_t q = psi_prime2(ffma2(vy, vy, ffma2(vx, vx, ffma2(uy, uy, fmul2(ux, ux)))));
+        st_pair(m.Ix + e, fmul2(half, ix));
+        st_pair(m.Iy + e, fmul2(half, iy));
+        st_pair(m.As + e, fmul2(dup(alpha_s), q));
+    }
+}
+
+// The systems of pixels (gx, gy), (gx + 1, gy), e their place in the windows;
+// i0, i0x, i0y: the template's values.  d1, d2: the diagonal; wl, wr, wu, wd:
+// the edge weights, 0 where the edge leaves the level.
+struct PairSystem {
+    float2 d1, d2, a12, b1, b2, wl, wr, wu, wd;
+};
+template <int WH>
+__device__ __forceinline__ PairSystem pair_system(const Windows<WH> &m, int e, int gx, int gy,
+                                                  int w, int h, bool inside, pair_t i0,
+                                                  pair_t i0x, pair_t i0y, float delta,
+                                                  float gamma)
+{
+    const float wm1 = (float)(w - 1), hm1 = (float)(h - 1);
+    const pair_t half = dup(0.5f);
+    auto cd2 = [&](pair_t hi, pair_t lo) { return fmul2(half, fsub2(hi, lo)); };
+    const bool top = !inside && gy <= 0, bottom = !inside && gy + 1 >= h;
+    const pair_t ix = ld_pair(m.Ix + e), iy = ld_pair(m.Iy + e);
+    const pair_t ixu = top ? ix : ld_pair(m.Ix + e - kLvW);
+    const pair_t ixd = bottom ? ix : ld_pair(m.Ix + e + kLvW);
+    const pair_t iyu = top ? iy : ld_pair(m.Iy + e - kLvW);
+    const pair_t iyd = bottom ? iy : ld_pair(m.Iy + e + kLvW);
+    const float2 ixv = upk(ix);
+    // clamped neighbours along x
+    const bool l0 = inside || gx > 0, r0 = inside || gx + 1 < w;
+    const bool l1 = inside || gx + 1 > 0, r1 = inside || gx + 2 < w;
+    const pair_t Ixx = fmul2(half, pk(fsub(r0 ? ixv.y : ixv.x, l0 ? m.Ix[e - 1] : ixv.x),
+                                      fsub(r1 ? m.Ix[e + 2] : ixv.y, l1 ? ixv.x : ixv.y)));
+    const pair_t Ixy = cd2(ixd, ixu), Iyy = cd2(iyd, iyu);
+    const pair_t Iz = fsub2(ld_pair(m.W + e), i0);
+    const pair_t Ixz = fsub2(ix, i0x), Iyz = fsub2(iy, i0y);
+    const pair_t z2 = dup(kZeta2);
+    const pair_t xx = fmul2(Ixx, Ixx), yy = fmul2(Ixy, Ixy);
+    const float2 n1 = upk(fadd2(ffma2(iy, iy, fmul2(ix, ix)), z2));
+    const float2 n2 = upk(fadd2(ffma2(Iyy, Iyy, ffma2(fmul2(dup(2.0f), Ixy), Ixy, xx)), z2));
+    const pair_t nd = pk(rcp_normal(n1.x), rcp_normal(n1.y));
+    const pair_t ng = pk(rcp_normal(n2.x), rcp_normal(n2.y));
+    float2 adv = upk(fmul2(fmul2(dup(delta), nd), psi_prime2(fmul2(fmul2(nd, Iz), Iz))));
+    float2 agv = upk(fmul2(fmul2(dup(gamma), ng),
+                           psi_prime2(fmul2(ng, ffma2(Iyz, Iyz, fmul2(Ixz, Ixz))))));
+    const pair_t u = ld_pair(m.U + e), v = ld_pair(m.V + e);
+    const float2 wx = upk(fadd2(pk((float)gx, (float)(gx + 1)), u));
+    const float2 wy = upk(fadd2(dup((float)gy), v));
+    if (wx.x < 0.0f || wx.x > wm1 || wy.x < 0.0f || wy.x > hm1) adv.x = agv.x = 0.0f;
+    if (wx.y < 0.0f || wx.y > wm1 || wy.y < 0.0f || wy.y > hm1) adv.y = agv.y = 0.0f;
+    const pair_t ad = pk(adv.x, adv.y), ag = pk(agv.x, agv.y);
+    const pair_t as = ld_pair(m.As + e);
+    const float2 av = upk(as);
+    const float mid = fmul(0.5f, fadd(av.x, av.y));
+    PairSystem ps;
+    ps.wl = make_float2(l0 ? fmul(0.5f, fadd(av.x, m.As[e - 1])) : 0.0f, l1 ? mid : 0.0f);
+    ps.wr = make_float2(r0 ? mid : 0.0f, r1 ? fmul(0.5f, fadd(av.y, m.As[e + 2])) : 0.0f);
+    const pair_t cl = pk(ps.wl.x, ps.wl.y), cr = pk(ps.wr.x, ps.wr.y);
+    const pair_t cu = top ? 0 : fmul2(half, fadd2(as, ld_pair(m.As + e - kLvW)));
+    const pair_t cd = bottom ? 0 : fmul2(half, fadd2(as, ld_pair(m.As + e + kLvW)));
+    ps.wu = upk(cu);
+    ps.wd = upk(cd);
+    const pair_t sw = fadd2(fadd2(fadd2(cl, cr), cu), cd);
+    auto smooth = [&](const float *q, pair_t c) {
+        const float2 n = upk(c);
+        const pair_t dl = pk(fsub(q[e - 1], n.x), fsub(n.x, n.y));
+        const pair_t dr = pk(fsub(n.y, n.x), fsub(q[e + 2], n.y));
+        return ffma2(cd, fsub2(ld_pair(q + e + kLvW), c),
+                     ffma2(cu, fsub2(ld_pair(q + e - kLvW), c), ffma2(cr, dr, fmul2(cl, dl))));
+    };
+    const pair_t su = smooth(m.U, u), sv = smooth(m.V, v);
+    const pair_t adx = fmul2(ad, ix), ady = fmul2(ad, iy), nag = neg2(ag);
+    ps.d1 = upk(fadd2(ffma2(ag, ffma2(Ixy, Ixy, xx), fmul2(adx, ix)), sw));
+    ps.d2 = upk(fadd2(ffma2(ag, ffma2(Iyy, Iyy, yy), fmul2(ady, iy)), sw));
+    ps.a12 = upk(ffma2(ag, ffma2(Ixy, Iyy, fmul2(Ixx, Ixy)), fmul2(adx, iy)));
+    ps.b1 = upk(ffma2(nag, ffma2(Ixy, Iyz, fmul2(Ixx, Ixz)), ffma2(neg2(adx), Iz, su)));
+    ps.b2 = upk(ffma2(nag, ffma2(Iyy, Iyz, fmul2(Ixy, Ixz)), ffma2(neg2(ady), Iz, sv)));
+    return ps;
+}
+
+// The linear systems of a level as planes: a block stages a tile of 64 columns
+// x TH rows (from an odd column, as the planes' pairs are aligned) and writes
+// its pixels' systems, two adjacent ones a thread and step.
+template <int TH, int NT, typename T>
+__device__ __forceinline__ void var_coeff_body(
+    float *smem, const T *__restrict__ I0, const T *__restrict__ I0x, const T *__restrict__ I0y,
+    const T *__restrict__ I1, int w, int h, int pitch, const float *__restrict__ U, size_t plane,
+    float *__restrict__ cf, float delta, float gamma, float alpha_s, float omega, int bx, int by)
+{
+    constexpr int WH = TH + 4, WARPS = NT / 32;
+    const Windows<WH> m(smem);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int tx = bx * 64 - 1, ty = by * TH;
+    const bool inside = tx >= 2 && ty >= 2 && tx + 66 <= w && ty + TH + 2 <= h;
+    stage_window<WH, NT, 3, false>(m, U, plane, I1, w, h, pitch, tx - 2, ty - 2, inside);
+    __syncthreads();
+    derive_window<WH, NT>(m, alpha_s);
+    __syncthreads();
+    const int gx = tx + 2 * lane, pl = (int)plane;
+    const bool c0 = inside || (gx >= 0 && gx < w), c1 = inside || gx + 1 < w;
+#pragma unroll 1
+    for (int r = wp; r < TH; r += WARPS) {
+        const int gy = ty + r, o = gy * pitch + gx;
+        if (gy >= h) break;
+        const pair_t i0 = pk(c0 ? ldp(I0 + o) : 0.0f, c1 ? ldp(I0 + o + 1) : 0.0f);
+        const pair_t i0x = pk(c0 ? ldp(I0x + o) : 0.0f, c1 ? ldp(I0x + o + 1) : 0.0f);
+        const pair_t i0y = pk(c0 ? ldp(I0y + o) : 0.0f, c1 ? ldp(I0y + o + 1) : 0.0f);
+        const int e = (r + 2) * kLvW + 2 * lane + 2;
+        const PairSystem ps = pair_system(m, e, gx, gy, w, h, inside, i0, i0x, i0y, delta, gamma);
+        float *c = cf + o;
+        auto st = [&](int k, float x, float y) {
+            if (c0 && c1) *reinterpret_cast<float2 *>(c + k * pl) = make_float2(x, y);
+            else if (c0) c[k * pl] = x;
+            else if (c1) c[k * pl + 1] = y;
+        };
+        st(kCI11, __fdividef(omega, ps.d1.x), __fdividef(omega, ps.d1.y));
+        st(kCI22, __fdividef(omega, ps.d2.x), __fdividef(omega, ps.d2.y));
+        st(kCA12, ps.a12.x, ps.a12.y);
+        st(kCB1, ps.b1.x, ps.b1.y);
+        st(kCB2, ps.b2.x, ps.b2.y);
+        st(kCAS, m.As[e], m.As[e + 1]);
+    }
+}
+
+// Tiles of 16 rows, 256 threads of 64 registers (four blocks an SM), or of 8
+// rows for grids of under two blocks an SM, where the chain of the three phases
+// counts.
+constexpr int kCoefThreads = 256, kCoefRows = 16, kCoefRowsSmall = 8;
+
+template <int TH, typename T>
+__global__ void __launch_bounds__(kCoefThreads, TH == kCoefRows ? 4 : 3)
+var_coeff_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
+                 const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h, int pitch,
+                 size_t pfs, const float *__restrict__ Ub, size_t ufs, size_t plane,
+                 float *__restrict__ coefb, size_t cfs, float delta, float gamma, float alpha_s,
+                 float omega)
+{
+    extern __shared__ __align__(16) float csm[];
+    const int f = blockIdx.z;
+    const size_t po = (size_t)f * pfs;
+    var_coeff_body<TH, kCoefThreads>(csm, I0b + po, I0xb + po, I0yb + po, I1b + po, w, h, pitch,
+                                     Ub + (size_t)f * ufs, plane, coefb + (size_t)f * cfs, delta,
+                                     gamma, alpha_s, omega, blockIdx.x, blockIdx.y);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCoefThreads, 4)
+seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
+{
+    extern __shared__ __align__(16) float csm[];
+    int b;
+    const SegCoeff &a = seg_of(tab, b);
+    const int r = b / a.gx;
+    const size_t f = r / a.gy, po = f * a.pfs;
+    var_coeff_body<kCoefRows, kCoefThreads>(
+        csm, (const T *)a.I0 + po, (const T *)a.I0x + po, (const T *)a.I0y + po,
+        (const T *)a.I1 + po, a.w, a.h, a.pitch, a.U + f * a.ufs, a.plane,
+        a.coef + kCoefShift + f * a.cfs, a.delta, a.gamma, a.alpha_s, a.omega, b % a.gx, r % a.gy);
+}
+
 // The whole variational refinement of a level in one launch.  The work is a
 // list of items (iteration, region of 64 x 16 VS), iteration by iteration; a
 // block claims them in order from a counter, the next one while it works on
@@ -1067,11 +930,10 @@ __device__ __forceinline__ pair_t bil_lerp2(const Taps2 &t)
 // ctl: [0] the claim counter, [1] blocks gone, [2 + r] finished iterations of
 // region r.  The last block to leave sets them to 0 for the next launch.  Waits
 // are bounded; a block whose wait runs out reports kErrTimeout and leaves.
-constexpr int kLvW = kVR + 4;  // staged columns
 template <int VS>
 constexpr size_t level_smem_bytes()
 {
-    return (size_t)6 * kLvW * (VS * kVWarps + 4) * sizeof(float);
+    return Windows<VS * kVWarps + 4>::kBytes;
 }
 
 template <int VS, typename T>
@@ -1082,17 +944,14 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                  int R, int nrx, int nry, float delta, float gamma, float alpha_s, float omega,
                  int blocks, unsigned *ctl, long long wait_limit, int *err)
 {
-    constexpr int RH = VS * kVWarps, WH = RH + 4, NP = kLvW / 2;  // pairs of a staged row
+    constexpr int RH = VS * kVWarps, WH = RH + 4;
     extern __shared__ __align__(16) float lsm[];
-    float *sU = lsm, *sV = sU + kLvW * WH, *sW = sV + kLvW * WH;
-    float *sIx = sW + kLvW * WH, *sIy = sIx + kLvW * WH, *sAs = sIy + kLvW * WH;
+    const Windows<WH> m(lsm);
     __shared__ StripEnds<kVWarps> ends;
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
     __shared__ int s_item;
     const int per_frame = nrx * nry, total = outer * blocks;
     clear_ends(ends);
-    const float wm1 = (float)(w - 1), hm1 = (float)(h - 1);
-    auto pr = [](const float *a) { return *reinterpret_cast<const pair_t *>(a); };
     if (t == 0) s_item = (int)atomicAdd(ctl, 1u);
     __syncthreads();
     for (int item = s_item; item < total; item = s_item) {
@@ -1142,155 +1001,39 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             if (t == 0) atomicOr(err, kErrTimeout);
             break;
         }
-        // A
-        constexpr int NI = NP * WH, KI = 3;
-#pragma unroll 1
-        for (int i0 = t; i0 < NI; i0 += kVThreads * KI) {
-            pair_t u[KI], v[KI], x[KI], y[KI];
-#pragma unroll
-            for (int j = 0; j < KI; ++j) {
-                const int i = min(i0 + kVThreads * j, NI - 1);
-                const int row = i / NP, gx = rx0 - 2 + 2 * (i - row * NP), gy = ry0 - 2 + row;
-                if (inside) {
-                    const float *q = a + gy * pitch + gx;
-                    const float2 uu = __ldcg(reinterpret_cast<const float2 *>(q));
-                    const float2 vv = __ldcg(reinterpret_cast<const float2 *>(q + plane));
-                    u[j] = pk(uu.x, uu.y);
-                    v[j] = pk(vv.x, vv.y);
-                    x[j] = pk((float)gx, (float)(gx + 1));
-                    y[j] = dup((float)gy);
-                } else {
-                    const int c0 = clampi(gx, 0, w - 1), c1 = clampi(gx + 1, 0, w - 1);
-                    const int cy = clampi(gy, 0, h - 1);
-                    const float *q = a + cy * pitch;
-                    u[j] = pk(__ldcg(q + c0), __ldcg(q + c1));
-                    v[j] = pk(__ldcg(q + plane + c0), __ldcg(q + plane + c1));
-                    x[j] = pk((float)c0, (float)c1);
-                    y[j] = dup((float)cy);
-                }
-            }
-            Taps2 tp[KI];
-#pragma unroll
-            for (int j = 0; j < KI; ++j)
-                tp[j] = bil_taps2(I1, w, h, pitch, fadd2(x[j], u[j]), fadd2(y[j], v[j]));
-#pragma unroll
-            for (int j = 0; j < KI; ++j) {
-                const int i = i0 + kVThreads * j;
-                if (i < NI) {
-                    *reinterpret_cast<pair_t *>(sU + 2 * i) = u[j];
-                    *reinterpret_cast<pair_t *>(sV + 2 * i) = v[j];
-                    *reinterpret_cast<pair_t *>(sW + 2 * i) = bil_lerp2(tp[j]);
-                }
-            }
-        }
+        stage_window<WH, kVThreads, 3, true>(m, a, plane, I1, w, h, pitch, rx0 - 2, ry0 - 2,
+                                             inside);
         __syncthreads();
-        // B: rows 1 .. WH - 2 (the first and last column's left and right
-        // neighbours are another row's; nothing reads those results)
-#pragma unroll 1
-        for (int i = NP + t; i < NP * (WH - 1); i += kVThreads) {
-            const int e = 2 * i;
-            const pair_t half = dup(0.5f);
-            const float2 u = upk(pr(sU + e)), v = upk(pr(sV + e)), wc = upk(pr(sW + e));
-            const float un = sU[e + 2], vn = sV[e + 2];
-            const pair_t ix = pk(fsub(wc.y, sW[e - 1]), fsub(sW[e + 2], wc.x));
-            const pair_t iy = fsub2(pr(sW + e + kLvW), pr(sW + e - kLvW));
-            const pair_t ux = pk(fsub(u.y, u.x), fsub(un, u.y));
-            const pair_t vx = pk(fsub(v.y, v.x), fsub(vn, v.y));
-            const pair_t uy = fsub2(pr(sU + e + kLvW), pk(u.x, u.y));
-            const pair_t vy = fsub2(pr(sV + e + kLvW), pk(v.x, v.y));
-            const pair_t q = psi_prime2(ffma2(vy, vy, ffma2(vx, vx, ffma2(uy, uy, fmul2(ux, ux)))));
-            *reinterpret_cast<pair_t *>(sIx + e) = fmul2(half, ix);
-            *reinterpret_cast<pair_t *>(sIy + e) = fmul2(half, iy);
-            *reinterpret_cast<pair_t *>(sAs + e) = fmul2(dup(alpha_s), q);
-        }
+        derive_window<WH, kVThreads>(m, alpha_s);
         __syncthreads();
-        // C
         Strip<VS> s;
 #pragma unroll
         for (int r = 0; r < VS; ++r) {
             const int e = (wp * VS + r + 2) * kLvW + 2 * lane + 2;
             const int gx = p.gx, gy = p.gy + r;
-            const pair_t half = dup(0.5f);
-            auto cd2 = [&](pair_t hi, pair_t lo) { return fmul2(half, fsub2(hi, lo)); };
-            const bool top = !inside && gy <= 0, bottom = !inside && gy + 1 >= h;
-            const bool c0 = inside || (gx >= 0 && gx < w), c1 = inside || (gx + 1 >= 0 && gx + 1 < w);
             const bool row_in = inside || (gy >= 0 && gy < h);
-            const bool in0 = c0 && row_in, in1 = c1 && row_in;
-            const pair_t ix = pr(sIx + e), iy = pr(sIy + e);
-            const pair_t ixu = top ? ix : pr(sIx + e - kLvW), ixd = bottom ? ix : pr(sIx + e + kLvW);
-            const pair_t iyu = top ? iy : pr(sIy + e - kLvW), iyd = bottom ? iy : pr(sIy + e + kLvW);
-            const float2 ixv = upk(ix);
-            // clamped neighbours along x
-            const bool l0 = inside || gx > 0, r0 = inside || gx + 1 < w;
-            const bool l1 = inside || gx + 1 > 0, r1 = inside || gx + 2 < w;
-            const pair_t Ixx = fmul2(half, pk(fsub(r0 ? ixv.y : ixv.x, l0 ? sIx[e - 1] : ixv.x),
-                                              fsub(r1 ? sIx[e + 2] : ixv.y, l1 ? ixv.x : ixv.y)));
-            const pair_t Ixy = cd2(ixd, ixu), Iyy = cd2(iyd, iyu);
-            const pair_t Iz = fsub2(pr(sW + e), i0[r]);
-            const pair_t Ixz = fsub2(ix, i0x[r]), Iyz = fsub2(iy, i0y[r]);
-            const pair_t z2 = dup(kZeta2);
-            const pair_t xx = fmul2(Ixx, Ixx), yy = fmul2(Ixy, Ixy);
-            const float2 n1 = upk(fadd2(ffma2(iy, iy, fmul2(ix, ix)), z2));
-            const float2 n2 =
-                upk(fadd2(ffma2(Iyy, Iyy, ffma2(fmul2(dup(2.0f), Ixy), Ixy, xx)), z2));
-            const pair_t nd = pk(rcp_normal(n1.x), rcp_normal(n1.y));
-            const pair_t ng = pk(rcp_normal(n2.x), rcp_normal(n2.y));
-            float2 adv =
-                upk(fmul2(fmul2(dup(delta), nd), psi_prime2(fmul2(fmul2(nd, Iz), Iz))));
-            float2 agv = upk(fmul2(fmul2(dup(gamma), ng),
-                                   psi_prime2(fmul2(ng, ffma2(Iyz, Iyz, fmul2(Ixz, Ixz))))));
-            const pair_t u = pr(sU + e), v = pr(sV + e);
-            const float2 wx = upk(fadd2(pk((float)gx, (float)(gx + 1)), u));
-            const float2 wy = upk(fadd2(dup((float)gy), v));
-            if (wx.x < 0.0f || wx.x > wm1 || wy.x < 0.0f || wy.x > hm1) adv.x = agv.x = 0.0f;
-            if (wx.y < 0.0f || wx.y > wm1 || wy.y < 0.0f || wy.y > hm1) adv.y = agv.y = 0.0f;
-            const pair_t ad = pk(adv.x, adv.y), ag = pk(agv.x, agv.y);
-            // edge weights, 0 where the edge leaves the level
-            const pair_t as = pr(sAs + e);
-            const float2 av = upk(as);
-            const float mid = fmul(0.5f, fadd(av.x, av.y));
-            const float wl = l0 ? fmul(0.5f, fadd(av.x, sAs[e - 1])) : 0.0f;
-            const float wr = r1 ? fmul(0.5f, fadd(av.y, sAs[e + 2])) : 0.0f;
-            const pair_t cl = pk(wl, l1 ? mid : 0.0f), cr = pk(r0 ? mid : 0.0f, wr);
-            const pair_t cu = top ? 0 : fmul2(half, fadd2(as, pr(sAs + e - kLvW)));
-            const pair_t cd = bottom ? 0 : fmul2(half, fadd2(as, pr(sAs + e + kLvW)));
-            const pair_t sw = fadd2(fadd2(fadd2(cl, cr), cu), cd);
-            auto smooth = [&](const float *q, pair_t c) {
-                const float2 m = upk(c);
-                const pair_t dl = pk(fsub(q[e - 1], m.x), fsub(m.x, m.y));
-                const pair_t dr = pk(fsub(m.y, m.x), fsub(q[e + 2], m.y));
-                return ffma2(cd, fsub2(pr(q + e + kLvW), c),
-                             ffma2(cu, fsub2(pr(q + e - kLvW), c), ffma2(cr, dr, fmul2(cl, dl))));
-            };
-            const pair_t su = smooth(sU, u), sv = smooth(sV, v);
-            const pair_t adx = fmul2(ad, ix), ady = fmul2(ad, iy), nag = neg2(ag);
-            const float2 d1 = upk(fadd2(ffma2(ag, ffma2(Ixy, Ixy, xx), fmul2(adx, ix)), sw));
-            const float2 d2 = upk(fadd2(ffma2(ag, ffma2(Iyy, Iyy, yy), fmul2(ady, iy)), sw));
-            const float2 a12 =
-                upk(ffma2(ag, ffma2(Ixy, Iyy, fmul2(Ixx, Ixy)), fmul2(adx, iy)));
-            const float2 b1 = upk(ffma2(nag, ffma2(Ixy, Iyz, fmul2(Ixx, Ixz)),
-                                        ffma2(neg2(adx), Iz, su)));
-            const float2 b2 = upk(ffma2(nag, ffma2(Iyy, Iyz, fmul2(Ixy, Ixz)),
-                                        ffma2(neg2(ady), Iz, sv)));
-            s.i11[r][0] = in0 ? __fdividef(omega, d1.x) : 0.0f;
-            s.i11[r][1] = in1 ? __fdividef(omega, d1.y) : 0.0f;
-            s.i22[r][0] = in0 ? __fdividef(omega, d2.x) : 0.0f;
-            s.i22[r][1] = in1 ? __fdividef(omega, d2.y) : 0.0f;
-            s.a12[r][0] = in0 ? a12.x : 0.0f;
-            s.a12[r][1] = in1 ? a12.y : 0.0f;
-            s.b[r][0] = in0 ? pk(b1.x, b2.x) : 0;
-            s.b[r][1] = in1 ? pk(b1.y, b2.y) : 0;
+            const bool in0 = row_in && (inside || (gx >= 0 && gx < w));
+            const bool in1 = row_in && (inside || (gx + 1 >= 0 && gx + 1 < w));
+            const PairSystem ps =
+                pair_system(m, e, gx, gy, w, h, inside, i0[r], i0x[r], i0y[r], delta, gamma);
+            s.i11[r][0] = in0 ? __fdividef(omega, ps.d1.x) : 0.0f;
+            s.i11[r][1] = in1 ? __fdividef(omega, ps.d1.y) : 0.0f;
+            s.i22[r][0] = in0 ? __fdividef(omega, ps.d2.x) : 0.0f;
+            s.i22[r][1] = in1 ? __fdividef(omega, ps.d2.y) : 0.0f;
+            s.a12[r][0] = in0 ? ps.a12.x : 0.0f;
+            s.a12[r][1] = in1 ? ps.a12.y : 0.0f;
+            s.b[r][0] = in0 ? pk(ps.b1.x, ps.b2.x) : 0;
+            s.b[r][1] = in1 ? pk(ps.b1.y, ps.b2.y) : 0;
             // the region's own edges carry no weight, nor do pixels outside
-            const float2 lv = upk(cl), uv = upk(cu), dv = upk(cd);
-            s.wl[r][0] = lane > 0 && in0 ? lv.x : 0.0f;
-            s.wl[r][1] = in1 ? lv.y : 0.0f;
-            s.wr[r] = lane < 31 && in1 ? wr : 0.0f;
             const bool up_in = !(r == 0 && wp == 0);
-            s.wu[r][0] = up_in && in0 ? uv.x : 0.0f;
-            s.wu[r][1] = up_in && in1 ? uv.y : 0.0f;
+            s.wl[r][0] = lane > 0 && in0 ? ps.wl.x : 0.0f;
+            s.wl[r][1] = in1 ? ps.wl.y : 0.0f;
+            s.wr[r] = lane < 31 && in1 ? ps.wr.y : 0.0f;
+            s.wu[r][0] = up_in && in0 ? ps.wu.x : 0.0f;
+            s.wu[r][1] = up_in && in1 ? ps.wu.y : 0.0f;
             if (r == VS - 1) {
-                s.wd[0] = wp < kVWarps - 1 && in0 ? dv.x : 0.0f;
-                s.wd[1] = wp < kVWarps - 1 && in1 ? dv.y : 0.0f;
+                s.wd[0] = wp < kVWarps - 1 && in0 ? ps.wd.x : 0.0f;
+                s.wd[1] = wp < kVWarps - 1 && in1 ? ps.wd.y : 0.0f;
             }
         }
         // D
@@ -1300,7 +1043,7 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             if (r < p.r0 || r >= p.r1) continue;
             const int e = (wp * VS + r + 2) * kLvW + 2 * lane + 2;
             float *q = b + (p.gy + r) * pitch + p.gx;
-            const float2 u = upk(pr(sU + e)), v = upk(pr(sV + e));
+            const float2 u = upk(ld_pair(m.U + e)), v = upk(ld_pair(m.V + e));
             const float2 d0 = upk(s.d[r][0]), d1 = upk(s.d[r][1]);
             if (p.c0 && p.c1) {
                 __stcg(reinterpret_cast<float2 *>(q), make_float2(u.x + d0.x, u.y + d1.x));
@@ -1409,18 +1152,16 @@ void init_var_attributes()
 
 int sor_halo(int var_sor) { return var_sor > 0 ? 2 * var_sor - 1 : 1; }
 int sor_tile(int R) { return kVR - 2 * R; }
-void coeff_tile_shape(int &x, int &y)
-{
-    x = kAX;
-    y = kAY;
-}
+int coeff_tiles_x(int w) { return (w + 64) / 64; }  // the first tile starts at column -1
+int coeff_tiles_y(int h) { return (h + kCoefRows - 1) / kCoefRows; }
 int coeff_planes() { return kCPlanes; }
 
 void launch_seg_coeff(const SegTable<SegCoeff> &t, int blocks, bool half, cudaStream_t st)
 {
     StageScope sc(kStVarCoeff, 1, st);
-    if (half) seg_var_coeff_kernel<__half><<<blocks, dim3(kAX, kAY), 0, st>>>(t);
-    else seg_var_coeff_kernel<float><<<blocks, dim3(kAX, kAY), 0, st>>>(t);
+    constexpr size_t smem = Windows<kCoefRows + 4>::kBytes;
+    if (half) seg_var_coeff_kernel<__half><<<blocks, kCoefThreads, smem, st>>>(t);
+    else seg_var_coeff_kernel<float><<<blocks, kCoefThreads, smem, st>>>(t);
 }
 
 void launch_seg_sor(const SegTable<SegSor> &t, int blocks, cudaStream_t st)
@@ -1445,17 +1186,9 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
     const int tile = sor_tile(R);           // interior side of a 64 x 64 region
     const int small = kVSmallRows - 2 * R;  // interior rows of a 64 x 32 region
     coef += kCoefShift;
-    const dim3 cgrd((lv.w + kAX - 1) / kAX, (lv.h + kAY - 1) / kAY, frames);
-    // the coefficient kernel's form depends on the level's width and the
-    // stream's parameters only, so single, batched and grouped windows of a
-    // level always run the same one (and give the same coefficients): by
-    // default the column walk from 1024 px wide (the finest level of 1280 x
-    // 720 frames), where it is the faster; smaller levels keep the tile form
-    const bool column_walk = lv.w >= fp.coeff_cw_min_width;
-    const int cw_rows = fp.coeff_cw_rows == 4 || fp.coeff_cw_rows == 16 ? fp.coeff_cw_rows
-                                                                       : kCWRows;
-    const dim3 wgrd((lv.w + kCWOut - 1) / kCWOut,
-                    ((lv.h + cw_rows - 1) / cw_rows + kCWWarps - 1) / kCWWarps, frames);
+    dim3 cgrd(coeff_tiles_x(lv.w), coeff_tiles_y(lv.h), frames);
+    const bool small_tiles = (long long)(cgrd.x * cgrd.y * cgrd.z) < 2LL * nsm;
+    if (small_tiles) cgrd.y = (lv.h + kCoefRowsSmall - 1) / kCoefRowsSmall;
     const dim3 sgrd((lv.w + tile - 1) / tile, (lv.h + tile - 1) / tile, frames);
     // small levels of a single frame: every outer iteration in one launch (same
     // flow bit for bit), where the regions fit one wave and a region's staged
@@ -1500,37 +1233,21 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
     }
     float *a = U, *b = Utmp;
     for (int k = 0; k < fp.var_outer; ++k) {
-        if (column_walk) {
+        {
             StageScope sc(kStVarCoeff, 1, st);
-#define EBOF_CW(R, T)                                                                          \
-    var_coeff_cw_kernel<R, T><<<wgrd, dim3(32, kCWWarps), 0, st>>>(                             \
-        (const T *)I0, (const T *)I0x, (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch,     \
-        pyr_frame_stride, a, u_frame_stride, lv.plane, coef, coef_frame_stride, fp.delta,       \
+#define EBOF_CF(TH, T)                                                                          \
+    var_coeff_kernel<TH, T><<<cgrd, kCoefThreads, Windows<TH + 4>::kBytes, st>>>(                \
+        (const T *)I0, (const T *)I0x, (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch,      \
+        pyr_frame_stride, a, u_frame_stride, lv.plane, coef, coef_frame_stride, fp.delta,        \
         fp.gamma, fp.alpha_s, fp.omega)
             if (fp.half) {
-                if (cw_rows == 4) EBOF_CW(4, __half);
-                else if (cw_rows == 16) EBOF_CW(16, __half);
-                else EBOF_CW(kCWRows, __half);
+                if (small_tiles) EBOF_CF(kCoefRowsSmall, __half);
+                else EBOF_CF(kCoefRows, __half);
             } else {
-                if (cw_rows == 4) EBOF_CW(4, float);
-                else if (cw_rows == 16) EBOF_CW(16, float);
-                else EBOF_CW(kCWRows, float);
+                if (small_tiles) EBOF_CF(kCoefRowsSmall, float);
+                else EBOF_CF(kCoefRows, float);
             }
-#undef EBOF_CW
-        } else {
-            StageScope sc(kStVarCoeff, 1, st);
-            if (fp.half)
-                var_coeff_kernel<__half><<<cgrd, dim3(kAX, kAY), 0, st>>>(
-                    (const __half *)I0, (const __half *)I0x, (const __half *)I0y,
-                    (const __half *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride, a,
-                    u_frame_stride, lv.plane, coef, coef_frame_stride, fp.delta, fp.gamma,
-                    fp.alpha_s, fp.omega);
-            else
-                var_coeff_kernel<float><<<cgrd, dim3(kAX, kAY), 0, st>>>(
-                    (const float *)I0, (const float *)I0x, (const float *)I0y,
-                    (const float *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride, a,
-                    u_frame_stride, lv.plane, coef, coef_frame_stride, fp.delta, fp.gamma,
-                    fp.alpha_s, fp.omega);
+#undef EBOF_CF
         }
         {
             StageScope sc(kStVarSor, 1, st);

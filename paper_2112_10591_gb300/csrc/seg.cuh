@@ -169,7 +169,8 @@ int search_blocks(int ps, bool wide, int npx, int npy);
 bool search_wide(int n_patches);
 int sor_halo(int var_sor);             // halo of a SOR region (odd)
 int sor_tile(int R);                   // interior side of a 64 x 64 SOR region
-void coeff_tile_shape(int &x, int &y);  // pixels of a coefficient tile
+int coeff_tiles_x(int w);              // coefficient tiles of a level
+int coeff_tiles_y(int h);
 int coeff_planes();                    // coefficient planes per level and frame
 int seg_max_levels();                  // pyramid levels the fused pyramid kernels build
 PyrDesc make_pyr_desc(const Geometry &geo);
