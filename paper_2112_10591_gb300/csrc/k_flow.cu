@@ -615,7 +615,9 @@ constexpr int kDenseX = 36, kDenseY = 12;
 // samples all lie inside the level takes them from the staged values, without
 // the floors, conversions and border tests of every pixel (each on the slow
 // pipe, nine times a pixel at 12 x 12 patches and stride 4); other blocks
-// sample patch by patch.  The arithmetic is the same.
+// sample patch by patch.  The arithmetic is the same.  Bound by issue and the
+// taps' latency.  1280x720 level 0, eight frames: 188 -> 164 us (194 while a
+// test stood before every patch's loads); 85 -> 65 us over the other levels.
 template <typename T, int NC>
 __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T *__restrict__ I1b,
                                              int w, int h, int pitch, size_t pfs,
