@@ -67,6 +67,8 @@ struct ebof_stream {
     unsigned long long *d_dropped_time = nullptr;
     int *d_err = nullptr;
     unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
+    char *d_xch = nullptr;      // and its packets: 2 x level_px x kPacketBytes
+    size_t level_px = 0;
     float *flow_stage = nullptr;  // device flow for the host-buffer call
     void *ev_stage = nullptr;     // device events for the host-buffer call
     size_t ev_stage_bytes = 0;
@@ -155,6 +157,8 @@ struct ebof_group {
     unsigned long long *d_dropped_time = nullptr;
     int *d_err = nullptr;
     unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
+    char *d_xch = nullptr;      // and its packets: 2 x level_px x kPacketBytes
+    size_t level_px = 0;
     ebof_window_desc *d_desc = nullptr;
     int64_t *h_events = nullptr;  // events given per stream in the last step
     int parity = 0;
@@ -284,6 +288,8 @@ ebof_status check_params(const ebof_params *p)
 // the one that fails; negative = disarmed.
 std::atomic<int> g_alloc_fail_after{-1};
 
+constexpr size_t kPacketBytes = 16;  // a pixel's u, v and 64-bit tag
+
 // Every device allocation of the library goes through here.
 template <class T>
 cudaError_t dmalloc(T **ptr, size_t bytes)
@@ -318,6 +324,7 @@ void free_all(ebof_stream *s)
     cudaFree(s->E); cudaFree(s->Ed); cudaFree(s->Edf); cudaFree(s->g); cudaFree(s->pyr);
     cudaFree(s->up); flow_free(s->Ua); flow_free(s->Ub); cudaFree(s->work);
     cudaFree(s->dstats); cudaFree(s->d_dropped_time); cudaFree(s->d_err); cudaFree(s->d_ctl);
+    cudaFree(s->d_xch);
     cudaFree(s->flow_stage); cudaFree(s->ev_stage); cudaFree(s->d_call);
     for (int b = 0; b < 2; ++b)
         if (s->graph[b]) cudaGraphExecDestroy(s->graph[b]);
@@ -394,6 +401,8 @@ FlowParams flow_params(const ebof_params &p)
     fp.sor_row_waves = p.sor_row_waves;
     fp.var_cluster_max = p.var_cluster_max;
     fp.level_ctl = nullptr;
+    fp.level_xch = nullptr;
+    fp.level_px = 0;
     return fp;
 }
 
@@ -473,7 +482,11 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
         for (int l = geo.levels - 1; l >= 0; --l) {
             tl_level = l;
             // windows in order: nothing else uses the counters meanwhile
-            if (parts == kPartAll) fp.level_ctl = s->d_ctl;
+            if (parts == kPartAll) {
+                fp.level_ctl = s->d_ctl;
+                fp.level_xch = s->d_xch;
+                fp.level_px = s->level_px;
+            }
             const Level &lv = geo.lv[l];
             const char *I0 = pyr + ((size_t)prev_first * s->pyr_fs + geo.pyr_off[l]) * es;
             const char *I1 = pyr + ((size_t)curf_first * s->pyr_fs + geo.pyr_off[l]) * es;
@@ -874,6 +887,7 @@ void free_group(ebof_group *g)
     cudaFree(g->E); cudaFree(g->Ed); cudaFree(g->Edf); cudaFree(g->g); cudaFree(g->pyr);
     cudaFree(g->up); flow_free(g->Ua); flow_free(g->Ub); cudaFree(g->work); cudaFree(g->flow);
     cudaFree(g->dstats); cudaFree(g->d_dropped_time); cudaFree(g->d_err); cudaFree(g->d_ctl);
+    cudaFree(g->d_xch);
     cudaFree(g->d_desc);
     delete[] g->h_events;
     if (g->cap) cudaStreamDestroy(g->cap);
@@ -923,6 +937,8 @@ void run_group_flow(ebof_group *g, bool with_flow, cudaStream_t st)
     if (with_flow && geo.levels > 0) {
         FlowParams fp = flow_params(p);
         fp.level_ctl = g->d_ctl;
+        fp.level_xch = g->d_xch;
+        fp.level_px = g->level_px;
         float *Ucur = nullptr, *Uc = nullptr;
         const Level *lvc = nullptr;
         for (int l = geo.levels - 1; l >= 0; --l) {
@@ -1490,6 +1506,8 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     ok &= dmalloc(&s->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&s->d_err, sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&s->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
+    s->level_px = level_pixels(geo, p->var_sor, p->var_cluster_max, B);
+    ok &= dmalloc(&s->d_xch, 2 * kPacketBytes * s->level_px) == cudaSuccess;
     ok &= dmalloc(&s->flow_stage, sizeof(float) * 2 * (size_t)p->width * p->height) == cudaSuccess;
     ok &= cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming) == cudaSuccess;
     const size_t call_bytes = (sizeof(ebof_window_desc) + sizeof(float *)) * B;
@@ -1509,6 +1527,7 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     }
     cudaMemset(s->d_err, 0, sizeof(int));
     cudaMemset(s->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
+    cudaMemset(s->d_xch, 0, 2 * kPacketBytes * s->level_px);
     cudaMemset(s->dstats, 0, sizeof(DevStats) * B);
     make_coef_maps(s->work, s->geo, B, &s->cmaps);
     cudaMemset(s->d_dropped_time, 0, sizeof(unsigned long long));
@@ -1531,7 +1550,8 @@ int64_t ebof_stream_device_bytes(const ebof_params *p)
     size_t total = 3 * r(plane0 * B) + r(4 * plane0 * B) + r(es * geo.pyr_floats * (B + 1));
     total += r(4 * 2 * (size_t)std::max(geo.max_patches, 1) * B);
     total += 2 * r(4 * (2 * plane0 * B + 1)) + r(4 * 9 * plane0 * B);
-    total += sizeof(unsigned) * kLevelCtl;
+    total += 256;  // the one-launch refinement's counters, then its packets
+    total += r(2 * kPacketBytes * level_pixels(geo, p->var_sor, p->var_cluster_max, p->max_batch));
     total += r(sizeof(DevStats) * B) + 2 * 256 + r(4 * 2 * (size_t)p->width * p->height) +
              r((sizeof(ebof_window_desc) + sizeof(float *)) * B);
     return (int64_t)total;
@@ -2034,6 +2054,8 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     ok &= dmalloc(&g->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&g->d_err, sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&g->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
+    g->level_px = level_pixels(g->geo, q.var_sor, q.var_cluster_max, n);
+    ok &= dmalloc(&g->d_xch, 2 * kPacketBytes * g->level_px) == cudaSuccess;
     ok &= dmalloc(&g->d_desc, sizeof(ebof_window_desc) * n) == cudaSuccess;
     ok &= cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking) == cudaSuccess;
     ok &= cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming) == cudaSuccess;
@@ -2045,6 +2067,7 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     }
     cudaMemset(g->d_err, 0, sizeof(int));
     cudaMemset(g->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
+    cudaMemset(g->d_xch, 0, 2 * kPacketBytes * g->level_px);
     cudaMemset(g->flow, 0, sizeof(float) * 2 * (size_t)q.width * q.height * n);
     make_coef_maps(g->work, g->geo, n, &g->cmaps);
     if (cudaDeviceSynchronize() != cudaSuccess) {

@@ -667,42 +667,38 @@ __device__ __forceinline__ void st_pair(float *a, pair_t v)
 
 // The flow of the window and the warped image there.  Positions outside the
 // level are those of the nearest pixel inside: the replicated borders of the
-// differences.  inside: the window lies in the level (block-uniform).  COH as
-// in ldf.
-template <int WH, int NT, int KI, bool COH, typename T>
-__device__ __forceinline__ void stage_window(const Windows<WH> &m, const float *a, size_t plane,
-                                             const T *__restrict__ I1, int w, int h, int pitch,
-                                             int ex, int ey, bool inside)
+// differences.  inside: the window lies in the level (block-uniform).
+// load(c0, c1, cy, u, v): the flow of KI pairs of pixels (c0, cy), (c1, cy);
+// all of a thread's loads come before their first use.
+template <int WH, int NT, int KI, typename T, class L>
+__device__ __forceinline__ void stage_window(const Windows<WH> &m, const T *__restrict__ I1,
+                                             int w, int h, int pitch, int ex, int ey, bool inside,
+                                             L load)
 {
     constexpr int NP = kLvW / 2, NI = NP * WH;
 #pragma unroll 1
     for (int i0 = threadIdx.x; i0 < NI; i0 += NT * KI) {
-        pair_t u[KI], v[KI], x[KI], y[KI];
+        pair_t u[KI], v[KI];
+        int c0[KI], c1[KI], cy[KI];
 #pragma unroll
         for (int j = 0; j < KI; ++j) {
             const int i = min(i0 + NT * j, NI - 1);
-            const int row = i / NP, gx = ex + 2 * (i - row * NP), gy = ey + row;
-            if (inside) {
-                const float *q = a + gy * pitch + gx;
-                const float2 uu = ldf2<COH>(q), vv = ldf2<COH>(q + plane);
-                u[j] = pk(uu.x, uu.y);
-                v[j] = pk(vv.x, vv.y);
-                x[j] = pk((float)gx, (float)(gx + 1));
-                y[j] = dup((float)gy);
-            } else {
-                const int c0 = clampi(gx, 0, w - 1), c1 = clampi(gx + 1, 0, w - 1);
-                const int cy = clampi(gy, 0, h - 1);
-                const float *q = a + cy * pitch;
-                u[j] = pk(ldf<COH>(q + c0), ldf<COH>(q + c1));
-                v[j] = pk(ldf<COH>(q + plane + c0), ldf<COH>(q + plane + c1));
-                x[j] = pk((float)c0, (float)c1);
-                y[j] = dup((float)cy);
+            const int row = i / NP;
+            c0[j] = ex + 2 * (i - row * NP);
+            c1[j] = c0[j] + 1;
+            cy[j] = ey + row;
+            if (!inside) {
+                c0[j] = clampi(c0[j], 0, w - 1);
+                c1[j] = clampi(c1[j], 0, w - 1);
+                cy[j] = clampi(cy[j], 0, h - 1);
             }
         }
+        load(c0, c1, cy, u, v);
         Taps2 tp[KI];
 #pragma unroll
         for (int j = 0; j < KI; ++j)
-            tp[j] = bil_taps2(I1, w, h, pitch, fadd2(x[j], u[j]), fadd2(y[j], v[j]));
+            tp[j] = bil_taps2(I1, w, h, pitch, fadd2(pk((float)c0[j], (float)c1[j]), u[j]),
+                              fadd2(dup((float)cy[j]), v[j]));
 #pragma unroll
         for (int j = 0; j < KI; ++j) {
             const int i = i0 + NT * j;
@@ -711,6 +707,26 @@ __device__ __forceinline__ void stage_window(const Windows<WH> &m, const float *
                 st_pair(m.V + 2 * i, v[j]);
                 st_pair(m.W + 2 * i, bil_lerp2(tp[j]));
             }
+        }
+    }
+}
+
+// The flow from its planes (an aligned pair where the window lies inside).
+template <int KI>
+__device__ __forceinline__ void load_planes(const float *__restrict__ a, size_t plane, int pitch,
+                                            bool inside, const int (&c0)[KI], const int (&c1)[KI],
+                                            const int (&cy)[KI], pair_t (&u)[KI],
+                                            pair_t (&v)[KI])
+{
+#pragma unroll
+    for (int j = 0; j < KI; ++j) {
+        const float *q = a + cy[j] * pitch;
+        if (inside) {
+            u[j] = ld_pair(q + c0[j]);
+            v[j] = ld_pair(q + plane + c0[j]);
+        } else {
+            u[j] = pk(q[c0[j]], q[c1[j]]);
+            v[j] = pk(q[plane + c0[j]], q[plane + c1[j]]);
         }
     }
 }
@@ -830,7 +846,10 @@ __device__ __forceinline__ void var_coeff_body(
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int tx = bx * 64 - 1, ty = by * TH;
     const bool inside = tx >= 2 && ty >= 2 && tx + 66 <= w && ty + TH + 2 <= h;
-    stage_window<WH, NT, 3, false>(m, U, plane, I1, w, h, pitch, tx - 2, ty - 2, inside);
+    stage_window<WH, NT, 3>(m, I1, w, h, pitch, tx - 2, ty - 2, inside,
+                            [&](auto &c0, auto &c1, auto &cy, auto &u, auto &v) {
+                                load_planes<3>(U, plane, pitch, inside, c0, c1, cy, u, v);
+                            });
     __syncthreads();
     derive_window<WH, NT>(m, alpha_s);
     __syncthreads();
@@ -900,17 +919,24 @@ seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
 // list of items (iteration, region of 64 x 16 VS), iteration by iteration; a
 // block claims them in order from a counter, the next one while it works on
 // the last:
-//  E. It waits for the previous iteration of the region and its eight
-//     neighbours (the halo and the 2 px around are no wider than an interior).
-//  A. It stages the flow of the region and 2 px around, and the warped image
-//     there (positions outside the level are those of the nearest pixel
-//     inside, which gives the replicated borders of the differences).
+//  A. It stages the flow of the region and 2 px around, which the region and
+//     its eight neighbours wrote in the previous iteration (the halo and the
+//     2 px are no wider than an interior), and the warped image there.
 //  B. The warped image's derivatives and the smoothness weights, 1 px around.
 //  C. Each thread builds the systems of its strip in registers, where the
 //     sweeps use them: they never leave the SM.
-//  D. The sweeps, then U + dU of the interior to the other flow buffer.
+//  D. The sweeps, then U + dU of the interior.
 // The arithmetic is that of the per-iteration kernels, pixel by pixel with the
 // same rounding, so the flow is the same bit for bit.
+//
+// Between iterations the flow travels as packets of a pixel's (u, v) and a
+// 64-bit tag, written and read as one 128-bit word: a reader polls the packets
+// it needs until they carry the iteration's tag.  No flag and no fence stands
+// between a write and its use: a release fence alone took about 2000 of an
+// item's 12500 cycles (the acknowledgements of the block's stores), the polls
+// of a flag 700 more.  Two buffers take turns: a region overwrites one only
+// after its neighbours have written the other, so after they read the first.
+// Tags never repeat: a launch's follow on the last one's.
 //
 // Items are claimed by running blocks and in order, so whatever an item waits
 // for is already claimed by a block that runs: the kernel ends with any number
@@ -920,16 +946,37 @@ seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
 // It pays where an iteration's two launches are latency: the launches
 // themselves, and three round trips through L2 (flow, image, coefficients)
 // before the sweeps start.  The halo's systems are built again by every region
-// that holds them (1.9 times at 64 x 64, 3.2 at 64 x 32).  A 64 x 32 item takes
-// about 12500 cycles: the wait and the release 3000, A 2400, B 1300, C 2700,
-// the sweeps 2700.  Measured, with the launches of one iteration each in
-// brackets: a 346 x 260 window 165 us (175; both inside a graph), outside a
-// graph, where every launch costs more, 613 x 397 windows with all outputs 234
-// us (315) and the flow block on 641 x 479 surfaces 401 us (497).
+// that holds them (1.9 times at 64 x 64, 3.2 at 64 x 32).
 //
-// ctl: [0] the claim counter, [1] blocks gone, [2 + r] finished iterations of
-// region r.  The last block to leave sets them to 0 for the next launch.  Waits
-// are bounded; a block whose wait runs out reports kErrTimeout and leaves.
+// ctl: [0] the claim counter, [1] blocks gone, [2..3] the tag that the
+// launch's follow.  The last block to leave prepares them for the next launch.
+// Polls are bounded; a block whose polls run out reports kErrTimeout and leaves.
+//
+// Measured, a window of all levels: 346 x 260 425 us with launches, 324 with
+// flags, 298 with packets; 641 x 479 741 -> 665 us with its finest level here.
+__device__ __forceinline__ void store_packet(float4 *q, float u, float v, unsigned long long tag)
+{
+    asm volatile("{ .reg .b64 uv; .reg .b128 p;\n\t"
+                 "mov.b64 uv, {%1, %2};\n\t"
+                 "mov.b128 p, {uv, %3};\n\t"
+                 "st.relaxed.gpu.global.b128 [%0], p; }" ::"l"(q),
+                 "f"(u), "f"(v), "l"(tag)
+                 : "memory");
+}
+__device__ __forceinline__ bool load_packet(const float4 *q, unsigned long long tag, float &u,
+                                            float &v)
+{
+    unsigned long long got;
+    asm volatile("{ .reg .b64 uv; .reg .b128 p;\n\t"
+                 "ld.relaxed.gpu.global.b128 p, [%3];\n\t"
+                 "mov.b128 {uv, %2}, p;\n\t"
+                 "mov.b64 {%0, %1}, uv; }"
+                 : "=f"(u), "=f"(v), "=l"(got)
+                 : "l"(q)
+                 : "memory");
+    return got == tag;
+}
+
 template <int VS>
 constexpr size_t level_smem_bytes()
 {
@@ -942,7 +989,8 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                  const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h, int pitch,
                  size_t pfs, float *Ua, float *Ub, size_t ufs, size_t plane, int outer, int n_half,
                  int R, int nrx, int nry, float delta, float gamma, float alpha_s, float omega,
-                 int blocks, unsigned *ctl, long long wait_limit, int *err)
+                 int blocks, unsigned *ctl, float4 *xch, size_t xch_px, long long wait_limit,
+                 int *err)
 {
     constexpr int RH = VS * kVWarps, WH = RH + 4;
     extern __shared__ __align__(16) float lsm[];
@@ -952,6 +1000,9 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
     __shared__ int s_item;
     const int per_frame = nrx * nry, total = outer * blocks;
     clear_ends(ends);
+    // written by a launch's last block only
+    unsigned long long *ctl_tag = reinterpret_cast<unsigned long long *>(ctl + 2);
+    const unsigned long long base = *ctl_tag;
     if (t == 0) s_item = (int)atomicAdd(ctl, 1u);
     __syncthreads();
     for (int item = s_item; item < total; item = s_item) {
@@ -964,8 +1015,6 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
         const T *I0 = I0b + po, *I0x = I0xb + po, *I0y = I0yb + po, *I1 = I1b + po;
         // the staged window lies in the level (block-uniform)
         const bool inside = rx0 >= 2 && ry0 >= 2 && rx0 + kVR + 2 <= w && ry0 + RH + 2 <= h;
-        const float *a = ((k & 1) ? Ub : Ua) + (size_t)f * ufs;
-        float *b = ((k & 1) ? Ua : Ub) + (size_t)f * ufs;
         // the strip's template values, which do not depend on the wait
         pair_t i0[VS], i0x[VS], i0y[VS];
 #pragma unroll
@@ -977,33 +1026,40 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             i0x[r] = pk(in0 ? ldp(I0x + o) : 0.0f, in1 ? ldp(I0x + o + 1) : 0.0f);
             i0y[r] = pk(in0 ? ldp(I0y + o) : 0.0f, in1 ? ldp(I0y + o + 1) : 0.0f);
         }
-        // E
         bool late = false;
-        if (k > 0 && t < 9) {
-            const int nx = bx + t % 3 - 1, ny = by + t / 3 - 1;
-            if (nx >= 0 && nx < nrx && ny >= 0 && ny < nry) {
-                const unsigned *q = ctl + 2 + f * per_frame + ny * nrx + nx;
-                late = true;
-                for (long long it = 0; it < wait_limit; ++it) {
-                    unsigned got;
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
-                                 : "=r"(got)
-                                 : "l"(q)
-                                 : "memory");
-                    if ((int)got >= k) {
-                        late = false;
+        stage_window<WH, kVThreads, 3>(
+            m, I1, w, h, pitch, rx0 - 2, ry0 - 2, inside,
+            [&](auto &c0, auto &c1, auto &cy, auto &u, auto &v) {
+                if (k == 0) {
+                    load_planes<3>(Ua + (size_t)f * ufs, plane, pitch, inside, c0, c1, cy, u, v);
+                    return;
+                }
+                const float4 *src = xch + ((k - 1) & 1) * xch_px + (size_t)f * w * h;
+                const unsigned long long tag = base + k;
+                float x0[3], x1[3], y0[3], y1[3];
+                for (long long it = 0;; ++it) {
+                    bool ok = true;
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        ok &= load_packet(src + cy[j] * w + c0[j], tag, x0[j], y0[j]);
+                        ok &= load_packet(src + cy[j] * w + c1[j], tag, x1[j], y1[j]);
+                    }
+                    if (ok) break;
+                    if (it >= wait_limit) {
+                        late = true;
                         break;
                     }
                 }
-            }
-        }
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    u[j] = pk(x0[j], x1[j]);
+                    v[j] = pk(y0[j], y1[j]);
+                }
+            });
         if (__syncthreads_or(late)) {
             if (t == 0) atomicOr(err, kErrTimeout);
             break;
         }
-        stage_window<WH, kVThreads, 3, true>(m, a, plane, I1, w, h, pitch, rx0 - 2, ry0 - 2,
-                                             inside);
-        __syncthreads();
         derive_window<WH, kVThreads>(m, alpha_s);
         __syncthreads();
         Strip<VS> s;
@@ -1042,37 +1098,39 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
         for (int r = 0; r < VS; ++r) {
             if (r < p.r0 || r >= p.r1) continue;
             const int e = (wp * VS + r + 2) * kLvW + 2 * lane + 2;
-            float *q = b + (p.gy + r) * pitch + p.gx;
             const float2 u = upk(ld_pair(m.U + e)), v = upk(ld_pair(m.V + e));
             const float2 d0 = upk(s.d[r][0]), d1 = upk(s.d[r][1]);
+            const float2 nu = make_float2(u.x + d0.x, u.y + d1.x);
+            const float2 nv = make_float2(v.x + d0.y, v.y + d1.y);
+            if (k + 1 < outer) {
+                const unsigned long long tag = base + k + 1;
+                float4 *q = xch + (k & 1) * xch_px + (size_t)f * w * h + (p.gy + r) * w + p.gx;
+                if (p.c0) store_packet(q, nu.x, nv.x, tag);
+                if (p.c1) store_packet(q + 1, nu.y, nv.y, tag);
+                continue;
+            }
+            float *q = ((outer & 1) ? Ub : Ua) + (size_t)f * ufs + (p.gy + r) * pitch + p.gx;
             if (p.c0 && p.c1) {
-                __stcg(reinterpret_cast<float2 *>(q), make_float2(u.x + d0.x, u.y + d1.x));
-                __stcg(reinterpret_cast<float2 *>(q + plane), make_float2(v.x + d0.y, v.y + d1.y));
+                *reinterpret_cast<float2 *>(q) = nu;
+                *reinterpret_cast<float2 *>(q + plane) = nv;
             } else if (p.c0) {
-                __stcg(q, u.x + d0.x);
-                __stcg(q + plane, v.x + d0.y);
+                q[0] = nu.x;
+                q[plane] = nv.x;
             } else if (p.c1) {
-                __stcg(q + 1, u.y + d1.x);
-                __stcg(q + plane + 1, v.y + d1.y);
+                q[1] = nu.y;
+                q[plane + 1] = nv.y;
             }
         }
         if (t == 0) s_item = (int)next;
-        __syncthreads();  // the block's stores, its reads of the stage
-        if (t == 0)  // releases the whole block's stores, which the barrier ordered before it
-            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ctl + 2 + reg), "r"(k + 1)
-                         : "memory");
+        __syncthreads();  // the block's reads of the stage
     }
-    // the last block to leave resets the counters
-    __shared__ bool s_last;
+    // the last block to leave prepares the counters of the next launch
     if (t == 0) {
         __threadfence();
-        s_last = atomicInc(ctl + 1, gridDim.x - 1) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        for (int i = t; i < blocks; i += kVThreads) ctl[2 + i] = 0;
-        if (t == 0) ctl[0] = 0;
+        if (atomicInc(ctl + 1, gridDim.x - 1) == gridDim.x - 1) {
+            ctl[0] = 0;
+            *ctl_tag = base + outer;
+        }
     }
 }
 
@@ -1150,6 +1208,20 @@ void init_var_attributes()
     cudaGetLastError();
 }
 
+size_t level_pixels(const Geometry &geo, int var_sor, int cluster_max, int frames)
+{
+    const int R = sor_halo(var_sor), tile = sor_tile(R);
+    size_t most = 0;
+    if (tile < R + 2) return 0;
+    for (int l = 0; l < geo.levels; ++l) {
+        const Level &lv = geo.lv[l];
+        const int per = ((lv.w + tile - 1) / tile) * ((lv.h + tile - 1) / tile);
+        const int f = cluster_max > 0 ? std::min(frames, kLevelBlocks / std::max(per, 1)) : 1;
+        if (per <= kLevelBlocks) most = std::max(most, (size_t)lv.w * lv.h * std::max(f, 1));
+    }
+    return most;
+}
+
 int sor_halo(int var_sor) { return var_sor > 0 ? 2 * var_sor - 1 : 1; }
 int sor_tile(int R) { return kVR - 2 * R; }
 int coeff_tiles_x(int w) { return (w + 64) / 64; }  // the first tile starts at column -1
@@ -1191,19 +1263,23 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
     if (small_tiles) cgrd.y = (lv.h + kCoefRowsSmall - 1) / kCoefRowsSmall;
     const dim3 sgrd((lv.w + tile - 1) / tile, (lv.h + tile - 1) / tile, frames);
     // small levels of a single frame: every outer iteration in one launch (same
-    // flow bit for bit), where the regions fit one wave and a region's staged
-    // window reaches no further than its neighbours' interiors; 64 x 32 regions
-    // if they fit, else 64 x 64 (640 x 360: 112 of them, no slower than ten
-    // launches inside a graph, 12 % faster outside one).  Not for levels of
-    // more than one wave (1280 x 720: 171 us against 145), nor, unless asked
-    // for, for several frames, whose launches fill the SMs (640 x 480, eight
-    // frames: 1.21 against 1.20 ms a call)
+    // flow bit for bit), where a region's staged window reaches no further than
+    // its neighbours' interiors: 64 x 32 regions if one wave holds them (more
+    // was slower at every size: 640 x 360, 364 of them, 582 us a window against
+    // 548 with 112 of 64 x 64), else 64 x 64 up to 1.75 waves.  There the items
+    // of all iterations fill the waves that a launch an iteration leaves open;
+    // one window (all levels) with the finest level here against per-iteration
+    // launches: 640 x 480, 154 regions, 605 against 640 us; 800 x 600, 252, 733
+    // against 739; 880 x 640, 280, 775 against 767; 1280 x 720, 448, 960 against
+    // 935.  Several frames fill the SMs either way (640 x 480, eight frames:
+    // 1.01 ms a call with and without), so only where asked for
     for (int vs : {kVSmallVS, kVS}) {
         const int ty = vs * kVWarps - 2 * R, nrx = (int)sgrd.x;
         const int nry = ty > 0 ? (lv.h + ty - 1) / ty : 0;
         const long long per = (long long)nrx * nry, blocks = per * frames;
+        const long long most = std::min(vs == kVS ? 7 * nsm / 4 : nsm, kLevelBlocks);
         if (!fp.level_ctl || fp.var_outer < 1 || ty < R + 2 || tile < R + 2 || lv.w < 2 ||
-            lv.h < 2 || nsm < 1 || blocks > std::min(nsm, kLevelBlocks) ||
+            lv.h < 2 || nsm < 1 || blocks > most || (size_t)lv.w * lv.h * frames > fp.level_px ||
             (frames > 1 && per > fp.var_cluster_max))
             continue;
         const bool small_form = vs == kVSmallVS;
@@ -1221,7 +1297,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
                        (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride,   \
                        U, Utmp, u_frame_stride, lv.plane, fp.var_outer, n_half, R, nrx, nry,    \
                        fp.delta, fp.gamma, fp.alpha_s, fp.omega, (int)blocks, fp.level_ctl,     \
-                       kWaitLimitDefault, err)
+                       (float4 *)fp.level_xch, fp.level_px, kWaitLimitDefault, err)
             if (fp.half)
                 e = small_form ? EBOF_LV(kVSmallVS, __half) : EBOF_LV(kVS, __half);
             else

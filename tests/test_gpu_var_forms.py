@@ -65,3 +65,34 @@ def test_forms_agree_and_match_the_oracle(eb, W, H, sor, batch):
                             var_sor=sor)[2]
     F = flows[0][0]
     assert np.hypot(F[0] - U[0], F[1] - U[1]).mean() <= 0.05
+
+
+@pytest.mark.parametrize("W,H,sor,outer", [
+    (46, 46, 5, 2), (93, 47, 5, 1), (139, 185, 5, 5), (71, 353, 0, 3), (230, 131, 3, 4),
+    (346, 260, 5, 5), (645, 479, 5, 5), (873, 645, 5, 2)])
+def test_one_launch_a_level_is_a_launch_an_iteration(eb, W, H, sor, outer):
+    """Windows one by one (small levels in one launch) and three a call (a
+    launch per iteration): equal bit for bit, with levels of one region, of
+    several, of more than a wave of them and of too many; twice, so that the
+    second pass starts from the packets and counters of the first."""
+    n = 3
+    ev = synth.translating_segments(width=W, height=H, n_windows=2 * n + 1, n_segments=14,
+                                    events_per_window=max(600, W * H // 8), seed=W + outer)
+    flows = []
+    for batch in (1, n):
+        p = eb.ebof_default_params(W, H)
+        p.var_sor, p.var_outer, p.max_batch = sor, outer, batch
+        st, s = eb.ebof_stream_create(p, 0)
+        eb.check(st)
+        flow = torch.zeros((2 * n + 1, 2, H, W), dtype=torch.float32, device="cuda")
+        for k in range(0, 2 * n + 1, batch if flows else 1):
+            m = min(batch, 2 * n + 1 - k)
+            a, b = int(ev.offsets[k]), int(ev.offsets[k + m])
+            eb.check(eb.ebof_process_windows(s, m, _dev(ev.x[a:b]), _dev(ev.y[a:b]),
+                                             _dev(ev.t[a:b]), None, int(ev.t_begin[k]), ev.dt,
+                                             flow[k:k + m]))
+        eb.check(eb.ebof_stream_sync(s, 1)[0])
+        flows.append(flow.cpu().numpy())
+        s.close()
+    assert np.array_equal(flows[0], flows[1])
+    assert np.abs(flows[0][-1]).max() > 0
