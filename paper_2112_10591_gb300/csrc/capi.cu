@@ -67,8 +67,8 @@ struct ebof_stream {
     unsigned long long *d_dropped_time = nullptr;
     int *d_err = nullptr;
     unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
-    char *d_xch = nullptr;      // and its packets: 2 x level_px x kPacketBytes
-    size_t level_px = 0;
+    char *d_xch = nullptr;      // and its packets: 2 x level_n x kPacketBytes
+    size_t level_n = 0;
     float *flow_stage = nullptr;  // device flow for the host-buffer call
     void *ev_stage = nullptr;     // device events for the host-buffer call
     size_t ev_stage_bytes = 0;
@@ -157,8 +157,8 @@ struct ebof_group {
     unsigned long long *d_dropped_time = nullptr;
     int *d_err = nullptr;
     unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
-    char *d_xch = nullptr;      // and its packets: 2 x level_px x kPacketBytes
-    size_t level_px = 0;
+    char *d_xch = nullptr;      // and its packets: 2 x level_n x kPacketBytes
+    size_t level_n = 0;
     ebof_window_desc *d_desc = nullptr;
     int64_t *h_events = nullptr;  // events given per stream in the last step
     int parity = 0;
@@ -402,7 +402,7 @@ FlowParams flow_params(const ebof_params &p)
     fp.var_cluster_max = p.var_cluster_max;
     fp.level_ctl = nullptr;
     fp.level_xch = nullptr;
-    fp.level_px = 0;
+    fp.level_n = 0;
     return fp;
 }
 
@@ -485,7 +485,7 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
             if (parts == kPartAll) {
                 fp.level_ctl = s->d_ctl;
                 fp.level_xch = s->d_xch;
-                fp.level_px = s->level_px;
+                fp.level_n = s->level_n;
             }
             const Level &lv = geo.lv[l];
             const char *I0 = pyr + ((size_t)prev_first * s->pyr_fs + geo.pyr_off[l]) * es;
@@ -938,7 +938,7 @@ void run_group_flow(ebof_group *g, bool with_flow, cudaStream_t st)
         FlowParams fp = flow_params(p);
         fp.level_ctl = g->d_ctl;
         fp.level_xch = g->d_xch;
-        fp.level_px = g->level_px;
+        fp.level_n = g->level_n;
         float *Ucur = nullptr, *Uc = nullptr;
         const Level *lvc = nullptr;
         for (int l = geo.levels - 1; l >= 0; --l) {
@@ -1506,8 +1506,8 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     ok &= dmalloc(&s->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&s->d_err, sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&s->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
-    s->level_px = level_pixels(geo, p->var_sor, p->var_cluster_max, B);
-    ok &= dmalloc(&s->d_xch, 2 * kPacketBytes * s->level_px) == cudaSuccess;
+    s->level_n = level_packets(geo, p->var_sor, p->var_cluster_max, B);
+    ok &= dmalloc(&s->d_xch, 2 * kPacketBytes * s->level_n) == cudaSuccess;
     ok &= dmalloc(&s->flow_stage, sizeof(float) * 2 * (size_t)p->width * p->height) == cudaSuccess;
     ok &= cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming) == cudaSuccess;
     const size_t call_bytes = (sizeof(ebof_window_desc) + sizeof(float *)) * B;
@@ -1527,7 +1527,7 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     }
     cudaMemset(s->d_err, 0, sizeof(int));
     cudaMemset(s->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
-    cudaMemset(s->d_xch, 0, 2 * kPacketBytes * s->level_px);
+    cudaMemset(s->d_xch, 0, 2 * kPacketBytes * s->level_n);
     cudaMemset(s->dstats, 0, sizeof(DevStats) * B);
     make_coef_maps(s->work, s->geo, B, &s->cmaps);
     cudaMemset(s->d_dropped_time, 0, sizeof(unsigned long long));
@@ -1551,7 +1551,7 @@ int64_t ebof_stream_device_bytes(const ebof_params *p)
     total += r(4 * 2 * (size_t)std::max(geo.max_patches, 1) * B);
     total += 2 * r(4 * (2 * plane0 * B + 1)) + r(4 * 9 * plane0 * B);
     total += 256;  // the one-launch refinement's counters, then its packets
-    total += r(2 * kPacketBytes * level_pixels(geo, p->var_sor, p->var_cluster_max, p->max_batch));
+    total += r(2 * kPacketBytes * level_packets(geo, p->var_sor, p->var_cluster_max, p->max_batch));
     total += r(sizeof(DevStats) * B) + 2 * 256 + r(4 * 2 * (size_t)p->width * p->height) +
              r((sizeof(ebof_window_desc) + sizeof(float *)) * B);
     return (int64_t)total;
@@ -2054,8 +2054,8 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     ok &= dmalloc(&g->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&g->d_err, sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&g->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
-    g->level_px = level_pixels(g->geo, q.var_sor, q.var_cluster_max, n);
-    ok &= dmalloc(&g->d_xch, 2 * kPacketBytes * g->level_px) == cudaSuccess;
+    g->level_n = level_packets(g->geo, q.var_sor, q.var_cluster_max, n);
+    ok &= dmalloc(&g->d_xch, 2 * kPacketBytes * g->level_n) == cudaSuccess;
     ok &= dmalloc(&g->d_desc, sizeof(ebof_window_desc) * n) == cudaSuccess;
     ok &= cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking) == cudaSuccess;
     ok &= cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming) == cudaSuccess;
@@ -2067,7 +2067,7 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     }
     cudaMemset(g->d_err, 0, sizeof(int));
     cudaMemset(g->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
-    cudaMemset(g->d_xch, 0, 2 * kPacketBytes * g->level_px);
+    cudaMemset(g->d_xch, 0, 2 * kPacketBytes * g->level_n);
     cudaMemset(g->flow, 0, sizeof(float) * 2 * (size_t)q.width * q.height * n);
     make_coef_maps(g->work, g->geo, n, &g->cmaps);
     if (cudaDeviceSynchronize() != cudaSuccess) {

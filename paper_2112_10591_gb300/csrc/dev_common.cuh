@@ -1,6 +1,7 @@
 // dev_common.cuh -- small device helpers shared by the flow kernels.
 #pragma once
 
+#include <cstdint>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -19,6 +20,14 @@ __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b)
 __device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float ffma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// x / s for x >= 0, s >= 1 and x s < 2^31, so that rounding the reciprocal up
+// never reaches the next integer.  magic = 2^31 / s + 1.
+inline uint32_t stride_magic(int s) { return (uint32_t)((1u << 31) / (uint32_t)s + 1); }
+__device__ __forceinline__ int div_stride(int x, uint32_t magic)
+{
+    return (int)(((unsigned long long)(uint32_t)x * magic) >> 31);
+}
 
 // Two floats in one 64-bit register: the packed FP32 instructions round each
 // half as the scalar ones do.  A packed multiply-add holds the FMA pipe as long

@@ -89,16 +89,16 @@ struct FlowParams {
     // variational layouts (ebof_params): none changes a result
     int sor_tma_min_per_sm, sor_row_waves, var_cluster_max;
     // the one-launch refinement's counters (kLevelCtl words, 0 at first) and
-    // two packet buffers of level_px pixels of 16 bytes (0 at first), used by
+    // two buffers of level_n packets of 16 bytes (0 at first), used by
     // no other launch at the same time; null: one launch per step
     unsigned *level_ctl;
     void *level_xch;
-    size_t level_px;
+    size_t level_n;
 };
 constexpr int kLevelBlocks = 266;  // most regions of a one-launch refinement
 constexpr int kLevelCtl = 4;
-// level_px for a stream or group of up to `frames` frames a call.
-size_t level_pixels(const Geometry &geo, int var_sor, int cluster_max, int frames);
+// level_n for a stream or group of up to `frames` frames a call.
+size_t level_packets(const Geometry &geo, int var_sor, int cluster_max, int frames);
 
 // Launchers (each enqueues on `st`; frames = batch size). ---------------------
 

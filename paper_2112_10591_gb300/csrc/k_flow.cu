@@ -561,14 +561,6 @@ seg_patch_search_kernel(const __grid_constant__ SegTable<SegSearch> tab)
 }
 
 // ---------------------------------------------------------------- A7
-// x / s for 0 <= x < 2^15 and 1 <= s < 2^15: x s < 2^31, so rounding the
-// reciprocal up never reaches the next integer.  magic = 2^31 / s + 1.
-inline uint32_t stride_magic(int s) { return (uint32_t)((1u << 31) / (uint32_t)s + 1); }
-__device__ __forceinline__ int div_stride(int x, uint32_t magic)
-{
-    return (int)(((unsigned long long)(uint32_t)x * magic) >> 31);
-}
-
 // The patches that cover x along an axis of n: the regular ones lo .. hi, and
 // whether the last one does.
 __device__ __forceinline__ void cover_range(int x, int n, int ps, int stride, uint32_t magic,

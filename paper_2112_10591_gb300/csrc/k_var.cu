@@ -669,7 +669,9 @@ __device__ __forceinline__ void st_pair(float *a, pair_t v)
 // level are those of the nearest pixel inside: the replicated borders of the
 // differences.  inside: the window lies in the level (block-uniform).
 // load(c0, c1, cy, u, v): the flow of KI pairs of pixels (c0, cy), (c1, cy);
-// all of a thread's loads come before their first use.
+// all of a thread's loads come before their first use.  A pair is half a row
+// apart, so that a warp's taps lie side by side (adjacent pixels a pair spread
+// them over twice the lines: 640 x 360 in one launch 60.0 us against 57.7).
 template <int WH, int NT, int KI, typename T, class L>
 __device__ __forceinline__ void stage_window(const Windows<WH> &m, const T *__restrict__ I1,
                                              int w, int h, int pitch, int ex, int ey, bool inside,
@@ -684,8 +686,8 @@ __device__ __forceinline__ void stage_window(const Windows<WH> &m, const T *__re
         for (int j = 0; j < KI; ++j) {
             const int i = min(i0 + NT * j, NI - 1);
             const int row = i / NP;
-            c0[j] = ex + 2 * (i - row * NP);
-            c1[j] = c0[j] + 1;
+            c0[j] = ex + i - row * NP;
+            c1[j] = c0[j] + NP;
             cy[j] = ey + row;
             if (!inside) {
                 c0[j] = clampi(c0[j], 0, w - 1);
@@ -703,9 +705,14 @@ __device__ __forceinline__ void stage_window(const Windows<WH> &m, const T *__re
         for (int j = 0; j < KI; ++j) {
             const int i = i0 + NT * j;
             if (i < NI) {
-                st_pair(m.U + 2 * i, u[j]);
-                st_pair(m.V + 2 * i, v[j]);
-                st_pair(m.W + 2 * i, bil_lerp2(tp[j]));
+                const int e = i + i / NP * NP;
+                const float2 uu = upk(u[j]), vv = upk(v[j]), ww = upk(bil_lerp2(tp[j]));
+                m.U[e] = uu.x;
+                m.U[e + NP] = uu.y;
+                m.V[e] = vv.x;
+                m.V[e + NP] = vv.y;
+                m.W[e] = ww.x;
+                m.W[e + NP] = ww.y;
             }
         }
     }
@@ -721,13 +728,8 @@ __device__ __forceinline__ void load_planes(const float *__restrict__ a, size_t 
 #pragma unroll
     for (int j = 0; j < KI; ++j) {
         const float *q = a + cy[j] * pitch;
-        if (inside) {
-            u[j] = ld_pair(q + c0[j]);
-            v[j] = ld_pair(q + plane + c0[j]);
-        } else {
-            u[j] = pk(q[c0[j]], q[c1[j]]);
-            v[j] = pk(q[plane + c0[j]], q[plane + c1[j]]);
-        }
+        u[j] = pk(q[c0[j]], q[c1[j]]);
+        v[j] = pk(q[plane + c0[j]], q[plane + c1[j]]);
     }
 }
 
@@ -917,8 +919,9 @@ seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
 
 // The whole variational refinement of a level in one launch.  The work is a
 // list of items (iteration, region of 64 x 16 VS), iteration by iteration; a
-// block claims them in order from a counter, the next one while it works on
-// the last:
+// block claims them in order from a counter, the next one during the sweeps
+// of the last (not before: a block that started early must not take an item
+// of one that starts a little later, which would then come an item late):
 //  A. It stages the flow of the region and 2 px around, which the region and
 //     its eight neighbours wrote in the previous iteration (the halo and the
 //     2 px are no wider than an interior), and the warped image there.
@@ -952,8 +955,17 @@ seg_var_coeff_kernel(const __grid_constant__ SegTable<SegCoeff> tab)
 // launch's follow.  The last block to leave prepares them for the next launch.
 // Polls are bounded; a block whose polls run out reports kErrTimeout and leaves.
 //
-// Measured, a window of all levels: 346 x 260 425 us with launches, 324 with
-// flags, 298 with packets; 641 x 479 741 -> 665 us with its finest level here.
+// Measured, two windows of all levels: 346 x 260 425 us with launches, 324 with
+// flags, 298 with packets; a window of 641 x 479 and its surface 741 us with
+// its finest level in launches, 647 here.
+//
+// The packets of odd and of even columns lie apart: regions start at odd ones,
+// so a warp's accesses, a pair of pixels a lane, are contiguous.
+__host__ __device__ __forceinline__ int packet_pitch(int w) { return (w + 1) >> 1; }
+__device__ __forceinline__ int packet_at(int x, int y, int w2, int h)
+{
+    return ((x & 1 ? 0 : h) + y) * w2 + (x >> 1);
+}
 __device__ __forceinline__ void store_packet(float4 *q, float u, float v, unsigned long long tag)
 {
     asm volatile("{ .reg .b64 uv; .reg .b128 p;\n\t"
@@ -989,16 +1001,19 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                  const T *__restrict__ I0yb, const T *__restrict__ I1b, int w, int h, int pitch,
                  size_t pfs, float *Ua, float *Ub, size_t ufs, size_t plane, int outer, int n_half,
                  int R, int nrx, int nry, float delta, float gamma, float alpha_s, float omega,
-                 int blocks, unsigned *ctl, float4 *xch, size_t xch_px, long long wait_limit,
+                 int blocks, uint3 mg, unsigned *ctl, float4 *xch, size_t xch_n, long long wait_limit,
                  int *err)
 {
     constexpr int RH = VS * kVWarps, WH = RH + 4;
+    // pairs a thread stages: all of them at once, one wait for the packets
+    constexpr int KI = (kLvW / 2 * WH + kVThreads - 1) / kVThreads;
     extern __shared__ __align__(16) float lsm[];
     const Windows<WH> m(lsm);
     __shared__ StripEnds<kVWarps> ends;
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
     __shared__ int s_item;
     const int per_frame = nrx * nry, total = outer * blocks;
+    const int w2 = packet_pitch(w), pk_fs = 2 * w2 * h;
     clear_ends(ends);
     // written by a launch's last block only
     unsigned long long *ctl_tag = reinterpret_cast<unsigned long long *>(ctl + 2);
@@ -1006,43 +1021,32 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
     if (t == 0) s_item = (int)atomicAdd(ctl, 1u);
     __syncthreads();
     for (int item = s_item; item < total; item = s_item) {
-        const unsigned next = t == 0 ? atomicAdd(ctl, 1u) : 0u;
-        const int k = item / blocks, reg = item - k * blocks, f = reg / per_frame;
-        const int rem = reg - f * per_frame, by = rem / nrx, bx = rem - by * nrx;
+        const int k = div_stride(item, mg.x), reg = item - k * blocks;
+        const int f = div_stride(reg, mg.y), rem = reg - f * per_frame;
+        const int by = div_stride(rem, mg.z), bx = rem - by * nrx;
         const StripPlace<VS, kVWarps> p(bx, by, R, w, h, pitch, lane, wp);
         const int rx0 = p.gx - 2 * lane, ry0 = p.gy - wp * VS;
         const size_t po = (size_t)f * pfs;
         const T *I0 = I0b + po, *I0x = I0xb + po, *I0y = I0yb + po, *I1 = I1b + po;
         // the staged window lies in the level (block-uniform)
         const bool inside = rx0 >= 2 && ry0 >= 2 && rx0 + kVR + 2 <= w && ry0 + RH + 2 <= h;
-        // the strip's template values, which do not depend on the wait
-        pair_t i0[VS], i0x[VS], i0y[VS];
-#pragma unroll
-        for (int r = 0; r < VS; ++r) {
-            const int gx = p.gx, gy = p.gy + r, o = gy * pitch + gx;
-            const bool in0 = inside || (gx >= 0 && gx < w && gy >= 0 && gy < h);
-            const bool in1 = inside || (gx + 1 >= 0 && gx + 1 < w && gy >= 0 && gy < h);
-            i0[r] = pk(in0 ? ldp(I0 + o) : 0.0f, in1 ? ldp(I0 + o + 1) : 0.0f);
-            i0x[r] = pk(in0 ? ldp(I0x + o) : 0.0f, in1 ? ldp(I0x + o + 1) : 0.0f);
-            i0y[r] = pk(in0 ? ldp(I0y + o) : 0.0f, in1 ? ldp(I0y + o + 1) : 0.0f);
-        }
         bool late = false;
-        stage_window<WH, kVThreads, 3>(
+        stage_window<WH, kVThreads, KI>(
             m, I1, w, h, pitch, rx0 - 2, ry0 - 2, inside,
             [&](auto &c0, auto &c1, auto &cy, auto &u, auto &v) {
                 if (k == 0) {
-                    load_planes<3>(Ua + (size_t)f * ufs, plane, pitch, inside, c0, c1, cy, u, v);
+                    load_planes<KI>(Ua + (size_t)f * ufs, plane, pitch, inside, c0, c1, cy, u, v);
                     return;
                 }
-                const float4 *src = xch + ((k - 1) & 1) * xch_px + (size_t)f * w * h;
+                const float4 *src = xch + ((k - 1) & 1) * xch_n + (size_t)f * pk_fs;
                 const unsigned long long tag = base + k;
-                float x0[3], x1[3], y0[3], y1[3];
+                float x0[KI], x1[KI], y0[KI], y1[KI];
                 for (long long it = 0;; ++it) {
                     bool ok = true;
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        ok &= load_packet(src + cy[j] * w + c0[j], tag, x0[j], y0[j]);
-                        ok &= load_packet(src + cy[j] * w + c1[j], tag, x1[j], y1[j]);
+                    for (int j = 0; j < KI; ++j) {
+                        ok &= load_packet(src + packet_at(c0[j], cy[j], w2, h), tag, x0[j], y0[j]);
+                        ok &= load_packet(src + packet_at(c1[j], cy[j], w2, h), tag, x1[j], y1[j]);
                     }
                     if (ok) break;
                     if (it >= wait_limit) {
@@ -1051,7 +1055,7 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                     }
                 }
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
+                for (int j = 0; j < KI; ++j) {
                     u[j] = pk(x0[j], x1[j]);
                     v[j] = pk(y0[j], y1[j]);
                 }
@@ -1059,6 +1063,18 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
         if (__syncthreads_or(late)) {
             if (t == 0) atomicOr(err, kErrTimeout);
             break;
+        }
+        // the strip's template values, in flight during B; no test between the
+        // loads, so that none waits for another (pixels outside the level: any
+        // value, their systems are 0)
+        pair_t i0[VS], i0x[VS], i0y[VS];
+        const int xa = clampi(p.gx, 0, w - 1), xb = clampi(p.gx + 1, 0, w - 1);
+#pragma unroll
+        for (int r = 0; r < VS; ++r) {
+            const int o = clampi(p.gy + r, 0, h - 1) * pitch;
+            i0[r] = pk(ldp(I0 + o + xa), ldp(I0 + o + xb));
+            i0x[r] = pk(ldp(I0x + o + xa), ldp(I0x + o + xb));
+            i0y[r] = pk(ldp(I0y + o + xa), ldp(I0y + o + xb));
         }
         derive_window<WH, kVThreads>(m, alpha_s);
         __syncthreads();
@@ -1093,6 +1109,7 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             }
         }
         // D
+        const unsigned next = t == 0 ? atomicAdd(ctl, 1u) : 0u;
         sor_sweeps<VS, kVWarps>(s, ends, lane, wp, (p.gx + p.gy) & 1, n_half, omega);
 #pragma unroll
         for (int r = 0; r < VS; ++r) {
@@ -1104,9 +1121,9 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             const float2 nv = make_float2(v.x + d0.y, v.y + d1.y);
             if (k + 1 < outer) {
                 const unsigned long long tag = base + k + 1;
-                float4 *q = xch + (k & 1) * xch_px + (size_t)f * w * h + (p.gy + r) * w + p.gx;
-                if (p.c0) store_packet(q, nu.x, nv.x, tag);
-                if (p.c1) store_packet(q + 1, nu.y, nv.y, tag);
+                float4 *q = xch + (k & 1) * xch_n + (size_t)f * pk_fs;
+                if (p.c0) store_packet(q + packet_at(p.gx, p.gy + r, w2, h), nu.x, nv.x, tag);
+                if (p.c1) store_packet(q + packet_at(p.gx + 1, p.gy + r, w2, h), nu.y, nv.y, tag);
                 continue;
             }
             float *q = ((outer & 1) ? Ub : Ua) + (size_t)f * ufs + (p.gy + r) * pitch + p.gx;
@@ -1208,7 +1225,10 @@ void init_var_attributes()
     cudaGetLastError();
 }
 
-size_t level_pixels(const Geometry &geo, int var_sor, int cluster_max, int frames)
+// The packets of a frame of a level.
+static size_t frame_packets(const Level &lv) { return 2 * (size_t)packet_pitch(lv.w) * lv.h; }
+
+size_t level_packets(const Geometry &geo, int var_sor, int cluster_max, int frames)
 {
     const int R = sor_halo(var_sor), tile = sor_tile(R);
     size_t most = 0;
@@ -1217,7 +1237,7 @@ size_t level_pixels(const Geometry &geo, int var_sor, int cluster_max, int frame
         const Level &lv = geo.lv[l];
         const int per = ((lv.w + tile - 1) / tile) * ((lv.h + tile - 1) / tile);
         const int f = cluster_max > 0 ? std::min(frames, kLevelBlocks / std::max(per, 1)) : 1;
-        if (per <= kLevelBlocks) most = std::max(most, (size_t)lv.w * lv.h * std::max(f, 1));
+        if (per <= kLevelBlocks) most = std::max(most, frame_packets(lv) * std::max(f, 1));
     }
     return most;
 }
@@ -1279,7 +1299,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
         const long long per = (long long)nrx * nry, blocks = per * frames;
         const long long most = std::min(vs == kVS ? 7 * nsm / 4 : nsm, kLevelBlocks);
         if (!fp.level_ctl || fp.var_outer < 1 || ty < R + 2 || tile < R + 2 || lv.w < 2 ||
-            lv.h < 2 || nsm < 1 || blocks > most || (size_t)lv.w * lv.h * frames > fp.level_px ||
+            lv.h < 2 || nsm < 1 || blocks > most || frame_packets(lv) * frames > fp.level_n ||
             (frames > 1 && per > fp.var_cluster_max))
             continue;
         const bool small_form = vs == kVSmallVS;
@@ -1289,6 +1309,9 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
         cfg.dynamicSmemBytes =
             small_form ? level_smem_bytes<kVSmallVS>() : level_smem_bytes<kVS>();
         cfg.stream = st;
+        // items < 1000 x 266, so the products stay below 2^31
+        const uint3 mg = make_uint3(stride_magic((int)blocks), stride_magic((int)per),
+                                    stride_magic(nrx));
         cudaError_t e;
         {
             StageScope sc(kStVarSor, 1, st);
@@ -1296,8 +1319,8 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
     cudaLaunchKernelEx(&cfg, var_level_kernel<VS, T>, (const T *)I0, (const T *)I0x,            \
                        (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride,   \
                        U, Utmp, u_frame_stride, lv.plane, fp.var_outer, n_half, R, nrx, nry,    \
-                       fp.delta, fp.gamma, fp.alpha_s, fp.omega, (int)blocks, fp.level_ctl,     \
-                       (float4 *)fp.level_xch, fp.level_px, kWaitLimitDefault, err)
+                       fp.delta, fp.gamma, fp.alpha_s, fp.omega, (int)blocks, mg, fp.level_ctl,     \
+                       (float4 *)fp.level_xch, fp.level_n, kWaitLimitDefault, err)
             if (fp.half)
                 e = small_form ? EBOF_LV(kVSmallVS, __half) : EBOF_LV(kVS, __half);
             else
