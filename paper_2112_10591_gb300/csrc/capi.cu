@@ -403,6 +403,7 @@ FlowParams flow_params(const ebof_params &p)
     fp.level_ctl = nullptr;
     fp.level_xch = nullptr;
     fp.level_n = 0;
+    fp.chained = false;
     return fp;
 }
 
@@ -455,8 +456,9 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
                 launch_scatter(x, y, t, nev, t_begin, dt, n, W, H, s->pitch0, s->E, s->e_fs,
                                s->dstats, s->d_dropped_time, st);
             launch_denoise_fill(s->E, s->Ed, s->Edf, W, H, s->pitch0, s->e_fs, n, p.connectivity,
-                                p.n_d, p.n_f, d_edge, s->dstats, st);
-            launch_edt_columns(s->Edf, s->pitch0, s->e_fs, W, H, s->g, s->pitch0, s->g_fs, n, st);
+                                p.n_d, p.n_f, d_edge, s->dstats, st, via_args || nev > 0);
+            launch_edt_columns(s->Edf, s->pitch0, s->e_fs, W, H, s->g, s->pitch0, s->g_fs, n, st,
+                               true);
             launch_edt_rows_surface(s->g, s->pitch0, s->g_fs, W, H, surface_map(p), d_edt,
                                     d_surface, I0cur, s->pitch0, s->pyr_fs, n, half, st);
         }
@@ -481,6 +483,7 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
         const Level *lvc = nullptr;
         for (int l = geo.levels - 1; l >= 0; --l) {
             tl_level = l;
+            fp.chained = parts == kPartAll || l + 1 < geo.levels;
             // windows in order: nothing else uses the counters meanwhile
             if (parts == kPartAll) {
                 fp.level_ctl = s->d_ctl;
@@ -915,8 +918,8 @@ void run_group(ebof_group *g, bool with_flow, cudaStream_t st)
     launch_scatter_desc(g->d_desc, n, W, H, g->pitch0, g->E, g->e_fs, g->dstats,
                         g->d_dropped_time, st);
     launch_denoise_fill(g->E, g->Ed, g->Edf, W, H, g->pitch0, g->e_fs, n, p.connectivity, p.n_d,
-                        p.n_f, nullptr, g->dstats, st);
-    launch_edt_columns(g->Edf, g->pitch0, g->e_fs, W, H, g->g, g->pitch0, g->g_fs, n, st);
+                        p.n_f, nullptr, g->dstats, st, true);
+    launch_edt_columns(g->Edf, g->pitch0, g->e_fs, W, H, g->g, g->pitch0, g->g_fs, n, st, true);
     launch_edt_rows_surface(g->g, g->pitch0, g->g_fs, W, H, surface_map(p), nullptr, nullptr, cur,
                             g->pitch0, g->pyr_fs, n, half, st);
     tl_level = 0;
@@ -943,6 +946,7 @@ void run_group_flow(ebof_group *g, bool with_flow, cudaStream_t st)
         const Level *lvc = nullptr;
         for (int l = geo.levels - 1; l >= 0; --l) {
             tl_level = l;
+            fp.chained = l + 1 < geo.levels;
             const Level &lv = geo.lv[l];
             const char *I0 = prv + geo.pyr_off[l] * es;
             const char *I1 = cur + geo.pyr_off[l] * es;

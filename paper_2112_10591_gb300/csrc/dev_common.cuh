@@ -21,6 +21,20 @@ __device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float ffma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
+// The first statement of every kernel of a window's chain.  A kernel launched
+// with launch_chained() may start before the one ahead of it on its stream has
+// ended, once that one's blocks have all called this: its launch, and its
+// blocks' start where there is room, then overlap the other's last wave.  Here
+// it waits until that kernel has ended and its writes are visible.  That one
+// waited in the same way, so everything before it has ended too.
+__device__ __forceinline__ void chain_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Of a chain's last kernel, which lets nothing start early.
+__device__ __forceinline__ void chain_end() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // x / s for x >= 0, s >= 1 and x s < 2^31, so that rounding the reciprocal up
 // never reaches the next integer.  magic = 2^31 / s + 1.
 inline uint32_t stride_magic(int s) { return (uint32_t)((1u << 31) / (uint32_t)s + 1); }

@@ -94,11 +94,37 @@ struct FlowParams {
     unsigned *level_ctl;
     void *level_xch;
     size_t level_n;
+    bool chained;  // the search's launch is behind a kernel of the same chain
 };
 constexpr int kLevelBlocks = 266;  // most regions of a one-launch refinement
 constexpr int kLevelCtl = 4;
 // level_n for a stream or group of up to `frames` frames a call.
 size_t level_packets(const Geometry &geo, int var_sor, int cluster_max, int frames);
+
+// Launches a kernel; chained: behind a kernel of the same chain, with nothing
+// between the two on the stream, as chain_begin() has it.  A window of 641 x 479
+// launched kernel by kernel: 585 us, 647 with full dependencies.  Inside a
+// graph full dependencies are the faster ones (two windows of 346 x 260 299 us,
+// 308 with early starts; one of 1280 x 720 463 against 480), so captured
+// launches keep them.
+template <class... P, class... A>
+cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t st, A... args)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (chained && cudaStreamIsCapturing(st, &capture) != cudaSuccess) chained = false;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained && capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
 
 // Launchers (each enqueues on `st`; frames = batch size). ---------------------
 
@@ -116,13 +142,14 @@ void launch_scatter_desc(const ebof_window_desc *desc, int frames, int W, int H,
 // A2: Alg. 1 then Alg. 2; writes E_df (pitched) and optional dense export.
 void launch_denoise_fill(const uint8_t *E, uint8_t *Ed, uint8_t *Edf, int W, int H, int pitch,
                          size_t frame_stride, int frames, int conn, int n_d, int n_f,
-                         uint8_t *export_dense, DevStats *stats, cudaStream_t st);
+                         uint8_t *export_dense, DevStats *stats, cudaStream_t st,
+                         bool chained = false);
 
 // A3: per column and 32 rows, the edge pixels' bits and the nearest edge rows
 // above and below; g: at least g_pitch * H int32 a frame.
 void launch_edt_columns(const uint8_t *E, int edge_pitch, size_t edge_frame_stride, int W,
                         int H, int32_t *g, int g_pitch, size_t g_frame_stride, int frames,
-                        cudaStream_t st);
+                        cudaStream_t st, bool chained = false);
 
 // A4: per-row lower envelope -> D, fused surface (Eq. 1 or an ablation
 // surface) and level-0 intensity.

@@ -28,6 +28,7 @@ template <typename T>
 __global__ void downsample_kernel(const T *__restrict__ I, int pitch, T *__restrict__ out,
                                   int wc, int hc, int pitch_c, size_t fs)
 {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= wc || y >= hc) return;
@@ -220,6 +221,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 pyramid_means_kernel(T *__restrict__ slots, size_t fs, PyrDesc d)
 {
+    chain_begin();
     pyramid_means_body(slots, fs, d, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -262,6 +264,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 pyramid_gradients_kernel(T *__restrict__ slots, size_t fs, PyrDesc d)
 {
+    chain_begin();
     pyramid_gradients_body(slots, fs, d, blockIdx.x, blockIdx.z);
 }
 
@@ -543,6 +546,7 @@ patch_search_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                     int hc, int pitch_c, size_t plane_c, size_t ucfs, float *__restrict__ upb,
                     size_t upfs, int stride, int iters, float kappa, int *err)
 {
+    chain_begin();
     patch_search_body<PS, CG, RG, T>(I0b, I0xb, I0yb, I1b, w, h, pitch, pfs, npx, npy, Ucb, wc, hc,
                                      pitch_c, plane_c, ucfs, upb, upfs, stride, iters, kappa, err,
                                      blockIdx.x, blockIdx.y);
@@ -730,6 +734,7 @@ densify_kernel(const T *__restrict__ I0b, const T *__restrict__ I1b, int w, int 
                float *__restrict__ Ub, size_t ufs, size_t plane, int ps, int stride,
                uint32_t magic)
 {
+    chain_begin();
     densify_body<T, NC>(I0b, I1b, w, h, pitch, pfs, upb, upfs, npx, npy, Ub, ufs, plane, ps,
                         stride, magic, blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -886,6 +891,7 @@ __device__ __forceinline__ void flow_out_body(const float *__restrict__ Ub, int 
 __global__ void flow_out_kernel(const float *__restrict__ Ub, int W, int H, int pitch,
                                 size_t ufs, size_t plane, float *__restrict__ flow)
 {
+    chain_end();
     flow_out_body(Ub, W, H, pitch, ufs, plane, flow, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -904,6 +910,7 @@ seg_flow_out_kernel(const __grid_constant__ SegTable<SegFlowOut> tab)
 __global__ void flow_out_ptr_kernel(const float *__restrict__ U, int W, int H, int pitch,
                                     size_t plane, size_t u_frame_stride, float *const *dst)
 {
+    chain_end();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= W) return;
@@ -924,7 +931,7 @@ void search_ps(const T *I0, const T *I0x, const T *I0y, const T *I1,
     dim3 grd(search_blocks(PS, wide, lv.npx, lv.npy), frames);
     auto kern = wide ? patch_search_kernel<PS, SS::kWideCG, SS::kWideRG, T>
                      : patch_search_kernel<PS, SS::kNarrowCG, SS::kNarrowRG, T>;
-    kern<<<grd, search_threads(wide), 0, st>>>(
+    launch_chained(fp.chained, kern, grd, search_threads(wide), 0, st,
         I0, I0x, I0y, I1, lv.w, lv.h, lv.pitch, pfs, lv.npx, lv.npy, Uc, lvc ? lvc->w : 0,
         lvc ? lvc->h : 0, lvc ? lvc->pitch : 0, lvc ? lvc->plane : 0, ucfs, up, upfs, fp.stride,
         fp.gn_iters, fp.gn_damping, err);
@@ -974,27 +981,31 @@ void launch_pyramid(void *slots, const Geometry &geo, size_t frame_stride, int f
         const dim3 grd((d.w[0] + 2 * kPyrTile - 1) / (2 * kPyrTile),
                        (d.h[0] + 2 * kPyrTile - 1) / (2 * kPyrTile), frames);
         if (half)
-            pyramid_means_kernel<__half><<<grd, blk, 0, st>>>((__half *)slots, frame_stride, d);
+            launch_chained(true, pyramid_means_kernel<__half>, grd, blk, 0, st, (__half *)slots,
+                           frame_stride, d);
         else
-            pyramid_means_kernel<float><<<grd, blk, 0, st>>>((float *)slots, frame_stride, d);
+            launch_chained(true, pyramid_means_kernel<float>, grd, blk, 0, st, (float *)slots,
+                           frame_stride, d);
     }
     for (int l = kPyrFused; l < d.levels; ++l) {  // levels beyond the fused tile
         char *base = (char *)slots;
         const dim3 grd = grid2d(d.w[l], d.h[l], frames, blk);
         if (half)
-            downsample_kernel<__half><<<grd, blk, 0, st>>>(
+            launch_chained(true, downsample_kernel<__half>, grd, blk, 0, st,
                 (const __half *)(base + d.off[l - 1] * es), d.pitch[l - 1],
                 (__half *)(base + d.off[l] * es), d.w[l], d.h[l], d.pitch[l], frame_stride);
         else
-            downsample_kernel<float><<<grd, blk, 0, st>>>(
+            launch_chained(true, downsample_kernel<float>, grd, blk, 0, st,
                 (const float *)(base + d.off[l - 1] * es), d.pitch[l - 1],
                 (float *)(base + d.off[l] * es), d.w[l], d.h[l], d.pitch[l], frame_stride);
     }
     const dim3 ggrd(nb, 1, frames);
     if (half)
-        pyramid_gradients_kernel<__half><<<ggrd, blk, 0, st>>>((__half *)slots, frame_stride, d);
+        launch_chained(true, pyramid_gradients_kernel<__half>, ggrd, blk, 0, st, (__half *)slots,
+                       frame_stride, d);
     else
-        pyramid_gradients_kernel<float><<<ggrd, blk, 0, st>>>((float *)slots, frame_stride, d);
+        launch_chained(true, pyramid_gradients_kernel<float>, ggrd, blk, 0, st, (float *)slots,
+                       frame_stride, d);
 }
 
 void launch_pyramid_export(const void *plane, bool half, int w, int h, int pitch, float *dst,
@@ -1057,11 +1068,11 @@ void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_
     // no patch beyond the border: a longer stride is the same grid
     const int stride = std::min(fp.stride, kMaxDim);
     const uint32_t magic = stride_magic(stride);
+    const bool chained = fp.chained || lv.npx * lv.npy > 0;  // the search is launched
 #define EBOF_DENSE(T, N)                                                                         \
-    densify_kernel<T, N><<<grd, blk, 0, st>>>((const T *)I0, (const T *)I1, lv.w, lv.h,         \
-                                              lv.pitch, pyr_frame_stride, up, up_frame_stride,   \
-                                              lv.npx, lv.npy, U, u_frame_stride, lv.plane, fp.ps,\
-                                              stride, magic)
+    launch_chained(chained, densify_kernel<T, N>, grd, blk, 0, st, (const T *)I0,                \
+                   (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride, up, up_frame_stride,   \
+                   lv.npx, lv.npy, U, u_frame_stride, lv.plane, fp.ps, stride, magic)
     if (fp.half) {
         if (nc == 2) EBOF_DENSE(__half, 2);
         else if (nc == 3) EBOF_DENSE(__half, 3);
@@ -1232,8 +1243,8 @@ void launch_flow_out_ptr(const float *U, int W, int H, int pitch, size_t u_frame
 {
     StageScope sc(kStFlowOut, 1, st);
     dim3 grd((W + 255) / 256, H, frames);
-    flow_out_ptr_kernel<<<grd, 256, 0, st>>>(U, W, H, pitch, (size_t)pitch * H, u_frame_stride,
-                                             dst);
+    launch_chained(true, flow_out_ptr_kernel, grd, 256, 0, st, U, W, H, pitch,
+                   (size_t)pitch * H, u_frame_stride, dst);
 }
 
 void launch_flow_out(const float *U, int W, int H, int pitch, size_t u_frame_stride,
@@ -1241,8 +1252,8 @@ void launch_flow_out(const float *U, int W, int H, int pitch, size_t u_frame_str
 {
     StageScope sc(kStFlowOut, 1, st);
     dim3 grd((W + 255) / 256, H, frames);
-    flow_out_kernel<<<grd, 256, 0, st>>>(U, W, H, pitch, u_frame_stride,
-                                         (size_t)pitch * H, flow);
+    launch_chained(true, flow_out_kernel, grd, 256, 0, st, U, W, H, pitch, u_frame_stride,
+                   (size_t)pitch * H, flow);
 }
 
 }  // namespace ebof

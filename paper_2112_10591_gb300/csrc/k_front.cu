@@ -6,6 +6,7 @@
 // parabolas), fused with Eq. 1, d_exp = 1 - exp(-sqrt(D) / alpha), and the
 // 8-bit intensity scale 255 * d_exp the flow block runs on.
 #include "ebof.h"
+#include "dev_common.cuh"
 #include "ebof_internal.cuh"
 #include "profiler.cuh"
 #include "seg.cuh"
@@ -48,6 +49,7 @@ __global__ void scatter_kernel(const uint16_t *__restrict__ x, const uint16_t *_
                                uint8_t *__restrict__ E, size_t fstride, DevStats *stats,
                                unsigned long long *dropped_time)
 {
+    chain_begin();
     const int64_t span = dt * (int64_t)n_windows;
     const int lane = threadIdx.x & 31;
     const int64_t per_block =
@@ -110,6 +112,7 @@ __global__ void scatter_desc_kernel(const ebof_window_desc *__restrict__ desc, i
                                     int pitch, uint8_t *__restrict__ E, size_t fstride,
                                     DevStats *stats, unsigned long long *dropped_time)
 {
+    chain_begin();
     const int f = blockIdx.y;
     const ebof_window_desc d = desc[f];
     const int lane = threadIdx.x & 31;
@@ -305,6 +308,7 @@ denoise_fill_kernel(const uint8_t *__restrict__ E, uint8_t *__restrict__ Edf, in
                     int pitch, size_t fstride, int conn, int n_d, int n_f,
                     uint8_t *__restrict__ export_dense, DevStats *stats)
 {
+    chain_begin();
     denoise_fill_body(E, Edf, W, H, pitch, fstride, conn, n_d, n_f, export_dense, stats,
                       blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -418,6 +422,7 @@ __global__ void __launch_bounds__(32 * kColWarps)
 edt_cols_kernel(const uint8_t *__restrict__ E, int epitch, size_t efs, int W, int H,
                 int32_t *__restrict__ g, int gpitch, size_t gfs)
 {
+    chain_begin();
     edt_cols_body(E, epitch, efs, W, H, g, gpitch, gfs, blockIdx.x, blockIdx.y);
 }
 
@@ -689,6 +694,7 @@ edt_rows_surface_kernel(const int32_t *__restrict__ g, int gpitch, size_t gfs, i
                         int rows_per_block, SurfaceMap sm, int32_t *__restrict__ D_dense,
                         float *__restrict__ S_dense, T *__restrict__ I0, int ipitch, size_t ifs)
 {
+    chain_begin();
     edt_rows_surface_body<WPR, T>(g, gpitch, gfs, W, H, rows_per_block, sm, D_dense, S_dense, I0,
                                   ipitch, ifs, blockIdx.x, blockIdx.y);
 }
@@ -717,6 +723,7 @@ template <typename T>
 __global__ void surface_to_intensity_kernel(const float *__restrict__ S, int W, int H,
                                             T *__restrict__ I0, int pitch, SurfaceMap sm)
 {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= W) return;
@@ -763,13 +770,13 @@ void launch_scatter_desc(const ebof_window_desc *desc, int frames, int W, int H,
 
 void launch_denoise_fill(const uint8_t *E, uint8_t *Ed, uint8_t *Edf, int W, int H, int pitch,
                          size_t frame_stride, int frames, int conn, int n_d, int n_f,
-                         uint8_t *export_dense, DevStats *stats, cudaStream_t st)
+                         uint8_t *export_dense, DevStats *stats, cudaStream_t st, bool chained)
 {
     (void)Ed;  // the denoised image stays in shared memory
     StageScope sc(kStDenoiseFill, 1, st);
     dim3 blk(kDfX, kDfY), grd((W + kDfX - 1) / kDfX, (H + kDfY - 1) / kDfY, frames);
-    denoise_fill_kernel<<<grd, blk, 0, st>>>(E, Edf, W, H, pitch, frame_stride, conn, n_d, n_f,
-                                             export_dense, stats);
+    launch_chained(chained, denoise_fill_kernel, grd, blk, 0, st, E, Edf, W, H, pitch,
+                   frame_stride, conn, n_d, n_f, export_dense, stats);
 }
 
 int edt_cols_warps(int H) { return std::min(col_words(H), kColWarps); }
@@ -777,12 +784,12 @@ size_t edt_cols_smem(int H) { return cols_smem_bytes(col_words(H)); }
 
 void launch_edt_columns(const uint8_t *E, int edge_pitch, size_t edge_frame_stride, int W,
                         int H, int32_t *g, int g_pitch, size_t g_frame_stride, int frames,
-                        cudaStream_t st)
+                        cudaStream_t st, bool chained)
 {
     StageScope sc(kStEdtCols, 1, st);
     dim3 blk(32, edt_cols_warps(H)), grd((W + 31) / 32, frames);
-    edt_cols_kernel<<<grd, blk, edt_cols_smem(H), st>>>(E, edge_pitch, edge_frame_stride, W, H, g,
-                                                        g_pitch, g_frame_stride);
+    launch_chained(chained, edt_cols_kernel, grd, blk, edt_cols_smem(H), st, E, edge_pitch,
+                   edge_frame_stride, W, H, g, g_pitch, g_frame_stride);
 }
 
 int edt_rows_block_rows(int W)
@@ -812,9 +819,8 @@ void edt_rows_t(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int
     dim3 grd((H + rows - 1) / rows, frames);
     auto kern = wpr == 1 ? edt_rows_surface_kernel<1, T>
                          : edt_rows_surface_kernel<kRowsPerBlock, T>;
-    kern<<<grd, 32 * (wpr == 1 ? rows : wpr), smem, st>>>(g, g_pitch, g_frame_stride, W, H, rows,
-                                                          sm, D_dense, S_dense, I0, i_pitch,
-                                                          i_frame_stride);
+    launch_chained(true, kern, grd, 32 * (wpr == 1 ? rows : wpr), smem, st, g, g_pitch,
+                   g_frame_stride, W, H, rows, sm, D_dense, S_dense, I0, i_pitch, i_frame_stride);
 }
 
 void launch_edt_direct(const uint8_t *edge, int W, int H, float alpha, int32_t *D_dense,

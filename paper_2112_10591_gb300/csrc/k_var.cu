@@ -431,6 +431,7 @@ var_sor_kernel(int w, int h, int pitch, const float *__restrict__ Uinb,
                float *__restrict__ Uoutb, size_t ufs, size_t plane,
                const float *__restrict__ coefb, size_t cfs, int R, int n_half, float omega)
 {
+    chain_begin();
     extern __shared__ float2 su[];
     __shared__ StripEnds<kVWarps> ends;
     sor_region<VS, kVWarps, false>(blockIdx.x, blockIdx.y, blockIdx.z, w, h, pitch, Uinb, Uoutb,
@@ -475,6 +476,7 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap, int w, int h, int p
                    size_t plane, int R, int nrx, int nry, int total, int n_half, float omega,
                    long long wait_limit, int *err)
 {
+    chain_begin();
     extern __shared__ __align__(1024) float tsm[];
     float *cbuf = tsm;  // [kCPlanes][kVR][kTmaBoxW]
     float2 *slot = reinterpret_cast<float2 *>(tsm + kTmaCoefFloats) + threadIdx.x;
@@ -894,6 +896,7 @@ var_coeff_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                  float *__restrict__ coefb, size_t cfs, float delta, float gamma, float alpha_s,
                  float omega)
 {
+    chain_begin();
     extern __shared__ __align__(16) float csm[];
     const int f = blockIdx.z;
     const size_t po = (size_t)f * pfs;
@@ -1004,6 +1007,7 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
                  int blocks, uint3 mg, unsigned *ctl, float4 *xch, size_t xch_n, long long wait_limit,
                  int *err)
 {
+    chain_begin();
     constexpr int RH = VS * kVWarps, WH = RH + 4;
     // pairs a thread stages: all of them at once, one wait for the packets
     constexpr int KI = (kLvW / 2 * WH + kVThreads - 1) / kVThreads;
@@ -1303,12 +1307,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
             (frames > 1 && per > fp.var_cluster_max))
             continue;
         const bool small_form = vs == kVSmallVS;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)std::min<long long>(blocks, nsm), 1, 1);
-        cfg.blockDim = dim3(kVThreads, 1, 1);
-        cfg.dynamicSmemBytes =
-            small_form ? level_smem_bytes<kVSmallVS>() : level_smem_bytes<kVS>();
-        cfg.stream = st;
+        const int lgrid = (int)std::min<long long>(blocks, nsm);
         // items < 1000 x 266, so the products stay below 2^31
         const uint3 mg = make_uint3(stride_magic((int)blocks), stride_magic((int)per),
                                     stride_magic(nrx));
@@ -1316,7 +1315,8 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
         {
             StageScope sc(kStVarSor, 1, st);
 #define EBOF_LV(VS, T)                                                                          \
-    cudaLaunchKernelEx(&cfg, var_level_kernel<VS, T>, (const T *)I0, (const T *)I0x,            \
+    launch_chained(true, var_level_kernel<VS, T>, lgrid, kVThreads, level_smem_bytes<VS>(), st, \
+                   (const T *)I0, (const T *)I0x,                                               \
                        (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride,   \
                        U, Utmp, u_frame_stride, lv.plane, fp.var_outer, n_half, R, nrx, nry,    \
                        fp.delta, fp.gamma, fp.alpha_s, fp.omega, (int)blocks, mg, fp.level_ctl,     \
@@ -1335,10 +1335,10 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
         {
             StageScope sc(kStVarCoeff, 1, st);
 #define EBOF_CF(TH, T)                                                                          \
-    var_coeff_kernel<TH, T><<<cgrd, kCoefThreads, Windows<TH + 4>::kBytes, st>>>(                \
-        (const T *)I0, (const T *)I0x, (const T *)I0y, (const T *)I1, lv.w, lv.h, lv.pitch,      \
-        pyr_frame_stride, a, u_frame_stride, lv.plane, coef, coef_frame_stride, fp.delta,        \
-        fp.gamma, fp.alpha_s, fp.omega)
+    launch_chained(true, var_coeff_kernel<TH, T>, cgrd, kCoefThreads,                            \
+                   Windows<TH + 4>::kBytes, st, (const T *)I0, (const T *)I0x, (const T *)I0y,   \
+                   (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride, a, u_frame_stride,     \
+                   lv.plane, coef, coef_frame_stride, fp.delta, fp.gamma, fp.alpha_s, fp.omega)
             if (fp.half) {
                 if (small_tiles) EBOF_CF(kCoefRowsSmall, __half);
                 else EBOF_CF(kCoefRows, __half);
@@ -1354,19 +1354,21 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
             const int row_waves = fp.sor_row_waves;
             const dim3 g1(sgrd.x, small > 0 ? (lv.h + small - 1) / small : 1, frames);
             if (coef_map && nsm > 0 && (long long)total >= (long long)fp.sor_tma_min_per_sm * nsm)
-                var_sor_tma_kernel<<<std::min(nsm, total), kVThreads, kTmaSmemBytes, st>>>(
-                    *coef_map, lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, R,
-                    (int)sgrd.x, (int)sgrd.y, total, n_half, fp.omega,
-                    fp.wait_limit >= 0 ? fp.wait_limit : kWaitLimitDefault, err);
+                launch_chained(true, var_sor_tma_kernel, std::min(nsm, total), kVThreads,
+                               kTmaSmemBytes, st, *coef_map, lv.w, lv.h, lv.pitch, a, b,
+                               u_frame_stride, lv.plane, R, (int)sgrd.x, (int)sgrd.y, total,
+                               n_half, fp.omega,
+                               fp.wait_limit >= 0 ? fp.wait_limit : kWaitLimitDefault, err);
             else if (small >= 8 && (long long)(g1.x * g1.y * g1.z) <= (long long)row_waves * nsm)
-                var_sor_kernel<kVSmallVS>
-                    <<<g1, kVThreads, flow_stage_bytes<kVSmallVS, kVWarps>(), st>>>(
-                        lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, coef,
-                        coef_frame_stride, R, n_half, fp.omega);
+                launch_chained(true, var_sor_kernel<kVSmallVS>, g1, kVThreads,
+                               flow_stage_bytes<kVSmallVS, kVWarps>(), st, lv.w, lv.h, lv.pitch,
+                               a, b, u_frame_stride, lv.plane, coef, coef_frame_stride, R, n_half,
+                               fp.omega);
             else
-                var_sor_kernel<kVS><<<sgrd, kVThreads, flow_stage_bytes<kVS, kVWarps>(), st>>>(
-                    lv.w, lv.h, lv.pitch, a, b, u_frame_stride, lv.plane, coef,
-                    coef_frame_stride, R, n_half, fp.omega);
+                launch_chained(true, var_sor_kernel<kVS>, sgrd, kVThreads,
+                               flow_stage_bytes<kVS, kVWarps>(), st, lv.w, lv.h, lv.pitch, a, b,
+                               u_frame_stride, lv.plane, coef, coef_frame_stride, R, n_half,
+                               fp.omega);
         }
         float *t = a;
         a = b;
