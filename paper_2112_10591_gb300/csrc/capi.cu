@@ -500,7 +500,7 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
             launch_densify(I0, I1, lv, s->pyr_fs, sc.up, s->up_fs, Ucur, s->u_fs, nf, fp, st);
             // the coarser flow is consumed by the search: its buffer is free
             float *Utmp = (Ucur == sc.Ua) ? sc.Ub : sc.Ua;
-            const CUtensorMap *cmap =
+            const SorMaps *cmap =
                 sc.cmaps && sc.cmaps->ok[l] ? &sc.cmaps->map[l] : nullptr;
             Ucur = launch_variational(I0, I0x, I0y, I1, lv, s->pyr_fs, Ucur, Utmp, s->u_fs,
                                       sc.work, s->work_fs, nf, fp, cmap, s->d_err, st);
@@ -752,7 +752,8 @@ ebof_status pipeline_ready(ebof_stream *s)
         pipeline_release(s);
         return EBOF_ERR_OOM;
     }
-    for (int f = 1; f < kPipeFlows; ++f) make_coef_maps(L.work[f], s->geo, 1, &L.cmaps[f]);
+    for (int f = 1; f < kPipeFlows; ++f)
+        make_coef_maps(L.work[f], L.Ua[f], L.Ub[f], s->u_fs, s->geo, s->p.var_sor, 1, &L.cmaps[f]);
     L.h_call.assign(kPipeSlots * kPipeCallBytes, 0);
     L.ready = true;
     return EBOF_OK;
@@ -1220,7 +1221,7 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
                 const FlowParams fp = flow_params(g->p);
                 const float *Uc = x.U;
                 const Level *lvc = x.lvc;
-                const CUtensorMap *cmap = g->cmaps.ok[l] ? &g->cmaps.map[l] : nullptr;
+                const SorMaps *cmap = g->cmaps.ok[l] ? &g->cmaps.map[l] : nullptr;
                 P.ops.push_back([=](cudaStream_t st) {
                     tl_level = l;
                     launch_patch_search(I0, I0x, I0y, I1, *lv, g->pyr_fs, Uc, lvc, g->u_fs, g->up,
@@ -1533,7 +1534,7 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     cudaMemset(s->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
     cudaMemset(s->d_xch, 0, 2 * kPacketBytes * s->level_n);
     cudaMemset(s->dstats, 0, sizeof(DevStats) * B);
-    make_coef_maps(s->work, s->geo, B, &s->cmaps);
+    make_coef_maps(s->work, s->Ua, s->Ub, s->u_fs, s->geo, p->var_sor, B, &s->cmaps);
     cudaMemset(s->d_dropped_time, 0, sizeof(unsigned long long));
     if (cudaDeviceSynchronize() != cudaSuccess) {
         free_all(s);
@@ -2073,7 +2074,7 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     cudaMemset(g->d_ctl, 0, sizeof(unsigned) * kLevelCtl);
     cudaMemset(g->d_xch, 0, 2 * kPacketBytes * g->level_n);
     cudaMemset(g->flow, 0, sizeof(float) * 2 * (size_t)q.width * q.height * n);
-    make_coef_maps(g->work, g->geo, n, &g->cmaps);
+    make_coef_maps(g->work, g->Ua, g->Ub, g->u_fs, g->geo, q.var_sor, n, &g->cmaps);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         free_group(g);
         delete g;

@@ -199,29 +199,36 @@ void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_
 // Tensor maps (TMA descriptors) of the variational coefficient planes of
 // each pyramid level in a stream's or group's work buffer: level l holds
 // frames x coeff_planes() planes of pitch_l x h_l floats.
+struct SorMaps {
+    CUtensorMap coef;
+    CUtensorMap u[2];       // of the flow buffers
+    const float *ubase[2];  // which these are
+};
 struct CoefMaps {
     bool ok[kMaxLevels];
-    CUtensorMap map[kMaxLevels];
+    SorMaps map[kMaxLevels];
 };
-// Fills m for `frames` frames of `work`; levels whose map cannot be encoded
-// are marked not ok (their SOR sweeps then load the planes directly).
-void make_coef_maps(float *work, const Geometry &geo, int frames, CoefMaps *m);
+// Fills m for `frames` frames of `work` and of the flow buffers Ua, Ub, as a
+// level lays them out; levels whose maps cannot be encoded are marked not ok
+// (their SOR sweeps then load directly).
+void make_coef_maps(float *work, const float *Ua, const float *Ub, size_t u_frame_stride,
+                    const Geometry &geo, int var_sor, int frames, CoefMaps *m);
 
 // A8: variational refinement of U.  Returns the buffer holding the result:
 // U itself, or Utmp (same shape as U) when the fused kernel ping-pongs.
-// coef_map: the level's coefficient tensor map, or nullptr; err: device
+// maps: the level's tensor maps, or nullptr; err: device
 // error word (kErrTimeout if a bounded wait runs out).
 float *launch_variational(const void *I0, const void *I0x, const void *I0y, const void *I1,
                           const Level &lv, size_t pyr_frame_stride, float *U, float *Utmp,
                           size_t u_frame_stride, float *work, size_t work_frame_stride,
-                          int frames, const FlowParams &fp, const CUtensorMap *coef_map,
+                          int frames, const FlowParams &fp, const SorMaps *maps,
                           int *err, cudaStream_t st);
 bool var_fused_supported(int var_sor);
 void init_var_attributes();
 float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y,
                                 const void *I1, const Level &lv, size_t pyr_frame_stride,
                                 float *U, float *Utmp, size_t u_frame_stride, float *coef,
-                                int frames, const FlowParams &fp, const CUtensorMap *coef_map,
+                                int frames, const FlowParams &fp, const SorMaps *maps,
                                 int *err, cudaStream_t st);
 
 // A9 for one window, destination pointer read from device memory.
