@@ -831,13 +831,13 @@ __device__ __forceinline__ void derive_window(const Windows<WH> &m, float alpha_
     }
 }
 
-// The systems of pixels (gx, gy), (gx + 1, gy), e their place in the windows;
-// i0, i0x, i0y: the template's values.  d1, d2: the diagonal; wl, wr, wu, wd:
-// the edge weights, 0 where the edge leaves the level.
+// The systems of pixels (gx, gy), (gx + D, gy), e the first one's place in the
+// windows; i0, i0x, i0y: the template's values.  d1, d2: the diagonal; wl, wr,
+// wu, wd: the edge weights, 0 where the edge leaves the level.
 struct PairSystem {
     float2 d1, d2, a12, b1, b2, wl, wr, wu, wd;
 };
-template <int WH>
+template <int D, int WH>
 __device__ __forceinline__ PairSystem pair_system(const Windows<WH> &m, int e, int gx, int gy,
                                                   int w, int h, bool inside, pair_t i0,
                                                   pair_t i0x, pair_t i0y, float delta,
@@ -845,21 +845,31 @@ __device__ __forceinline__ PairSystem pair_system(const Windows<WH> &m, int e, i
 {
     const float wm1 = (float)(w - 1), hm1 = (float)(h - 1);
     const pair_t half = dup(0.5f);
+    // a window's values at the two pixels and beside them; of adjacent pixels
+    // either is the other's neighbour
+    auto at = [&](const float *q) { return D == 1 ? ld_pair(q + e) : pk(q[e], q[e + D]); };
+    auto left = [&](const float *q, float2 c) {
+        return make_float2(q[e - 1], D == 1 ? c.x : q[e + D - 1]);
+    };
+    auto right = [&](const float *q, float2 c) {
+        return make_float2(D == 1 ? c.y : q[e + 1], q[e + D + 1]);
+    };
     auto cd2 = [&](pair_t hi, pair_t lo) { return fmul2(half, fsub2(hi, lo)); };
     const bool top = !inside && gy <= 0, bottom = !inside && gy + 1 >= h;
-    const pair_t ix = ld_pair(m.Ix + e), iy = ld_pair(m.Iy + e);
-    const pair_t ixu = top ? ix : ld_pair(m.Ix + e - kLvW);
-    const pair_t ixd = bottom ? ix : ld_pair(m.Ix + e + kLvW);
-    const pair_t iyu = top ? iy : ld_pair(m.Iy + e - kLvW);
-    const pair_t iyd = bottom ? iy : ld_pair(m.Iy + e + kLvW);
+    const pair_t ix = at(m.Ix), iy = at(m.Iy);
+    const pair_t ixu = top ? ix : at(m.Ix - kLvW);
+    const pair_t ixd = bottom ? ix : at(m.Ix + kLvW);
+    const pair_t iyu = top ? iy : at(m.Iy - kLvW);
+    const pair_t iyd = bottom ? iy : at(m.Iy + kLvW);
     const float2 ixv = upk(ix);
     // clamped neighbours along x
     const bool l0 = inside || gx > 0, r0 = inside || gx + 1 < w;
-    const bool l1 = inside || gx + 1 > 0, r1 = inside || gx + 2 < w;
-    const pair_t Ixx = fmul2(half, pk(fsub(r0 ? ixv.y : ixv.x, l0 ? m.Ix[e - 1] : ixv.x),
-                                      fsub(r1 ? m.Ix[e + 2] : ixv.y, l1 ? ixv.x : ixv.y)));
+    const bool l1 = inside || gx + D > 0, r1 = inside || gx + D + 1 < w;
+    const float2 ixl = left(m.Ix, ixv), ixr = right(m.Ix, ixv);
+    const pair_t Ixx = fmul2(half, pk(fsub(r0 ? ixr.x : ixv.x, l0 ? ixl.x : ixv.x),
+                                      fsub(r1 ? ixr.y : ixv.y, l1 ? ixl.y : ixv.y)));
     const pair_t Ixy = cd2(ixd, ixu), Iyy = cd2(iyd, iyu);
-    const pair_t Iz = fsub2(ld_pair(m.W + e), i0);
+    const pair_t Iz = fsub2(at(m.W), i0);
     const pair_t Ixz = fsub2(ix, i0x), Iyz = fsub2(iy, i0y);
     const pair_t z2 = dup(kZeta2);
     const pair_t xx = fmul2(Ixx, Ixx), yy = fmul2(Ixy, Ixy);
@@ -870,30 +880,32 @@ __device__ __forceinline__ PairSystem pair_system(const Windows<WH> &m, int e, i
     float2 adv = upk(fmul2(fmul2(dup(delta), nd), psi_prime2(fmul2(fmul2(nd, Iz), Iz))));
     float2 agv = upk(fmul2(fmul2(dup(gamma), ng),
                            psi_prime2(fmul2(ng, ffma2(Iyz, Iyz, fmul2(Ixz, Ixz))))));
-    const pair_t u = ld_pair(m.U + e), v = ld_pair(m.V + e);
-    const float2 wx = upk(fadd2(pk((float)gx, (float)(gx + 1)), u));
+    const pair_t u = at(m.U), v = at(m.V);
+    const float2 wx = upk(fadd2(pk((float)gx, (float)(gx + D)), u));
     const float2 wy = upk(fadd2(dup((float)gy), v));
     if (wx.x < 0.0f || wx.x > wm1 || wy.x < 0.0f || wy.x > hm1) adv.x = agv.x = 0.0f;
     if (wx.y < 0.0f || wx.y > wm1 || wy.y < 0.0f || wy.y > hm1) adv.y = agv.y = 0.0f;
     const pair_t ad = pk(adv.x, adv.y), ag = pk(agv.x, agv.y);
-    const pair_t as = ld_pair(m.As + e);
+    const pair_t as = at(m.As);
     const float2 av = upk(as);
-    const float mid = fmul(0.5f, fadd(av.x, av.y));
+    const float2 al = left(m.As, av), ar = right(m.As, av);
+    auto mean = [](float p, float q) { return fmul(0.5f, fadd(p, q)); };
     PairSystem ps;
-    ps.wl = make_float2(l0 ? fmul(0.5f, fadd(av.x, m.As[e - 1])) : 0.0f, l1 ? mid : 0.0f);
-    ps.wr = make_float2(r0 ? mid : 0.0f, r1 ? fmul(0.5f, fadd(av.y, m.As[e + 2])) : 0.0f);
+    ps.wl = make_float2(l0 ? mean(av.x, al.x) : 0.0f, l1 ? mean(av.y, al.y) : 0.0f);
+    ps.wr = make_float2(r0 ? mean(av.x, ar.x) : 0.0f, r1 ? mean(av.y, ar.y) : 0.0f);
     const pair_t cl = pk(ps.wl.x, ps.wl.y), cr = pk(ps.wr.x, ps.wr.y);
-    const pair_t cu = top ? 0 : fmul2(half, fadd2(as, ld_pair(m.As + e - kLvW)));
-    const pair_t cd = bottom ? 0 : fmul2(half, fadd2(as, ld_pair(m.As + e + kLvW)));
+    const pair_t cu = top ? 0 : fmul2(half, fadd2(as, at(m.As - kLvW)));
+    const pair_t cd = bottom ? 0 : fmul2(half, fadd2(as, at(m.As + kLvW)));
     ps.wu = upk(cu);
     ps.wd = upk(cd);
     const pair_t sw = fadd2(fadd2(fadd2(cl, cr), cu), cd);
     auto smooth = [&](const float *q, pair_t c) {
         const float2 n = upk(c);
-        const pair_t dl = pk(fsub(q[e - 1], n.x), fsub(n.x, n.y));
-        const pair_t dr = pk(fsub(n.y, n.x), fsub(q[e + 2], n.y));
-        return ffma2(cd, fsub2(ld_pair(q + e + kLvW), c),
-                     ffma2(cu, fsub2(ld_pair(q + e - kLvW), c), ffma2(cr, dr, fmul2(cl, dl))));
+        const float2 ql = left(q, n), qr = right(q, n);
+        const pair_t dl = pk(fsub(ql.x, n.x), fsub(ql.y, n.y));
+        const pair_t dr = pk(fsub(qr.x, n.x), fsub(qr.y, n.y));
+        return ffma2(cd, fsub2(at(q + kLvW), c),
+                     ffma2(cu, fsub2(at(q - kLvW), c), ffma2(cr, dr, fmul2(cl, dl))));
     };
     const pair_t su = smooth(m.U, u), sv = smooth(m.V, v);
     const pair_t adx = fmul2(ad, ix), ady = fmul2(ad, iy), nag = neg2(ag);
@@ -906,8 +918,11 @@ __device__ __forceinline__ PairSystem pair_system(const Windows<WH> &m, int e, i
 }
 
 // The linear systems of a level as planes: a block stages a tile of 64 columns
-// x TH rows (from an odd column, as the planes' pairs are aligned) and writes
-// its pixels' systems, two adjacent ones a thread and step.
+// x TH rows and writes its pixels' systems, two a thread and step, 32 columns
+// apart: every access of a warp is to 32 columns side by side, from any column
+// (adjacent pixels a pair want odd ones, one tile more at widths of 64 k).
+// Bound by L1 (78 % of its cycles) and issue (59 %): eight frames of 1280 x 720
+// 93 us a launch, 354 MB of planes 50.
 template <int TH, int NT, typename T>
 __device__ __forceinline__ void var_coeff_body(
     float *smem, const T *__restrict__ I0, const T *__restrict__ I0x, const T *__restrict__ I0y,
@@ -917,38 +932,50 @@ __device__ __forceinline__ void var_coeff_body(
     constexpr int WH = TH + 4, WARPS = NT / 32;
     const Windows<WH> m(smem);
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int tx = bx * 64 - 1, ty = by * TH;
+    const int tx = bx * 64, ty = by * TH;
     const bool inside = tx >= 2 && ty >= 2 && tx + 66 <= w && ty + TH + 2 <= h;
     stage_window<WH, NT, 3>(m, I1, w, h, pitch, tx - 2, ty - 2, inside,
                             [&](auto &c0, auto &c1, auto &cy, auto &u, auto &v) {
                                 load_planes<3>(U, plane, pitch, inside, c0, c1, cy, u, v);
                             });
     __syncthreads();
+    const int gx = tx + lane, pl = (int)plane;
+    const bool c0 = inside || gx < w, c1 = inside || gx + 32 < w;
+    // the template's values of a row are loaded while the row before, or the
+    // derivatives, are computed; no test between the loads (columns outside:
+    // any value, nothing is written there)
+    const int xa = min(gx, w - 1), xb = min(gx + 32, w - 1);
+    T t0[2], tx0[2], ty0[2];
+    auto fetch = [&](int r) {
+        const int o = min(ty + r, h - 1) * pitch;
+        t0[0] = I0[o + xa], t0[1] = I0[o + xb];
+        tx0[0] = I0x[o + xa], tx0[1] = I0x[o + xb];
+        ty0[0] = I0y[o + xa], ty0[1] = I0y[o + xb];
+    };
+    fetch(wp);
     derive_window<WH, NT>(m, alpha_s);
     __syncthreads();
-    const int gx = tx + 2 * lane, pl = (int)plane;
-    const bool c0 = inside || (gx >= 0 && gx < w), c1 = inside || gx + 1 < w;
 #pragma unroll 1
     for (int r = wp; r < TH; r += WARPS) {
         const int gy = ty + r, o = gy * pitch + gx;
         if (gy >= h) break;
-        const pair_t i0 = pk(c0 ? ldp(I0 + o) : 0.0f, c1 ? ldp(I0 + o + 1) : 0.0f);
-        const pair_t i0x = pk(c0 ? ldp(I0x + o) : 0.0f, c1 ? ldp(I0x + o + 1) : 0.0f);
-        const pair_t i0y = pk(c0 ? ldp(I0y + o) : 0.0f, c1 ? ldp(I0y + o + 1) : 0.0f);
-        const int e = (r + 2) * kLvW + 2 * lane + 2;
-        const PairSystem ps = pair_system(m, e, gx, gy, w, h, inside, i0, i0x, i0y, delta, gamma);
+        const pair_t i0 = pk((float)t0[0], (float)t0[1]);
+        const pair_t i0x = pk((float)tx0[0], (float)tx0[1]);
+        const pair_t i0y = pk((float)ty0[0], (float)ty0[1]);
+        if (r + WARPS < TH) fetch(r + WARPS);
+        const int e = (r + 2) * kLvW + lane + 2;
+        const PairSystem ps = pair_system<32>(m, e, gx, gy, w, h, inside, i0, i0x, i0y, delta, gamma);
         float *c = cf + o;
         auto st = [&](int k, float x, float y) {
-            if (c0 && c1) *reinterpret_cast<float2 *>(c + k * pl) = make_float2(x, y);
-            else if (c0) c[k * pl] = x;
-            else if (c1) c[k * pl + 1] = y;
+            if (c0) c[k * pl] = x;
+            if (c1) c[k * pl + 32] = y;
         };
         st(kCI11, __fdividef(omega, ps.d1.x), __fdividef(omega, ps.d1.y));
         st(kCI22, __fdividef(omega, ps.d2.x), __fdividef(omega, ps.d2.y));
         st(kCA12, ps.a12.x, ps.a12.y);
         st(kCB1, ps.b1.x, ps.b1.y);
         st(kCB2, ps.b2.x, ps.b2.y);
-        st(kCAS, m.As[e], m.As[e + 1]);
+        st(kCAS, m.As[e], m.As[e + 32]);
     }
 }
 
@@ -1160,7 +1187,7 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             const bool in0 = row_in && (inside || (gx >= 0 && gx < w));
             const bool in1 = row_in && (inside || (gx + 1 >= 0 && gx + 1 < w));
             const PairSystem ps =
-                pair_system(m, e, gx, gy, w, h, inside, i0[r], i0x[r], i0y[r], delta, gamma);
+                pair_system<1>(m, e, gx, gy, w, h, inside, i0[r], i0x[r], i0y[r], delta, gamma);
             s.i11[r][0] = in0 ? __fdividef(omega, ps.d1.x) : 0.0f;
             s.i11[r][1] = in1 ? __fdividef(omega, ps.d1.y) : 0.0f;
             s.i22[r][0] = in0 ? __fdividef(omega, ps.d2.x) : 0.0f;
@@ -1329,7 +1356,7 @@ size_t level_packets(const Geometry &geo, int var_sor, int cluster_max, int fram
 
 int sor_halo(int var_sor) { return var_sor > 0 ? 2 * var_sor - 1 : 1; }
 int sor_tile(int R) { return kVR - 2 * R; }
-int coeff_tiles_x(int w) { return (w + 64) / 64; }  // the first tile starts at column -1
+int coeff_tiles_x(int w) { return (w + 63) / 64; }
 int coeff_tiles_y(int h) { return (h + kCoefRows - 1) / kCoefRows; }
 int coeff_planes() { return kCPlanes; }
 
