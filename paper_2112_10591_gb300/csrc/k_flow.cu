@@ -603,18 +603,23 @@ __device__ __forceinline__ float dense_sample(const T *__restrict__ I1, int w, i
 }
 
 // The patches that cover a block's tile, staged once: their displacement, its
-// fraction and its whole-pixel part as an offset.  At most 36 x 12 of them
-// where NC <= 4 (a stride of 1 with 4 x 4 patches).
-constexpr int kDenseX = 36, kDenseY = 12;
+// fraction and its whole-pixel part as an offset.  At most 36 x 20 of them
+// where NC <= 4 (a stride of 1 with 4 x 4 patches, two rows a thread).
+constexpr int kDenseX = 36;
+template <int PY>
+constexpr int kDenseY = 8 * PY + 4;
 
-// (bx, by): the 32 x 8 tile, f: the frame.  NC > 0: a block whose patches'
-// samples all lie inside the level takes them from the staged values, without
-// the floors, conversions and border tests of every pixel (each on the slow
-// pipe, nine times a pixel at 12 x 12 patches and stride 4); other blocks
-// sample patch by patch.  The arithmetic is the same.  Bound by issue and the
-// taps' latency.  1280x720 level 0, eight frames: 188 -> 164 us (194 while a
-// test stood before every patch's loads); 85 -> 65 us over the other levels.
-template <typename T, int NC>
+// (bx, by): the tile of 32 x 8 PY, f: the frame; a thread's PY pixels lie one
+// above the other.  NC > 0: a block whose patches' samples all lie inside the
+// level takes them from the staged values, without the floors, conversions and
+// border tests of every pixel (each on the slow pipe, nine times a pixel at
+// 12 x 12 patches and stride 4); other blocks sample patch by patch.  PY == 2
+// (even strides that divide the patch): away from the borders both pixels have
+// the same patches, so one load of a patch serves both, and the taps' middle
+// row is interpolated once.  The arithmetic is the same.  Bound by issue.
+// 1280x720 level 0, eight frames: 188 -> 164 us with the staged patches, -> 116
+// us with two pixels a thread.
+template <typename T, int NC, int PY>
 __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T *__restrict__ I1b,
                                              int w, int h, int pitch, size_t pfs,
                                              const float *__restrict__ upb, size_t upfs, int npx,
@@ -622,35 +627,41 @@ __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T 
                                              size_t plane, int ps, int stride, uint32_t magic,
                                              unsigned bx, unsigned by, unsigned f)
 {
+    constexpr int TY = 8 * PY;
     const int x = bx * 32 + threadIdx.x;
-    const int y = by * 8 + threadIdx.y;
-    const bool px = x < w && y < h;
+    const int y = by * TY + PY * threadIdx.y;
     const T *I0 = I0b + (size_t)f * pfs, *I1 = I1b + (size_t)f * pfs;
     const float *up = upb + (size_t)f * upfs;
     const float *vp = up + npx * npy;
     const int p = y * pitch + x;
-    const float i0 = px ? ldp(&I0[p]) : 0.0f;
-    int ilo, ihi, jlo, jhi;
-    bool ilast, jlast;
+    bool px[PY];
+    float i0[PY], nu[PY], nv[PY], den[PY];
+#pragma unroll
+    for (int k = 0; k < PY; ++k) {
+        px[k] = x < w && y + k < h;
+        i0[k] = px[k] ? ldp(&I0[p + k * pitch]) : 0.0f;
+        nu[k] = nv[k] = den[k] = 0.0f;
+    }
+    int ilo, ihi;
+    bool ilast;
     cover_range(x, w, ps, stride, magic, npx, ilo, ihi, ilast);
-    cover_range(y, h, ps, stride, magic, npy, jlo, jhi, jlast);
-    float nu = 0.0f, nv = 0.0f, den = 0.0f;
-    auto weigh = [&](float sample, float u, float v) {
-        const float r = sample - i0;
+    auto weigh = [&](int k, float sample, float u, float v) {
+        const float r = sample - i0[k];
         const float lam = 1.0f / fmaxf(1.0f, fabsf(r));
-        nu += lam * u; nv += lam * v; den += lam;
+        nu[k] += lam * u; nv[k] += lam * v; den[k] += lam;
     };
-    bool staged = false;
+    bool staged = false, done = false;
     if (NC > 0) {
-        __shared__ float4 s_uv[kDenseY][kDenseX];
-        __shared__ int s_off[kDenseY][kDenseX];
+        __shared__ float4 s_uv[kDenseY<PY>][kDenseX];
+        __shared__ int s_off[kDenseY<PY>][kDenseX];
         // the tile's patches: columns ti .. ti + ni - 1, then the flush one
+        const int xe = min((int)bx * 32 + 31, w - 1), ye = min((int)by * TY + TY - 1, h - 1);
         int ti, tj, ie, je, lo;
         bool fx, fy;
-        cover_range(min((int)bx * 32 + 31, w - 1), w, ps, stride, magic, npx, lo, ie, fx);
-        cover_range(min((int)by * 8 + 7, h - 1), h, ps, stride, magic, npy, lo, je, fy);
+        cover_range(xe, w, ps, stride, magic, npx, lo, ie, fx);
+        cover_range(ye, h, ps, stride, magic, npy, lo, je, fy);
         ti = div_stride(max((int)bx * 32 - ps + stride, 0), magic);
-        tj = div_stride(max((int)by * 8 - ps + stride, 0), magic);
+        tj = div_stride(max((int)by * TY - ps + stride, 0), magic);
         const int ni = max(ie - ti + 1, 0), nj = max(je - tj + 1, 0);
         bool in = true;
         for (int jj = threadIdx.y; jj < nj + fy; jj += 8)
@@ -667,67 +678,89 @@ __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T 
                 s_off[jj][ii] = ok ? (int)fv * pitch + (int)fu : 0;
             }
         staged = __syncthreads_and(in);
-        if (staged && px) {
+        // every pixel of the tile has exactly NC x NC regular patches: no test
+        // stands between the loads of one patch and the next
+        if (staged && NC * stride == ps && (int)bx * 32 >= ps - stride && ie <= npx - 2 && !fx &&
+            (int)by * TY >= ps - stride && je <= npy - 2 && !fy &&
+            div_stride(xe, magic) <= npx - 2 && div_stride(ye, magic) <= npy - 2) {
+            const int j0 = div_stride(y - ps + stride, magic) - tj;
+            const float4 *m4 = &s_uv[j0][ilo - ti];
+            const int *o = &s_off[j0][ilo - ti];
             const T *q = I1 + p;
-            auto add = [&](const float4 *m4, const int *off) {
-                const float4 m = *m4;
-                const float ax = m.z, ay = m.w;
-                const T *r0 = q + *off, *r1 = r0 + pitch;
-                const float a = ldp(&r0[0]), b = ldp(&r0[1]), c = ldp(&r1[0]), d = ldp(&r1[1]);
-                weigh((1.0f - ay) * ((1.0f - ax) * a + ax * b) +
-                          ay * ((1.0f - ax) * c + ax * d),
-                      m.x, m.y);
-            };
-            // every pixel of the tile has exactly NC x NC regular patches:
-            // no test stands between the loads of one patch and the next
-            if (NC * stride == ps && (int)bx * 32 >= ps - stride && ie <= npx - 2 && !fx &&
-                (int)by * 8 >= ps - stride && je <= npy - 2 && !fy &&
-                div_stride(min((int)bx * 32 + 31, w - 1), magic) <= npx - 2 &&
-                div_stride(min((int)by * 8 + 7, h - 1), magic) <= npy - 2) {
-                const float4 *m = &s_uv[jlo - tj][ilo - ti];
-                const int *o = &s_off[jlo - tj][ilo - ti];
-#pragma unroll
-                for (int dj = 0; dj < (NC > 0 ? NC : 1); ++dj)
-#pragma unroll
-                    for (int di = 0; di < (NC > 0 ? NC : 1); ++di)
-                        add(m + dj * kDenseX + di, o + dj * kDenseX + di);
-                ilo = INT_MAX / 2;  // done
-                ilast = jlast = false;
-                jhi = -1;
-            }
-            auto row = [&](int jj) {
-                const float4 *m = &s_uv[jj][ilo - ti];
-                const int *o = &s_off[jj][ilo - ti];
-#pragma unroll
-                for (int di = 0; di < (NC > 0 ? NC : 1); ++di)
-                    if (ilo + di <= ihi) add(m + di, o + di);
-                if (ilast) add(&s_uv[jj][ni], &s_off[jj][ni]);
-            };
 #pragma unroll
             for (int dj = 0; dj < (NC > 0 ? NC : 1); ++dj)
-                if (jlo + dj <= jhi) row(jlo - tj + dj);
-            if (jlast) row(nj);
+#pragma unroll
+                for (int di = 0; di < (NC > 0 ? NC : 1); ++di) {
+                    const float4 m = m4[dj * kDenseX + di];
+                    const float ax = m.z, ay = m.w;
+                    const T *r0 = q + o[dj * kDenseX + di];
+                    float row[PY + 1];
+#pragma unroll
+                    for (int k = 0; k <= PY; ++k, r0 += pitch)
+                        row[k] = (1.0f - ax) * ldp(&r0[0]) + ax * ldp(&r0[1]);
+#pragma unroll
+                    for (int k = 0; k < PY; ++k)
+                        weigh(k, (1.0f - ay) * row[k] + ay * row[k + 1], m.x, m.y);
+                }
+            done = true;
+        } else if (staged) {
+#pragma unroll
+            for (int k = 0; k < PY; ++k) {
+                if (!px[k]) continue;
+                int jlo, jhi;
+                bool jlast;
+                cover_range(y + k, h, ps, stride, magic, npy, jlo, jhi, jlast);
+                const T *q = I1 + p + k * pitch;
+                auto add = [&](const float4 *m4, const int *off) {
+                    const float4 m = *m4;
+                    const float ax = m.z, ay = m.w;
+                    const T *r0 = q + *off, *r1 = r0 + pitch;
+                    const float a = ldp(&r0[0]), b = ldp(&r0[1]), c = ldp(&r1[0]), d = ldp(&r1[1]);
+                    weigh(k, (1.0f - ay) * ((1.0f - ax) * a + ax * b) +
+                                 ay * ((1.0f - ax) * c + ax * d),
+                          m.x, m.y);
+                };
+                auto row = [&](int jj) {
+                    const float4 *m = &s_uv[jj][ilo - ti];
+                    const int *o = &s_off[jj][ilo - ti];
+#pragma unroll
+                    for (int di = 0; di < (NC > 0 ? NC : 1); ++di)
+                        if (ilo + di <= ihi) add(m + di, o + di);
+                    if (ilast) add(&s_uv[jj][ni], &s_off[jj][ni]);
+                };
+#pragma unroll
+                for (int dj = 0; dj < (NC > 0 ? NC : 1); ++dj)
+                    if (jlo + dj <= jhi) row(jlo - tj + dj);
+                if (jlast) row(nj);
+            }
+            done = true;
         }
     }
-    if (!px) return;
-    if (!staged) {
-        auto add = [&](int id) {
-            const float u = up[id], v = vp[id];
-            weigh(dense_sample(I1, w, h, pitch, x, y, u, v), u, v);
-        };
-        auto row = [&](int j) {
-            for (int i = ilo; i <= ihi; ++i) add(j * npx + i);
-            if (ilast) add(j * npx + npx - 1);
-        };
-        for (int j = jlo; j <= jhi; ++j) row(j);
-        if (jlast) row(npy - 1);
+#pragma unroll
+    for (int k = 0; k < PY; ++k) {
+        if (!px[k]) return;
+        if (!done) {
+            int jlo, jhi;
+            bool jlast;
+            cover_range(y + k, h, ps, stride, magic, npy, jlo, jhi, jlast);
+            auto add = [&](int id) {
+                const float u = up[id], v = vp[id];
+                weigh(k, dense_sample(I1, w, h, pitch, x, y + k, u, v), u, v);
+            };
+            auto row = [&](int j) {
+                for (int i = ilo; i <= ihi; ++i) add(j * npx + i);
+                if (ilast) add(j * npx + npx - 1);
+            };
+            for (int j = jlo; j <= jhi; ++j) row(j);
+            if (jlast) row(npy - 1);
+        }
+        float *U = Ub + (size_t)f * ufs + p + k * pitch;
+        U[0] = den[k] > 0.0f ? nu[k] / den[k] : 0.0f;
+        U[plane] = den[k] > 0.0f ? nv[k] / den[k] : 0.0f;
     }
-    float *U = Ub + (size_t)f * ufs;
-    U[p] = den > 0.0f ? nu / den : 0.0f;
-    (U + plane)[p] = den > 0.0f ? nv / den : 0.0f;
 }
 
-template <typename T, int NC>
+template <typename T, int NC, int PY>
 __global__ void __launch_bounds__(256)
 densify_kernel(const T *__restrict__ I0b, const T *__restrict__ I1b, int w, int h, int pitch,
                size_t pfs, const float *__restrict__ upb, size_t upfs, int npx, int npy,
@@ -735,7 +768,7 @@ densify_kernel(const T *__restrict__ I0b, const T *__restrict__ I1b, int w, int 
                uint32_t magic)
 {
     chain_begin();
-    densify_body<T, NC>(I0b, I1b, w, h, pitch, pfs, upb, upfs, npx, npy, Ub, ufs, plane, ps,
+    densify_body<T, NC, PY>(I0b, I1b, w, h, pitch, pfs, upb, upfs, npx, npy, Ub, ufs, plane, ps,
                         stride, magic, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -746,7 +779,7 @@ seg_densify_kernel(const __grid_constant__ SegTable<SegDensify> tab)
     int b;
     const SegDensify &a = seg_of(tab, b);
     const int r = b / a.gx;
-    densify_body<T, NC>((const T *)a.I0, (const T *)a.I1, a.w, a.h, a.pitch, a.pfs, a.up, a.upfs,
+    densify_body<T, NC, 1>((const T *)a.I0, (const T *)a.I1, a.w, a.h, a.pitch, a.pfs, a.up, a.upfs,
                         a.npx, a.npy, a.U, a.ufs, a.plane, a.ps, a.stride, a.magic, b % a.gx,
                         r % a.gy, r / a.gy);
 }
@@ -1056,34 +1089,49 @@ void launch_patch_search(const void *I0, const void *I0x, const void *I0y, const
                               up, up_frame_stride, frames, fp, err, st);
 }
 
+// Blocks of 32 x 8 from which two pixels a thread are faster (16 a SM): 40
+// windows of 1280 x 720 10.12 -> 9.82 ms; with a line at 400 blocks 641 x 479
+// took 588 us against 583, its two levels of 300 and 1260 blocks left with too
+// few warps.
+constexpr long long kDensePairBlocks = 2432;
+
 void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_frame_stride,
                     const float *up, size_t up_frame_stride, float *U, size_t u_frame_stride,
                     int frames, const FlowParams &fp, cudaStream_t st)
 {
     StageScope sc(kStDensify, 1, st);
     dim3 blk(32, 8);
-    const dim3 grd = grid2d(lv.w, lv.h, frames, blk);
+    dim3 grd = grid2d(lv.w, lv.h, frames, blk);
     // regular patches covering a pixel per axis: at most ceil(ps / stride)
     const int nc = (fp.ps + fp.stride - 1) / fp.stride;
     // no patch beyond the border: a longer stride is the same grid
     const int stride = std::min(fp.stride, kMaxDim);
     const uint32_t magic = stride_magic(stride);
     const bool chained = fp.chained || lv.npx * lv.npy > 0;  // the search is launched
-#define EBOF_DENSE(T, N)                                                                         \
-    launch_chained(chained, densify_kernel<T, N>, grd, blk, 0, st, (const T *)I0,                \
+    const bool two = nc >= 2 && nc <= 4 && nc * stride == fp.ps && stride % 2 == 0 &&
+                     (long long)grd.x * grd.y * frames >= kDensePairBlocks;
+    if (two) grd.y = (lv.h + 15) / 16;
+#define EBOF_DENSE2(T, N)                                                                        \
+    do {                                                                                         \
+        if (two) EBOF_DENSE(T, N, 2);                                                            \
+        else EBOF_DENSE(T, N, 1);                                                                \
+    } while (0)
+#define EBOF_DENSE(T, N, PY)                                                                     \
+    launch_chained(chained, densify_kernel<T, N, PY>, grd, blk, 0, st, (const T *)I0,            \
                    (const T *)I1, lv.w, lv.h, lv.pitch, pyr_frame_stride, up, up_frame_stride,   \
                    lv.npx, lv.npy, U, u_frame_stride, lv.plane, fp.ps, stride, magic)
     if (fp.half) {
-        if (nc == 2) EBOF_DENSE(__half, 2);
-        else if (nc == 3) EBOF_DENSE(__half, 3);
-        else if (nc == 4) EBOF_DENSE(__half, 4);
-        else EBOF_DENSE(__half, 0);
+        if (nc == 2) EBOF_DENSE2(__half, 2);
+        else if (nc == 3) EBOF_DENSE2(__half, 3);
+        else if (nc == 4) EBOF_DENSE2(__half, 4);
+        else EBOF_DENSE(__half, 0, 1);
     } else {
-        if (nc == 2) EBOF_DENSE(float, 2);
-        else if (nc == 3) EBOF_DENSE(float, 3);
-        else if (nc == 4) EBOF_DENSE(float, 4);
-        else EBOF_DENSE(float, 0);
+        if (nc == 2) EBOF_DENSE2(float, 2);
+        else if (nc == 3) EBOF_DENSE2(float, 3);
+        else if (nc == 4) EBOF_DENSE2(float, 4);
+        else EBOF_DENSE(float, 0, 1);
     }
+#undef EBOF_DENSE2
 #undef EBOF_DENSE
 }
 
