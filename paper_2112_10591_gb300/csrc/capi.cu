@@ -65,6 +65,7 @@ struct ebof_stream {
     float *up = nullptr, *Ua = nullptr, *Ub = nullptr, *work = nullptr;
     DevStats *dstats = nullptr;
     unsigned long long *d_dropped_time = nullptr;
+    char *counters = nullptr;  // dstats, d_dropped_time and E, see front_alloc
     int *d_err = nullptr;
     unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
     char *d_xch = nullptr;      // and its packets: 2 x level_n x kPacketBytes
@@ -155,6 +156,7 @@ struct ebof_group {
     float *flow = nullptr;  // [n][2][H][W]
     DevStats *dstats = nullptr;
     unsigned long long *d_dropped_time = nullptr;
+    char *counters = nullptr;  // dstats, d_dropped_time and E, see front_alloc
     int *d_err = nullptr;
     unsigned *d_ctl = nullptr;  // counters of the one-launch refinement
     char *d_xch = nullptr;      // and its packets: 2 x level_n x kPacketBytes
@@ -319,11 +321,38 @@ void flow_free(float *u)
     cudaFree(u ? u - 1 : nullptr);
 }
 
+// What a window's front part finds cleared, in one allocation: the counters of
+// all frames, the dropped events' counter, the edge images.  A call of as many
+// frames clears it at once.
+size_t front_head(int frames) { return (sizeof(DevStats) * frames + 8 + 255) / 256 * 256; }
+
+template <class S>
+bool front_alloc(S *s, int frames)
+{
+    static_assert(sizeof(DevStats) % 8 == 0, "the dropped events' counter is aligned");
+    if (dmalloc(&s->counters, front_head(frames) + s->e_fs * frames) != cudaSuccess) return false;
+    s->dstats = (DevStats *)s->counters;
+    s->d_dropped_time = (unsigned long long *)(s->counters + sizeof(DevStats) * frames);
+    s->E = (uint8_t *)s->counters + front_head(frames);
+    return true;
+}
+
+// Clears the counters of n of the `frames` frames and, with them, their edge
+// images.
+template <class S>
+void front_clear(S *s, int frames, int n, bool edges, cudaStream_t st)
+{
+    char *from = n == frames ? (char *)s->dstats : (char *)s->d_dropped_time;
+    char *to = edges ? (char *)s->E + s->e_fs * n : (char *)(s->d_dropped_time + 1);
+    if (n != frames) cudaMemsetAsync(s->dstats, 0, sizeof(DevStats) * n, st);
+    cudaMemsetAsync(from, 0, to - from, st);
+}
+
 void free_all(ebof_stream *s)
 {
-    cudaFree(s->E); cudaFree(s->Ed); cudaFree(s->Edf); cudaFree(s->g); cudaFree(s->pyr);
+    cudaFree(s->counters); cudaFree(s->Ed); cudaFree(s->Edf); cudaFree(s->g); cudaFree(s->pyr);
     cudaFree(s->up); flow_free(s->Ua); flow_free(s->Ub); cudaFree(s->work);
-    cudaFree(s->dstats); cudaFree(s->d_dropped_time); cudaFree(s->d_err); cudaFree(s->d_ctl);
+    cudaFree(s->d_err); cudaFree(s->d_ctl);
     cudaFree(s->d_xch);
     cudaFree(s->flow_stage); cudaFree(s->ev_stage); cudaFree(s->d_call);
     for (int b = 0; b < 2; ++b)
@@ -441,14 +470,11 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
     const size_t es = s->es;
     char *I0cur = pyr + (size_t)cur_first * s->pyr_fs * es;
     if (parts & kPartFront) {
-        cudaMemsetAsync(s->dstats, 0, sizeof(DevStats) * n, st);
-        cudaMemsetAsync(s->d_dropped_time, 0, sizeof(unsigned long long), st);
-
+        front_clear(s, p.max_batch, n, !surface_in, st);
         if (surface_in) {
             launch_surface_to_intensity(surface_in, W, H, I0cur, s->pitch0, half,
                                         surface_map(p), st);
         } else {
-            cudaMemsetAsync(s->E, 0, s->e_fs * n, st);
             if (via_args)
                 launch_scatter_desc(d_wins, n, W, H, s->pitch0, s->E, s->e_fs, s->dstats,
                                     s->d_dropped_time, st);
@@ -888,9 +914,9 @@ void free_group(ebof_group *g)
 {
     for (int b = 0; b < 2; ++b)
         if (g->graph[b]) cudaGraphExecDestroy(g->graph[b]);
-    cudaFree(g->E); cudaFree(g->Ed); cudaFree(g->Edf); cudaFree(g->g); cudaFree(g->pyr);
+    cudaFree(g->counters); cudaFree(g->Ed); cudaFree(g->Edf); cudaFree(g->g); cudaFree(g->pyr);
     cudaFree(g->up); flow_free(g->Ua); flow_free(g->Ub); cudaFree(g->work); cudaFree(g->flow);
-    cudaFree(g->dstats); cudaFree(g->d_dropped_time); cudaFree(g->d_err); cudaFree(g->d_ctl);
+    cudaFree(g->d_err); cudaFree(g->d_ctl);
     cudaFree(g->d_xch);
     cudaFree(g->d_desc);
     delete[] g->h_events;
@@ -913,9 +939,7 @@ void run_group(ebof_group *g, bool with_flow, cudaStream_t st)
     const size_t es = g->es;
     char *cur = g->pyr + (size_t)g->parity * n * g->pyr_fs * es;
     tl_level = -1;
-    cudaMemsetAsync(g->dstats, 0, sizeof(DevStats) * n, st);
-    cudaMemsetAsync(g->d_dropped_time, 0, sizeof(unsigned long long), st);
-    cudaMemsetAsync(g->E, 0, g->e_fs * n, st);
+    front_clear(g, n, n, true, st);
     launch_scatter_desc(g->d_desc, n, W, H, g->pitch0, g->E, g->e_fs, g->dstats,
                         g->d_dropped_time, st);
     launch_denoise_fill(g->E, g->Ed, g->Edf, W, H, g->pitch0, g->e_fs, n, p.connectivity, p.n_d,
@@ -1054,9 +1078,7 @@ void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
     for (GS &x : gs) {
         ebof_group *g = x.g;
         P.ops.push_back([g](cudaStream_t st) {
-            cudaMemsetAsync(g->dstats, 0, sizeof(DevStats) * g->n, st);
-            cudaMemsetAsync(g->d_dropped_time, 0, sizeof(unsigned long long), st);
-            cudaMemsetAsync(g->E, 0, g->e_fs * g->n, st);
+            front_clear(g, g->n, g->n, true, st);
         });
     }
     // A1: the work list of all windows
@@ -1497,7 +1519,7 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     s->work_fs = 9 * plane0;
     s->nslots = B + 1;
     bool ok = true;
-    ok &= dmalloc(&s->E, s->e_fs * B) == cudaSuccess;
+    ok &= front_alloc(s, B);
     ok &= dmalloc(&s->Ed, s->e_fs * B) == cudaSuccess;
     ok &= dmalloc(&s->Edf, s->e_fs * B) == cudaSuccess;
     ok &= dmalloc(&s->g, sizeof(int32_t) * s->g_fs * B) == cudaSuccess;
@@ -1507,8 +1529,6 @@ ebof_status ebof_stream_create(const ebof_params *p, int device, ebof_stream **o
     ok &= flow_alloc(&s->Ua, s->u_fs * B) == cudaSuccess;
     ok &= flow_alloc(&s->Ub, s->u_fs * B) == cudaSuccess;
     ok &= dmalloc(&s->work, sizeof(float) * s->work_fs * B) == cudaSuccess;
-    ok &= dmalloc(&s->dstats, sizeof(DevStats) * B) == cudaSuccess;
-    ok &= dmalloc(&s->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&s->d_err, sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&s->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
     s->level_n = level_packets(geo, p->var_sor, p->var_cluster_max, B);
@@ -1552,12 +1572,12 @@ int64_t ebof_stream_device_bytes(const ebof_params *p)
     const size_t B = (size_t)p->max_batch, plane0 = geo.lv[0].plane;
     const size_t es = p->storage == EBOF_STORAGE_FP16 ? 2 : 4;
     auto r = [](size_t b) { return std::max<size_t>(b, 256); };
-    size_t total = 3 * r(plane0 * B) + r(4 * plane0 * B) + r(es * geo.pyr_floats * (B + 1));
+    size_t total = 2 * r(plane0 * B) + r(front_head((int)B) + plane0 * B) + r(4 * plane0 * B) + r(es * geo.pyr_floats * (B + 1));
     total += r(4 * 2 * (size_t)std::max(geo.max_patches, 1) * B);
     total += 2 * r(4 * (2 * plane0 * B + 1)) + r(4 * 9 * plane0 * B);
     total += 256;  // the one-launch refinement's counters, then its packets
     total += r(2 * kPacketBytes * level_packets(geo, p->var_sor, p->var_cluster_max, p->max_batch));
-    total += r(sizeof(DevStats) * B) + 2 * 256 + r(4 * 2 * (size_t)p->width * p->height) +
+    total += 256 + r(4 * 2 * (size_t)p->width * p->height) +
              r((sizeof(ebof_window_desc) + sizeof(float *)) * B);
     return (int64_t)total;
 }
@@ -2045,7 +2065,7 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     g->es = q.storage == EBOF_STORAGE_FP16 ? 2 : 4;
     g->h_events = new (std::nothrow) int64_t[n];
     bool ok = g->h_events != nullptr;
-    ok &= dmalloc(&g->E, g->e_fs * n) == cudaSuccess;
+    ok &= front_alloc(g, n);
     ok &= dmalloc(&g->Ed, g->e_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->Edf, g->e_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->g, sizeof(int32_t) * g->g_fs * n) == cudaSuccess;
@@ -2055,8 +2075,6 @@ ebof_status ebof_group_create(const ebof_params *p, int32_t n_streams, int devic
     ok &= flow_alloc(&g->Ub, g->u_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->work, sizeof(float) * g->work_fs * n) == cudaSuccess;
     ok &= dmalloc(&g->flow, sizeof(float) * 2 * (size_t)q.width * q.height * n) == cudaSuccess;
-    ok &= dmalloc(&g->dstats, sizeof(DevStats) * n) == cudaSuccess;
-    ok &= dmalloc(&g->d_dropped_time, sizeof(unsigned long long)) == cudaSuccess;
     ok &= dmalloc(&g->d_err, sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&g->d_ctl, sizeof(unsigned) * kLevelCtl) == cudaSuccess;
     g->level_n = level_packets(g->geo, q.var_sor, q.var_cluster_max, n);
