@@ -98,9 +98,10 @@ typedef struct {
                                    of two-row strips take that form; 0 = never (1) */
     int32_t var_cluster_max;    /* small levels: the whole refinement of a level in one
                                    launch (every outer iteration).  A single frame in
-                                   order always takes it where its regions fit one
-                                   wave; calls of several frames do so for levels of
-                                   at most this many regions a frame; 0 = never (0) */
+                                   order always takes it where its 64x64 regions fill
+                                   at most 1.75 waves; calls of several frames do so
+                                   for levels of at most this many regions a frame;
+                                   0 = never (0) */
     int32_t coeff_cw_rows;      /* 4, 8 or 16 (8); checked, without effect */
 } ebof_params;
 
@@ -577,12 +578,12 @@ uint64_t ebof_kernel_launches(void);
  * paper has no counterpart; they let tests drive the error paths above
  * without faulting a GPU. */
 
-/* Bound, in mbarrier try-wait rounds, of the first wait of the batched SOR
- * kernel (the copy-ahead form, used when a call's variational grid has at
- * least sor_tma_min_per_sm regions per SM) for a region's coefficient copy.  When it runs
- * out the kernel latches EBOF_ERR_TIMEOUT, reported by ebof_stream_sync, lets
- * the copy in flight land under a second wait at the default bound, and
- * leaves the flow of that call undefined.  Applies to launches enqueued
+/* Bound, in mbarrier try-wait rounds, of the waits of the batched SOR kernel
+ * (the copy-ahead form, used when a call's variational grid has at least
+ * sor_tma_min_per_sm regions per SM) for a region's copies, its coefficients'
+ * and its flow's.  When one runs out the kernel latches EBOF_ERR_TIMEOUT,
+ * reported by ebof_stream_sync, lets the copies in flight land under a second
+ * wait at the default bound, and leaves the flow of that call undefined.  Applies to launches enqueued
  * after the call (graphs captured earlier keep their bound); iterations < 0
  * restores the default, 2^22; 0 makes every such wait run out at once.
  * EBOF_ERR_BUSY while another thread uses the stream. */
