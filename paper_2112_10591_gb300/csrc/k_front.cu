@@ -809,7 +809,7 @@ int edt_rows_wpr(int frames) { return frames > 2 ? 1 : kRowsPerBlock; }
 template <typename T>
 void edt_rows_t(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
                 const SurfaceMap &sm, int32_t *D_dense, float *S_dense, T *I0, int i_pitch,
-                size_t i_frame_stride, int frames, cudaStream_t st)
+                size_t i_frame_stride, int frames, bool chained, cudaStream_t st)
 {
     const int wpr = edt_rows_wpr(frames);
     // one warp a row: four rows per block, fewer where a row's shared memory
@@ -819,9 +819,7 @@ void edt_rows_t(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int
     dim3 grd((H + rows - 1) / rows, frames);
     auto kern = wpr == 1 ? edt_rows_surface_kernel<1, T>
                          : edt_rows_surface_kernel<kRowsPerBlock, T>;
-    // with full dependencies: started early, its blocks fill the SMs beside the
-    // column kernel's and slow it (1920 x 1080: 45 us the transform, 36 so)
-    launch_chained(false, kern, grd, 32 * (wpr == 1 ? rows : wpr), smem, st, g, g_pitch,
+    launch_chained(chained, kern, grd, 32 * (wpr == 1 ? rows : wpr), smem, st, g, g_pitch,
                    g_frame_stride, W, H, rows, sm, D_dense, S_dense, I0, i_pitch, i_frame_stride);
 }
 
@@ -833,27 +831,41 @@ void launch_edt_direct(const uint8_t *edge, int W, int H, float alpha, int32_t *
         edge, W, H, exp_surface(alpha), D_dense, S_dense);
 }
 
+static void edt_rows(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
+                     const SurfaceMap &sm, int32_t *D_dense, float *S_dense, void *I0,
+                     int i_pitch, size_t i_frame_stride, int frames, bool half, bool chained,
+                     cudaStream_t st)
+{
+    StageScope sc(kStEdtRows, 1, st);
+    if (half)
+        edt_rows_t(g, g_pitch, g_frame_stride, W, H, sm, D_dense, S_dense, (__half *)I0,
+                   i_pitch, i_frame_stride, frames, chained, st);
+    else
+        edt_rows_t(g, g_pitch, g_frame_stride, W, H, sm, D_dense, S_dense, (float *)I0,
+                   i_pitch, i_frame_stride, frames, chained, st);
+}
+
 void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
                              const SurfaceMap &sm, int32_t *D_dense, float *S_dense, void *I0,
                              int i_pitch, size_t i_frame_stride, int frames, bool half,
                              cudaStream_t st)
 {
-    StageScope sc(kStEdtRows, 1, st);
-    if (half)
-        edt_rows_t(g, g_pitch, g_frame_stride, W, H, sm, D_dense, S_dense, (__half *)I0,
-                   i_pitch, i_frame_stride, frames, st);
-    else
-        edt_rows_t(g, g_pitch, g_frame_stride, W, H, sm, D_dense, S_dense, (float *)I0,
-                   i_pitch, i_frame_stride, frames, st);
+    edt_rows(g, g_pitch, g_frame_stride, W, H, sm, D_dense, S_dense, I0, i_pitch, i_frame_stride,
+             frames, half, false, st);
 }
 
+// The stand-alone transform: the rows start while the columns end where they
+// are few (four blocks an SM; 640 x 480 14.4 -> 12.4 us); more of them fill the
+// SMs beside the column kernel's blocks and slow it (1280 x 720 22.6 either way,
+// 1920 x 1080 45.1 against 34.9 with full dependencies).  Within a
+// window they start late (613 x 397 with exports 386 us, early 388).
 void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
                              float alpha, int32_t *D_dense, float *S_dense, void *I0,
                              int i_pitch, size_t i_frame_stride, int frames, bool half,
                              cudaStream_t st)
 {
-    launch_edt_rows_surface(g, g_pitch, g_frame_stride, W, H, exp_surface(alpha), D_dense,
-                            S_dense, I0, i_pitch, i_frame_stride, frames, half, st);
+    edt_rows(g, g_pitch, g_frame_stride, W, H, exp_surface(alpha), D_dense, S_dense, I0, i_pitch,
+             i_frame_stride, frames, half, (long long)H * frames <= 608, st);
 }
 
 void init_front_attributes()
