@@ -307,8 +307,12 @@ ebof_status ebof_stream_sync(ebof_stream *s, ebof_window_stats *out, int32_t n_o
 
 /* Exact squared EDT and Eq. 1 surface of a caller-given binary edge image
  * d_edge [H][W] (non-zero = edge pixel): the separable passes of §III-C.
- * d_scratch: caller-owned device buffer of at least width*height int32
- * (column distances).  d_edt [H][W] required; d_surface [H][W] optional.
+ * d_scratch: caller-owned device buffer of at least width*height int32 (the
+ * columns' edge bits and nearest edge rows).  It may be one of the results or
+ * overlap them: column distances are then kept in a result until its rows are
+ * written, which costs one pass over width*height int32 more.  d_edge may
+ * overlap a result, but not d_scratch.
+ * d_edt [H][W] required; d_surface [H][W] optional.
  * No per-stream state is used. */
 ebof_status ebof_edt(const uint8_t *d_edge, int32_t width, int32_t height, int32_t *d_scratch,
                      int32_t *d_edt, float *d_surface, float alpha, void *cuda_stream);
@@ -319,7 +323,7 @@ ebof_status ebof_edt(const uint8_t *d_edge, int32_t width, int32_t height, int32
  * or code inside a host framework that owns all device memory through its
  * own allocator.  The paper has no counterpart; this is a deployment variant
  * of the separable EDT entry point above.
- * Same inputs, outputs and result as ebof_edt, but the column distances are
+ * Same inputs, outputs and result as ebof_edt, but the columns' words are
  * kept in a static device array of 2^21 int32 (8 MiB) that every device
  * which loads the library holds until the process exits, so width*height
  * must not exceed 2^21 (EBOF_ERR_INVALID_ARG otherwise).  The call

@@ -2012,14 +2012,22 @@ ebof_status ebof_edt(const uint8_t *d_edge, int32_t width, int32_t height, int32
     cudaGetLastError();
     const size_t plane = (size_t)width * height;
     // a row's words serve 32 rows, so the scratch must outlive the first
-    // results: where the caller lets it overlap them, the column distances are
-    // read off the edge image instead
-    auto overlaps = [&](const void *out) {
-        return out && (const char *)out < (const char *)(d_scratch + plane) &&
-               (const char *)d_scratch < (const char *)out + 4 * plane;
+    // results: where the caller lets it overlap them, the column distances
+    // themselves are kept, in place in a result.  In the scratch's own place if
+    // that is a result (the caller keeps the edge image out of the scratch), else
+    // in a result that the edge image is not in.
+    auto overlaps = [&](const void *a, size_t an, const void *b, size_t bn) {
+        return a && b && (const char *)a < (const char *)b + bn &&
+               (const char *)b < (const char *)a + an;
     };
-    if (overlaps(d_edt) || overlaps(d_surface)) {
-        launch_edt_direct(d_edge, width, height, alpha, d_edt, d_surface, st);
+    if (overlaps(d_scratch, 4 * plane, d_edt, 4 * plane) ||
+        overlaps(d_scratch, 4 * plane, d_surface, 4 * plane)) {
+        const void *s = d_scratch;
+        int32_t *g = s == d_edt || s == d_surface ? d_scratch
+                     : d_surface && overlaps(d_edge, plane, d_edt, 4 * plane)
+                         ? (int32_t *)d_surface
+                         : d_edt;
+        launch_edt_inplace(d_edge, width, height, alpha, g, d_edt, d_surface, st);
     } else {
         launch_edt_columns(d_edge, width, plane, width, height, d_scratch, width, plane, 1, st);
         launch_edt_rows_surface(d_scratch, width, plane, width, height, alpha, d_edt, d_surface,

@@ -163,10 +163,10 @@ void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_strid
                              int i_pitch, size_t i_frame_stride, int frames, bool half,
                              cudaStream_t st);
 
-// A3 and A4 with the Eq. 1 surface straight from a dense edge image, without
-// scratch (slower: every pixel walks its column).
-void launch_edt_direct(const uint8_t *edge, int W, int H, float alpha, int32_t *D_dense,
-                       float *S_dense, cudaStream_t st);
+// A3 and A4 with the Eq. 1 surface of a dense edge image, the column distances
+// kept in g [H][W], which may be D_dense or S_dense itself.
+void launch_edt_inplace(const uint8_t *edge, int W, int H, float alpha, int32_t *g,
+                        int32_t *D_dense, float *S_dense, cudaStream_t st);
 
 // Per-device kernel attributes (opt-in shared memory); call with the device current.
 void init_front_attributes();

@@ -1,5 +1,5 @@
 // edt_static.cu -- ebof_edt_static: the exact EDT entry point for callers that
-// cannot allocate device memory.  Its scratch (the column distances of the
+// cannot allocate device memory.  Its scratch (the columns' words of the
 // separable EDT) lives in a file-scope __device__ array instead of a buffer
 // the caller passes in.
 #include "ebof.h"

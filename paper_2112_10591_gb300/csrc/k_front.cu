@@ -338,14 +338,21 @@ seg_denoise_fill_kernel(const __grid_constant__ SegTable<SegDenoise> tab)
 // of its columns (a word's 32 byte loads in flight together) and publishes
 // their first and last edge rows; one warp then runs down and one up the
 // column's words.
+//
+// DIST: the distances themselves, a pixel an int32, for a stand-alone call whose
+// scratch is one of its results: a row of distances is read by that row's block
+// only, before it writes the row's results there, where a word serves 32 rows.
+// The words then stay in shared memory.  It writes the 4 bytes a pixel that the
+// words save: 640x480 @@A, 1920x1080 @@B us a call, against @@C and @@D.
 constexpr int kColWarps = 32;
 constexpr int kNoneAbove = -32768, kNoneBelow = 32767;
 
 __host__ __device__ __forceinline__ int col_words(int H) { return (H + 31) / 32; }
-// shared memory of a block: the first and last edge rows of its words
-__host__ __device__ __forceinline__ size_t cols_smem_bytes(int nw)
+// shared memory of a block: the first and last edge rows of its words (dist:
+// and the words, 128 KB in all for 16384 rows)
+__host__ __device__ __forceinline__ size_t cols_smem_bytes(int nw, bool dist)
 {
-    return (size_t)nw * 32 * 2 * sizeof(int16_t);
+    return (size_t)nw * 32 * (2 * sizeof(int16_t) + (dist ? sizeof(uint32_t) : 0));
 }
 // the nearest edge rows above and below, 16 bits each
 __device__ __forceinline__ int pack_rows(int above, int below)
@@ -355,14 +362,26 @@ __device__ __forceinline__ int pack_rows(int above, int below)
 __device__ __forceinline__ int row_above(int v) { return (int)(int16_t)(v & 0xffff); }
 __device__ __forceinline__ int row_below(int v) { return v >> 16; }
 
+// Column distance from a pixel's words; above kMaxDim - 1: no edge pixel.
+__device__ __forceinline__ int word_distance(uint32_t m, int ab, int y)
+{
+    const int b = y & 31;
+    const uint32_t us = m << (31 - b), ds = m >> b;
+    const int up = us ? __clz(us) : y - row_above(ab);
+    const int dn = ds ? __clz(__brev(ds)) : row_below(ab) - y;
+    return min(up, dn);
+}
+
 // bx: the block of 32 columns, f: the frame.
+template <bool DIST>
 __device__ __forceinline__ void edt_cols_body(const uint8_t *__restrict__ E, int epitch,
                                               size_t efs, int W, int H, int32_t *__restrict__ g,
                                               int gpitch, size_t gfs, unsigned bx, unsigned f)
 {
-    extern __shared__ int16_t s_rows[];
+    extern __shared__ __align__(4) int16_t s_rows[];
     const int nw = col_words(H), c = threadIdx.x, x = bx * 32 + c;
     int16_t *s_last = s_rows + c, *s_first = s_last + nw * 32;
+    uint32_t *s_words = reinterpret_cast<uint32_t *>(s_rows + nw * 64) + c;  // DIST
     const bool colok = x < W;
     const uint8_t *e = E + (size_t)f * efs + min(x, W - 1);
     uint32_t *words = reinterpret_cast<uint32_t *>(g + (size_t)f * gfs) + x;
@@ -377,11 +396,12 @@ __device__ __forceinline__ void edt_cols_body(const uint8_t *__restrict__ E, int
         for (int b = 0; b < 32; ++b)
             if (ev[b]) m |= 1u << b;
         if (wi == nw - 1 && (H & 31)) m &= (1u << (H & 31)) - 1;
-        if (colok) words[(size_t)wi * gpitch] = m;
+        if (DIST) s_words[wi * 32] = m;
+        else if (colok) words[(size_t)wi * gpitch] = m;
         s_last[wi * 32] = (int16_t)(m ? wi * 32 + 31 - __clz(m) : kNoneAbove);
         s_first[wi * 32] = (int16_t)(m ? wi * 32 + __ffs(m) - 1 : kNoneBelow);
     }
-    if (nw == 1) return;
+    if (!DIST && nw == 1) return;
     __syncthreads();
     // one warp runs down the column's words and one up, eight at a time (the
     // loads before the chain of maxima)
@@ -414,16 +434,25 @@ __device__ __forceinline__ void edt_cols_body(const uint8_t *__restrict__ E, int
     }
     __syncthreads();
     if (!colok) return;
-    for (int wi = threadIdx.y; wi < nw; wi += blockDim.y)
-        words[(size_t)(nw + wi) * gpitch] = pack_rows(s_last[wi * 32], s_first[wi * 32]);
+    for (int wi = threadIdx.y; wi < nw; wi += blockDim.y) {
+        const int ab = pack_rows(s_last[wi * 32], s_first[wi * 32]);
+        if (!DIST) {
+            words[(size_t)(nw + wi) * gpitch] = ab;
+            continue;
+        }
+        const uint32_t m = s_words[wi * 32];
+        const int y1 = min(wi * 32 + 32, H);
+        for (int y = wi * 32; y < y1; ++y) words[(size_t)y * gpitch] = word_distance(m, ab, y);
+    }
 }
 
+template <bool DIST>
 __global__ void __launch_bounds__(32 * kColWarps)
 edt_cols_kernel(const uint8_t *__restrict__ E, int epitch, size_t efs, int W, int H,
                 int32_t *__restrict__ g, int gpitch, size_t gfs)
 {
     chain_begin();
-    edt_cols_body(E, epitch, efs, W, H, g, gpitch, gfs, blockIdx.x, blockIdx.y);
+    edt_cols_body<DIST>(E, epitch, efs, W, H, g, gpitch, gfs, blockIdx.x, blockIdx.y);
 }
 
 __global__ void __launch_bounds__(32 * kColWarps)
@@ -431,7 +460,7 @@ seg_edt_cols_kernel(const __grid_constant__ SegTable<SegEdtCols> tab)
 {
     int b;
     const SegEdtCols &a = seg_of(tab, b);
-    edt_cols_body(a.E, a.epitch, a.efs, a.W, a.H, a.g, a.gpitch, a.gfs, b % a.gx, b / a.gx);
+    edt_cols_body<false>(a.E, a.epitch, a.efs, a.W, a.H, a.g, a.gpitch, a.gfs, b % a.gx, b / a.gx);
 }
 
 // ---------------------------------------------------------------- A4
@@ -474,16 +503,6 @@ __host__ __device__ __forceinline__ size_t rows_smem_bytes(int W)
 {
     const size_t nb = ((size_t)W + 31) / 32;
     return 4 * (((size_t)W + 3) & ~(size_t)3) + ((4 * (nb + 1) + 15) & ~(size_t)15);
-}
-
-// Column distance from a pixel's words; above kMaxDim - 1: no edge pixel.
-__device__ __forceinline__ int word_distance(uint32_t m, int ab, int y)
-{
-    const int b = y & 31;
-    const uint32_t us = m << (31 - b), ds = m >> b;
-    const int up = us ? __clz(us) : y - row_above(ab);
-    const int dn = ds ? __clz(__brev(ds)) : row_below(ab) - y;
-    return min(up, dn);
 }
 
 // Owners of the NP pixels x, x + dx, ... (NP * dx columns of pixels) among the
@@ -553,14 +572,14 @@ __device__ __forceinline__ float ablation_surface(const SurfaceMap &sm, float d)
 // warp-level barriers only.  WPR > 1: one row per block.  D is exact whatever
 // WPR, so the layout never changes a result.  bx: the block of rows, f: the
 // frame.  A warp past the block's rows_per_block rows (a fused launch sized for
-// another segment's) exits (WPR = 1 has warp-level barriers only).  Edge: where
-// set, the column distances are read off the edge image itself instead of g.
-template <int WPR, typename T>
+// another segment's) exits (WPR = 1 has warp-level barriers only).  DIST: g holds
+// distances instead of words, and D_dense or S_dense may be g itself: a row is
+// read before row_sync() and written after it, by its own warps.
+template <int WPR, bool DIST, typename T>
 __device__ __forceinline__ void edt_rows_surface_body(
-    const int32_t *__restrict__ g, int gpitch, size_t gfs, int W, int H, int rows_per_block,
-    const SurfaceMap &sm, int32_t *D_dense, float *__restrict__ S_dense,
-    T *__restrict__ I0, int ipitch, size_t ifs, int bx, int f,
-    const uint8_t *__restrict__ edge = nullptr)
+    const int32_t *g, int gpitch, size_t gfs, int W, int H, int rows_per_block,
+    const SurfaceMap &sm, int32_t *D_dense, float *S_dense, T *__restrict__ I0, int ipitch,
+    size_t ifs, int bx, int f)
 {
     constexpr int NT = 32 * WPR;
     constexpr int FAC = 4;  // how many times finer each level of step 2 is
@@ -581,8 +600,8 @@ __device__ __forceinline__ void edt_rows_surface_body(
     // 1. loads issued in batches of kRowLoads before their first use
     {
         const int nw = col_words(H);
-        const uint32_t *words =
-            reinterpret_cast<const uint32_t *>(g + (size_t)f * gfs) + (size_t)(y >> 5) * gpitch;
+        const uint32_t *words = reinterpret_cast<const uint32_t *>(g + (size_t)f * gfs) +
+                                (size_t)(DIST ? y : y >> 5) * gpitch;
         const size_t ab_off = (size_t)nw * gpitch;
         const int none = pack_rows(kNoneAbove, kNoneBelow);
         for (int x0 = tr; x0 < Wp; x0 += NT * kRowLoads) {
@@ -591,30 +610,16 @@ __device__ __forceinline__ void edt_rows_surface_body(
 #pragma unroll
             for (int u = 0; u < kRowLoads; ++u) {
                 const int x = x0 + NT * u;
-                m[u] = 0;
+                m[u] = DIST ? kMaxDim : 0;
                 ab[u] = none;
-                if (x < W && !edge) {
+                if (x < W) {
                     m[u] = words[x];
-                    if (nw > 1) ab[u] = (int)words[ab_off + x];
+                    if (!DIST && nw > 1) ab[u] = (int)words[ab_off + x];
                 }
             }
 #pragma unroll
-            for (int u = 0; u < kRowLoads; ++u) d[u] = word_distance(m[u], ab[u], y);
-            if (edge) {
-#pragma unroll 1
-                for (int u = 0; u < kRowLoads; ++u) {
-                    const int x = x0 + NT * u;
-                    d[u] = kMaxDim;
-                    for (int k = 0; x < W && k < H; ++k) {
-                        if ((y - k >= 0 && edge[(size_t)(y - k) * W + x]) ||
-                            (y + k < H && edge[(size_t)(y + k) * W + x])) {
-                            d[u] = k;
-                            break;
-                        }
-                        if (y - k < 0 && y + k >= H) break;
-                    }
-                }
-            }
+            for (int u = 0; u < kRowLoads; ++u)
+                d[u] = DIST ? (int)m[u] : word_distance(m[u], ab[u], y);
 #pragma unroll
             for (int u = 0; u < kRowLoads; ++u) {
                 const int x = x0 + NT * u;
@@ -695,17 +700,18 @@ edt_rows_surface_kernel(const int32_t *__restrict__ g, int gpitch, size_t gfs, i
                         float *__restrict__ S_dense, T *__restrict__ I0, int ipitch, size_t ifs)
 {
     chain_begin();
-    edt_rows_surface_body<WPR, T>(g, gpitch, gfs, W, H, rows_per_block, sm, D_dense, S_dense, I0,
-                                  ipitch, ifs, blockIdx.x, blockIdx.y);
+    edt_rows_surface_body<WPR, false, T>(g, gpitch, gfs, W, H, rows_per_block, sm, D_dense,
+                                         S_dense, I0, ipitch, ifs, blockIdx.x, blockIdx.y);
 }
 
-// The row pass straight from a dense edge image, without scratch.
+// The row pass from distances that lie in one of its results (no restrict: it
+// writes where it has read).
 __global__ void __launch_bounds__(32 * kRowsPerBlock)
-edt_direct_kernel(const uint8_t *__restrict__ edge, int W, int H, SurfaceMap sm,
-                  int32_t *__restrict__ D_dense, float *__restrict__ S_dense)
+edt_rows_inplace_kernel(const int32_t *g, int W, int H, SurfaceMap sm, int32_t *D_dense,
+                        float *S_dense)
 {
-    edt_rows_surface_body<kRowsPerBlock, float>(nullptr, 0, 0, W, H, 1, sm, D_dense, S_dense,
-                                                nullptr, 0, 0, blockIdx.x, 0, edge);
+    edt_rows_surface_body<kRowsPerBlock, true, float>(g, W, 0, W, H, 1, sm, D_dense, S_dense,
+                                                      nullptr, 0, 0, blockIdx.x, 0);
 }
 
 template <typename T>
@@ -714,8 +720,8 @@ seg_edt_rows_kernel(const __grid_constant__ SegTable<SegEdtRows> tab)
 {
     int b;
     const SegEdtRows &a = seg_of(tab, b);
-    edt_rows_surface_body<1, T>(a.g, a.gpitch, a.gfs, a.W, a.H, a.rows, a.sm, nullptr, nullptr,
-                                (T *)a.I0, a.ipitch, a.ifs, b % a.gx, b / a.gx);
+    edt_rows_surface_body<1, false, T>(a.g, a.gpitch, a.gfs, a.W, a.H, a.rows, a.sm, nullptr,
+                                       nullptr, (T *)a.I0, a.ipitch, a.ifs, b % a.gx, b / a.gx);
 }
 
 // Caller-given surface (dense, d_exp in [0, 1]) to the level-0 intensity.
@@ -780,7 +786,7 @@ void launch_denoise_fill(const uint8_t *E, uint8_t *Ed, uint8_t *Edf, int W, int
 }
 
 int edt_cols_warps(int H) { return std::min(col_words(H), kColWarps); }
-size_t edt_cols_smem(int H) { return cols_smem_bytes(col_words(H)); }
+size_t edt_cols_smem(int H, bool dist) { return cols_smem_bytes(col_words(H), dist); }
 
 void launch_edt_columns(const uint8_t *E, int edge_pitch, size_t edge_frame_stride, int W,
                         int H, int32_t *g, int g_pitch, size_t g_frame_stride, int frames,
@@ -788,8 +794,8 @@ void launch_edt_columns(const uint8_t *E, int edge_pitch, size_t edge_frame_stri
 {
     StageScope sc(kStEdtCols, 1, st);
     dim3 blk(32, edt_cols_warps(H)), grd((W + 31) / 32, frames);
-    launch_chained(chained, edt_cols_kernel, grd, blk, edt_cols_smem(H), st, E, edge_pitch,
-                   edge_frame_stride, W, H, g, g_pitch, g_frame_stride);
+    launch_chained(chained, edt_cols_kernel<false>, grd, blk, edt_cols_smem(H, false), st, E,
+                   edge_pitch, edge_frame_stride, W, H, g, g_pitch, g_frame_stride);
 }
 
 int edt_rows_block_rows(int W)
@@ -823,12 +829,17 @@ void edt_rows_t(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int
                    g_frame_stride, W, H, rows, sm, D_dense, S_dense, I0, i_pitch, i_frame_stride);
 }
 
-void launch_edt_direct(const uint8_t *edge, int W, int H, float alpha, int32_t *D_dense,
-                       float *S_dense, cudaStream_t st)
+void launch_edt_inplace(const uint8_t *edge, int W, int H, float alpha, int32_t *g,
+                        int32_t *D_dense, float *S_dense, cudaStream_t st)
 {
+    {
+        StageScope sc(kStEdtCols, 1, st);
+        edt_cols_kernel<true><<<(W + 31) / 32, dim3(32, edt_cols_warps(H)), edt_cols_smem(H, true),
+                                st>>>(edge, W, 0, W, H, g, W, 0);
+    }
     StageScope sc(kStEdtRows, 1, st);
-    edt_direct_kernel<<<H, 32 * kRowsPerBlock, edt_rows_smem(W, 1), st>>>(
-        edge, W, H, exp_surface(alpha), D_dense, S_dense);
+    edt_rows_inplace_kernel<<<H, 32 * kRowsPerBlock, edt_rows_smem(W, 1), st>>>(
+        g, W, H, exp_surface(alpha), D_dense, S_dense);
 }
 
 static void edt_rows(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
@@ -877,8 +888,9 @@ void init_front_attributes()
     opt_in((const void *)edt_rows_surface_kernel<kRowsPerBlock, float>);
     opt_in((const void *)edt_rows_surface_kernel<1, __half>);
     opt_in((const void *)edt_rows_surface_kernel<kRowsPerBlock, __half>);
-    opt_in((const void *)edt_direct_kernel);
-    opt_in((const void *)edt_cols_kernel);
+    opt_in((const void *)edt_rows_inplace_kernel);
+    opt_in((const void *)edt_cols_kernel<false>);
+    opt_in((const void *)edt_cols_kernel<true>);
     opt_in((const void *)seg_edt_cols_kernel);
     opt_in((const void *)seg_edt_rows_kernel<float>);
     opt_in((const void *)seg_edt_rows_kernel<__half>);
@@ -899,7 +911,8 @@ void launch_seg_denoise_fill(const SegTable<SegDenoise> &t, int blocks, cudaStre
 void launch_seg_edt_cols(const SegTable<SegEdtCols> &t, int blocks, int max_h, cudaStream_t st)
 {
     StageScope sc(kStEdtCols, 1, st);
-    seg_edt_cols_kernel<<<blocks, dim3(32, edt_cols_warps(max_h)), edt_cols_smem(max_h), st>>>(t);
+    const dim3 blk(32, edt_cols_warps(max_h));
+    seg_edt_cols_kernel<<<blocks, blk, edt_cols_smem(max_h, false), st>>>(t);
 }
 
 void launch_seg_edt_rows(const SegTable<SegEdtRows> &t, int blocks, int rows_max, size_t smem,
