@@ -168,6 +168,8 @@ void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_strid
 void launch_edt_inplace(const uint8_t *edge, int W, int H, float alpha, int32_t *g,
                         int32_t *D_dense, float *S_dense, cudaStream_t st);
 
+int sm_count();  // of the current device; 0: unknown
+
 // Per-device kernel attributes (opt-in shared memory); call with the device current.
 void init_front_attributes();
 void init_flow_attributes();

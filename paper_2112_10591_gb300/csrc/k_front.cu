@@ -14,6 +14,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 
 namespace ebof {
 
@@ -865,18 +866,38 @@ void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_strid
              frames, half, false, st);
 }
 
-// The stand-alone transform: the rows start while the columns end where they
-// are few (four blocks an SM; 640 x 480 14.4 -> 12.4 us); more of them fill the
-// SMs beside the column kernel's blocks and slow it (1280 x 720 22.6 either way,
-// 1920 x 1080 45.1 against 34.9 with full dependencies).  Within a
-// window they start late (613 x 397 with exports 386 us, early 388).
+// Whether a stand-alone transform's rows start while its columns end: that saves
+// a launch's latency (2 us), but rows started early fill the SMs that the column
+// blocks leave, and only those.  So they do where those SMs take at most one row
+// more each than all of them would (measured, early against late: 346x260 8.3
+// and 10.3 us, 640x480 12.4 and 14.4, 1024x640 18.5 and 20.4, 2048x200 20.6 and
+// 21.3, 3500x40 30.8 and 32.9, 3500x80 32.8 both; beyond it 1280x720 22.6 both,
+// 1920x1080 45.1 and 35.4, 4096x300 82.0 and 37.0, 8192x200 90.2 and 62.6).
+// Within a window rows start late (613x397 with exports 386 us, early 388).
+static bool rows_start_early(int W, int H)
+{
+    const int sms = sm_count(), left = sms - (W + 31) / 32;
+    return left > 0 && (H + left - 1) / left <= (H + sms - 1) / sms + 1;
+}
+
 void launch_edt_rows_surface(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
                              float alpha, int32_t *D_dense, float *S_dense, void *I0,
                              int i_pitch, size_t i_frame_stride, int frames, bool half,
                              cudaStream_t st)
 {
     edt_rows(g, g_pitch, g_frame_stride, W, H, exp_surface(alpha), D_dense, S_dense, I0, i_pitch,
-             i_frame_stride, frames, half, (long long)H * frames <= 608, st);
+             i_frame_stride, frames, half, frames == 1 && rows_start_early(W, H), st);
+}
+
+int sm_count()
+{
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int n = known[dev].load(std::memory_order_relaxed);
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        known[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 void init_front_attributes()

@@ -94,8 +94,6 @@ constexpr size_t flow_stage_bytes()
 __host__ __device__ constexpr int u_box_width(int tile) { return (tile + 3 + 3) & ~3; }
 constexpr size_t kTmaSmemBytes =
     (kTmaCoefFloats + (2 * (kVR - 2) + kVS - 1) * u_box_width(kVR - 2)) * sizeof(float);
-constexpr int kMaxDevs = 64;
-int g_num_sms[kMaxDevs];
 constexpr unsigned kFull = 0xffffffffu;
 
 // Loads of data that the same launch may have written on another SM earlier
@@ -1315,12 +1313,6 @@ bool var_fused_supported(int var_sor)
 
 void init_var_attributes()
 {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevs) {
-        int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        g_num_sms[dev] = n;
-    }
     cudaFuncSetAttribute(var_sor_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kTmaSmemBytes);
     cudaFuncSetAttribute(var_sor_kernel<kVS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1382,9 +1374,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
 {
     // the level's planes are packed: frame stride kCPlanes planes of this level
     const size_t coef_frame_stride = (size_t)kCPlanes * lv.plane;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const int nsm = (dev >= 0 && dev < kMaxDevs && g_num_sms[dev] > 0) ? g_num_sms[dev] : 0;
+    const int nsm = sm_count();
     const int n_half = 2 * fp.var_sor;
     const int R = sor_halo(fp.var_sor);
     const int tile = sor_tile(R);           // interior side of a 64 x 64 region
