@@ -582,15 +582,18 @@ uint64_t ebof_kernel_launches(void);
  * paper has no counterpart; they let tests drive the error paths above
  * without faulting a GPU. */
 
-/* Bound, in mbarrier try-wait rounds, of the waits of the batched SOR kernel
+/* Bound of the waits inside the variational kernels.  Of the batched SOR kernel
  * (the copy-ahead form, used when a call's variational grid has at least
- * sor_tma_min_per_sm regions per SM) for a region's copies, its coefficients'
- * and its flow's.  When one runs out the kernel latches EBOF_ERR_TIMEOUT,
- * reported by ebof_stream_sync, lets the copies in flight land under a second
- * wait at the default bound, and leaves the flow of that call undefined.  Applies to launches enqueued
- * after the call (graphs captured earlier keep their bound); iterations < 0
- * restores the default, 2^22; 0 makes every such wait run out at once.
- * EBOF_ERR_BUSY while another thread uses the stream. */
+ * sor_tma_min_per_sm regions per SM), in mbarrier try-wait rounds: the waits for
+ * a region's copies, its coefficients' and its flow's.  Of the refinement of a
+ * level in one launch, in polls: the waits for the flow that other regions
+ * publish between the outer iterations.  When one runs out the kernel latches
+ * EBOF_ERR_TIMEOUT, reported by ebof_stream_sync, lets the copies in flight land
+ * under a second wait at the default bound, and leaves the flow of that call
+ * undefined.  Applies to launches enqueued after the call (graphs captured
+ * earlier keep their bound, which steady in-order windows and lists replay);
+ * iterations < 0 restores the default, 2^22; 0 makes every such wait run out at
+ * once.  EBOF_ERR_BUSY while another thread uses the stream. */
 ebof_status ebof_stream_set_wait_limit(ebof_stream *s, int64_t iterations);
 
 /* The next n device allocations of this library (all threads, all streams)

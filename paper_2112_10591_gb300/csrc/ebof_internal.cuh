@@ -85,7 +85,7 @@ struct FlowParams {
     float gn_damping;
     int var_outer, var_sor;
     float delta, gamma, alpha_s, omega;
-    long long wait_limit;  // first wait of the copy-ahead SOR kernel (rounds)
+    long long wait_limit;  // rounds of the variational kernels' waits
     // variational layouts (ebof_params): none changes a result
     int sor_tma_min_per_sm, sor_row_waves, var_cluster_max;
     // the one-launch refinement's counters (kLevelCtl words, 0 at first) and
