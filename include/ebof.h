@@ -578,7 +578,7 @@ const char *ebof_stage_name(int32_t stage);
 uint64_t ebof_kernel_launches(void);
 
 /* ---- diagnostics: failure injection for tests ------------------------------
- * Both act on the host side only and change nothing a kernel computes.  The
+ * They act on the host side only and change nothing a kernel computes.  The
  * paper has no counterpart; they let tests drive the error paths above
  * without faulting a GPU. */
 
@@ -595,6 +595,11 @@ uint64_t ebof_kernel_launches(void);
  * iterations < 0 restores the default, 2^22; 0 makes every such wait run out at
  * once.  EBOF_ERR_BUSY while another thread uses the stream. */
 ebof_status ebof_stream_set_wait_limit(ebof_stream *s, int64_t iterations);
+
+/* The bound of one of these waits alone, the batched SOR kernel's for a region's
+ * flow, which comes after the sweeps: with 0 here the coefficients' wait
+ * succeeds and this one runs out.  ebof_stream_set_wait_limit sets it too. */
+ebof_status ebof_debug_flow_wait_limit(ebof_stream *s, int64_t iterations);
 
 /* The next n device allocations of this library (all threads, all streams)
  * succeed and the one after fails the way cudaMalloc fails when the device is

@@ -182,6 +182,7 @@ def _declare(L):
     L.ebof_status_string.argtypes = [ctypes.c_int]
     L.ebof_status_string.restype = ctypes.c_char_p
     L.ebof_stream_set_wait_limit.argtypes = [vp, i64]
+    L.ebof_debug_flow_wait_limit.argtypes = [vp, i64]
     L.ebof_debug_fail_allocation.argtypes = [i32]
     L.ebof_debug_fail_allocation.restype = None
     for name in ("ebof_stream_create", "ebof_stream_destroy", "ebof_stream_reset",
@@ -196,7 +197,8 @@ def _declare(L):
                  "ebof_process_window_list", "ebof_server_create", "ebof_fwl", "ebof_server_destroy",
                  "ebof_server_open_stream", "ebof_server_close_stream", "ebof_server_submit",
                  "ebof_server_poll", "ebof_server_drain", "ebof_server_get_info",
-                 "ebof_stream_set_wait_limit", "ebof_multigroup_create",
+                 "ebof_stream_set_wait_limit", "ebof_debug_flow_wait_limit",
+                 "ebof_multigroup_create",
                  "ebof_multigroup_destroy", "ebof_multigroup_process",
                  "ebof_multigroup_set_fused"):
         getattr(L, name).restype = ctypes.c_int
@@ -586,6 +588,10 @@ EBOF_STAGE_COUNT = 12
 
 def ebof_stream_set_wait_limit(stream: Stream, iterations: int) -> int:
     return load().ebof_stream_set_wait_limit(stream.handle, int(iterations))
+
+
+def ebof_debug_flow_wait_limit(stream: Stream, iterations: int) -> int:
+    return load().ebof_debug_flow_wait_limit(stream.handle, int(iterations))
 
 
 def ebof_debug_fail_allocation(n: int) -> None:

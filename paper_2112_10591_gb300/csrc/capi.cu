@@ -82,6 +82,7 @@ struct ebof_stream {
     bool have_last = false;
     std::atomic<int> busy{0};
     long long wait_limit = kWaitLimitDefault;  // ebof_stream_set_wait_limit
+    long long flow_wait_limit = kWaitLimitDefault;  // ebof_debug_flow_wait_limit
     Profiler prof;
     // Per-call window descriptors and flow destinations, read on the device by
     // the descriptor-driven paths: [max_batch] ebof_window_desc followed by
@@ -425,7 +426,7 @@ FlowParams flow_params(const ebof_params &p)
     fp.gamma = p.var_gamma;
     fp.alpha_s = p.var_alpha;
     fp.omega = p.sor_omega;
-    fp.wait_limit = kWaitLimitDefault;
+    fp.wait_limit = fp.flow_wait_limit = kWaitLimitDefault;
     fp.sor_tma_min_per_sm = p.sor_tma_min_per_sm;
     fp.sor_row_waves = p.sor_row_waves;
     fp.var_cluster_max = p.var_cluster_max;
@@ -503,6 +504,7 @@ void enqueue(ebof_stream *s, int n, const uint16_t *x, const uint16_t *y, const 
         const int curf_first = cur_first + ff;
         FlowParams fp = flow_params(p);
         fp.wait_limit = s->wait_limit;
+        fp.flow_wait_limit = s->flow_wait_limit;
         const FlowScratch own = {s->up, s->Ua, s->Ub, s->work, &s->cmaps};
         const FlowScratch &sc = scratch ? *scratch : own;
         float *Ucur = nullptr, *Uc = nullptr;
@@ -1949,6 +1951,16 @@ ebof_status ebof_stream_set_wait_limit(ebof_stream *s, int64_t iterations)
     BusyGuard bg(s->busy);
     if (!bg.ok) return EBOF_ERR_BUSY;
     s->wait_limit = iterations < 0 ? kWaitLimitDefault : (long long)iterations;
+    s->flow_wait_limit = s->wait_limit;
+    return EBOF_OK;
+}
+
+ebof_status ebof_debug_flow_wait_limit(ebof_stream *s, int64_t iterations)
+{
+    if (!s) return EBOF_ERR_INVALID_ARG;
+    BusyGuard bg(s->busy);
+    if (!bg.ok) return EBOF_ERR_BUSY;
+    s->flow_wait_limit = iterations < 0 ? kWaitLimitDefault : (long long)iterations;
     return EBOF_OK;
 }
 

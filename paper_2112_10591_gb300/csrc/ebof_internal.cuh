@@ -86,6 +86,7 @@ struct FlowParams {
     int var_outer, var_sor;
     float delta, gamma, alpha_s, omega;
     long long wait_limit;  // rounds of the variational kernels' waits
+    long long flow_wait_limit;  // of the copy-ahead kernel's for a region's flow
     // variational layouts (ebof_params): none changes a result
     int sor_tma_min_per_sm, sor_row_waves, var_cluster_max;
     // the one-launch refinement's counters (kLevelCtl words, 0 at first) and

@@ -493,7 +493,8 @@ __global__ void __launch_bounds__(kVThreads, 1)
 var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap,
                    const __grid_constant__ CUtensorMap umap, int w, int h, int pitch,
                    float *__restrict__ Uoutb, size_t ufs, size_t plane, int R, int nrx, int nry,
-                   int total, int n_half, float omega, long long wait_limit, int *err)
+                   int total, int n_half, float omega, long long wait_limit,
+                   long long flow_wait_limit, int *err)
 {
     chain_begin();
     extern __shared__ __align__(1024) float tsm[];
@@ -599,7 +600,7 @@ var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap,
         else
             edge_weights<kVS, false>(s, as, lane, first, last, p.gx, p.gy, w, h);
         sor_sweeps<kVS, kVWarps>(s, ends, lane, wp, (p.gx + p.gy) & 1, n_half, omega);
-        late = !mbar_wait(ubar, parity, wait_limit);
+        late = !mbar_wait(ubar, parity, flow_wait_limit);
         parity ^= 1u;
         if (p.r0 < p.r1) {
             // loads before the tests of what is stored; those of pixels that
@@ -1458,7 +1459,7 @@ float *launch_variational_fused(const void *I0, const void *I0x, const void *I0y
                 launch_chained(true, var_sor_tma_kernel, std::min(nsm, total), kVThreads,
                                kTmaSmemBytes, st, maps->coef, maps->u[ub], lv.w, lv.h, lv.pitch, b,
                                u_frame_stride, lv.plane, R, (int)sgrd.x, (int)sgrd.y, total,
-                               n_half, fp.omega, fp.wait_limit, err);
+                               n_half, fp.omega, fp.wait_limit, fp.flow_wait_limit, err);
             else if (small >= 8 && (long long)(g1.x * g1.y * g1.z) <= (long long)row_waves * nsm)
                 launch_chained(true, var_sor_kernel<kVSmallVS>, g1, kVThreads,
                                flow_stage_bytes<kVSmallVS, kVWarps>(), st, lv.w, lv.h, lv.pitch,
