@@ -9,10 +9,11 @@
 //   2. fwl_sums_kernel: per-block sums of I and I^2 of both images in a fixed
 //      order; the last block to finish adds the blocks' in a fixed order and
 //      writes FWL = var(I_comp) / var(I_uncomp) with the two variances.
-// The sums are kept as unevaluated pairs of floats (about 48 bits) inside a
-// warp and as doubles beyond it: this chip's FP64 rate made the sums in double
-// the longest step.  Measured at 1280x720 with 276k events: the sums 16.9 + 6.6
-// us in two launches -> about 7 us in one, a call 43.7 -> 26.0 us.  The rest is
+// The sums are kept as unevaluated triples of floats (about 70 bits) inside a
+// block and as doubles beyond it: this chip's FP64 rate made the sums in double
+// the longest step, and two floats (48 bits) held less than a double does.
+// Measured at 1280x720 with 276k events: the sums in double 16.9 + 6.6 us in two
+// launches, a call 44.9; pairs 10.2 and 25.3; triples 11.1 and 27.3.  The rest is
 // the splat, 15 us of L1 requests for scattered votes (L1 at 76 %).
 // Traffic: 16 B per event read (x, y, t, p) plus 8 B of flow at its pixel,
 // the two images written by atomics and read once (8 B per pixel each way).
@@ -75,26 +76,55 @@ __global__ void fwl_splat_kernel(const uint16_t *__restrict__ x, const uint16_t 
     }
 }
 
-// A sum held as an unevaluated pair of floats; every operation rounds once and
-// is never fused, so the error terms are exact.
-struct PairSum {
-    float h = 0.0f, l = 0.0f;
-    __device__ __forceinline__ void add(float x, float e)  // x + e, |e| <= ulp(x)
+// The sum s + e of two floats, exactly (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// A sum held as three floats h + l + m, each the rounding errors of the one
+// before: only m's additions lose anything, 2^-24 of 2^-48 of the sum.  Every
+// operation rounds once and is never fused, so the error terms are exact.
+struct TripleSum {
+    float h = 0.0f, l = 0.0f, m = 0.0f;
+    __device__ __forceinline__ void add(float x)
     {
-        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-        const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b));
-        h = s;
-        l = __fadd_rn(l, __fadd_rn(err, e));
+        float e;
+        two_sum(h, x, h, e);
+        add_low(e);
     }
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+    __device__ __forceinline__ void add_low(float x)
+    {
+        float e;
+        two_sum(l, x, l, e);
+        m = __fadd_rn(m, e);
+    }
+    __device__ __forceinline__ void add(const TripleSum &o)
+    {
+        add(o.h);
+        add_low(o.l);
+        m = __fadd_rn(m, o.m);
+    }
+    __device__ __forceinline__ TripleSum of_lane(int mask) const  // lane ^ mask
+    {
+        TripleSum o;
+        o.h = __shfl_xor_sync(0xffffffffu, h, mask);
+        o.l = __shfl_xor_sync(0xffffffffu, l, mask);
+        o.m = __shfl_xor_sync(0xffffffffu, m, mask);
+        return o;
+    }
+    __device__ __forceinline__ double value() const { return (double)h + ((double)l + (double)m); }
 };
 
-// v and v^2 of one pixel into the two sums.
-__device__ __forceinline__ void add_moments(PairSum &m1, PairSum &m2, float v)
+// v and v^2 of one pixel into the two sums; the square is p + e exactly.
+__device__ __forceinline__ void add_moments(TripleSum &m1, TripleSum &m2, float v)
 {
     const float p = __fmul_rn(v, v);
-    m1.add(v, 0.0f);
-    m2.add(p, __fmaf_rn(v, v, -p));
+    m1.add(v);
+    m2.add(p);
+    m2.add_low(__fmaf_rn(v, v, -p));
 }
 
 // Four adjacent pixels from i on (VEC: an aligned quad), 0 past the image.
@@ -118,7 +148,7 @@ fwl_sums_kernel(const float *__restrict__ comp, const float *__restrict__ uncomp
 {
     constexpr int kWarps = kFwlThreads / 32;
     static_assert(kWarps == 8, "a warp adds the eight warps' four sums");
-    __shared__ float2 sh[4][kWarps];
+    __shared__ TripleSum sh[4][kWarps];
     __shared__ double shd[kWarps];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -133,7 +163,7 @@ fwl_sums_kernel(const float *__restrict__ comp, const float *__restrict__ uncomp
             c[k] = load4<VEC>(comp, i, P);
             u[k] = load4<VEC>(uncomp, i, P);
         }
-        PairSum m[4];
+        TripleSum m[4];
 #pragma unroll
         for (int k = 0; k < kQuads; ++k) {
             add_moments(m[0], m[1], c[k].x);
@@ -145,31 +175,24 @@ fwl_sums_kernel(const float *__restrict__ comp, const float *__restrict__ uncomp
             add_moments(m[0], m[1], c[k].w);
             add_moments(m[2], m[3], u[k].w);
         }
-        // over the warp, then over the warps, still in pairs
+        // over the warp, then over the warps, still in triples.  The lanes share
+        // the four sums: halves keep two each, quarters one each (6 additions of
+        // triples, 20 with every lane carrying all four)
+        const bool hi = lane & 16, hi8 = lane & 8;
+        TripleSum a = hi ? m[2] : m[0], b = hi ? m[3] : m[1];
+        a.add((hi ? m[0] : m[2]).of_lane(16));
+        b.add((hi ? m[1] : m[3]).of_lane(16));
+        TripleSum q = hi8 ? b : a;
+        q.add((hi8 ? a : b).of_lane(8));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float h = __shfl_down_sync(0xffffffffu, m[k].h, o);
-                const float l = __shfl_down_sync(0xffffffffu, m[k].l, o);
-                m[k].add(h, l);
-            }
+        for (int o = 4; o > 0; o >>= 1) q.add(q.of_lane(o));
         __syncthreads();  // the last pass's sums are read
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) sh[k][warp] = make_float2(m[k].h, m[k].l);
+        if (lane % 8 == 0) sh[lane / 8][warp] = q;  // quarter k has sum k
         __syncthreads();
         if (warp == 0) {
-            PairSum t;
-            const float2 q = sh[lane / kWarps][lane % kWarps];
-            t.h = q.x;
-            t.l = q.y;
+            TripleSum t = sh[lane / kWarps][lane % kWarps];
 #pragma unroll
-            for (int o = kWarps / 2; o > 0; o >>= 1) {
-                const float h = __shfl_down_sync(0xffffffffu, t.h, o);
-                const float l = __shfl_down_sync(0xffffffffu, t.l, o);
-                t.add(h, l);
-            }
+            for (int o = kWarps / 2; o > 0; o >>= 1) t.add(t.of_lane(o));
             if (lane % kWarps == 0) v += t.value();
         }
     }
