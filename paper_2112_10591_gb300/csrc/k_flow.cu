@@ -577,6 +577,19 @@ __device__ __forceinline__ void cover_range(int x, int n, int ps, int stride, ui
     last = x >= n - ps;
 }
 
+// (1 - f) a + f b, and between two rows, rounded in one order in every form of
+// the densification, whatever the compiler fuses: one or two pixels a thread,
+// staged patches or not, a launch of its own or a fused one give the same flow.
+__device__ __forceinline__ float dense_lerp(float a, float b, float f)
+{
+    return ffma(fsub(1.0f, f), a, fmul(f, b));
+}
+__device__ __forceinline__ float dense_lerp2(float a, float b, float c, float d, float fx,
+                                             float fy)
+{
+    return dense_lerp(dense_lerp(a, b, fx), dense_lerp(c, d, fx), fy);
+}
+
 // Thread per pixel.  NC = ceil(ps / stride) bounds the regular patches that
 // cover a pixel per axis: their loops are unrolled and predicated so that the
 // loads of all of them are in flight together, and the patch flush with the
@@ -597,7 +610,7 @@ __device__ __forceinline__ float dense_sample(const T *__restrict__ I1, int w, i
         const float ax = u - fu, ay = v - fv;
         const T *r0 = I1 + (int)syf * pitch + (int)sxf, *r1 = r0 + pitch;
         const float a = ldp(&r0[0]), b = ldp(&r0[1]), c = ldp(&r1[0]), d = ldp(&r1[1]);
-        return (1.0f - ay) * ((1.0f - ax) * a + ax * b) + ay * ((1.0f - ax) * c + ax * d);
+        return dense_lerp2(a, b, c, d, ax, ay);
     }
     return bilinear_i(I1, w, h, pitch, (float)x + u, (float)y + v);
 }
@@ -646,9 +659,11 @@ __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T 
     bool ilast;
     cover_range(x, w, ps, stride, magic, npx, ilo, ihi, ilast);
     auto weigh = [&](int k, float sample, float u, float v) {
-        const float r = sample - i0[k];
+        const float r = fsub(sample, i0[k]);
         const float lam = 1.0f / fmaxf(1.0f, fabsf(r));
-        nu[k] += lam * u; nv[k] += lam * v; den[k] += lam;
+        nu[k] = ffma(lam, u, nu[k]);
+        nv[k] = ffma(lam, v, nv[k]);
+        den[k] = fadd(den[k], lam);
     };
     bool staged = false, done = false;
     if (NC > 0) {
@@ -697,10 +712,10 @@ __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T 
                     float row[PY + 1];
 #pragma unroll
                     for (int k = 0; k <= PY; ++k, r0 += pitch)
-                        row[k] = (1.0f - ax) * ldp(&r0[0]) + ax * ldp(&r0[1]);
+                        row[k] = dense_lerp(ldp(&r0[0]), ldp(&r0[1]), ax);
 #pragma unroll
                     for (int k = 0; k < PY; ++k)
-                        weigh(k, (1.0f - ay) * row[k] + ay * row[k + 1], m.x, m.y);
+                        weigh(k, dense_lerp(row[k], row[k + 1], ay), m.x, m.y);
                 }
             done = true;
         } else if (staged) {
@@ -716,9 +731,7 @@ __device__ __forceinline__ void densify_body(const T *__restrict__ I0b, const T 
                     const float ax = m.z, ay = m.w;
                     const T *r0 = q + *off, *r1 = r0 + pitch;
                     const float a = ldp(&r0[0]), b = ldp(&r0[1]), c = ldp(&r1[0]), d = ldp(&r1[1]);
-                    weigh(k, (1.0f - ay) * ((1.0f - ax) * a + ax * b) +
-                                 ay * ((1.0f - ax) * c + ax * d),
-                          m.x, m.y);
+                    weigh(k, dense_lerp2(a, b, c, d, ax, ay), m.x, m.y);
                 };
                 auto row = [&](int jj) {
                     const float4 *m = &s_uv[jj][ilo - ti];
