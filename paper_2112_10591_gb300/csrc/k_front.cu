@@ -493,7 +493,6 @@ seg_edt_cols_kernel(const __grid_constant__ SegTable<SegEdtCols> tab)
 // without edge pixels gets h = 2^30.
 constexpr int kNoColumn = 1 << 30;
 
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRowsPerBlock = 4;                  // rows (warps) per block
 constexpr int kRowLoads = 4;                      // pixels in flight per lane
 constexpr size_t kRowsSmemCap = 200 * 1024;       // bytes; 16384-px rows fit

@@ -96,26 +96,10 @@ constexpr size_t kTmaSmemBytes =
     (kTmaCoefFloats + (2 * (kVR - 2) + kVS - 1) * u_box_width(kVR - 2)) * sizeof(float);
 constexpr unsigned kFull = 0xffffffffu;
 
-// Loads of data that the same launch may have written on another SM earlier
-// (COH: through L2 with ld.global.cg, never from a possibly stale L1 or the
-// read-only path); plain loads otherwise.  The values are the same.
-template <bool COH>
-__device__ __forceinline__ float ldf(const float *p)
+__device__ __forceinline__ float2 ld2(const float *p)
 {
-    if constexpr (COH)
-        return __ldcg(p);
-    else
-        return *p;
+    return *reinterpret_cast<const float2 *>(p);
 }
-template <bool COH>
-__device__ __forceinline__ float2 ldf2(const float *p)
-{
-    if constexpr (COH)
-        return __ldcg(reinterpret_cast<const float2 *>(p));
-    else
-        return *reinterpret_cast<const float2 *>(p);
-}
-
 
 // A thread's strip of 2 columns x VS rows: the pixels' systems, the weights of
 // their edges (right: of column 1 only, column 0's is column 1's left one;
@@ -334,37 +318,27 @@ __device__ __forceinline__ void store_row(const StripPlace<VS, WARPS> &p, float 
     }
 }
 
-// U + dU of the output pixels.  staged: this thread's slots after stage_flow,
-// or null: the flow is read here, through L2 (another SM may have written it
-// earlier in the launch).
+// U + dU of the output pixels.  staged: this thread's slots after stage_flow.
 template <int VS, int WARPS>
 __device__ __forceinline__ void store_flow(const StripPlace<VS, WARPS> &p, const Strip<VS> &s,
-                                           const float *Uin, float *Uout, size_t plane,
-                                           const float2 *staged)
+                                           float *Uout, size_t plane, const float2 *staged)
 {
-    if (staged) asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
     for (int r = 0; r < VS; ++r) {
         if (r < p.r0 || r >= p.r1) continue;
         const int o = (p.gy + r) * p.pitch + p.gx;
         const float2 d0 = upk(s.d[r][0]), d1 = upk(s.d[r][1]);
-        float2 u = make_float2(0.0f, 0.0f), v = u;
-        if (staged) {
-            u = staged[(2 * r) * 32 * WARPS];
-            v = staged[(2 * r + 1) * 32 * WARPS];
-        } else {
-            if (p.c0) u.x = __ldcg(Uin + o), v.x = __ldcg(Uin + plane + o);
-            if (p.c1) u.y = __ldcg(Uin + o + 1), v.y = __ldcg(Uin + plane + o + 1);
-        }
+        const float2 u = staged[(2 * r) * 32 * WARPS];
+        const float2 v = staged[(2 * r + 1) * 32 * WARPS];
         store_row(p, Uout, plane, o, make_float2(u.x + d0.x, u.y + d1.x),
                   make_float2(v.x + d0.y, v.y + d1.y));
     }
 }
 
 // A region of 64 columns x VS * WARPS rows, its coefficients loaded straight
-// into registers.  COH: the planes and U were written earlier in the launch.
-// su: the block's flow stage (COH: none).
-template <int VS, int WARPS, bool COH>
+// into registers.  su: the block's flow stage.
+template <int VS, int WARPS>
 __device__ __forceinline__ void sor_region(int bx, int by, int f, int w, int h, int pitch,
                                            const float *__restrict__ Uinb,
                                            float *__restrict__ Uoutb, size_t ufs, size_t plane,
@@ -387,9 +361,9 @@ __device__ __forceinline__ void sor_region(int bx, int by, int f, int w, int h, 
 #pragma unroll
         for (int r = 0; r < VS; ++r) {
             const float *c = c0 + r * pitch;
-            const float2 i1 = ldf2<COH>(c + kCI11 * pl), i2 = ldf2<COH>(c + kCI22 * pl);
-            const float2 a = ldf2<COH>(c + kCA12 * pl), g = ldf2<COH>(c + kCAS * pl);
-            const float2 b1 = ldf2<COH>(c + kCB1 * pl), b2 = ldf2<COH>(c + kCB2 * pl);
+            const float2 i1 = ld2(c + kCI11 * pl), i2 = ld2(c + kCI22 * pl);
+            const float2 a = ld2(c + kCA12 * pl), g = ld2(c + kCAS * pl);
+            const float2 b1 = ld2(c + kCB1 * pl), b2 = ld2(c + kCB2 * pl);
             s.i11[r][0] = i1.x, s.i11[r][1] = i1.y;
             s.i22[r][0] = i2.x, s.i22[r][1] = i2.y;
             s.a12[r][0] = a.x, s.a12[r][1] = a.y;
@@ -399,8 +373,8 @@ __device__ __forceinline__ void sor_region(int bx, int by, int f, int w, int h, 
         }
         const float *ca = c0 + kCAS * pl;
         const float2 z = make_float2(0.0f, 0.0f);
-        const float2 gu = first ? z : ldf2<COH>(ca - pitch);
-        const float2 gd = last ? z : ldf2<COH>(ca + VS * pitch);
+        const float2 gu = first ? z : ld2(ca - pitch);
+        const float2 gd = last ? z : ld2(ca + VS * pitch);
         as[0][0] = gu.x, as[0][1] = gu.y;
         as[VS + 1][0] = gd.x, as[VS + 1][1] = gd.y;
     } else {
@@ -412,7 +386,7 @@ __device__ __forceinline__ void sor_region(int bx, int by, int f, int w, int h, 
                 const int gx = p.gx + q;
                 const bool in = gx >= 0 && gx < w && gy >= 0 && gy < h;
                 const float *c = cf + (in ? gy * pitch + gx : 0);
-                auto ld = [&](int k) { return in ? ldf<COH>(c + k * pl) : 0.0f; };
+                auto ld = [&](int k) { return in ? c[k * pl] : 0.0f; };
                 as[r + 1][q] = ld(kCAS);
                 if (r >= 0 && r < VS) {
                     s.i11[r][q] = ld(kCI11);
@@ -424,14 +398,14 @@ __device__ __forceinline__ void sor_region(int bx, int by, int f, int w, int h, 
         }
     }
     float2 *slot = su + threadIdx.x;
-    if (!COH) stage_flow(p, Uin, plane, smem_u32(slot));
+    stage_flow(p, Uin, plane, smem_u32(slot));
     clear_ends(ends);
     if (inside)
         edge_weights<VS, true>(s, as, lane, first, last, p.gx, p.gy, w, h);
     else
         edge_weights<VS, false>(s, as, lane, first, last, p.gx, p.gy, w, h);
     sor_sweeps<VS, WARPS>(s, ends, lane, wp, (p.gx + p.gy) & 1, n_half, omega);
-    store_flow(p, s, Uin, Uoutb + (size_t)f * ufs, plane, COH ? nullptr : slot);
+    store_flow(p, s, Uoutb + (size_t)f * ufs, plane, slot);
 }
 
 template <int VS>
@@ -443,8 +417,8 @@ var_sor_kernel(int w, int h, int pitch, const float *__restrict__ Uinb,
     chain_begin();
     extern __shared__ float2 su[];
     __shared__ StripEnds<kVWarps> ends;
-    sor_region<VS, kVWarps, false>(blockIdx.x, blockIdx.y, blockIdx.z, w, h, pitch, Uinb, Uoutb,
-                                   ufs, plane, coefb, cfs, R, n_half, omega, ends, su);
+    sor_region<VS, kVWarps>(blockIdx.x, blockIdx.y, blockIdx.z, w, h, pitch, Uinb, Uoutb, ufs,
+                            plane, coefb, cfs, R, n_half, omega, ends, su);
 }
 
 // The 64 x 64 regions of several groups' levels in one launch.
@@ -456,9 +430,9 @@ seg_var_sor_kernel(const __grid_constant__ SegTable<SegSor> tab)
     int b;
     const SegSor &a = seg_of(tab, b);
     const int r = b / a.gx;
-    sor_region<kVS, kVWarps, false>(b % a.gx, r % a.gy, r / a.gy, a.w, a.h, a.pitch, a.Uin,
-                                    a.Uout, a.ufs, a.plane, a.coef + kCoefShift, a.cfs, a.R,
-                                    a.n_half, a.omega, ends, su);
+    sor_region<kVS, kVWarps>(b % a.gx, r % a.gy, r / a.gy, a.w, a.h, a.pitch, a.Uin, a.Uout,
+                             a.ufs, a.plane, a.coef + kCoefShift, a.cfs, a.R, a.n_half, a.omega,
+                             ends, su);
 }
 
 // Bounded wait for the mbarrier phase with the given parity: at most
@@ -788,10 +762,10 @@ __device__ __forceinline__ void stage_window(const Windows<WH> &m, const T *__re
     }
 }
 
-// The flow from its planes (an aligned pair where the window lies inside).
+// The flow of the pairs from its planes.
 template <int KI>
 __device__ __forceinline__ void load_planes(const float *__restrict__ a, size_t plane, int pitch,
-                                            bool inside, const int (&c0)[KI], const int (&c1)[KI],
+                                            const int (&c0)[KI], const int (&c1)[KI],
                                             const int (&cy)[KI], pair_t (&u)[KI],
                                             pair_t (&v)[KI])
 {
@@ -935,7 +909,7 @@ __device__ __forceinline__ void var_coeff_body(
     const bool inside = tx >= 2 && ty >= 2 && tx + 66 <= w && ty + TH + 2 <= h;
     stage_window<WH, NT, 3>(m, I1, w, h, pitch, tx - 2, ty - 2, inside,
                             [&](auto &c0, auto &c1, auto &cy, auto &u, auto &v) {
-                                load_planes<3>(U, plane, pitch, inside, c0, c1, cy, u, v);
+                                load_planes<3>(U, plane, pitch, c0, c1, cy, u, v);
                             });
     __syncthreads();
     const int gx = tx + lane, pl = (int)plane;
@@ -1136,7 +1110,7 @@ var_level_kernel(const T *__restrict__ I0b, const T *__restrict__ I0xb,
             m, I1, w, h, pitch, rx0 - 2, ry0 - 2, inside,
             [&](auto &c0, auto &c1, auto &cy, auto &u, auto &v) {
                 if (k == 0) {
-                    load_planes<KI>(Ua + (size_t)f * ufs, plane, pitch, inside, c0, c1, cy, u, v);
+                    load_planes<KI>(Ua + (size_t)f * ufs, plane, pitch, c0, c1, cy, u, v);
                     return;
                 }
                 const float4 *src = xch + ((k - 1) & 1) * xch_n + (size_t)f * pk_fs;
