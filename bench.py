@@ -9,7 +9,10 @@ search, densification, variational refinement) over every window of the
 stream, with all events resident in HBM before the timed region (715 MB
 of events per step, larger than the 129 MB L2).
 
-Prints one JSON line (rank 0).  `value` is one window per call through the
+Prints one JSON line (rank 0): the contract's keys whole and the other sections'
+main figures, 8 KB at most, so that a reader of a bounded tail gets all of it.
+The full record (every stage, run and setting) goes to standard error, one line
+behind the word `details`.  `value` is one window per call through the
 pipelined ebof_process_window_async (a window's front end overlaps the
 previous window's flow levels; CUDA events on the caller's stream, the step
 closed by ebof_stream_join); `in_order` the same windows through
@@ -297,6 +300,39 @@ class ClockSampler:
         return {"sm_mhz": float(np.median(sm)) if sm else None,
                 "sm_max_mhz": max(mx) if mx else None, "reasons": sorted(reasons),
                 "samples": len(sm)}
+
+
+# ---------------------------------------------------------------- the line
+LINE_LIMIT = 8000  # bytes
+CONTRACT_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                 "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "clocks",
+                 "e2e", "gpu_launches", "cpu_baseline")
+
+
+def _brief(v, depth):
+    """The scalars and short texts of a record, down to `depth` dicts below it."""
+    return {k: _brief(x, depth - 1) if isinstance(x, dict) else x for k, x in v.items()
+            if (depth > 0 if isinstance(x, dict) else
+                not isinstance(x, (list, tuple)) and len(str(x)) <= 100)}
+
+
+def headline(record, limit=LINE_LIMIT):
+    """The JSON line of a full record: contract keys as they are, the other
+    sections' scalars, the longest of those left out while the line is longer
+    than `limit`."""
+    out = {k: v if k in CONTRACT_KEYS or not isinstance(v, dict) else _brief(v, 1)
+           for k, v in record.items()}
+    for k in ("stage_share", "stage_ms_per_frame", "stage_roofline"):
+        for section in ("roofline", "batched"):
+            if isinstance(out.get(section), dict):
+                out[section].pop(k, None)
+    left = sorted((k for k in out if k not in CONTRACT_KEYS and k != "roofline"),
+                  key=lambda k: len(json.dumps(out[k])))
+    line = json.dumps(out)
+    while len(line) > limit and left:
+        del out[left.pop()]
+        line = json.dumps(out)
+    return line
 
 
 # ---------------------------------------------------------------- roofline
@@ -1374,7 +1410,8 @@ def main():
             "gpu_launches": int(launches),
             "clocks": clocks,
         }
-        print(json.dumps(out), flush=True)
+        print("details " + json.dumps(out), file=sys.stderr, flush=True)
+        print(headline(out), flush=True)
     s.close()
     if world > 1:
         dist.destroy_process_group()
