@@ -337,9 +337,10 @@ def headline(record, limit=LINE_LIMIT):
 
 # ---------------------------------------------------------------- roofline
 def algorithmic_bytes_per_launch(stage, level, geo, n_events_per_window, P):
-    """Algorithmic bytes of ONE launch of a stage for one window: each
-    kernel's inputs read once and outputs written once, by the per-stage
-    formulas below.  geo: [(w, h, npx, npy)] per pyramid level."""
+    """Algorithmic bytes of ONE launch of a stage for one window: its inputs
+    read once and outputs written once, in the method's plain layout (int32
+    column distances, seven coefficient planes with both edge weights).  geo:
+    [(w, h, npx, npy)] per pyramid level."""
     if level >= 0:
         w, h, npx, npy = geo[level]
         Pl, npl = w * h, npx * npy
@@ -358,6 +359,19 @@ def algorithmic_bytes_per_launch(stage, level, geo, n_events_per_window, P):
     }
     f = per.get(stage)
     return float(f()) if f else 0.0
+
+
+def kernel_io_bytes_per_launch(stage, level, geo, n_events_per_window, P):
+    """What the present kernels read and write, each byte once: the plain
+    layout's bytes but for the column pass, whose words hold 32 rows of a column
+    in 8 bytes, and the coefficients, of which one plane holds the weights of
+    both edges (six planes in all)."""
+    Pl = geo[level][0] * geo[level][1] if level >= 0 else 0
+    own = {"edt_cols": 1.25 * P,           # E_df bytes in, words out
+           "edt_rows_surface": 4.25 * P,   # words in, float intensity out
+           "var_coeff": 48.0 * Pl,         # U, I1, I0, I0x, I0y in; 6 planes out
+           "var_sor": 40.0 * Pl}           # 6 planes and U in, U out
+    return own.get(stage, algorithmic_bytes_per_launch(stage, level, geo, n_events_per_window, P))
 
 
 PER_LEVEL = ("pyramid", "patch_search", "densify", "var_coeff", "var_sor")
@@ -1136,7 +1150,7 @@ def main():
     dom_ms, dom_launches = (prof0 if level == 0 else profn)[dom]
     gl = geo_levels(prm)
     n_ev_win = int(off[-1]) / nwin
-    per_launch_bytes = algorithmic_bytes_per_launch(dom, level, gl, n_ev_win, P)
+    per_launch_bytes = kernel_io_bytes_per_launch(dom, level, gl, n_ev_win, P)
     per_launch_s = dom_ms / 1000.0 / max(dom_launches, 1)
     achieved = per_launch_bytes / per_launch_s / 1e9
     peak, peak_kind = load_peaks()
@@ -1159,7 +1173,8 @@ def main():
         "stage_ms_per_frame_by_level": by_level,
         "stage_timing": "CUDA events around each stage's launches on the caller's stream "
                         "(eager launches, gaps included; the graph-replayed path times "
-                        "the whole window only)"})
+                        "the whole window only); a level refined in one launch appears "
+                        "under var_sor whole, without var_coeff launches"})
     # the whole path at the pipelined rate: every stage's algorithmic bytes
     # per frame times the frames per second of `value`
     allb = roofline["stage_roofline"].get("all stages", {}).get("bytes_per_frame")

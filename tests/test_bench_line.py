@@ -64,3 +64,22 @@ def test_sections_go_before_the_contract_does(bench):
     out = json.loads(bench.headline(rec))
     assert all(out[k] == rec[k] for k in bench.CONTRACT_KEYS) and "roofline" in out
     assert len(json.dumps(out)) <= bench.LINE_LIMIT
+
+
+def test_kernel_io_counts_what_the_kernels_move(bench):
+    """Against the sources: six coefficient planes, one flow and the four images
+    of a coefficient launch, and 8 bytes of column words per 32 rows."""
+    import re
+    src = open(os.path.join(ROOT, "paper_2112_10591_gb300", "csrc", "k_var.cu")).read()
+    names = re.search(r"enum \{ (kCI11[^}]*), kCPlanes \};", src).group(1)
+    planes = len(names.split(","))
+    geo = [(1280, 720, 318, 178), (640, 360, 158, 88)]
+    P = 1280 * 720
+    io = lambda s, l: bench.kernel_io_bytes_per_launch(s, l, geo, 275_000, P)
+    assert io("var_coeff", 1) == (8 + 4 * 4 + 4 * planes) * 640 * 360
+    assert io("var_sor", 0) == (4 * planes + 8 + 8) * P
+    assert io("edt_cols", -1) == P + 8 * P / 32
+    assert io("edt_rows_surface", -1) == 8 * P / 32 + 4 * P
+    # the other stages have one layout
+    for s, l in (("scatter", -1), ("patch_search", 0), ("densify", 1), ("flow_out", -1)):
+        assert io(s, l) == bench.algorithmic_bytes_per_launch(s, l, geo, 275_000, P) > 0
