@@ -97,7 +97,9 @@ struct FlowParams {
     size_t level_n;
     bool chained;  // the search's launch is behind a kernel of the same chain
 };
-constexpr int kLevelBlocks = 266;  // most regions of a one-launch refinement
+// most regions of a one-launch refinement: 1.75 an SM of 152 (the launch asks the
+// device; this bounds the packets that a stream or group holds)
+constexpr int kLevelBlocks = 266;
 constexpr int kLevelCtl = 4;
 // level_n for a stream or group of up to `frames` frames a call.
 size_t level_packets(const Geometry &geo, int var_sor, int cluster_max, int frames);

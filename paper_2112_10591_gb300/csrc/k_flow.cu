@@ -1102,11 +1102,11 @@ void launch_patch_search(const void *I0, const void *I0x, const void *I0y, const
                               up, up_frame_stride, frames, fp, err, st);
 }
 
-// Blocks of 32 x 8 from which two pixels a thread are faster (16 a SM): 40
+// Blocks of 32 x 8 an SM from which two pixels a thread are faster: 40
 // windows of 1280 x 720 10.12 -> 9.82 ms; with a line at 400 blocks 641 x 479
 // took 588 us against 583, its two levels of 300 and 1260 blocks left with too
 // few warps.
-constexpr long long kDensePairBlocks = 2432;
+constexpr long long kDensePairBlocksPerSM = 16;
 
 void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_frame_stride,
                     const float *up, size_t up_frame_stride, float *U, size_t u_frame_stride,
@@ -1122,7 +1122,7 @@ void launch_densify(const void *I0, const void *I1, const Level &lv, size_t pyr_
     const uint32_t magic = stride_magic(stride);
     const bool chained = fp.chained || lv.npx * lv.npy > 0;  // the search is launched
     const bool two = nc >= 2 && nc <= 4 && nc * stride == fp.ps && stride % 2 == 0 &&
-                     (long long)grd.x * grd.y * frames >= kDensePairBlocks;
+                     (long long)grd.x * grd.y * frames >= kDensePairBlocksPerSM * sm_count();
     if (two) grd.y = (lv.h + 15) / 16;
 #define EBOF_DENSE2(T, N)                                                                        \
     do {                                                                                         \
