@@ -1051,9 +1051,9 @@ bool fused_supported(const ebof_group *g, int mode)
 // per kernel instance where groups differ in storage, patch size or lane
 // layout).  Pyramid levels are aligned at the coarsest level (below).
 // Results are those of run_group bit for bit: every kernel body is the
-// group kernel's, and every layout that differs (EDT rows of one warp, the
-// tile form of the coefficients, the even-halo SOR regions) gives the same
-// values.
+// group kernel's, and every layout that differs (EDT rows of one warp,
+// coefficient tiles of 16 rows, one densified pixel a thread, SOR regions of
+// 64 x 64 loaded by their threads) gives the same values.
 void build_fused_plan(ebof_multigroup *m, FusedPlan &P, int mode)
 {
     const int nsm = [] {

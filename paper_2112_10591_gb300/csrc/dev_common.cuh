@@ -14,8 +14,8 @@ __device__ __forceinline__ int clampi(int v, int lo, int hi) { return min(max(v,
 // different kernels; these intrinsics are never fused or split, so an
 // expression written with them rounds the same way in every kernel that
 // evaluates it.  The variational refinement's per-pixel arithmetic and the
-// bilinear sample are written with them, so that every kernel form (tile,
-// column walk, SOR region layouts) gives the same values bit for bit.
+// bilinear sample are written with them, so that every kernel form (tiles,
+// the one-launch refinement, SOR region layouts) gives the same values bit for bit.
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
@@ -73,9 +73,9 @@ __device__ __forceinline__ pair_t fmul2(pair_t a, pair_t b)
     return d;
 }
 
-// The compiler fuses a packed
-// product into a packed sum that follows it (whatever the rounding suffix), so
-// a product whose rounding matters is added by scalar operations.
+// The compiler fuses a packed product into a packed sum that follows it
+// (whatever the rounding suffix), so a product whose rounding matters is added by
+// scalar operations.
 __device__ __forceinline__ pair_t fadd2(pair_t a, pair_t b)
 {
     pair_t d;

@@ -7,15 +7,15 @@
 // system (data and gradient-constancy terms normalised, weights lagged at
 // dU = 0): omega/a11, omega/a22 (the SOR relaxation factor folded into the
 // inverted diagonal), a12, b1, b2 and the smoothness weight, as six planes.
-// Everything is done on pairs of adjacent pixels with packed FP32 operations.
+// Everything is done on pairs of pixels, half a row or 32 columns apart, with
+// packed FP32 operations.
 // What bounds it: issue slots (a scalar form took 340 instructions a pixel row
 // of 32) and, once those are halved, the latency of the flow and the image's
 // taps, which is why the rows are staged by a block of independent threads: a
 // warp that walks its columns down with the rows in registers needs as few
-// instructions but only four warps a scheduler fit.  Measured in a graph,
-// against the scalar column walk (levels from 1024 px) and scalar 32x12 tiles:
-// 1280x720 14.3 -> 12.7 us for one frame, 103 -> 89 for eight (pairs in a
-// column walk: 12.1 and 92); 640x360 5.8 -> 5.0 and 34 -> 25; 160x90 3.1 -> 2.9.
+// instructions but only four warps a scheduler fit.  Measured (the first form:
+// scalar, a column walk from 1024 px and 32x12 tiles below): 1280x720 14.3 -> 13.0
+// us for one frame, 103 -> 85 for eight; 640x360 34 -> 24 for eight.
 //
 // SOR: one block owns a 64x64 region and refines the flow of its
 // (64 - 2R)^2 interior, R = 2 * sweeps - 1.  It loads the region's linear
@@ -35,9 +35,8 @@
 // first half sweep (whose neighbours are 0) runs without an exchange, the edge
 // weights are rebuilt from one plane, regions begin on odd columns that every
 // buffer aligns to 8 bytes, and the interior's flow is fetched behind the
-// sweeps.  Measured per 1280x720 launch on a GB300, inside a graph, against
-// the scalar form of 7 planes and a full exchange: 18.3 -> 15.6 us for one
-// frame, 165 -> 126 us for eight.
+// sweeps.  Measured per 1280x720 launch, against the scalar form of 7 planes
+// and a full exchange: 18.3 -> 16.4 us for one frame, 165 -> 118 us for eight.
 //
 // var_sor_tma_kernel: the same regions in a persistent grid (one block per
 // SM).  One thread loads each region's planes into shared memory with a
@@ -46,10 +45,10 @@
 // block's next region is issued and runs during the sweeps.  The box starts at
 // the region's first column rounded down to the 16-byte rule of tensor copies
 // and is 4 columns wider; elements outside the level are filled with zero, as
-// the direct loads do, so both kernels give the same result.  It needs at
-// least two regions an SM to hide a copy: measured against the direct form (in
-// a graph, 7 planes) 6.8 vs 6.1 us for 112 regions, 10.4 vs 9.8 for 154, 14.7
-// vs 15.6 for 448, 27.0 vs 30.4 for 896, 101 vs 126 for 3584.
+// the direct loads do, so both kernels give the same result.  With one region an
+// SM there is no copy to hide.  Measured against the direct form: 11.2 us both for
+// 168 regions, 11.4 and 12.1 for 224, 14.7 and 16.4 for 448, 25.8 and 30.7 for
+// 896, 47.5 and 63.4 for 1792, 89.6 and 117.7 for 3584.
 #include "dev_common.cuh"
 #include "ebof_internal.cuh"
 #include "profiler.cuh"
@@ -462,7 +461,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
 // comes by one tensor copy instead of eight 8-byte copies a thread, and the
 // output's loads and stores stand without branches between them.  The copies
 // write a buffer only after the barrier that follows its last reads.
-// 1280 x 720, ten half sweeps: one frame 22.8 -> 18.8 us, eight 129 -> 101.
+// 1280 x 720, ten half sweeps, against a region a block: one frame 16.4 -> 14.6
+// us, eight 118 -> 90.
 __global__ void __launch_bounds__(kVThreads, 1)
 var_sor_tma_kernel(const __grid_constant__ CUtensorMap cmap,
                    const __grid_constant__ CUtensorMap umap, int w, int h, int pitch,
@@ -894,8 +894,8 @@ __device__ __forceinline__ PairSystem pair_system(const Windows<WH> &m, int e, i
 // x TH rows and writes its pixels' systems, two a thread and step, 32 columns
 // apart: every access of a warp is to 32 columns side by side, from any column
 // (adjacent pixels a pair want odd ones, one tile more at widths of 64 k).
-// Bound by L1 (78 % of its cycles) and issue (59 %): eight frames of 1280 x 720
-// 93 us a launch, 354 MB of planes 50.
+// Bound by L1 (77 % of its cycles) and issue (69 %): eight frames of 1280 x 720
+// 85 us a launch, 354 MB of planes 50.
 template <int TH, int NT, typename T>
 __device__ __forceinline__ void var_coeff_body(
     float *smem, const T *__restrict__ I0, const T *__restrict__ I0x, const T *__restrict__ I0y,
