@@ -494,6 +494,7 @@ seg_edt_cols_kernel(const __grid_constant__ SegTable<SegEdtCols> tab)
 constexpr int kNoColumn = 1 << 30;
 
 constexpr int kRowsPerBlock = 4;                  // rows (warps) per block
+constexpr int kWarpsLongRow = 16;                 // warps of a long row
 constexpr int kRowLoads = 4;                      // pixels in flight per lane
 constexpr size_t kRowsSmemCap = 200 * 1024;       // bytes; 16384-px rows fit
 
@@ -694,7 +695,7 @@ __device__ __forceinline__ void edt_rows_surface_body(
 }
 
 template <int WPR, typename T>
-__global__ void __launch_bounds__(32 * kRowsPerBlock)
+__global__ void __launch_bounds__(32 * (WPR > kRowsPerBlock ? WPR : kRowsPerBlock))
 edt_rows_surface_kernel(const int32_t *__restrict__ g, int gpitch, size_t gfs, int W, int H,
                         int rows_per_block, SurfaceMap sm, int32_t *__restrict__ D_dense,
                         float *__restrict__ S_dense, T *__restrict__ I0, int ipitch, size_t ifs)
@@ -706,12 +707,13 @@ edt_rows_surface_kernel(const int32_t *__restrict__ g, int gpitch, size_t gfs, i
 
 // The row pass from distances that lie in one of its results (no restrict: it
 // writes where it has read).
-__global__ void __launch_bounds__(32 * kRowsPerBlock)
+template <int WPR>
+__global__ void __launch_bounds__(32 * WPR)
 edt_rows_inplace_kernel(const int32_t *g, int W, int H, SurfaceMap sm, int32_t *D_dense,
                         float *S_dense)
 {
-    edt_rows_surface_body<kRowsPerBlock, true, float>(g, W, 0, W, H, 1, sm, D_dense, S_dense,
-                                                      nullptr, 0, 0, blockIdx.x, 0);
+    edt_rows_surface_body<WPR, true, float>(g, W, 0, W, H, 1, sm, D_dense, S_dense, nullptr, 0, 0,
+                                            blockIdx.x, 0);
 }
 
 template <typename T>
@@ -809,22 +811,29 @@ size_t edt_rows_smem(int W, int rows) { return (size_t)rows * rows_smem_bytes(W)
 
 // Warps per row: one for batches (fewest instructions per frame), four for
 // single windows (one or two frames per launch), one row per block, to shorten
-// a row's chain.
-int edt_rows_wpr(int frames) { return frames > 2 ? 1 : kRowsPerBlock; }
+// a row's chain; sixteen for long rows that leave each an SM (stand-alone, against
+// four warps: 2048x16 16.5 -> 10.4 us, 4096x150 54.6 -> 20.6, 8192x16 86 -> 29,
+// 16384x1 109 -> 53, 16384x150 133 -> 55).
+int edt_rows_wpr(int W, int H, int frames)
+{
+    if (frames > 2) return 1;
+    return W >= 2048 && (long long)H * frames <= sm_count() ? kWarpsLongRow : kRowsPerBlock;
+}
 
 template <typename T>
 void edt_rows_t(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
                 const SurfaceMap &sm, int32_t *D_dense, float *S_dense, T *I0, int i_pitch,
                 size_t i_frame_stride, int frames, bool chained, cudaStream_t st)
 {
-    const int wpr = edt_rows_wpr(frames);
+    const int wpr = edt_rows_wpr(W, H, frames);
     // one warp a row: four rows per block, fewer where a row's shared memory
     // is large; the wider layout: one row per block
     const int rows = wpr == 1 ? edt_rows_block_rows(W) : 1;
     const size_t smem = edt_rows_smem(W, rows);
     dim3 grd((H + rows - 1) / rows, frames);
-    auto kern = wpr == 1 ? edt_rows_surface_kernel<1, T>
-                         : edt_rows_surface_kernel<kRowsPerBlock, T>;
+    auto kern = wpr == 1               ? edt_rows_surface_kernel<1, T>
+                : wpr == kWarpsLongRow ? edt_rows_surface_kernel<kWarpsLongRow, T>
+                                       : edt_rows_surface_kernel<kRowsPerBlock, T>;
     launch_chained(chained, kern, grd, 32 * (wpr == 1 ? rows : wpr), smem, st, g, g_pitch,
                    g_frame_stride, W, H, rows, sm, D_dense, S_dense, I0, i_pitch, i_frame_stride);
 }
@@ -838,8 +847,10 @@ void launch_edt_inplace(const uint8_t *edge, int W, int H, float alpha, int32_t 
                                 st>>>(edge, W, 0, W, H, g, W, 0);
     }
     StageScope sc(kStEdtRows, 1, st);
-    edt_rows_inplace_kernel<<<H, 32 * kRowsPerBlock, edt_rows_smem(W, 1), st>>>(
-        g, W, H, exp_surface(alpha), D_dense, S_dense);
+    const int wpr = edt_rows_wpr(W, H, 1);
+    auto kern = wpr == kWarpsLongRow ? edt_rows_inplace_kernel<kWarpsLongRow>
+                                     : edt_rows_inplace_kernel<kRowsPerBlock>;
+    kern<<<H, 32 * wpr, edt_rows_smem(W, 1), st>>>(g, W, H, exp_surface(alpha), D_dense, S_dense);
 }
 
 static void edt_rows(const int32_t *g, int g_pitch, size_t g_frame_stride, int W, int H,
@@ -908,7 +919,10 @@ void init_front_attributes()
     opt_in((const void *)edt_rows_surface_kernel<kRowsPerBlock, float>);
     opt_in((const void *)edt_rows_surface_kernel<1, __half>);
     opt_in((const void *)edt_rows_surface_kernel<kRowsPerBlock, __half>);
-    opt_in((const void *)edt_rows_inplace_kernel);
+    opt_in((const void *)edt_rows_surface_kernel<kWarpsLongRow, float>);
+    opt_in((const void *)edt_rows_surface_kernel<kWarpsLongRow, __half>);
+    opt_in((const void *)edt_rows_inplace_kernel<kRowsPerBlock>);
+    opt_in((const void *)edt_rows_inplace_kernel<kWarpsLongRow>);
     opt_in((const void *)edt_cols_kernel<false>);
     opt_in((const void *)edt_cols_kernel<true>);
     opt_in((const void *)seg_edt_cols_kernel);
