@@ -86,7 +86,9 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 
 // A sum held as three floats h + l + m, each the rounding errors of the one
 // before: only m's additions lose anything, 2^-24 of 2^-48 of the sum.  Every
-// operation rounds once and is never fused, so the error terms are exact.
+// operation rounds once and is never fused, so the error terms are exact.  FP32's
+// range holds the squares: pixels are at most 2^31 (128 times the 2^24 at which a
+// float stops counting), and what falls below 2^-149 is that small in the sum.
 struct TripleSum {
     float h = 0.0f, l = 0.0f, m = 0.0f;
     __device__ __forceinline__ void add(float x)
