@@ -311,7 +311,8 @@ ebof_status ebof_stream_sync(ebof_stream *s, ebof_window_stats *out, int32_t n_o
  * columns' edge bits and nearest edge rows).  It may be one of the results or
  * overlap them: column distances are then kept in a result until its rows are
  * written, which costs one pass over width*height int32 more.  d_edge may
- * overlap a result, but not d_scratch.
+ * overlap a result, but not d_scratch, and, where d_scratch overlaps a result,
+ * not every result.
  * d_edt [H][W] required; d_surface [H][W] optional.
  * No per-stream state is used. */
 ebof_status ebof_edt(const uint8_t *d_edge, int32_t width, int32_t height, int32_t *d_scratch,
